@@ -84,8 +84,9 @@ typedef struct cp_stats {
     int64_t top_survivors;    /* facets left for the dual union-find after pruning */
     int64_t h0_roots;         /* local minima (roots of the H0 forest) */
     int64_t top_roots;        /* top cells left as roots of the dual forest */
-    int64_t h0_rounds;        /* rounds of the H0 union-find */
-    int64_t top_rounds;       /* rounds of the dual union-find */
+    int64_t h0_rounds;        /* passes of the H0 union-find: 1 (0: no survivors), or its rounds
+                                 (slab split, CP_TUNE_UF_VARIANT = 1, cross-pruning) */
+    int64_t top_rounds;       /* likewise of the dual union-find */
     int64_t pairs;            /* reported pairs (nonzero persistence + essential) */
     uint32_t status;          /* raw device status bits */
     uint32_t mst_rounds;      /* Borůvka rounds (CP_TUNE_UF_VARIANT = 1), else 0 */
@@ -428,7 +429,8 @@ int cubical_persistence_backward_noalloc(const cp_pair *d_pairs, int64_t n_pairs
 
 /*
  * Union-find trace of the last forward call that used this workspace (waits
- * for `stream`): for round i (up to min(cap, 48) rounds, plus the final
+ * for `stream`; the merge tree's single pass counts as one round without
+ * times): for round i (up to min(cap, 48) rounds, plus the final
  * empty one), h_active[i] = survivors still unresolved at its start and
  * h_us[i] = microseconds since the start of round 0.  dual = 0 for H0, 1 for
  * the top dimension.  Returns the number of entries or a CP_ERR_* code.
@@ -499,13 +501,14 @@ int cubical_persistence_debug_wait_timeout(void *d_workspace, size_t ws_bytes, i
  *                        alone while the others wait, until more than twice
  *                        as many enter one (0 .. 1024; 0: every round on the
  *                        whole grid; default 16).  Same pairs.
- *   CP_TUNE_UF_VARIANT   0 (default): the elder-rule union-find runs in
- *                        reservation rounds over every survivor; 1: Borůvka's
- *                        minimum spanning forest of the survivor graph first
- *                        (the survivors the union-find commits), then the
- *                        rounds over the forest's edges alone.  Same pairs.
- *                        Calls with H1 or with cross-pruning of images keep
- *                        0.  Read when the workspace is sized: set it before
+ *   CP_TUNE_UF_VARIANT   0 (default): the elder-rule union-find is a merge
+ *                        tree that takes the survivors unsorted, in one pass;
+ *                        1: the survivors are sorted, Borůvka's minimum
+ *                        spanning forest of the survivor graph is built (the
+ *                        survivors the union-find commits), then reservation
+ *                        rounds run over the forest's edges alone.  Same
+ *                        pairs.  Calls with H1 keep 0; cross-pruning of images
+ *                        runs reservation rounds over every sorted survivor.  Read when the workspace is sized: set it before
  *                        the _workspace_size call.
  * cp_set_tuning returns CP_OK or CP_ERR_ARG; cp_get_tuning the value or -1.
  * The autotuner in the Python package picks these per GPU and shape.

@@ -1,7 +1,8 @@
 // C-ABI entry points: argument checks, workspace layout, lookup-table set-up
 // and the enqueueing of the pipeline
-//   init -> K1 prune -> K2 sort (H0) -> K3 H0 union-find (+ 2D cross-pruning)
-//        -> K2 sort (dual) -> K3 dual union-find -> essential pairs
+//   init -> K1 prune -> root walks -> K3 merge trees of both lists -> essential pairs
+//        (slab split, Borůvka variant: K2 sort of both lists -> K3 rounds; 2D
+//        cross-pruning: sort and rounds of H0, then of the dual)
 //        [-> H1 of the volumes: columns, sort, reduction, pairs]
 //        -> K2 sort (pairs, canonical order) -> gather.
 #include <algorithm>
@@ -90,6 +91,7 @@ struct Plan {
     size_t o_ctr, o_uf0, o_uft, o_s0, o_st, o_salt, o_age0, o_res0, o_aget, o_rest;
     size_t o_act0, o_act1, o_yn, o_on, o_na0, o_na1, o_nb0, o_nb1, o_pairs, o_pvals, o_pvalt, o_hist, o_status;
     size_t o_hist2, o_status2;
+    size_t o_node0, o_nodet;  // merge-tree nodes
     // H1 of the volumes (calls that ask for it): see H1Bufs
     bool h1 = false;
     uint32_t h1_mcap = 0, h1_neg = 0, h1_posq = 0;
@@ -220,6 +222,8 @@ int make_plan(int n_items, const int32_t* ndims, const int64_t* dims, const floa
     P.o_res0 = take(sizeof(uint64_t) * P.cap_r0);
     P.o_aget = take(sizeof(uint64_t) * P.cap_rt);
     P.o_rest = take(sizeof(uint64_t) * P.cap_rt);
+    P.o_node0 = take(sizeof(TreeNode) * P.cap_r0);
+    P.o_nodet = take(sizeof(TreeNode) * P.cap_rt);
     P.o_act0 = take(sizeof(uint32_t) * P.cap_big);
     P.o_act1 = take(sizeof(uint32_t) * P.cap_big);
     P.o_yn = take(sizeof(uint32_t) * P.cap_s);
@@ -370,24 +374,32 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
     StageRanges nv;
     nv.next("cp.prune");
     CP_TRY(cudaMemsetAsync(ctr, 0, sizeof(Counters), s));
-    CP_TRY(launch_init(P.tab, ctr, uft, aget, rest, s));
+    // the merge tree takes both lists at once; the slab split, the Borůvka
+    // variant and cross-pruning of images need the sorted lists and the rounds
+    const bool joint = P.tab.n2d == 0 || !P.tab.cross2d;
+    const bool tree = joint && P.slabs == 0 && !P.boruvka;
+    TreeNode* node0 = tree ? at<TreeNode>(ws, P.o_node0) : nullptr;
+    TreeNode* nodet = tree ? at<TreeNode>(ws, P.o_nodet) : nullptr;
+    CP_TRY(launch_init(P.tab, ctr, uft, aget, rest, nodet, s));
     mark(0, s);
+    PruneOuts po;
+    po.uf0 = uf0;
+    po.uft = uft;
+    po.s0 = s0;
+    po.st = st;
+    po.age0 = age0;
+    po.res0 = res0;
+    po.aget = aget;
+    po.rest = rest;
+    po.node0 = node0;
+    po.nodet = nodet;
+    po.cap_s = P.cap_s;
+    po.cap_r0 = P.cap_r0;
+    po.cap_rt = P.cap_rt;
+    po.ctr = ctr;
+    po.n_uf0 = uint32_t(P.ntot);
+    po.n_uft = uint32_t(P.ttot);
     if (prune_only) {
-        PruneOuts po;
-        po.uf0 = uf0;
-        po.uft = uft;
-        po.s0 = s0;
-        po.st = st;
-        po.age0 = age0;
-        po.res0 = res0;
-        po.aget = aget;
-        po.rest = rest;
-        po.cap_s = P.cap_s;
-        po.cap_r0 = P.cap_r0;
-        po.cap_rt = P.cap_rt;
-        po.ctr = ctr;
-        po.n_uf0 = uint32_t(P.ntot);
-        po.n_uft = uint32_t(P.ttot);
         CP_TRY(launch_prune(P.tab, po, P.tma, s));
         mark(1, s);
         return CP_OK;
@@ -418,21 +430,6 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
         CP_TRY(cudaMemsetAsync(hb.pos_q, 0, sizeof(uint32_t) * P.h1_words, s));
     }
 
-    PruneOuts po;
-    po.uf0 = uf0;
-    po.uft = uft;
-    po.s0 = s0;
-    po.st = st;
-    po.age0 = age0;
-    po.res0 = res0;
-    po.aget = aget;
-    po.rest = rest;
-    po.cap_s = P.cap_s;
-    po.cap_r0 = P.cap_r0;
-    po.cap_rt = P.cap_rt;
-    po.ctr = ctr;
-    po.n_uf0 = uint32_t(P.ntot);
-    po.n_uft = uint32_t(P.ttot);
     CP_TRY(launch_prune(P.tab, po, P.tma, s));
     if (tm) CP_TRY(launch_t_flatten(uf0, tm->items, s));
     mark(1, s);
@@ -486,31 +483,37 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
     };
     // The two lists are independent unless 2D items use cross-pruning (their
     // dual list then waits for the H0 union-find).
-    const bool joint = P.tab.n2d == 0 || !P.tab.cross2d;
+    RootArgs rt = ra;
+    rt.keys = st;
+    rt.d_n = &ctr->n_st;
+    rt.uf = uft;
+    rt.n_nodes = uint32_t(P.ttot);
+    rt.dual = 1;
     if (joint) {
-        // both lists walked, then sorted together (one launch per pass), then
-        // placed side by side; the dual list's scratch sits in the pairs buffer
-        uint64_t* salt2 = reinterpret_cast<uint64_t*>(pairs);
-        uint32_t* raT = reinterpret_cast<uint32_t*>(salt2 + P.cap_s);
-        uint32_t* rbT = raT + P.cap_s;
-        uint32_t* posT = rbT + P.cap_s;
-        RootArgs rt = ra;
-        rt.keys = st;
-        rt.d_n = &ctr->n_st;
-        rt.uf = uft;
-        rt.n_nodes = uint32_t(P.ttot);
-        rt.dual = 1;
-        rt.ra = raT;
-        rt.rb = rbT;
-        rt.pos = posT;
-        rt.sorted_pos = posT;
-        rt.d_n_before = &ctr->n_s0;
         ra.keys = s0;
         ra.d_n = &ctr->n_s0;
         ra.uf = uf0;
         ra.n_nodes = uint32_t(P.ntot);
         ra.dual = 0;
         ra.d_n_before = nullptr;
+    }
+    if (tree) {
+        ra.pos = rt.pos = nullptr;
+        rt.ra = na0;
+        rt.rb = nb0;
+        CP_TRY(launch_roots2(ra, rt, s));
+    } else if (joint) {
+        // both lists walked, then sorted together (one launch per pass), then
+        // placed side by side; the dual list's scratch sits in the pairs buffer
+        uint64_t* salt2 = reinterpret_cast<uint64_t*>(pairs);
+        uint32_t* raT = reinterpret_cast<uint32_t*>(salt2 + P.cap_s);
+        uint32_t* rbT = raT + P.cap_s;
+        uint32_t* posT = rbT + P.cap_s;
+        rt.ra = raT;
+        rt.rb = rbT;
+        rt.pos = posT;
+        rt.sorted_pos = posT;
+        rt.d_n_before = &ctr->n_s0;
         CP_TRY(launch_roots2(ra, rt, s));
         SortBufs two[2] = {sb, sb};
         two[0].keys = s0;
@@ -715,11 +718,27 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
         CP_TRY(launch_uf(P.tab, u, 2, s));
         mark(5, s);
     } else {
-        // both union-finds share one launch and its rounds (the dual list after
-        // the H0 list)
+        // both lists into their merge trees, and the pairs from the trees
         mark(3, s);
         g_ev_joint = true;
-        CP_TRY(launch_uf(P.tab, up, 2, s));
+        TreeArgs ta;
+        ta.l[0] = TreeList{s0, &ctr->n_s0, ra.ra, ra.rb, node0, P.cap_r0};
+        ta.l[1] = TreeList{st, &ctr->n_st, rt.ra, rt.rb, nodet, P.cap_rt};
+        ta.cap = P.cap_s;
+        ta.ctr = ctr;
+        CP_TRY(launch_tree(ta, s));
+        TreeEmitArgs te;
+        te.tab = P.tab;
+        te.node[0] = node0;
+        te.node[1] = nodet;
+        te.n_rids[0] = P.cap_r0;
+        te.n_rids[1] = P.cap_rt;
+        te.h1flags[0] = up[0].h1flags;
+        te.h1flags[1] = up[1].h1flags;
+        te.pairs = pairs;
+        te.pair_cap = P.cap_p;
+        te.ctr = ctr;
+        CP_TRY(launch_tree_emit(te, s));
         mark(4, s);
         mark(5, s);
     }

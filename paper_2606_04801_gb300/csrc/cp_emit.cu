@@ -10,13 +10,15 @@ constexpr int kT = 256;
 
 // One outside vertex per item: the oldest dual vertex (Sec. 3.1), never
 // paired (Appendix A.4); it takes dual root id = item index.
-__global__ void k_init(ItemTable tab, Counters* ctr, uint32_t* uft, uint64_t* aget, uint64_t* rest) {
+__global__ void k_init(ItemTable tab, Counters* ctr, uint32_t* uft, uint64_t* aget, uint64_t* rest,
+                       TreeNode* nodet) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < tab.n) {
         const Item& it = tab.it[i];
         uft[it.toff + it.T] = kTag | uint32_t(i);
         aget[i] = ~0ull;
         rest[i] = 0;
+        if (nodet) nodet[i] = TreeNode{~0ull, uint64_t(i), 0, 0};  // older than every top cell
         ctr->gmin[i] = ~0ull;
     }
     if (i == 0) ctr->n_rt = uint32_t(tab.n);
@@ -203,8 +205,8 @@ cudaError_t launch_loss_backward(const cp_pair* pairs, int64_t n, const int64_t*
 }
 
 cudaError_t launch_init(const ItemTable& tab, Counters* ctr, uint32_t* uft, uint64_t* aget, uint64_t* rest,
-                        cudaStream_t s) {
-    k_init<<<1, kMaxItems, 0, s>>>(tab, ctr, uft, aget, rest);
+                        TreeNode* nodet, cudaStream_t s) {
+    k_init<<<1, kMaxItems, 0, s>>>(tab, ctr, uft, aget, rest, nodet);
     note_launches(1);
     return cudaGetLastError();
 }

@@ -9,6 +9,14 @@
 namespace cp {
 
 // ---- K1 pruning
+// A root of a pruned forest in the merge tree (cp_tree.cu): connected with the
+// older root `parent` by survivors of key at most `key`.  One 32-byte sector.
+struct alignas(32) TreeNode {
+    uint64_t key;     // ~0: connected with nothing older yet
+    uint64_t parent;  // root id
+    uint64_t age;     // smaller is older (the dual's age keys complemented)
+    uint64_t pad;
+};
 struct PruneOuts {
     uint32_t* uf0;   // H0 forest over global vertices
     uint32_t* uft;   // dual forest over global top cells (+ one outside vertex per item)
@@ -18,6 +26,8 @@ struct PruneOuts {
     uint64_t* res0;  // reservation word of each H0 root id
     uint64_t* aget;  // age of each dual root id
     uint64_t* rest;  // reservation word of each dual root id
+    TreeNode* node0; // merge-tree nodes of the roots (then age / res are not written), or nullptr
+    TreeNode* nodet;
     uint32_t cap_s, cap_r0, cap_rt;
     Counters* ctr;
     uint32_t n_uf0, n_uft;  // forest sizes (for the bounds-checked build)
@@ -106,7 +116,7 @@ struct RootArgs {
     int dual;
     uint32_t* ra;                // root id of each survivor's endpoints, by unsorted position
     uint32_t* rb;
-    uint32_t* pos;               // sort payload: the unsorted position
+    uint32_t* pos;               // sort payload: the unsorted position (k_roots2: or nullptr)
     const uint32_t* sorted_pos;  // k_place_roots: the payload after the sort
     const uint32_t* d_n_before;  // dual list after the H0 list: the H0 count (else nullptr)
     uint32_t scratch_cap;
@@ -125,6 +135,32 @@ cudaError_t launch_place_roots(const RootArgs& r, cudaStream_t s);
 // the same rounds.  Two problems share the scratch lists (the pointers of p[0])
 // side by side when both fit, else they run one after the other.
 cudaError_t launch_uf(const ItemTable& tab, const UfParams* p, int nprob, cudaStream_t s);
+
+// ---- K3 as a merge tree (cp_tree.cu)
+struct TreeList {
+    const uint64_t* keys;   // survivor keys, unsorted (ascending order is the list's order)
+    const uint32_t* d_n;
+    const uint32_t* ra;     // root ids of each survivor's endpoints (k_roots2)
+    const uint32_t* rb;
+    TreeNode* node;
+    uint32_t n_rids;        // nodes (bounds-checked build)
+};
+struct TreeArgs {
+    TreeList l[2];          // H0, dual
+    uint32_t cap;           // survivors per list at most
+    Counters* ctr;
+};
+cudaError_t launch_tree(const TreeArgs& a, cudaStream_t s);
+struct TreeEmitArgs {
+    ItemTable tab;
+    const TreeNode* node[2];
+    uint32_t n_rids[2];
+    uint32_t* h1flags[2];   // as UfParams::h1flags
+    cp_pair* pairs;
+    uint32_t pair_cap;
+    Counters* ctr;
+};
+cudaError_t launch_tree_emit(const TreeEmitArgs& a, cudaStream_t s);
 
 // ---- slab decomposition of the union-finds (cp_slab.cu)
 struct SlabCtr {
@@ -255,7 +291,7 @@ int get_h1_solo_cols();
 
 // ---- K4 emission, K5 backward
 cudaError_t launch_init(const ItemTable& tab, Counters* ctr, uint32_t* uft, uint64_t* aget, uint64_t* rest,
-                        cudaStream_t s);
+                        TreeNode* nodet, cudaStream_t s);
 // T-filtration by duality (cp_tfilt.cu), per item by the caller's index.
 struct TDims {
     int ndim;
@@ -291,7 +327,7 @@ cudaError_t launch_backward(const cp_pair* pairs, int64_t n, const float* gb, co
 int device_sm_count();
 // init() run once per device and slot (thread-safe), its result cached: the
 // launch set-up of a kernel (attributes, occupancy-derived grid size).
-enum { kCachePrune3d, kCachePrune2d, kCacheSort, kCacheUf, kCacheRoots, kCacheH1, kCacheBoruvka, kCacheSlots };
+enum { kCachePrune3d, kCachePrune2d, kCacheSort, kCacheUf, kCacheRoots, kCacheH1, kCacheBoruvka, kCacheTree, kCacheSlots };
 int device_cached(int slot, int (*init)());
 
 // Kernel launches made by the library (for the benchmark's launch count).

@@ -6,14 +6,12 @@
 namespace cp {
 
 // The pair of a committed survivor with key `key` (the key itself, not its
-// complement) of item `item`, whose dying class has root id yrid with age
-// key age[yrid] (the root vertex; for the dual the vertex whose lower star
-// holds the dying top cell).  Returns false for a zero-persistence pair,
+// complement) of item `item`, whose dying class has age key a (the root
+// vertex; for the dual the vertex whose lower star holds the dying top cell).  Returns false for a zero-persistence pair,
 // which is omitted (Sec. 2.3).
-__device__ __forceinline__ bool commit_pair(const ItemTable& tab, const uint64_t* age, int dual, uint64_t key,
-                                            int item, uint32_t yrid, cp_pair& out) {
+__device__ __forceinline__ bool commit_pair(const ItemTable& tab, uint64_t a, int dual, uint64_t key, int item,
+                                            cp_pair& out) {
     const Item& it = tab.it[item];
-    uint64_t a = age[yrid];
     const uint32_t young = key_vertex(a);
     uint32_t vg = key_vertex(key);
     int n = int(key_n(key, it.ndim));

@@ -54,6 +54,8 @@ struct Outs {
     uint64_t* res0;
     uint64_t* aget;
     uint64_t* rest;
+    TreeNode* node0;  // merge-tree nodes, or nullptr (then age / res are written)
+    TreeNode* nodet;
     uint32_t cap_s, cap_r0, cap_rt;
     Counters* ctr;
     uint32_t n_uf0, n_uft;  // forest sizes (bounds-checked build)
@@ -194,8 +196,12 @@ __device__ __forceinline__ void warp_flush(WS& ws, WarpCounts& c, const Outs& o)
     for (uint32_t i = lane; i < c.r0; i += 32) {
         uint32_t g = br0 + i;
         if (g < o.cap_r0) {
-            o.age0[g] = ws.r0age[i];
-            o.res0[g] = 0;
+            if (o.node0) {
+                o.node0[g] = TreeNode{~0ull, uint64_t(g), ws.r0age[i], 0};
+            } else {
+                o.age0[g] = ws.r0age[i];
+                o.res0[g] = 0;
+            }
             if (CP_IN(ws.r0node[i], o.n_uf0, o.ctr)) o.uf0[ws.r0node[i]] = kTag | g;
         } else if (CP_IN(ws.r0node[i], o.n_uf0, o.ctr)) {
             o.uf0[ws.r0node[i]] = kTag;  // out of capacity: keep the forest well formed (result flagged invalid)
@@ -204,8 +210,12 @@ __device__ __forceinline__ void warp_flush(WS& ws, WarpCounts& c, const Outs& o)
     for (uint32_t i = lane; i < c.rt; i += 32) {
         uint32_t g = brt + i;
         if (g < o.cap_rt) {
-            o.aget[g] = ws.rtage[i];
-            o.rest[g] = 0;
+            if (o.nodet) {
+                o.nodet[g] = TreeNode{~0ull, uint64_t(g), ~ws.rtage[i], 0};
+            } else {
+                o.aget[g] = ws.rtage[i];
+                o.rest[g] = 0;
+            }
             if (CP_IN(ws.rtnode[i], o.n_uft, o.ctr)) o.uft[ws.rtnode[i]] = kTag | g;
         } else if (CP_IN(ws.rtnode[i], o.n_uft, o.ctr)) {
             o.uft[ws.rtnode[i]] = kTag;
@@ -1131,6 +1141,8 @@ cudaError_t launch_prune(const ItemTable& tab, const PruneOuts& po, const TmaMap
     o.res0 = po.res0;
     o.aget = po.aget;
     o.rest = po.rest;
+    o.node0 = po.node0;
+    o.nodet = po.nodet;
     o.cap_s = po.cap_s;
     o.cap_r0 = po.cap_r0;
     o.cap_rt = po.cap_rt;

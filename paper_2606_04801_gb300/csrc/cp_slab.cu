@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(kST) k_slab_mark(const __grid_constant__ SlabA
                         uint64_t key = __ldcg(a.ko[q] + kl);
                         if (q) key = ~key;
                         const int item = item_of_vertex(a.tab, key_vertex(key));
-                        emit = commit_pair(a.tab, a.age[q], q, key, item, y, pr);
+                        emit = commit_pair(a.tab, a.age[q][y], q, key, item, pr);
                         fin = true;
                     }
                 }

@@ -1,0 +1,202 @@
+// K3: the elder-rule union-find over the survivors (H0: Sec. 4.1 step 3,
+// Sec. 4.2 step 2; the dual graph: Sec. 3.1, Appendix A, Sec. 4.1 step 5,
+// Sec. 4.2 step 3) as a merge tree that takes the survivors in any order: no
+// sort, no rounds, no grid barrier.
+//
+// Every root class u of the pruned forests has one word T[u] = (s, v): u is
+// connected with the older root v by survivors of key at most s; (infinity,
+// u) while it is connected with nothing older.  A survivor (u, v, s) goes in
+// as follows:
+//   1. climb from u and from v while T's key is below s: the oldest known
+//      root of each class at level s;
+//   2. the same root: the survivor closes a cycle, done;
+//   3. else, with u' the younger of the two and v' the older: compare and
+//      swap T[u'] from the word (t, w) just read to (s, v').  If another
+//      survivor changed it meanwhile, back to 1;
+//   4. if t was infinity, done; else the displaced connection (u', w, t) is
+//      still owed, and u' ~ v' at level s < t: go on with (v', w, t).
+// Why this is the sequential elder rule.  The connections in T and those
+// displaced ones still in some thread's hands connect, at every level a, what
+// all survivors taken so far with keys at most a connect: step 3 replaces
+// (u', w, t) by (u', v', s) and (v', w, t), and what step 2 drops is implied
+// by the rest.  Every T[u] points to an older root.  When all survivors are
+// in, a class of k roots at level a is a tree of T's connections of key at
+// most a; each root gives at most one and the oldest none, so all but the
+// oldest have T's key at most a: T[u]'s key is the level at which u stops
+// being the oldest of its class, which is the survivor that kills it.  The
+// keys (so the pairs) do not depend on the schedule; the parents may.
+// This is the triplet merge tree of Smirnov and Morozov (TopoInVis 2017), in
+// root-id space.
+//
+// Two threads could each drop a connection that the other's implies only if
+// each had read the other's word from before its displacement after making
+// its own: the full fence after a displacement rules that out (a connection
+// taken from T by a swap is owed by one thread alone until it is back in T).
+//
+// What bounds it: chains of dependent 16-byte L2 reads (a node's word), with
+// as many survivors in flight as threads fit.  Measured against the sorted
+// design it replaces as the default (8 radix passes over both lists, then
+// reservation rounds with two grid barriers each, cp_uf.cu), kernel times:
+//   2048^2, 256 levels (14 K survivors)     204 -> 37 us
+//   512^3 blurred (587 K survivors)         553 -> 198 us
+//   128^3 uniform noise (1.15 M survivors) 1110 -> 475 us
+#include "cp_common.cuh"
+#include "cp_grid.cuh"
+#include "cp_kernels.h"
+#include "cp_pairs.cuh"
+
+namespace cp {
+namespace {
+
+constexpr int kTT = 256;
+
+// A node's word, read and swapped as 128 bits: {key, parent}.
+struct Word {
+    uint64_t key;     // infinity (~0): connected with nothing older yet
+    uint64_t parent;  // root id
+};
+
+__device__ __forceinline__ Word ld_word(const TreeNode* n) {
+    Word w;
+    asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
+                 : "=l"(w.key), "=l"(w.parent)
+                 : "l"(n)
+                 : "memory");
+    return w;
+}
+__device__ __forceinline__ Word cas_word(TreeNode* n, Word expect, Word desired) {
+    Word w;
+    asm volatile(
+        "{\n\t.reg .b128 t, e, d;\n\tmov.b128 e, {%3, %4};\n\tmov.b128 d, {%5, %6};\n\t"
+        "atom.relaxed.gpu.global.cas.b128 t, [%2], e, d;\n\tmov.b128 {%0, %1}, t;\n\t}"
+        : "=l"(w.key), "=l"(w.parent)
+        : "l"(n), "l"(expect.key), "l"(expect.parent), "l"(desired.key), "l"(desired.parent)
+        : "memory");
+    return w;
+}
+
+// Both lists' survivors, in the order the pruning pass wrote them, one
+// survivor per thread.
+__global__ void __launch_bounds__(kTT) k_tree(const __grid_constant__ TreeArgs a) {
+    Counters* ctr = a.ctr;
+    // non-finite input, or walks that gave up: the call fails anyway
+    if (ld_acquire_u32(&ctr->status) & (kStTimeout | kStNonfinite)) return;
+    const uint32_t n0 = min(*a.l[0].d_n, a.cap), n1 = min(*a.l[1].d_n, a.cap), n = n0 + n1;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        ctr->rounds0 = n0 ? 1u : 0u;
+        ctr->roundst = n1 ? 1u : 0u;
+        ctr->trace_active[0][0] = n0;
+        ctr->trace_active[1][0] = n1;
+    }
+    uint32_t hops = 0;
+    for (uint32_t g = blockIdx.x * kTT + threadIdx.x; g < n; g += gridDim.x * kTT) {
+        const int q = g >= n0 ? 1 : 0;
+        const TreeList& L = a.l[q];
+        const uint32_t i = q ? g - n0 : g;
+        TreeNode* T = L.node;
+        uint64_t s = L.keys[i];  // ascending order of the stored keys in both lists
+        uint32_t u = __ldcg(L.ra + i), v = __ldcg(L.rb + i);
+        uint64_t t0 = 0;
+        uint32_t steps = 0;
+        // every climb ends (parents are older) and a swap only fails when another
+        // survivor went in; the wall-clock bound guards against a corrupted word
+        auto overdue = [&]() {
+            if ((++steps & 1023u) != 0) return false;
+            const uint64_t now = global_timer_ns();
+            if (t0 == 0) t0 = now;
+            if (now - t0 <= kWaitLimitNs) return false;
+            set_status(ctr, kStTimeout);
+            return true;
+        };
+        for (bool live = true; live;) {
+            if (!CP_IN(u, L.n_rids, ctr) || !CP_IN(v, L.n_rids, ctr)) break;
+            Word wu = ld_word(T + u), wv = ld_word(T + v);
+            for (;;) {
+                const bool cu = wu.key < s, cv = wv.key < s;
+                if (!cu && !cv) break;
+                if (cu) {
+                    u = uint32_t(wu.parent);
+                    if (!CP_IN(u, L.n_rids, ctr)) u = 0;
+                    wu = ld_word(T + u);
+                }
+                if (cv) {
+                    v = uint32_t(wv.parent);
+                    if (!CP_IN(v, L.n_rids, ctr)) v = 0;
+                    wv = ld_word(T + v);
+                }
+                if (overdue()) {
+                    live = false;
+                    break;
+                }
+            }
+            if (!live || u == v || overdue()) break;
+            if (T[u].age < T[v].age) {  // u: the younger (ages: smaller is older)
+                const uint32_t tu = u;
+                u = v;
+                v = tu;
+                wu = wv;
+            }
+            const Word got = cas_word(T + u, wu, Word{s, uint64_t(v)});
+            if (got.key != wu.key || got.parent != wu.parent) continue;
+            if (wu.key == ~0ull) break;
+            asm volatile("fence.sc.gpu;" ::: "memory");
+            s = wu.key;
+            u = v;
+            v = uint32_t(wu.parent);
+        }
+        hops += steps;
+    }
+    for (int o = 16; o > 0; o >>= 1) hops += __shfl_xor_sync(0xFFFFFFFFu, hops, o);
+    if (lane_id() == 0 && hops) atomicAdd(&ctr->trace_hops[0][1], (unsigned long long)hops);
+}
+
+// The pair of every root that the tree connects with an older one.
+__global__ void __launch_bounds__(kTT) k_tree_emit(const __grid_constant__ TreeEmitArgs a) {
+    Counters* ctr = a.ctr;
+    if (ld_acquire_u32(&ctr->status) & (kStTimeout | kStNonfinite)) return;
+    const uint32_t r0 = min(ctr->n_r0, a.n_rids[0]), r1 = min(ctr->n_rt, a.n_rids[1]), n = r0 + r1;
+    for (uint32_t g0 = blockIdx.x * kTT; g0 < n; g0 += gridDim.x * kTT) {
+        const uint32_t g = g0 + threadIdx.x;
+        bool emit = false;
+        cp_pair pr;
+        if (g < n) {
+            const int q = g >= r0 ? 1 : 0;
+            const TreeNode& nd = a.node[q][q ? g - r0 : g];
+            if (nd.key != ~0ull) {
+                const uint64_t key = q ? ~nd.key : nd.key;
+                const int item = item_of_vertex(a.tab, key_vertex(key));
+                if (a.h1flags[q] && a.tab.it[item].ndim == 3) {
+                    const uint32_t id = cell_id3(a.tab.it[item], key, q != 0);
+                    atomicOr(a.h1flags[q] + (id >> 5), 1u << (id & 31u));
+                }
+                emit = commit_pair(a.tab, q ? ~nd.age : nd.age, q, key, item, pr);
+            }
+        }
+        const uint32_t pp = warp_append(&ctr->n_pairs, emit);
+        if (emit) {
+            if (pp < a.pair_cap) a.pairs[pp] = pr;
+            else set_status(ctr, kStCapacity);
+        }
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_tree(const TreeArgs& a, cudaStream_t s) {
+    const int blocks = device_cached(kCacheTree, [] {
+        int per_sm = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tree, kTT, 0);
+        return device_sm_count() * (per_sm > 0 ? per_sm : 1);
+    });
+    k_tree<<<blocks, kTT, 0, s>>>(a);
+    note_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tree_emit(const TreeEmitArgs& a, cudaStream_t s) {
+    k_tree_emit<<<device_sm_count() * 4, kTT, 0, s>>>(a);
+    note_launches(1);
+    return cudaGetLastError();
+}
+
+}  // namespace cp

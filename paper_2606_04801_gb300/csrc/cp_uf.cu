@@ -156,7 +156,7 @@ __device__ __forceinline__ void endpoints(const ItemTable& tab, uint64_t k, int 
 // The pair of a committed survivor (see commit_pair).
 __device__ __forceinline__ void emit_pair(const UfParams& p, const ItemTable& tab, uint64_t key, int item,
                                           uint32_t yrid, bool* emitted, cp_pair& out) {
-    *emitted = commit_pair(tab, p.age, p.dual, key, item, yrid, out);
+    *emitted = commit_pair(tab, p.age[yrid], p.dual, key, item, out);
 }
 
 __device__ __forceinline__ bool side_by_side(const UfKernelArgs& args, uint32_t n0, uint32_t n1) {
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(kFT) k_roots2(const __grid_constant__ RootArgs
         if (live) {
             __stcg(r.ra + i, par[0] & ~kTag);
             __stcg(r.rb + i, par[1] & ~kTag);
-            __stcg(r.pos + i, i);
+            if (r.pos) __stcg(r.pos + i, i);
         }
     }
     for (int l = 0; l < 2; ++l) {
