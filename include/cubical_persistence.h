@@ -123,8 +123,9 @@ int cp_lut_lookup(int ndim, uint32_t raw, uint32_t *relevant, uint64_t *entry);
  * and collapses them there with a few multiplications and masks (Sec. 3.3's
  * rule that an offset matters only when every nonzero sub-offset precedes).
  * This runs that collapse on the host for all 2^26 raw masks and compares it
- * with the definition; *n_mismatch receives the number of masks that
- * differ (0 when the layout is right).  Takes a few seconds.  Returns CP_OK,
+ * with the definition, and the pruning kernel's closed forms with the table
+ * on all 15,935 classes; *n_mismatch receives the number of masks and
+ * classes that differ (0 when both are right).  Takes a few seconds.  Returns CP_OK,
  * or CP_ERR_ARG for a null pointer.
  */
 int cp_lut_check_layout(uint64_t *n_mismatch);
@@ -478,7 +479,8 @@ int cubical_persistence_debug_wait_timeout(void *d_workspace, size_t ws_bytes, i
 /*
  * Tuning of the pruning pass (process-wide; read by the following calls;
  * results never depend on it).  Keys:
- *   CP_TUNE_ZCHUNK_3D    planes per 3D pruning task (4..4096, default 64)
+ *   CP_TUNE_ZCHUNK_3D    planes per 3D pruning task at most (4..4096, default 64;
+ *                        small volumes get smaller tasks, to fill the chip)
  *   CP_TUNE_CTAS_PER_SM  3D pruning CTAs per SM (0 = as many as fit, default)
  *   CP_TUNE_ROWS_2D      rows per 2D pruning task (4 .. 4096; default 64)
  *   CP_TUNE_CROSS_PRUNE_2D  1: the top dimension of 2D images waits for H0

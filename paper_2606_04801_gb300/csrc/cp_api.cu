@@ -75,8 +75,9 @@ int ensure_device_tables() {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return CP_ERR_CUDA;
     if (dev < 64 && (g_dev_ready >> dev) & 1u) return CP_OK;
+    if (check_words3(g_lut3d) != 0) return CP_ERR_INTERNAL;
     const cudaError_t ue = upload_luts(g_lut2d.data(), g_lut3d.disp.data(), g_lut3d.entry.data(), g_lut3d.key.data());
-    if (ue == cudaErrorInvalidValue) return CP_ERR_INTERNAL;  // the table failed its consistency checks
+    if (ue == cudaErrorInvalidValue) return CP_ERR_INTERNAL;
     if (ue != cudaSuccess) return CP_ERR_CUDA;
     if (dev < 64) g_dev_ready |= 1ull << dev;
     return CP_OK;
@@ -92,6 +93,8 @@ struct Plan {
     size_t o_act0, o_act1, o_yn, o_on, o_na0, o_na1, o_nb0, o_nb1, o_pairs, o_pvals, o_pvalt, o_hist, o_status;
     size_t o_hist2, o_status2;
     size_t o_node0, o_nodet;  // merge-tree nodes
+    size_t o_code;            // link codes of the 3D items
+    uint64_t n_code = 0;
     // H1 of the volumes (calls that ask for it): see H1Bufs
     bool h1 = false;
     uint32_t h1_mcap = 0, h1_neg = 0, h1_posq = 0;
@@ -113,6 +116,32 @@ struct Plan {
 
 size_t align_up(size_t x) { return (x + 255) & ~size_t(255); }
 void plan_boruvka(Plan& P);
+
+// Owned planes per 3D pruning task, at most the tuned bound: the value that
+// makes the fewest plane steps on the busiest CTA, counting kStart steps for
+// a task's start (its planes' first loads and the lead-in and lead-out steps).
+// One value for all items of a call; 456 CTAs run at once (152 SMs x 3).
+int plan_zchunk(const ItemTable& tab) {
+    constexpr int kSlots = 456, kStart = 6;
+    const int hi = prune_zchunk3d();
+    int best = hi;
+    int64_t best_cost = INT64_MAX;
+    for (int c = 4; c <= hi; ++c) {
+        int64_t tasks = 0;
+        int dmax = 0;
+        for (int j = tab.n2d; j < tab.n; ++j) {
+            const Item& it = tab.it[j];
+            tasks += int64_t(it.tx) * it.ty * ((it.D + c - 1) / c);
+            dmax = std::max(dmax, it.D);
+        }
+        const int64_t cost = (tasks + kSlots - 1) / kSlots * (std::min(c, dmax) + kStart);
+        if (cost <= best_cost) {
+            best_cost = cost;
+            best = c;
+        }
+    }
+    return best;
+}
 
 // h1: also lay out the H1 stage of the 3D items, with h1_pool pool entries
 // for the columns that additions create (0: 4 per column + 2^20).
@@ -164,9 +193,6 @@ int make_plan(int n_items, const int32_t* ndims, const int64_t* dims, const floa
         } else {
             it.tx = int32_t((W + prune_tile_x3d() - 1) / prune_tile_x3d());
             it.ty = int32_t((H + prune_tile_y3d() - 1) / prune_tile_y3d());
-            it.tz = int32_t((D + prune_tile_z3d() - 1) / prune_tile_z3d());
-            it.tile0 = t3;
-            t3 += it.tx * it.ty * it.tz;
             P.tab.n3d++;
             edges += D * H * (W - 1) + D * (H - 1) * W + (D - 1) * H * W;
             facets += D * (H - 1) * (W - 1) + (D - 1) * H * (W - 1) + (D - 1) * (H - 1) * W;
@@ -175,6 +201,17 @@ int make_plan(int n_items, const int32_t* ndims, const int64_t* dims, const floa
             h1_posq += it.T;
         }
         if (voff > (int64_t(1) << kVBits) || toff > (int64_t(1) << kVBits) + kMaxItems) return CP_ERR_ARG;
+    }
+    const int zc = plan_zchunk(P.tab);
+    for (int j = P.tab.n2d; j < n_items; ++j) {
+        Item& it = P.tab.it[j];
+        it.zc = zc;
+        it.pitch = (it.W + 3) & ~3;
+        it.coff = int64_t(P.n_code);
+        P.n_code += uint64_t(it.D) * uint64_t(it.H) * uint64_t(it.pitch);
+        it.tz = (it.D + zc - 1) / zc;
+        it.tile0 = t3;
+        t3 += it.tx * it.ty * it.tz;
     }
     P.tab.tiles2d = t2;
     P.tab.tiles3d = t3;
@@ -185,7 +222,7 @@ int make_plan(int n_items, const int32_t* ndims, const int64_t* dims, const floa
             it.tma = ntma++;
     }
     P.tab.rows2d = prune_tile_y2d();
-    P.tab.zchunk3d = prune_tile_z3d();
+    P.tab.zchunk3d = prune_zchunk3d();
     P.tab.cross2d = prune_cross2d();
     P.ntot = voff;
     P.ttot = toff;
@@ -215,6 +252,7 @@ int make_plan(int n_items, const int32_t* ndims, const int64_t* dims, const floa
     P.o_ctr = take(sizeof(Counters));
     P.o_uf0 = take(sizeof(uint32_t) * size_t(P.ntot));
     P.o_uft = take(sizeof(uint32_t) * size_t(P.ttot));
+    P.o_code = take(size_t(P.n_code) + 16);
     P.o_s0 = take(sizeof(uint64_t) * P.cap_big);
     P.o_st = take(sizeof(uint64_t) * P.cap_s);
     P.o_salt = take(sizeof(uint64_t) * P.cap_big);
@@ -385,6 +423,8 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
     PruneOuts po;
     po.uf0 = uf0;
     po.uft = uft;
+    po.code = at<uint8_t>(ws, P.o_code);
+    po.n_code = P.n_code;
     po.s0 = s0;
     po.st = st;
     po.age0 = age0;
@@ -402,6 +442,7 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
     if (prune_only) {
         CP_TRY(launch_prune(P.tab, po, P.tma, s));
         mark(1, s);
+        CP_TRY(launch_expand(P.tab, po, s));
         return CP_OK;
     }
 
@@ -431,7 +472,7 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
     }
 
     CP_TRY(launch_prune(P.tab, po, P.tma, s));
-    if (tm) CP_TRY(launch_t_flatten(uf0, tm->items, s));
+    if (tm) CP_TRY(launch_t_flatten(uf0, po.code, tm->items, s));
     mark(1, s);
     nv.next("cp.roots+sort");
 
@@ -445,6 +486,8 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
     uint32_t* nb1 = at<uint32_t>(ws, P.o_nb1);
     uint32_t* ynode = at<uint32_t>(ws, P.o_yn);
     RootArgs ra;
+    ra.code = po.code;
+    ra.n_code = P.n_code;
     ra.tab = P.tab;
     ra.cap = P.cap_s;
     ra.ra = na1;
@@ -540,6 +583,8 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
     up[0].d_nkeys = &ctr->n_s0;
     up[0].cap_keys = P.cap_s;
     up[0].uf = uf0;
+    up[0].code = po.code;
+    up[0].n_code = P.n_code;
     up[0].age = age0;
     up[0].res = res0;
     up[0].act[0] = act0;
@@ -865,7 +910,12 @@ int t_run(int n_items, const float* const* h_images, const int32_t* ndims, const
     Plan P;
     rc = make_plan(n_items, ndims, jd.data(), jptr.data(), max_survivors, P);
     if (rc != CP_OK) return rc;
-    for (int j = 0; j < P.tab.n; ++j) tm.items.voff[P.tab.it[j].user] = P.tab.it[j].voff;
+    for (int j = 0; j < P.tab.n; ++j) {
+        const Item& it = P.tab.it[j];
+        tm.items.voff[it.user] = it.voff;
+        tm.items.coff[it.user] = it.ndim == 3 ? it.coff : 0;
+        tm.items.pitch[it.user] = it.ndim == 3 ? it.pitch : 0;
+    }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (launch_t_build(tm.items, bad, s) != cudaSuccess) return CP_ERR_CUDA;
     tm.bad = bad;
@@ -960,7 +1010,9 @@ int cp_lut_lookup(int ndim, uint32_t raw, uint32_t* relevant, uint64_t* entry) {
 
 int cp_lut_check_layout(uint64_t* n_mismatch) {
     if (!n_mismatch) return CP_ERR_ARG;
-    *n_mismatch = check_mask3_layout();
+    std::lock_guard<std::mutex> lk(g_mu);
+    if (!build_host_luts()) return CP_ERR_INTERNAL;
+    *n_mismatch = check_mask3_layout() + check_words3(g_lut3d);
     return CP_OK;
 }
 

@@ -33,6 +33,9 @@ struct Item {
     int32_t tx, ty, tz;       // pruning tiles along x, y, z
     int32_t user;             // the caller's index of the item
     int32_t tma;              // 3D: index of the item's plane tensor map (TMA loads), or -1
+    int32_t zc;               // 3D: owned planes per pruning task
+    int32_t pitch;            // 3D: row pitch of the item's link codes (its width, rounded up to 4)
+    int64_t coff;             // 3D: the item's first link code
 };
 
 struct ItemTable {
@@ -40,7 +43,7 @@ struct ItemTable {
     int32_t n2d, n3d;         // items 0..n2d-1 are 2D, n2d..n-1 are 3D
     int32_t tiles2d, tiles3d; // total pruning tiles of each kind
     int32_t rows2d;           // vertex rows per 2D pruning task (4 .. 4096)
-    int32_t zchunk3d;         // planes per 3D pruning task
+    int32_t zchunk3d;         // tuned bound on the planes of a 3D pruning task
     int32_t cross2d;          // 2D items: 1 = the dual list waits for H0 (cross-pruning), 0 = both at once
     Item it[kMaxItems];
 };
@@ -59,7 +62,7 @@ struct Counters {
     uint32_t act_count[2][3]; // active survivors of the next round (H0 / dual list), rotating
     uint32_t sort_tile[64];   // tile tickets of the sort passes of one call
     uint32_t find_ctr;        // work counter of the first union-find round's root walks
-    uint32_t tma_tasks;       // 3D pruning tasks whose planes came by TMA (a check that the path runs)
+    uint32_t tma_tasks;       // 3D pruning work whose planes came by TMA, in blocks of 31 x 8 columns x zchunk3d planes
     uint32_t t_keep;          // T-filtration calls: pairs kept after the mapping (the output count)
     uint32_t mst_rounds;      // Borůvka rounds (the spanning-forest union-find variant), else 0
     unsigned long long gmin[kMaxItems];  // (ord bits << 32 | local vertex) of each item's minimum

@@ -18,8 +18,10 @@ struct alignas(32) TreeNode {
     uint64_t pad;
 };
 struct PruneOuts {
-    uint32_t* uf0;   // H0 forest over global vertices
-    uint32_t* uft;   // dual forest over global top cells (+ one outside vertex per item)
+    uint32_t* uf0;   // H0 forest over global vertices (3D items: root words only)
+    uint32_t* uft;   // dual forest over global top cells (+ one outside vertex per item; 3D: root words only)
+    uint8_t* code;   // 3D items: both links of each vertex (cp_walk.cuh)
+    uint64_t n_code;
     uint64_t* s0;    // H0 survivor keys
     uint64_t* st;    // dual survivor keys (complemented: ascending sort = descending order)
     uint64_t* age0;  // age of each H0 root id
@@ -38,7 +40,7 @@ int prune_tile_x();
 int prune_tile_x3d();
 int prune_tile_y2d();
 int prune_tile_y3d();
-int prune_tile_z3d();
+int prune_zchunk3d();
 int prune_cross2d();
 int set_tuning(int key, int value);
 int get_tuning(int key);
@@ -54,6 +56,8 @@ struct TmaMaps {
 // Encodes the plane map of a D x H x W float volume; false if it cannot be used.
 bool encode_plane_map(CUtensorMap* map, const float* img, int64_t D, int64_t H, int64_t W);
 cudaError_t launch_prune(const ItemTable& tab, const PruneOuts& po, const TmaMaps& maps, cudaStream_t s);
+// The 3D items' forests as words, from their codes (stage tests).
+cudaError_t launch_expand(const ItemTable& tab, const PruneOuts& po, cudaStream_t s);
 
 // ---- K2 radix sort (LSD, 8-bit digits, decoupled look-back)
 struct SortBufs {
@@ -82,6 +86,8 @@ struct UfParams {
     const uint32_t* d_nkeys;
     uint32_t cap_keys;
     uint32_t* uf;
+    const uint8_t* code = nullptr;  // 3D items' links (cp_walk.cuh)
+    uint64_t n_code = 0;
     const uint64_t* age;
     uint64_t* res;
     uint32_t* act[2];         // survivor index of each active slot (ping-pong)
@@ -113,6 +119,8 @@ struct RootArgs {
     const uint32_t* d_n;
     uint32_t cap;
     const uint32_t* uf;
+    const uint8_t* code;         // 3D items' links (cp_walk.cuh)
+    uint64_t n_code;
     int dual;
     uint32_t* ra;                // root id of each survivor's endpoints, by unsorted position
     uint32_t* rb;
@@ -303,13 +311,15 @@ struct TItems {
     const float* img[kMaxItems];  // the image
     float* J[kMaxItems];          // its dual image: extents +2 along each image axis
     int64_t voff[kMaxItems];      // J's first vertex in the call's vertex space
+    int64_t coff[kMaxItems];      // 3D: J's first code and its codes' row pitch
+    int32_t pitch[kMaxItems];
 };
 // J <- -image flipped along every axis, inside a one-voxel frame at -FLT_MAX;
 // *bad <- 1 if a pixel is not below FLT_MAX (the frame would not come first).
 cudaError_t launch_t_build(const TItems& t, uint32_t* bad, cudaStream_t s);
 // After the pruning pass: every frame vertex's H0 link points at the item's
-// vertex 0.
-cudaError_t launch_t_flatten(uint32_t* uf0, const TItems& t, cudaStream_t s);
+// vertex 0 (3D: has the code that says so).
+cudaError_t launch_t_flatten(uint32_t* uf0, uint8_t* code, const TItems& t, cudaStream_t s);
 // V pairs of J -> T pairs of the images, in place; each item's frame class
 // gets item index n (it sorts after every kept pair), ctr->t_keep the count
 // without them, and a set *bad flags the call as non-finite.

@@ -26,6 +26,7 @@
 //      for the global dual union-find.
 #include "cp_lut.h"
 #include "cp_mask3.cuh"
+#include "cp_words3.cuh"
 
 #include <algorithm>
 #include <cstring>
@@ -295,6 +296,40 @@ uint64_t check_mask3_layout() {
     for (uint32_t raw = 0; raw < (1u << 27); ++raw) {
         if (raw & (1u << 13)) continue;
         if (collapse3_lattice(dev(raw)) != dev(collapse(st, raw))) ++bad;
+    }
+    return bad;
+}
+
+uint64_t check_words3(const Lut3D& lut) {
+    const Stencil& st = stencil(3);
+    const std::vector<uint32_t> masks = relevant_masks(st);
+    uint64_t bad = 0;
+    for (size_t i = 0; i < masks.size(); i += 32) {
+        const int n = int(std::min<size_t>(32, masks.size() - i));
+        uint32_t r[27] = {0};
+        for (int k = 0; k < n; ++k)
+            for (int b = 0; b < 27; ++b) r[b] |= ((masks[i + k] >> b) & 1u) << k;
+        Star3 s;
+        star_words3(r, s);
+        uint32_t b0, b1, b2;
+        slot7_target(s.co, b0, b1, b2);
+        for (int k = 0; k < n; ++k) {
+            auto bit = [&](uint32_t w) { return int((w >> k) & 1u); };
+            const uint32_t m = masks[i + k];
+            const uint64_t e = lut.entry[hash_slot(m, lut.disp[hash_bucket(m)])];
+            const int direct = lut_direct(e) == 7 ? 6 : lut_direct(e);
+            bool ok = direct == bit(s.h[0]) + 2 * bit(s.h[1]) + 4 * bit(s.h[2]);
+            for (int t = 0; t < 8; ++t) {
+                int want = 15;
+                if (bit(s.co[t])) {
+                    want = t < 7 ? slot_target(t) : bit(b0) + 2 * bit(b1) + 4 * bit(b2);
+                    if (want == t) want = 8;  // slot 7 towards itself: a dual root
+                }
+                ok = ok && want == int(lut_dual(e, t));
+            }
+            const bool needs = lut_h0_surv(e) || lut_dual_surv(e) || direct == 6 || lut_dual(e, 7) == 8;
+            if (!ok || (needs && !bit(s.event))) ++bad;
+        }
     }
     return bad;
 }

@@ -68,6 +68,11 @@ uint32_t collapse(const Stencil& st, uint32_t raw);
 // that layout; 0 when the layout is right.
 uint64_t check_mask3_layout();
 
+struct Lut3D;
+// Disagreements between the table and the closed forms that the pruning
+// kernel uses (cp_words3.cuh), over every class; 0 when they are right.
+uint64_t check_words3(const Lut3D& lut);
+
 // Lookup entry of a relevant mask.
 uint64_t classify(const Stencil& st, uint32_t rel);
 

@@ -51,6 +51,17 @@ CP_HD constexpr int mask3_pos(int n) {
     return kM3YZ + py + pz;
 }
 
+// all 26 bits; the bits of the neighbours on one side of an axis (0: z, 1: y, 2: x)
+CP_HD constexpr uint32_t mask3_side(int axis, int sign) {
+    uint32_t m = 0;
+    for (int n = 0; n < 27; ++n) {
+        const int d = axis == 0 ? n / 9 - 1 : (axis == 1 ? (n / 3) % 3 - 1 : n % 3 - 1);
+        if (n != 13 && (d == sign || sign == 2)) m |= 1u << mask3_pos(n);
+    }
+    return m;
+}
+constexpr uint32_t kM3All = mask3_side(0, 2);
+
 // canonical mask -> device layout
 CP_HD inline uint32_t mask3_from_canonical(uint32_t raw) {
     uint32_t m = 0;

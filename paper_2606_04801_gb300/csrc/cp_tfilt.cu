@@ -90,10 +90,13 @@ __global__ void __launch_bounds__(kTT) k_t_build(const __grid_constant__ TItems 
 // ancestor of every frame vertex (every frame vertex but 0 has an earlier
 // neighbour in the frame, and equal values order by index), so the shortcut
 // changes no root.  Item blockIdx.y.
-__global__ void __launch_bounds__(kTT) k_t_flatten(uint32_t* __restrict__ uf0, const __grid_constant__ TItems t) {
+__global__ void __launch_bounds__(kTT) k_t_flatten(uint32_t* __restrict__ uf0, uint8_t* __restrict__ code,
+                                                   const __grid_constant__ TItems t) {
     const int item = blockIdx.y;
     const TDims& d = t.d[item];
     uint32_t* __restrict__ uf = uf0 + t.voff[item];
+    uint8_t* __restrict__ cd = code + t.coff[item];
+    const int64_t P = t.pitch[item];
     const uint32_t root = uint32_t(t.voff[item]);
     const int64_t Dj = d.ndim == 3 ? d.D + 2 : 1, Hj = d.H + 2, Wj = d.W + 2;
     // whole frame rows, one block per row: both y faces of every plane, and
@@ -111,8 +114,12 @@ __global__ void __launch_bounds__(kTT) k_t_flatten(uint32_t* __restrict__ uf0, c
             y = (g & 1) ? Hj - 1 : 0;
         }
         uint32_t* row = uf + (z * Hj + y) * Wj;
+        uint8_t* crow = cd + (z * Hj + y) * P;
         for (int64_t x = threadIdx.x; x < Wj; x += kTT)
-            if (z != 0 || y != 0 || x != 0) row[x] = root;
+            if (z != 0 || y != 0 || x != 0) {
+                if (d.ndim == 3) crow[x] |= 7u;
+                else row[x] = root;
+            }
     }
     // the two x faces of the other rows
     const int64_t zi = d.ndim == 3 ? Dj - 2 : 1, yi = Hj - 2;
@@ -120,7 +127,9 @@ __global__ void __launch_bounds__(kTT) k_t_flatten(uint32_t* __restrict__ uf0, c
     for (int64_t k = int64_t(blockIdx.x) * kTT + threadIdx.x; k < nside; k += int64_t(gridDim.x) * kTT) {
         const int64_t q = k >> 1;
         const int64_t z = d.ndim == 3 ? 1 + q / yi : 0, y = 1 + q % yi;
-        uf[(z * Hj + y) * Wj + ((k & 1) ? Wj - 1 : 0)] = root;
+        const int64_t x = (k & 1) ? Wj - 1 : 0;
+        if (d.ndim == 3) cd[(z * Hj + y) * P + x] |= 7u;
+        else uf[(z * Hj + y) * Wj + x] = root;
     }
 }
 
@@ -212,10 +221,10 @@ cudaError_t launch_t_build(const TItems& t, uint32_t* bad, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_t_flatten(uint32_t* uf0, const TItems& t, cudaStream_t s) {
+cudaError_t launch_t_flatten(uint32_t* uf0, uint8_t* code, const TItems& t, cudaStream_t s) {
     if (t.n < 1 || t.n > kMaxItems) return cudaErrorInvalidValue;
     const int gx = (device_sm_count() * 8 + t.n - 1) / t.n;
-    k_t_flatten<<<dim3(gx, t.n), kTT, 0, s>>>(uf0, t);
+    k_t_flatten<<<dim3(gx, t.n), kTT, 0, s>>>(uf0, code, t);
     note_launches(1);
     return cudaGetLastError();
 }

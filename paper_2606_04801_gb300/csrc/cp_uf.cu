@@ -32,6 +32,7 @@
 #include "cp_grid.cuh"
 #include "cp_kernels.h"
 #include "cp_pairs.cuh"
+#include "cp_walk.cuh"
 
 namespace cp {
 namespace {
@@ -44,49 +45,6 @@ struct UfKernelArgs {
     UfParams p[2];
     int nprob;
 };
-
-// Roots of a and b, walking both paths in lockstep (two independent loads in
-// flight per thread).  The walks only read: the active survivors carry their
-// roots from round to round, so nothing needs compressing, and random partial
-// writes into the large forest array would cost read-modify-write traffic.
-// Paths end at roots (the forests are acyclic); the wall-clock bound only
-// guards against a corrupted forest (the walk then stops and reports false).
-// (Bounds-checked build: a parent outside the forest ends the walk, flagged.)
-__device__ __forceinline__ bool walk(const uint32_t* uf, uint32_t n_nodes, Counters* ctr, uint32_t& a, uint32_t& pa,
-                                     uint32_t& b, uint32_t& pb, uint32_t& hops) {
-    uint64_t t0 = 0;
-    (void)n_nodes;
-    (void)ctr;
-    while (!(pa & kTag) || !(pb & kTag)) {
-        ++hops;
-        if (!(pa & kTag)) {
-            a = pa;
-            pa = CP_IN(a, n_nodes, ctr) ? __ldcg(uf + a) : kTag;
-        }
-        if (!(pb & kTag)) {
-            b = pb;
-            pb = CP_IN(b, n_nodes, ctr) ? __ldcg(uf + b) : kTag;
-        }
-        if ((hops & 1023u) == 0) {
-            const uint64_t now = global_timer_ns();
-            if (t0 == 0) t0 = now;
-            else if (now - t0 > kWaitLimitNs) return false;
-        }
-    }
-    return true;
-}
-
-__device__ __forceinline__ bool find_two(const uint32_t* uf, uint32_t n_nodes, Counters* ctr, uint32_t a, uint32_t b,
-                                         uint32_t& rida, uint32_t& ridb, uint32_t& ra, uint32_t& rb, uint32_t& hops) {
-    uint32_t pa = CP_IN(a, n_nodes, ctr) ? __ldcg(uf + a) : kTag, pb = CP_IN(b, n_nodes, ctr) ? __ldcg(uf + b) : kTag;
-    const bool ok = walk(uf, n_nodes, ctr, a, pa, b, pb, hops);
-    ra = a;
-    rb = b;
-    rida = pa & ~kTag;
-    ridb = pb & ~kTag;
-    return ok;
-}
-
 
 // Current root id of a class given a root id it once had.
 // (Bounds-checked build: an id outside the root ids becomes 0, flagged.)
@@ -117,40 +75,6 @@ __device__ __forceinline__ bool find_rid(const uint64_t* res, uint32_t n_rids, C
 // thread does not wait for it (the grid barrier orders it before the checks).
 __device__ __forceinline__ void reserve(uint64_t* res, uint32_t rid, uint64_t stamp) {
     atomicMax(reinterpret_cast<unsigned long long*>(res + rid), (unsigned long long)stamp);
-}
-
-// Endpoints of survivor key k (H0: the edge's two vertices; dual: the two top
-// cells on either side of the facet, or the item's outside vertex).
-__device__ __forceinline__ void endpoints(const ItemTable& tab, uint64_t k, int dual, uint32_t& a, uint32_t& b,
-                                          int& item) {
-    uint32_t vg = key_vertex(k);
-    item = item_of_vertex(tab, vg);
-    const Item& it = tab.it[item];
-    int n = int(key_n(k, it.ndim));
-    int dz, dy, dx;
-    stencil_off(it.ndim, n, dz, dy, dx);
-    if (!dual) {
-        a = vg;
-        b = uint32_t(int64_t(vg) + (int64_t(dz) * it.H + dy) * it.W + dx);
-        return;
-    }
-    const uint32_t local = vg - uint32_t(it.voff), W = uint32_t(it.W), H = uint32_t(it.H);
-    const uint32_t row = local / W;
-    const int x = int(local - row * W), y = int(row % H), z = int(row / H);
-    // the facet's zero coordinate (on one of the item's axes) picks the side
-    int sz0 = dz, sy0 = dy, sx0 = dx, sz1 = dz, sy1 = dy, sx1 = dx;
-    if (it.ndim == 3 && dz == 0) {
-        sz0 = -1;
-        sz1 = 1;
-    } else if (dy == 0) {
-        sy0 = -1;
-        sy1 = 1;
-    } else {
-        sx0 = -1;
-        sx1 = 1;
-    }
-    a = top_of_octant(it, z, y, x, sz0, sy0, sx0);
-    b = top_of_octant(it, z, y, x, sz1, sy1, sx1);
 }
 
 // The pair of a committed survivor (see commit_pair).
@@ -186,8 +110,19 @@ __device__ __forceinline__ void cross_prune(const ItemTable& tab, const UfParams
 // separate, non-cooperative launch: warps take 32 survivors at a time from a
 // counter, so a warp held up by a long path delays no other warp.
 constexpr int kFT = 256;
-constexpr int kRootsPerLane = 1;  // survivors per lane (more paths in lockstep measured slower: the walks are
-                                  // bound by random DRAM accesses, and lockstep waste grows)
+
+__device__ __forceinline__ Forest forest_of(const RootArgs& r) { return Forest{r.uf, r.code, r.n_nodes, r.n_code, r.dual}; }
+
+// Survivor i of the list r (one lane): its endpoints' root ids and its position.
+__device__ __forceinline__ void place_walk(const ItemTable& tab, const RootArgs& r, uint32_t i, uint32_t& hops) {
+    uint64_t key = r.keys[i];
+    if (r.dual) key = ~key;
+    uint32_t ra, rb;
+    if (!walk_roots(tab, forest_of(r), r.ctr, key, ra, rb, hops)) set_status(r.ctr, kStTimeout);
+    __stcg(r.ra + i, ra);
+    __stcg(r.rb + i, rb);
+    if (r.pos) __stcg(r.pos + i, i);
+}
 
 __global__ void __launch_bounds__(kFT) k_roots(const __grid_constant__ RootArgs r) {
     Counters* ctr = r.ctr;
@@ -197,66 +132,17 @@ __global__ void __launch_bounds__(kFT) k_roots(const __grid_constant__ RootArgs 
     uint32_t hops = 0;
     for (;;) {
         uint32_t base = 0;
-        if (lane == 0) base = atomicAdd(&ctr->find_ctr, 32u * kRootsPerLane);
+        if (lane == 0) base = atomicAdd(&ctr->find_ctr, 32u);
         base = __shfl_sync(0xFFFFFFFFu, base, 0);
         if (base >= n) break;
-        // the endpoints of this lane's survivors and their first parents (all loads in flight together)
-        uint32_t node[2 * kRootsPerLane], par[2 * kRootsPerLane];
-#pragma unroll
-        for (int s = 0; s < kRootsPerLane; ++s) {
-            const uint32_t i = base + 32u * s + lane;
-            node[2 * s] = node[2 * s + 1] = 0;
-            if (i < n) {
-                uint64_t key = r.keys[i];
-                if (r.dual) key = ~key;
-                int item;
-                endpoints(r.tab, key, r.dual, node[2 * s], node[2 * s + 1], item);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < 2 * kRootsPerLane; ++k)
-            par[k] = base + 32u * (k >> 1) + lane < n && CP_IN(node[k], r.n_nodes, ctr) ? __ldcg(r.uf + node[k]) : kTag;
-        // walk all paths one hop per step until every one has reached its root
-        uint64_t t0 = 0;
-        uint32_t steps = 0;
-        for (;;) {
-            bool more = false;
-#pragma unroll
-            for (int k = 0; k < 2 * kRootsPerLane; ++k) {
-                if (!(par[k] & kTag)) {
-                    node[k] = par[k];
-                    par[k] = CP_IN(node[k], r.n_nodes, ctr) ? __ldcg(r.uf + node[k]) : kTag;
-                    more = true;
-                }
-            }
-            if (!more) break;
-            ++hops;
-            if ((++steps & 1023u) == 0) {
-                const uint64_t now = global_timer_ns();
-                if (t0 == 0) t0 = now;
-                else if (now - t0 > kWaitLimitNs) {  // only a corrupted forest gets here
-                    set_status(ctr, kStTimeout);
-#pragma unroll
-                    for (int k = 0; k < 2 * kRootsPerLane; ++k) par[k] = kTag;
-                    break;
-                }
-            }
-        }
-#pragma unroll
-        for (int s = 0; s < kRootsPerLane; ++s) {
-            const uint32_t i = base + 32u * s + lane;
-            if (i < n) {
-                __stcg(r.ra + i, par[2 * s] & ~kTag);
-                __stcg(r.rb + i, par[2 * s + 1] & ~kTag);
-                __stcg(r.pos + i, i);
-            }
-        }
+        if (base + lane < n) place_walk(r.tab, r, base + lane, hops);
+        __syncwarp();
     }
     for (int o = 16; o > 0; o >>= 1) hops += __shfl_xor_sync(0xFFFFFFFFu, hops, o);
     if (lane == 0 && hops) atomicAdd(&ctr->trace_hops[r.dual][0], (unsigned long long)hops);
 }
 
-// Both lists' first-round walks in one launch (volumes): warps take 32
+// Both lists' first-round walks in one launch: warps take 32
 // survivors at a time from one counter running over the H0 list and then the
 // dual list, so the long walks of one list overlap those of the other instead
 // of following them.  Each lane walks its own list's forest.
@@ -274,48 +160,9 @@ __global__ void __launch_bounds__(kFT) k_roots2(const __grid_constant__ RootArgs
         base = __shfl_sync(0xFFFFFFFFu, base, 0);
         if (base >= n) break;
         const uint32_t g = base + lane;
-        const bool live = g < n;
         const int l = g >= n0 ? 1 : 0;  // this lane's list
-        const RootArgs& r = l ? r1 : r0;
-        const uint32_t i = l ? g - n0 : g;
-        uint32_t node[2] = {0, 0}, par[2] = {kTag, kTag};
-        if (live) {
-            uint64_t key = r.keys[i];
-            if (r.dual) key = ~key;
-            int item;
-            endpoints(r0.tab, key, r.dual, node[0], node[1], item);
-            par[0] = CP_IN(node[0], r.n_nodes, ctr) ? __ldcg(r.uf + node[0]) : kTag;
-            par[1] = CP_IN(node[1], r.n_nodes, ctr) ? __ldcg(r.uf + node[1]) : kTag;
-        }
-        uint64_t t0 = 0;
-        uint32_t steps = 0;
-        for (;;) {
-            bool more = false;
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                if (!(par[k] & kTag)) {
-                    node[k] = par[k];
-                    par[k] = CP_IN(node[k], r.n_nodes, ctr) ? __ldcg(r.uf + node[k]) : kTag;
-                    more = true;
-                }
-            }
-            if (!more) break;
-            ++hops[l];
-            if ((++steps & 1023u) == 0) {
-                const uint64_t now = global_timer_ns();
-                if (t0 == 0) t0 = now;
-                else if (now - t0 > kWaitLimitNs) {  // only a corrupted forest gets here
-                    set_status(ctr, kStTimeout);
-                    par[0] = par[1] = kTag;
-                    break;
-                }
-            }
-        }
-        if (live) {
-            __stcg(r.ra + i, par[0] & ~kTag);
-            __stcg(r.rb + i, par[1] & ~kTag);
-            if (r.pos) __stcg(r.pos + i, i);
-        }
+        if (g < n) place_walk(r0.tab, l ? r1 : r0, l ? g - n0 : g, hops[l]);
+        __syncwarp();
     }
     for (int l = 0; l < 2; ++l) {
         uint32_t h = hops[l];
@@ -357,10 +204,7 @@ __device__ __forceinline__ void fresh_roots(const UfKernelArgs& args, const UfPa
                                             uint32_t& rb, uint32_t& hops) {
     uint64_t key = p.keys[i];
     if (p.dual) key = ~key;
-    uint32_t a, b, va, vb;
-    int item;
-    endpoints(args.tab, key, p.dual, a, b, item);
-    if (!find_two(p.uf, p.n_nodes, p.ctr, a, b, ra, rb, va, vb, hops)) {
+    if (!walk_roots(args.tab, Forest{p.uf, p.code, p.n_nodes, p.n_code, p.dual}, p.ctr, key, ra, rb, hops)) {
         set_status(p.ctr, kStTimeout);
         rb = ra;
     }
