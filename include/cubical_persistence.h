@@ -493,7 +493,8 @@ int cubical_persistence_debug_wait_timeout(void *d_workspace, size_t ws_bytes, i
  *                        then finds closing dual cycles.  Same pairs.
  *   CP_TUNE_H1_BUDGET_MS wall-clock budget in milliseconds of the cross-star
  *                        reduction rounds of the _full calls (0 .. 3,600,000;
- *                        default 30,000).  Those rounds run in one
+ *                        default 30,000).  Those rounds (and, with the same
+ *                        budget, the rewriting of the columns before them) run in one
  *                        non-preemptible cooperative launch; once the budget
  *                        is spent, every block leaves at the next round
  *                        boundary and the call returns CP_ERR_TIMEOUT (no

@@ -1216,7 +1216,7 @@ int cubical_persistence_full_info(const void* d_workspace, int n_items, const in
         return CP_ERR_CUDA;
     h_info[0] = c.m;
     h_info[1] = c.rounds;
-    h_info[2] = int64_t(c.grown);
+    h_info[2] = int64_t(c.grown + std::min<uint64_t>(c.flow_grown, P.h1_pool / 4));
     if (cap >= 10) {
         h_info[4] = c.neg_e;
         h_info[5] = c.pos_q;

@@ -34,8 +34,9 @@
 // (6 through m, 24 that miss it).  A column that ends holding an edge
 // through m is final: its pair has zero persistence, and the column is the
 // pivot of that edge.  The others (their lowest entry left the star: every
-// pair of nonzero persistence, and with distinct values only those) are
-// reduced across stars in rounds
+// pair of nonzero persistence, and with distinct values only those) are first
+// rewritten, each by a warp on its own, in terms of the edges that no star
+// column owns (k_h1_flow), and then reduced against each other in rounds
 // inside one cooperative kernel (the last rounds, once few columns change,
 // in its first CTA alone, with CTA barriers): every column whose lowest entry changed
 // bids for that row with an atomic minimum of its key (the filtration order)
@@ -663,6 +664,14 @@ __device__ uint32_t cta_merge(const H1Bufs& b, const ColSrc& c, const ColSrc& p,
     return written;
 }
 
+// The star replacement (below) may use this much of the pool; the rounds keep the rest, and
+// what of it is not used (flow_base: where theirs starts).
+__device__ __forceinline__ uint64_t flow_room(const H1Bufs& b) { return b.pool_cap / 4; }
+__device__ __forceinline__ uint64_t flow_base(const H1Bufs& b) {
+    const uint64_t g = __ldcg(&b.ctl->flow_grown);
+    return g < flow_room(b) ? g : flow_room(b);
+}
+
 // Column q lost its row to an older column: add that column (F2: the
 // symmetric difference; the common lowest entry cancels).  Columns that no
 // addition has reached yet are read from their star masks.  A column that
@@ -730,7 +739,7 @@ __device__ void add_winner_warp(const ReduceArgs& a, uint32_t q, uint32_t r, uin
         while (cap < need) cap <<= 1;
         cap <<= 1;
         uint64_t got = 0;
-        if (lane == 0) got = atomicAdd(&b.ctl->grown, (unsigned long long)(2ull * cap));
+        if (lane == 0) got = flow_base(b) + atomicAdd(&b.ctl->grown, (unsigned long long)(2ull * cap));
         base = __shfl_sync(0xFFFFFFFFu, got, 0);
         if (base + 2ull * cap > b.pool_cap) return stop(kStCapacity);
         into = 0u;
@@ -766,6 +775,378 @@ __device__ void add_winner_warp(const ReduceArgs& a, uint32_t q, uint32_t r, uin
         __stcg(b.clen + q, k);
     }
     if (k == 0) stop(kStInternal);
+}
+
+// ---- the columns that left their star, in terms of the edges no star owns
+//
+// A column may add the star column of any of its entries, not only of its
+// lowest: that column's square lies in the entry's star, which is older, so
+// the addition is left to right and changes no pair.  Replacing every entry
+// that a star column owns, until none is left, needs no other column that left
+// its star: the columns are independent, one per warp, with no rounds.  What
+// remains are the entries without a star owner, as many over the volume as
+// there are columns (the boundary matrix of the Morse complex of the star
+// pairs): the rounds below then add short columns, and few of them in a row.
+//
+// A warp keeps the column sorted (descending) and takes its first 32 entries
+// at a time: each lane looks up its entry's owner, the owners' other entries
+// are decoded together, sorted, and merged into the rest; equal entries cancel
+// in pairs.  (Over F2 the order of the replacements does not matter; taking
+// the largest first keeps an entry from being replaced twice.)  An entry
+// without owner is final once nothing larger is pending.
+//
+// What bounds it: latency.  A batch is three dependent L2 reads, a sort of up to
+// 128 keys and a merge, and a column takes some 100 batches.  Whole-diagram
+// forward with the rounds alone (each addition of a star column a round of its
+// own) and with this first:
+//   128^3 sigma 2 (10,223 columns)   84 -> 2.4 ms (5,650 -> 97 rounds)
+//   256^3 sigma 3 (25,771 columns)  840 -> 7.9 ms
+//   96^3 uniform noise (162,770)     17 -> 6.0 ms (657 -> 280 rounds)
+//   24^3 uniform noise (2,392)      2.2 -> 1.15 ms
+//
+// Two launches: most columns stay short and go through the first, whose warps
+// have little shared memory, so that many are in flight; the ones that outgrow
+// it start again in the second, whose columns may go on in the pool.
+constexpr int kFW = 8;                   // warps per CTA
+constexpr uint32_t kFNew = 128;          // entries that one batch adds at most
+constexpr uint32_t kFMax = 1u << 16;     // entries of a column in global scratch at most
+struct FlowSmall {
+    static constexpr bool kBig = false;
+    static constexpr uint32_t kCur = 384;  // entries of a column in shared memory
+    static constexpr uint32_t kOut = 128;  // entries of a finished column at most
+    uint64_t buf[2][kCur];
+    uint64_t out[kOut];
+    uint64_t add[kFNew + 1];  // from index 1
+    uint16_t slot[kFNew];
+};
+struct FlowBig {
+    static constexpr bool kBig = true;
+    static constexpr uint32_t kCur = 768;
+    static constexpr uint32_t kOut = 1024;
+    uint64_t buf[2][kCur];
+    uint64_t out[kOut];
+    uint64_t add[kFNew + 1];
+    uint16_t slot[kFNew];
+    MergeTile tile;
+};
+
+// Descending bitonic sort of 32 R keys of a warp, key 32 i + lane in v[i].
+template <int R>
+__device__ __forceinline__ void warp_sort_desc(uint64_t (&v)[R]) {
+    const unsigned lane = lane_id();
+#pragma unroll
+    for (int k = 2; k <= 32 * R; k <<= 1) {
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            if (j >= 32) {
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    const int l = i ^ (j >> 5);
+                    if (l > i) {
+                        const bool down = ((32 * i) & k) == 0;
+                        const uint64_t x = v[i], y = v[l];
+                        const bool swap = down ? x < y : x > y;
+                        v[i] = swap ? y : x;
+                        v[l] = swap ? x : y;
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    const uint64_t x = v[i], y = __shfl_xor_sync(0xFFFFFFFFu, x, j);
+                    const bool down = (((32 * i) | int(lane)) & k) == 0, first = (lane & unsigned(j)) == 0;
+                    v[i] = (down == first) ? (x > y ? x : y) : (x < y ? x : y);
+                }
+            }
+        }
+    }
+}
+
+// Sorts the warp's fresh keys (v[i] = entry 32 i + lane of n; 0 past the end),
+// cancels equal ones in pairs and writes the rest to add[1 ..]; their count.
+template <int R>
+__device__ __forceinline__ uint32_t sort_cancel(uint64_t (&v)[R], uint64_t* add) {
+    const unsigned lane = lane_id();
+    warp_sort_desc(v);
+    uint32_t na = 0;
+    // runs of equal keys are short: a key stays if it starts a run of odd length
+#pragma unroll
+    for (int i = 0; i < R; ++i) add[1 + 32 * i + lane] = v[i];
+    __syncwarp();
+    bool keep[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const uint32_t t = 32 * i + lane;
+        keep[i] = v[i] != 0 && (t == 0 || add[t] != v[i]);
+        if (keep[i]) {
+            uint32_t e = t + 1;
+            while (e < 32u * R && add[1 + e] == v[i]) ++e;
+            keep[i] = (e - t) & 1u;
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const unsigned kb = __ballot_sync(0xFFFFFFFFu, keep[i]);
+        if (keep[i]) add[1 + na + __popc(kb & ((1u << lane) - 1u))] = v[i];
+        na += __popc(kb);
+    }
+    __syncwarp();
+    return na;
+}
+
+// The symmetric difference of two descending arrays in shared memory (see
+// warp_merge); returns its length.
+__device__ uint32_t merge_shared(const uint64_t* c, uint32_t nc, const uint64_t* p, uint32_t np, uint64_t* out) {
+    const unsigned lane = lane_id();
+    const uint32_t total = nc + np, per = (total + 31) / 32;
+    const uint32_t d0 = min(total, lane * per), d1 = min(total, d0 + per);
+    uint32_t lo = d0 > np ? d0 - np : 0u, hi = min(d0, nc);
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (c[mid] >= p[d0 - mid - 1u]) lo = mid + 1u;
+        else hi = mid;
+    }
+    const uint32_t i0 = lo, j0 = d0 - lo;
+    uint32_t kept = 0, written = 0;
+    for (int pass = 0; pass < 2; ++pass) {
+        uint64_t* w = nullptr;
+        if (pass == 1) {
+            uint32_t incl = kept;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                if (lane >= unsigned(o)) incl += v;
+            }
+            w = out + (incl - kept);
+            written = __shfl_sync(0xFFFFFFFFu, incl, 31);
+        }
+        uint32_t i = i0, j = j0;
+        uint64_t x = i < nc ? c[i] : 0, y = j < np ? p[j] : 0, prevc = i > 0 ? c[i - 1] : ~0ull;
+        for (uint32_t d = d0; d < d1; ++d) {
+            if (j >= np || (i < nc && x >= y)) {
+                const bool keep = !(j < np && y == x);
+                if (pass == 0) kept += keep ? 1u : 0u;
+                else if (keep) *w++ = x;
+                prevc = x;
+                ++i;
+                x = i < nc ? c[i] : 0;
+            } else {
+                const bool keep = prevc != y;
+                if (pass == 0) kept += keep ? 1u : 0u;
+                else if (keep) *w++ = y;
+                ++j;
+                y = j < np ? p[j] : 0;
+            }
+        }
+    }
+    __syncwarp();
+    return written;
+}
+
+struct FlowArgs {
+    ItemTable tab;
+    H1Bufs b;
+    Counters* ctr;
+    uint64_t budget_ns;
+};
+
+// The warp takes n entries of the replacement's part of the pool; ~0: none
+// left.  (A plain addition: with a compare-and-swap that never takes too much,
+// the retries of a thousand warps were 95% of the kernel.)
+__device__ uint64_t pool_take(const H1Bufs& b, uint64_t n) {
+    unsigned long long at = 0;
+    if (lane_id() == 0) at = atomicAdd(&b.ctl->flow_grown, (unsigned long long)n);
+    at = __shfl_sync(0xFFFFFFFFu, at, 0);
+    return at + n <= flow_room(b) ? at : ~0ull;
+}
+
+// One column; false: left as it is (no room).
+template <class W>
+__device__ bool flow_column(const FlowArgs& a, W& s, uint32_t q, uint64_t& scratch, uint32_t& scratch_cap,
+                            uint64_t t_start) {
+    const H1Bufs& b = a.b;
+    const unsigned lane = lane_id();
+    const Item* itq;
+    int64_t mq;
+    column_key(a.tab, q, itq, mq);
+    uint64_t* cur = s.buf[0];
+    uint32_t n = warp_decode(*itq, mq, __ldcg(b.cmask + q), cur);
+    uint32_t which = 0, nout = 0, batches = 0;
+    bool in_smem = true, changed = false;
+    while (n > 0) {
+        if ((batches++ & 15u) == 0 && global_timer_ns() - t_start > a.budget_ns) {
+            if (lane == 0) set_status(a.ctr, kStTimeout);
+            return false;
+        }
+        // ---- the first entries and their owners
+        const uint32_t take = min(32u, n);
+        const uint64_t key = lane < take ? (in_smem ? cur[lane] : __ldcg(cur + lane)) : 0ull;
+        uint64_t pv = ~0ull;
+        int item = 0;
+        if (lane < take) {
+            item = item_of_vertex(a.tab, key_vertex(key));
+            const uint32_t eid = cell_id3(a.tab.it[item], key, false);
+            if (CP_IN(eid, b.n_ids, a.ctr)) pv = __ldcg(b.pivot + eid);
+        }
+        const bool owned = lane < take && pv != ~0ull;
+        const unsigned has = __ballot_sync(0xFFFFFFFFu, owned);
+        const uint32_t lead = has ? uint32_t(__ffs(has) - 1) : take;  // entries that are final
+        if (nout + lead > W::kOut) return false;
+        if (lane < lead) s.out[nout + lane] = key;
+        nout += lead;
+        uint32_t used = lead, na = 0;
+        if (has) {
+            // the other entries of the owners (an entry without owner behind an
+            // owned one goes back in), for as many lanes as fit
+            uint32_t mask = 0;
+            if (owned) {
+                const uint32_t p = cell_id3(a.tab.it[item], pv, true);
+                if (CP_IN(p, b.n_ids, a.ctr)) mask = __ldcg(b.cmask + p) & 0x3FFFFFFFu;
+                mask &= ~(1u << (31 - __clz(mask | 1u)));  // without the entry itself: the last edge through m
+            }
+            const bool back = lane < take && lane >= lead && !owned;
+            const uint32_t c = back ? 1u : __popc(mask);
+            uint32_t incl = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                if (lane >= unsigned(o)) incl += v;
+            }
+            used = uint32_t(__popc(__ballot_sync(0xFFFFFFFFu, lane < take && incl <= kFNew)));  // a prefix of the lanes
+            const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, int(used) - 1);
+            if (lane < used) {
+                uint32_t at = incl - c;
+                if (back) s.slot[at] = uint16_t(lane << 5 | 31u);
+                while (mask) {
+                    const int sl = __ffs(mask) - 1;
+                    mask &= mask - 1;
+                    s.slot[at++] = uint16_t(lane << 5 | sl);
+                }
+            }
+            __syncwarp();
+            uint64_t v[kFNew / 32];
+#pragma unroll
+            for (int i = 0; i < int(kFNew) / 32; ++i) {
+                v[i] = 0;
+                if (32u * i < total) {  // (the same for all lanes)
+                    const uint32_t t = 32u * i + lane, e = t < total ? s.slot[t] : 0u;
+                    const uint64_t ko = __shfl_sync(0xFFFFFFFFu, key, int(e >> 5));
+                    const Item& it = a.tab.it[__shfl_sync(0xFFFFFFFFu, item, int(e >> 5))];
+                    if (t < total)
+                        v[i] = (e & 31u) == 31u ? ko
+                                                : slot_key(it, int64_t(key_vertex(ko)) - it.voff, int(e & 31u));
+                }
+            }
+            changed = true;
+            if (total <= 32) {
+                uint64_t w[1] = {v[0]};
+                na = sort_cancel(w, s.add);
+            } else if (total <= 64) {
+                uint64_t w[2] = {v[0], v[1]};
+                na = sort_cancel(w, s.add);
+            } else {
+                na = sort_cancel(v, s.add);
+            }
+        }
+        if (na == 0) {  // nothing to merge
+            cur += used;
+            n -= used;
+            continue;
+        }
+        // ---- merged into the rest
+        const uint32_t rest = n - used, need = rest + na;
+        if (in_smem && need <= W::kCur) {
+            which ^= 1u;
+            n = merge_shared(cur + used, rest, s.add + 1, na, s.buf[which]);
+            cur = s.buf[which];
+            continue;
+        }
+        if constexpr (!W::kBig) {
+            return false;
+        } else {
+            uint64_t* dst;
+            const bool dst_smem = need <= W::kCur;
+            if (dst_smem) {
+                which ^= 1u;
+                dst = s.buf[which];
+            } else {
+                if (need > kFMax) return false;
+                if (need > scratch_cap) {
+                    uint32_t cap = 4096;
+                    while (cap < need) cap <<= 1;
+                    const uint64_t got = pool_take(b, 2ull * cap);
+                    if (got == ~0ull) return false;
+                    scratch = got;
+                    scratch_cap = cap;
+                    dst = b.pool + scratch;
+                } else {
+                    // the half that cur does not lie in
+                    dst = b.pool + scratch + ((!in_smem && cur < b.pool + scratch + scratch_cap) ? scratch_cap : 0u);
+                }
+            }
+            ColSrc c, p;
+            c.off = in_smem ? ~0ull : uint64_t(cur - b.pool) + used - 1u;
+            c.sm = cur + used - 1;
+            c.len = rest + 1u;
+            p.off = ~0ull;
+            p.sm = s.add;
+            p.len = na + 1u;
+            n = warp_merge(b, c, p, dst, s.tile);
+            __syncwarp();
+            cur = dst;
+            in_smem = dst_smem;
+        }
+    }
+    if (!changed) return true;
+    if (nout == 0) {  // never: a column reduces to a nonzero column
+        if (lane == 0) set_status(a.ctr, kStInternal);
+        return false;
+    }
+    uint32_t cap = 4u;
+    while (cap < nout) cap <<= 1;
+    const uint64_t base = pool_take(b, 2ull * cap);
+    if (base == ~0ull) return false;
+    __syncwarp();
+    for (uint32_t i = lane; i < nout; i += 32) __stcg(b.pool + base + i, s.out[i]);
+    if (lane == 0) {
+        __stcg(b.ccap + q, cap);
+        __stcg(b.clen + q, nout);
+        __stcg(b.coff + q, base);
+    }
+    __syncwarp();
+    return true;
+}
+
+// The columns of list0 (FlowSmall), then those it left (FlowBig), one per warp
+// at a time.
+template <class W>
+__global__ void __launch_bounds__(kFW * 32, W::kBig ? 1 : 3) k_h1_flow(const __grid_constant__ FlowArgs a) {
+    extern __shared__ __align__(16) unsigned char sh_flow[];
+    Counters* ctr = a.ctr;
+    if (ld_acquire_u32(&ctr->status) & kStSkip) return;
+    const H1Bufs& b = a.b;
+    W& s = reinterpret_cast<W*>(sh_flow)[threadIdx.x >> 5];
+    const uint32_t nl = min(b.ctl->nl, b.mcap);
+    const uint32_t n = W::kBig ? b.ctl->flow_left : nl;
+    const uint32_t* list = W::kBig ? b.list[0] : b.list0;
+    uint32_t* next = W::kBig ? &b.ctl->flow_next2 : &b.ctl->flow_next;
+    const uint64_t t_start = global_timer_ns();
+    uint64_t scratch = 0;
+    uint32_t scratch_cap = 0;
+    for (;;) {
+        uint32_t i = 0;
+        if (lane_id() == 0) i = atomicAdd(next, 1u);
+        i = __shfl_sync(0xFFFFFFFFu, i, 0);
+        if (i >= n || (ld_acquire_u32(&ctr->status) & kStSkip)) break;
+        const uint32_t q = list[i];
+        if (!CP_IN(q, b.n_ids, ctr)) continue;
+        if (!flow_column(a, s, q, scratch, scratch_cap, t_start) && !W::kBig && lane_id() == 0) {
+            const uint32_t k = atomicAdd(&b.ctl->flow_left, 1u);
+            if (k < b.mcap) b.list[0][k] = q;
+        }
+        __syncwarp();
+    }
 }
 
 __global__ void __launch_bounds__(kRT) k_h1_reduce(const __grid_constant__ ReduceArgs a) {
@@ -1036,7 +1417,22 @@ cudaError_t launch_h1(const ItemTable& tab, const H1Bufs& b, Counters* ctr, cp_p
     if (e != cudaSuccess) return e;
     k_h1_direct<<<grid_of(v1 - v0), kHT, 0, s>>>(tab, b, v0, v1);
     k_h1_local<<<grid_of(v1 - v0), kHT, 0, s>>>(tab, b, v0, v1);
-    note_launches(2);
+    const int flow_blocks = device_cached(kCacheFlow, [] {
+        const bool ok = cudaFuncSetAttribute(k_h1_flow<FlowSmall>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             int(sizeof(FlowSmall) * kFW)) == cudaSuccess &&
+                        cudaFuncSetAttribute(k_h1_flow<FlowBig>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             int(sizeof(FlowBig) * kFW)) == cudaSuccess;
+        return ok ? device_sm_count() : -1;
+    });
+    if (flow_blocks <= 0) return cudaErrorLaunchOutOfResources;
+    FlowArgs fa;
+    fa.tab = tab;
+    fa.b = b;
+    fa.ctr = ctr;
+    fa.budget_ns = uint64_t(get_h1_budget_ms()) * 1000000ull;
+    k_h1_flow<FlowSmall><<<3 * flow_blocks, kFW * 32, sizeof(FlowSmall) * kFW, s>>>(fa);
+    k_h1_flow<FlowBig><<<flow_blocks, kFW * 32, sizeof(FlowBig) * kFW, s>>>(fa);
+    note_launches(4);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     ReduceArgs ra;
     ra.tab = tab;

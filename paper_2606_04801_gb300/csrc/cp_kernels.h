@@ -253,12 +253,14 @@ struct H1Ctl {
     uint32_t stop[2];             // a round's merges hit an error (read one round later, by parity)
     uint32_t solo_round;          // the round from which the first CTA ran the rounds alone (0: never)
     unsigned long long grown;     // pool entries taken by merged columns
+    unsigned long long flow_grown;  // pool entries asked for by the star replacement (before them in the pool)
     unsigned long long t_grid_ns, t_solo_ns;  // wall time of the rounds on the whole grid / in one CTA
     unsigned long long t_phase_ns[4];  // thread 0 of CTA 0, summed over rounds: its bids, the wait after
                                        // them, its merges, the wait after them
     unsigned long long additions, merged;  // column additions, and the entries they read
     uint32_t park_gen, park_exit, park_round, park_nchg;  // the first CTA wakes the parked ones
     uint32_t solo_entries;        // times the first CTA went on alone
+    uint32_t flow_next, flow_left, flow_next2;  // star replacement: columns taken, left to the second launch, taken there
     uint32_t nw_hist[16];         // rounds by losing columns: bucket floor(log2(count)), capped at 15
 };
 struct H1Bufs {
@@ -337,7 +339,7 @@ cudaError_t launch_backward(const cp_pair* pairs, int64_t n, const float* gb, co
 int device_sm_count();
 // init() run once per device and slot (thread-safe), its result cached: the
 // launch set-up of a kernel (attributes, occupancy-derived grid size).
-enum { kCachePrune3d, kCachePrune2d, kCacheSort, kCacheUf, kCacheRoots, kCacheH1, kCacheBoruvka, kCacheTree, kCacheSlots };
+enum { kCachePrune3d, kCachePrune2d, kCacheSort, kCacheUf, kCacheRoots, kCacheH1, kCacheFlow, kCacheBoruvka, kCacheTree, kCacheSlots };
 int device_cached(int slot, int (*init)());
 
 // Kernel launches made by the library (for the benchmark's launch count).
