@@ -90,8 +90,14 @@ struct Plan {
     uint32_t cap_s = 0, cap_r0 = 0, cap_rt = 0, cap_p = 0, cap_big = 0;
     // byte offsets into the workspace
     size_t o_ctr, o_uf0, o_uft, o_s0, o_st, o_salt, o_age0, o_res0, o_aget, o_rest;
-    size_t o_act0, o_act1, o_yn, o_on, o_na0, o_na1, o_nb0, o_nb1, o_pairs, o_pvals, o_pvalt, o_hist, o_status;
+    size_t o_act0, o_act1, o_yn, o_on, o_na0, o_na1, o_nb0, o_nb1, o_pairs, o_hist, o_status;
     size_t o_hist2, o_status2;
+    // output order: places, buckets and their counts (behind the counters: zeroed with them)
+    uint64_t base[kMaxItems], cells[kMaxItems];
+    int order_shift = 0;
+    uint32_t buckets = 0;
+    int chunk_shift = 0;
+    size_t o_count, o_chunk, o_start, zero_bytes;
     size_t o_node0, o_nodet;  // merge-tree nodes
     size_t o_code;            // link codes of the 3D items
     uint64_t n_code = 0;
@@ -146,7 +152,7 @@ int plan_zchunk(const ItemTable& tab) {
 // h1: also lay out the H1 stage of the 3D items, with h1_pool pool entries
 // for the columns that additions create (0: 4 per column + 2^20).
 int make_plan(int n_items, const int32_t* ndims, const int64_t* dims, const float* const* imgs,
-              int64_t max_survivors, Plan& P, bool h1 = false, int64_t h1_pool = 0) {
+              int64_t max_survivors, Plan& P, bool h1 = false, int64_t h1_pool = 0, bool t_mode = false) {
     if (n_items <= 0 || n_items > kMaxItems || !ndims || !dims) return CP_ERR_ARG;
     std::memset(&P.tab, 0, sizeof(P.tab));
     P.tab.n = n_items;
@@ -250,6 +256,22 @@ int make_plan(int n_items, const int32_t* ndims, const int64_t* dims, const floa
         return at;
     };
     P.o_ctr = take(sizeof(Counters));
+    // places of the output order: per item (as the caller counts them) and
+    // dimension class, the cells of its doubled grid (T calls: of the image
+    // that the dual image stands for)
+    uint64_t places = 0;
+    for (int i = 0; i < n_items; ++i) {
+        uint64_t g = 1;
+        for (int k = ndims[i] == 3 ? 0 : 1; k < 3; ++k) g *= uint64_t(t_mode ? 2 * (dims[3 * i + k] - 2) + 1 : 2 * dims[3 * i + k] - 1);
+        P.base[i] = places;
+        P.cells[i] = g;
+        places += g * (P.h1 ? 3u : 2u);
+    }
+    plan_order(places, &P.order_shift, &P.chunk_shift, &P.buckets);
+    P.o_count = take(sizeof(uint32_t) * ((size_t(P.buckets) + 3) & ~size_t(3)));
+    P.zero_bytes = o;
+    P.o_chunk = take(sizeof(uint32_t) * order_chunks());
+    P.o_start = take(sizeof(uint32_t) * ((size_t(P.buckets) + 3) & ~size_t(3)));
     P.o_uf0 = take(sizeof(uint32_t) * size_t(P.ntot));
     P.o_uft = take(sizeof(uint32_t) * size_t(P.ttot));
     P.o_code = take(size_t(P.n_code) + 16);
@@ -273,8 +295,6 @@ int make_plan(int n_items, const int32_t* ndims, const int64_t* dims, const floa
     // the pairs buffer also holds the dual list's sort scratch (key ping-pong,
     // endpoint root ids, payload) while both survivor lists are sorted together
     P.o_pairs = take(std::max(sizeof(cp_pair) * size_t(P.cap_p), size_t(8 + 4 + 4 + 4) * P.cap_s + 1024));
-    P.o_pvals = P.o_act0;  // the active lists are dead once both union-finds are done
-    P.o_pvalt = P.o_act1;
     P.o_hist = take(sizeof(uint32_t) * 8 * 256);
     P.o_status = take(sizeof(uint64_t) * sort_status_words(P.cap_big));
     P.o_hist2 = take(sizeof(uint32_t) * 8 * 256);
@@ -363,9 +383,17 @@ void plan_boruvka(Plan& P) {
     P.bytes = o;
 }
 
+// The plans' arrays start at the first 256-byte boundary of the caller's
+// workspace (whose size counts kWsSlack bytes for it).
+constexpr size_t kWsSlack = 256;
+template <class P>
+P* ws_base(P* ws) {
+    return reinterpret_cast<P*>((reinterpret_cast<uintptr_t>(ws) + 255) & ~uintptr_t(255));
+}
+
 template <class T>
 T* at(void* ws, size_t off) {
-    return reinterpret_cast<T*>(static_cast<char*>(ws) + off);
+    return reinterpret_cast<T*>(static_cast<char*>(ws_base(ws)) + off);
 }
 
 int status_to_code(uint32_t st) {
@@ -386,7 +414,8 @@ struct TMode {
 
 int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, int64_t* d_out_count, void* ws,
         size_t ws_bytes, cudaStream_t s, bool prune_only = false, const TMode* tm = nullptr) {
-    if (!ws || ws_bytes < P.bytes || (!d_out && capacity > 0) || capacity < 0) return CP_ERR_ARG;
+    if (!ws || (!d_out && capacity > 0) || capacity < 0) return CP_ERR_ARG;
+    if (ws_bytes < P.bytes + kWsSlack) return CP_ERR_ARG;
     int rc = ensure_device_tables();
     if (rc != CP_OK) return rc;
     Counters* ctr = at<Counters>(ws, P.o_ctr);
@@ -411,7 +440,7 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
     } while (0)
     StageRanges nv;
     nv.next("cp.prune");
-    CP_TRY(cudaMemsetAsync(ctr, 0, sizeof(Counters), s));
+    CP_TRY(cudaMemsetAsync(ctr, 0, P.zero_bytes, s));
     // the merge tree takes both lists at once; the slab split, the Borůvka
     // variant and cross-pruning of images need the sorted lists and the rounds
     const bool joint = P.tab.n2d == 0 || !P.tab.cross2d;
@@ -772,6 +801,12 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
         ta.cap = P.cap_s;
         ta.ctr = ctr;
         CP_TRY(launch_tree(ta, s));
+        mark(4, s);
+        mark(5, s);
+    }
+
+    nv.next("cp.emit");
+    if (tree && P.h1) {
         TreeEmitArgs te;
         te.tab = P.tab;
         te.node[0] = node0;
@@ -784,48 +819,44 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
         te.pair_cap = P.cap_p;
         te.ctr = ctr;
         CP_TRY(launch_tree_emit(te, s));
-        mark(4, s);
-        mark(5, s);
     }
-
-    nv.next("cp.emit");
-    CP_TRY(launch_essential(P.tab, ctr, pairs, P.cap_p, s));
+    // (T calls have no other essential class than the one their pairs map to)
+    const bool from_trees = tree && !P.h1;
+    if (!from_trees && !tm) CP_TRY(launch_essential(P.tab, ctr, pairs, P.cap_p, s));
     if (P.h1) {
         nv.next("cp.h1");
         CP_TRY(launch_h1(P.tab, hb, ctr, pairs, P.cap_p, s));
         nv.next("cp.emit");
     }
-    uint32_t* pvals = at<uint32_t>(ws, P.o_pvals);
-    uint32_t* pvalt = at<uint32_t>(ws, P.o_pvalt);
-    // output order (item, dim, birth cell): only as many key bytes as this call's
-    // item count and largest doubled grid need (4 for one 512^3 volume)
-    int cell_bits = 1, item_bits = 0;
-    for (int i = 0; i < P.tab.n; ++i) {
-        const Item& it = P.tab.it[i];
-        int64_t G = int64_t(2 * it.D - 1) * (2 * it.H - 1) * (2 * it.W - 1);
-        if (tm) {  // the T-complex of the original image
-            const TDims& d = tm->items.d[it.user];
-            G = (d.ndim == 3 ? 2 * d.D + 1 : 1) * (2 * d.H + 1) * (2 * d.W + 1);
-        }
-        while ((int64_t(1) << cell_bits) < G) ++cell_bits;
-    }
-    if (tm) CP_TRY(launch_t_map(pairs, &ctr->n_pairs, P.cap_p, tm->items, tm->bad, ctr, s));
-    // T calls: one more item index, for the dropped frame classes
-    while ((1 << item_bits) < P.tab.n + (tm ? 1 : 0)) ++item_bits;
-    const int dim_bits = P.h1 ? 2 : 1;
-    int pair_passes = (item_bits + dim_bits + cell_bits + 7) / 8;
-    pair_passes += pair_passes & 1;  // an even count leaves the result in place
-    CP_TRY(launch_pair_keys(pairs, &ctr->n_pairs, P.cap_p, s0, pvals, cell_bits, dim_bits, s));
-    sb.keys = s0;
-    sb.keys_alt = salt;
-    sb.vals = pvals;
-    sb.vals_alt = pvalt;
-    sb.d_count = &ctr->n_pairs;
-    sb.cap = P.cap_p;
-    sb.tile_ctr = ctr->sort_tile + 16;
-    CP_TRY(sort_keys(sb, 0, pair_passes, 17, s));
-    CP_TRY(launch_gather(pairs, pvals, tm ? &ctr->t_keep : &ctr->n_pairs, P.cap_p, d_out, capacity, d_out_count, ctr,
-                         s));
+    OrderArgs oa;
+    oa.tab = P.tab;
+    oa.node[0] = node0;
+    oa.node[1] = nodet;
+    oa.n_rids[0] = P.cap_r0;
+    oa.n_rids[1] = P.cap_rt;
+    oa.from_trees = from_trees ? 1 : 0;
+    oa.t_mode = tm ? 1 : 0;
+    if (tm) std::memcpy(oa.t, tm->items.d, sizeof(oa.t));
+    oa.t_bad = tm ? tm->bad : nullptr;
+    oa.classes = P.h1 ? 3 : 2;
+    std::memcpy(oa.base, P.base, sizeof(oa.base));
+    std::memcpy(oa.cells, P.cells, sizeof(oa.cells));
+    oa.shift = P.order_shift;
+    oa.buckets = P.buckets;
+    oa.count = at<uint32_t>(ws, P.o_count);
+    oa.chunk_shift = P.chunk_shift;
+    oa.chunk = at<uint32_t>(ws, P.o_chunk);
+    oa.start = at<uint32_t>(ws, P.o_start);
+    oa.slot = act0;  // the union-finds' lists and logs are dead by now
+    oa.sorted = reinterpret_cast<uint2*>(salt);
+    oa.pairs = pairs;
+    oa.pair_cap = P.cap_p;
+    oa.out = d_out;
+    oa.out_cap = capacity;
+    oa.out16 = (reinterpret_cast<uintptr_t>(d_out) & 15u) == 0 ? 1 : 0;
+    oa.d_out_count = d_out_count;
+    oa.ctr = ctr;
+    CP_TRY(launch_order(oa, s));
     mark(6, s);
 #undef CP_TRY
     if (h_out_count) {
@@ -877,9 +908,9 @@ size_t t_workspace(int n_items, const int32_t* ndims, const int64_t* dims, int64
     std::vector<int64_t> jd;
     if (!t_extents(n_items, ndims, dims, t, jd)) return 0;
     Plan P;
-    if (make_plan(n_items, ndims, jd.data(), nullptr, max_survivors, P) != CP_OK) return 0;
+    if (make_plan(n_items, ndims, jd.data(), nullptr, max_survivors, P, false, 0, true) != CP_OK) return 0;
     if (v_bytes) *v_bytes = P.bytes;
-    size_t b = align_up(P.bytes) + 256;
+    size_t b = align_up(P.bytes) + 256 + kWsSlack;
     for (int i = 0; i < n_items; ++i) b += align_up(sizeof(float) * size_t(jd[3 * i] * jd[3 * i + 1] * jd[3 * i + 2]));
     return b;
 }
@@ -893,10 +924,10 @@ int t_run(int n_items, const float* const* h_images, const int32_t* ndims, const
     if (!t_extents(n_items, ndims, dims, tm.items, jd)) return CP_ERR_ARG;
     size_t v_bytes = 0;
     const size_t need = t_workspace(n_items, ndims, dims, max_survivors, &v_bytes);
+    char* base = static_cast<char*>(ws_base(ws));
     if (need == 0 || ws_bytes < need) return CP_ERR_ARG;
     int rc = ensure_device_tables();
     if (rc != CP_OK) return rc;
-    char* base = static_cast<char*>(ws);
     uint32_t* bad = reinterpret_cast<uint32_t*>(base + align_up(v_bytes));
     size_t off = align_up(v_bytes) + 256;
     std::vector<const float*> jptr(static_cast<size_t>(n_items));
@@ -908,7 +939,7 @@ int t_run(int n_items, const float* const* h_images, const int32_t* ndims, const
         off += align_up(sizeof(float) * size_t(jd[3 * i] * jd[3 * i + 1] * jd[3 * i + 2]));
     }
     Plan P;
-    rc = make_plan(n_items, ndims, jd.data(), jptr.data(), max_survivors, P);
+    rc = make_plan(n_items, ndims, jd.data(), jptr.data(), max_survivors, P, false, 0, true);
     if (rc != CP_OK) return rc;
     for (int j = 0; j < P.tab.n; ++j) {
         const Item& it = P.tab.it[j];
@@ -919,7 +950,7 @@ int t_run(int n_items, const float* const* h_images, const int32_t* ndims, const
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (launch_t_build(tm.items, bad, s) != cudaSuccess) return CP_ERR_CUDA;
     tm.bad = bad;
-    return run(P, d_out, capacity, h_out_count, d_out_count, ws, v_bytes, s, false, &tm);
+    return run(P, d_out, capacity, h_out_count, d_out_count, base, v_bytes + kWsSlack, s, false, &tm);
 }
 
 int t_single(int ndim, const float* d_image, const int64_t* dims, cp_pair* d_out, int64_t capacity,
@@ -1022,7 +1053,7 @@ size_t cubical_persistence_workspace_size(int ndim, const int64_t* dims, int64_t
     int64_t d3[3] = {ndim == 3 ? dims[0] : 1, dims[ndim - 2], dims[ndim - 1]};
     Plan P;
     if (make_plan(1, &nd, d3, nullptr, max_survivors, P) != CP_OK) return 0;
-    return P.bytes;
+    return P.bytes + kWsSlack;
 }
 
 int cubical_persistence_2d(const float* d_image, const int64_t dims[2], cp_pair* d_out_pairs, int64_t capacity,
@@ -1046,7 +1077,7 @@ size_t cubical_persistence_slabs_workspace_size(int ndim, const int64_t* dims, i
     Plan P;
     if (make_plan(1, &nd, d3, nullptr, max_survivors, P) != CP_OK) return 0;
     if (plan_slabs(P, n_slabs) != CP_OK) return 0;
-    return P.bytes;
+    return P.bytes + kWsSlack;
 }
 
 int cubical_persistence_slabs(int ndim, const float* d_image, const int64_t* dims, int n_slabs, cp_pair* d_out_pairs,
@@ -1150,7 +1181,7 @@ size_t cubical_persistence_batched_workspace_size(int n_items, const int32_t* nd
                                                   int64_t max_survivors) {
     Plan P;
     if (make_plan(n_items, ndims, dims, nullptr, max_survivors, P) != CP_OK) return 0;
-    return P.bytes;
+    return P.bytes + kWsSlack;
 }
 
 int cubical_persistence_batched(int n_items, const float* const* h_images, const int32_t* ndims, const int64_t* dims,
@@ -1168,7 +1199,7 @@ size_t cubical_persistence_full_batched_workspace_size(int n_items, const int32_
                                                        int64_t max_survivors, int64_t pool_entries) {
     Plan P;
     if (make_plan(n_items, ndims, dims, nullptr, max_survivors, P, true, pool_entries) != CP_OK) return 0;
-    return P.bytes;
+    return P.bytes + kWsSlack;
 }
 
 int cubical_persistence_full_batched(int n_items, const float* const* h_images, const int32_t* ndims,
@@ -1210,7 +1241,7 @@ int cubical_persistence_full_info(const void* d_workspace, int n_items, const in
     if (!P.h1) return CP_OK;
     H1Ctl c;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemcpyAsync(&c, static_cast<const char*>(d_workspace) + P.o_h1_ctl, sizeof(c), cudaMemcpyDeviceToHost,
+    if (cudaMemcpyAsync(&c, static_cast<const char*>(ws_base(d_workspace)) + P.o_h1_ctl, sizeof(c), cudaMemcpyDeviceToHost,
                         s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return CP_ERR_CUDA;
@@ -1244,7 +1275,7 @@ int cubical_persistence_stats(const void* d_workspace, cp_stats* h_stats, void* 
     if (!d_workspace || !h_stats) return CP_ERR_ARG;
     Counters h;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemcpyAsync(&h, d_workspace, sizeof(Counters), cudaMemcpyDeviceToHost, s) != cudaSuccess) return CP_ERR_CUDA;
+    if (cudaMemcpyAsync(&h, ws_base(d_workspace), sizeof(Counters), cudaMemcpyDeviceToHost, s) != cudaSuccess) return CP_ERR_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return CP_ERR_CUDA;
     std::memset(h_stats, 0, sizeof(*h_stats));
     h_stats->h0_survivors = h.n_s0;
@@ -1306,7 +1337,7 @@ int cubical_persistence_uf_trace2(const void* d_workspace, int dual, uint32_t* h
     if (!d_workspace || !h_active || !h_us || cap <= 0 || (dual != 0 && dual != 1)) return CP_ERR_ARG;
     Counters h;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (cudaMemcpyAsync(&h, d_workspace, sizeof(Counters), cudaMemcpyDeviceToHost, s) != cudaSuccess) return CP_ERR_CUDA;
+    if (cudaMemcpyAsync(&h, ws_base(d_workspace), sizeof(Counters), cudaMemcpyDeviceToHost, s) != cudaSuccess) return CP_ERR_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return CP_ERR_CUDA;
     uint32_t rounds = dual ? h.roundst : h.rounds0;
     int n = int(std::min<uint32_t>(rounds + 1, uint32_t(kTraceRounds)));

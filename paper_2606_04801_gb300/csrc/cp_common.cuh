@@ -12,6 +12,7 @@ constexpr int kVBits = 27;                        // global vertex id bits in a 
 constexpr uint64_t kVMask = (1ull << kVBits) - 1;
 constexpr uint32_t kTag = 0x80000000u;            // union-find word: root tag | root id
 constexpr int kMaxItems = CP_MAX_ITEMS;
+constexpr float kTFrame = -3.40282347e38f;        // T-filtration: value of the dual image's frame
 
 // status bits (device word)
 constexpr uint32_t kStNonfinite = 1u << 0;
@@ -63,7 +64,7 @@ struct Counters {
     uint32_t sort_tile[64];   // tile tickets of the sort passes of one call
     uint32_t find_ctr;        // work counter of the first union-find round's root walks
     uint32_t tma_tasks;       // 3D pruning work whose planes came by TMA, in blocks of 31 x 8 columns x zchunk3d planes
-    uint32_t t_keep;          // T-filtration calls: pairs kept after the mapping (the output count)
+    uint32_t order_bar;       // grid barrier of k_order
     uint32_t mst_rounds;      // Borůvka rounds (the spanning-forest union-find variant), else 0
     unsigned long long gmin[kMaxItems];  // (ord bits << 32 | local vertex) of each item's minimum
     int64_t out_count;

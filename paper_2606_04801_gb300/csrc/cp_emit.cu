@@ -1,7 +1,8 @@
-// K4: pair emission (outside vertices, essential class, canonical order) and
-// K5: the backward scatter.
+// The start of a call (outside vertices), the essential classes of calls whose
+// pairs are not emitted in k_order, and K5: the backward scatter.
 #include "cp_common.cuh"
 #include "cp_kernels.h"
+#include "cp_pairs.cuh"
 
 namespace cp {
 namespace {
@@ -10,7 +11,7 @@ constexpr int kT = 256;
 
 // One outside vertex per item: the oldest dual vertex (Sec. 3.1), never
 // paired (Appendix A.4); it takes dual root id = item index.
-__global__ void k_init(ItemTable tab, Counters* ctr, uint32_t* uft, uint64_t* aget, uint64_t* rest,
+__global__ void k_init(const __grid_constant__ ItemTable tab, Counters* ctr, uint32_t* uft, uint64_t* aget, uint64_t* rest,
                        TreeNode* nodet) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < tab.n) {
@@ -18,68 +19,20 @@ __global__ void k_init(ItemTable tab, Counters* ctr, uint32_t* uft, uint64_t* ag
         uft[it.toff + it.T] = kTag | uint32_t(i);
         aget[i] = ~0ull;
         rest[i] = 0;
-        if (nodet) nodet[i] = TreeNode{~0ull, uint64_t(i), 0, 0};  // older than every top cell
+        if (nodet) nodet[i] = TreeNode{~0ull, uint64_t(i), 0, uint64_t(i)};  // older than every top cell
         ctr->gmin[i] = ~0ull;
     }
     if (i == 0) ctr->n_rt = uint32_t(tab.n);
 }
 
-// The essential H0 class of each item: born at its minimum, never dies.
-__global__ void k_essential(ItemTable tab, Counters* ctr, cp_pair* pairs, uint32_t cap) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= tab.n) return;
-    const Item& it = tab.it[i];
-    unsigned long long g = ctr->gmin[i];
-    if (g == ~0ull) {
-        set_status(ctr, kStInternal);
-        return;
-    }
-    uint32_t v = uint32_t(g & 0xFFFFFFFFu);
-    int x = int(v % uint32_t(it.W)), y = int((v / uint32_t(it.W)) % uint32_t(it.H)), z = int(v / uint32_t(it.W * it.H));
+// The essential H0 class of each item.
+__global__ void k_essential(const __grid_constant__ ItemTable tab, Counters* ctr, cp_pair* pairs, uint32_t cap) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     cp_pair p;
-    p.birth = ord_float(uint32_t(g >> 32));
-    p.death = __int_as_float(0x7F800000);
-    p.birth_cell = int32_t(doubled_index(it, z, y, x, 0, 0, 0));
-    p.death_cell = -1;
-    p.birth_pixel = int32_t(v);
-    p.death_pixel = -1;
-    p.dim = 0;
-    p.item = it.user;
-    uint32_t pos = atomicAdd(&ctr->n_pairs, 1u);
+    if (i >= tab.n || !essential_pair(tab, ctr, i, p)) return;
+    const uint32_t pos = atomicAdd(&ctr->n_pairs, 1u);
     if (pos < cap) pairs[pos] = p;
     else set_status(ctr, kStCapacity);
-}
-
-// Canonical order: (item, dim, birth cell).
-// Sort key of the canonical output order (item, dim, birth cell), packed in
-// as few bits as the call needs: birth cells take cell_bits bits.
-__global__ void k_pair_keys(const cp_pair* __restrict__ pairs, const uint32_t* d_n, uint32_t cap,
-                            uint64_t* __restrict__ keys, uint32_t* __restrict__ vals, int cell_bits,
-                            int dim_bits) {
-    uint32_t n = min(*d_n, cap);
-    for (uint32_t i = blockIdx.x * kT + threadIdx.x; i < n; i += gridDim.x * kT) {
-        const cp_pair& p = pairs[i];
-        const uint32_t dc = dim_bits == 1 ? (p.dim > 0 ? 1u : 0u) : uint32_t(p.dim);
-        keys[i] = (uint64_t(uint32_t(p.item)) << (cell_bits + dim_bits)) | (uint64_t(dc) << cell_bits) |
-                  uint32_t(p.birth_cell);
-        vals[i] = i;
-    }
-}
-
-__global__ void k_gather(const cp_pair* __restrict__ pairs, const uint32_t* __restrict__ vals, const uint32_t* d_n,
-                         uint32_t cap, cp_pair* __restrict__ out, int64_t out_cap, int64_t* d_out_count,
-                         Counters* ctr) {
-    uint32_t n = min(*d_n, cap);
-    int64_t m = int64_t(n) < out_cap ? int64_t(n) : out_cap;
-    for (int64_t j = int64_t(blockIdx.x) * kT + threadIdx.x; j < m; j += int64_t(gridDim.x) * kT) {
-        uint32_t v = vals[j];
-        if (v < n) out[j] = pairs[v];  // always true unless a bounded wait gave up
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        ctr->out_count = int64_t(n);
-        if (d_out_count) *d_out_count = int64_t(n);
-        if (int64_t(n) > out_cap) set_status(ctr, kStCapacity);
-    }
 }
 
 __global__ void k_scatter(const cp_pair* __restrict__ pairs, int64_t n, const float* __restrict__ gb,
@@ -213,20 +166,6 @@ cudaError_t launch_init(const ItemTable& tab, Counters* ctr, uint32_t* uft, uint
 
 cudaError_t launch_essential(const ItemTable& tab, Counters* ctr, cp_pair* pairs, uint32_t cap, cudaStream_t s) {
     k_essential<<<1, kMaxItems, 0, s>>>(tab, ctr, pairs, cap);
-    note_launches(1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_pair_keys(const cp_pair* pairs, const uint32_t* d_n, uint32_t cap, uint64_t* keys, uint32_t* vals,
-                             int cell_bits, int dim_bits, cudaStream_t s) {
-    k_pair_keys<<<grid_for(cap), kT, 0, s>>>(pairs, d_n, cap, keys, vals, cell_bits, dim_bits);
-    note_launches(1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_gather(const cp_pair* pairs, const uint32_t* vals, const uint32_t* d_n, uint32_t cap,
-                          cp_pair* out, int64_t out_cap, int64_t* d_out_count, Counters* ctr, cudaStream_t s) {
-    k_gather<<<grid_for(cap), kT, 0, s>>>(pairs, vals, d_n, cap, out, out_cap, d_out_count, ctr);
     note_launches(1);
     return cudaGetLastError();
 }

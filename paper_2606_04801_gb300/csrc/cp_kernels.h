@@ -15,7 +15,7 @@ struct alignas(32) TreeNode {
     uint64_t key;     // ~0: connected with nothing older yet
     uint64_t parent;  // root id
     uint64_t age;     // smaller is older (the dual's age keys complemented)
-    uint64_t pad;
+    uint64_t item;    // index of its item in the call's table
 };
 struct PruneOuts {
     uint32_t* uf0;   // H0 forest over global vertices (3D items: root words only)
@@ -322,24 +322,45 @@ cudaError_t launch_t_build(const TItems& t, uint32_t* bad, cudaStream_t s);
 // After the pruning pass: every frame vertex's H0 link points at the item's
 // vertex 0 (3D: has the code that says so).
 cudaError_t launch_t_flatten(uint32_t* uf0, uint8_t* code, const TItems& t, cudaStream_t s);
-// V pairs of J -> T pairs of the images, in place; each item's frame class
-// gets item index n (it sorts after every kept pair), ctr->t_keep the count
-// without them, and a set *bad flags the call as non-finite.
-cudaError_t launch_t_map(cp_pair* pairs, const uint32_t* d_n, uint32_t cap, const TItems& t, const uint32_t* bad,
-                         Counters* ctr, cudaStream_t s);
 cudaError_t launch_essential(const ItemTable& tab, Counters* ctr, cp_pair* pairs, uint32_t pair_cap, cudaStream_t s);
-// dim_bits 1: dimension 0 or top; 2: dimension 0, 1 or 2 (calls with H1)
-cudaError_t launch_pair_keys(const cp_pair* pairs, const uint32_t* d_n, uint32_t cap, uint64_t* keys, uint32_t* vals,
-                             int cell_bits, int dim_bits, cudaStream_t s);
-cudaError_t launch_gather(const cp_pair* pairs, const uint32_t* vals, const uint32_t* d_n, uint32_t cap,
-                          cp_pair* out, int64_t out_cap, int64_t* d_out_count, Counters* ctr, cudaStream_t s);
+// Emission (tree calls), output order and gather (cp_order.cu).
+struct OrderArgs {
+    ItemTable tab;
+    const TreeNode* node[2];    // from_trees
+    uint32_t n_rids[2];
+    int from_trees;             // 1: the pairs come from the merge trees; 0: they are in `pairs` already
+    int t_mode;                 // map the V pairs of the dual images to T pairs (extents t, by the caller's index)
+    TDims t[kMaxItems];
+    const uint32_t* t_bad;      // T calls: set if a pixel does not lie below the largest finite float
+    int classes;                // dimension classes of an item's places (2: 0 and top; 3: calls with H1)
+    uint64_t base[kMaxItems];   // first place of an item, by the caller's index
+    uint64_t cells[kMaxItems];  // places per class: the cells of its doubled grid
+    int shift;
+    uint32_t buckets;
+    int chunk_shift;            // buckets per chunk of the scan
+    uint32_t* count;            // per bucket, zeroed
+    uint32_t* start;
+    uint32_t* chunk;            // per chunk: its pairs
+    uint32_t* slot;             // per pair: its number in its bucket
+    uint2* sorted;              // (place in the bucket, pair) in bucket order
+    cp_pair* pairs;
+    uint32_t pair_cap;
+    cp_pair* out;
+    int64_t out_cap;
+    int out16;                  // out is 16-byte aligned
+    int64_t* d_out_count;
+    Counters* ctr;
+};
+void plan_order(uint64_t places, int* shift, int* chunk_shift, uint32_t* buckets);
+size_t order_chunks();
+cudaError_t launch_order(const OrderArgs& a, cudaStream_t s);
 cudaError_t launch_backward(const cp_pair* pairs, int64_t n, const float* gb, const float* gd, const int64_t* offs,
                             double* acc, float* grad, int64_t n_pixels, cudaStream_t s);
 
 int device_sm_count();
 // init() run once per device and slot (thread-safe), its result cached: the
 // launch set-up of a kernel (attributes, occupancy-derived grid size).
-enum { kCachePrune3d, kCachePrune2d, kCacheSort, kCacheUf, kCacheRoots, kCacheH1, kCacheFlow, kCacheBoruvka, kCacheTree, kCacheSlots };
+enum { kCachePrune3d, kCachePrune2d, kCacheSort, kCacheUf, kCacheRoots, kCacheH1, kCacheFlow, kCacheBoruvka, kCacheTree, kCacheOrder, kCacheSlots };
 int device_cached(int slot, int (*init)());
 
 // Kernel launches made by the library (for the benchmark's launch count).

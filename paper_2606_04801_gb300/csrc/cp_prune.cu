@@ -78,13 +78,13 @@ __device__ __forceinline__ int tile_item(const ItemTable& t, int first, int last
 // reservation words.  Beyond the capacity: a bare tag keeps the forest well
 // formed (the call is flagged).
 __device__ __forceinline__ void put_root(uint32_t* word, uint32_t g, uint32_t cap, uint64_t age, TreeNode* node,
-                                         uint64_t* ages, uint64_t* res, bool dual) {
+                                         uint64_t* ages, uint64_t* res, bool dual, int item) {
     if (g >= cap) {
         *word = kTag;
         return;
     }
     if (node) {
-        node[g] = TreeNode{~0ull, uint64_t(g), dual ? ~age : age, 0};
+        node[g] = TreeNode{~0ull, uint64_t(g), dual ? ~age : age, uint64_t(item)};
     } else {
         ages[g] = age;
         res[g] = 0;
@@ -170,6 +170,7 @@ struct Task3 {
     const float* img;
     int D, H, W, x0, y0, z0, z1, zlast;  // owned planes [z0, z1), zlast = z1 - 1
     uint32_t HW, W1, HW1, voff, toff, pitch;
+    int item;                // its index in the call's table
     uint8_t* code;           // the item's link codes
     const CUtensorMap* map;  // nullptr: the planes come by cp.async
     uint32_t own[2], cube[2];       // even / odd columns whose vertex / top cell the task owns
@@ -603,12 +604,12 @@ __device__ __noinline__ unsigned long long event_batch(Smem3& sm, const Outs& o,
     unsigned long long gmin = ~0ull;
     if (root0 && CP_IN(vg, o.n_uf0, o.ctr)) {
         gmin = (unsigned long long)(uint64_t(ord) << 32 | vl);
-        put_root(o.uf0 + vg, g0, o.cap_r0, make_key(ord, vg, 0), o.node0, o.age0, o.res0, false);
+        put_root(o.uf0 + vg, g0, o.cap_r0, make_key(ord, vg, 0), o.node0, o.age0, o.res0, false, t.item);
     }
     if (rootT) {  // the top cell whose smallest corner is this vertex, in slot 7 of its lower star
         const uint32_t self = t.toff + uint32_t(z) * t.HW1 + uint32_t(y) * t.W1 + uint32_t(x);
         if (CP_IN(self, o.n_uft, o.ctr))
-            put_root(o.uft + self, gt, o.cap_rt, make_key(ord, vg, 26u), o.nodet, o.aget, o.rest, true);
+            put_root(o.uft + self, gt, o.cap_rt, make_key(ord, vg, 26u), o.nodet, o.aget, o.rest, true, t.item);
     }
     uint32_t bits = __reduce_or_sync(0xFFFFFFFFu, h0s);
     while (bits) {
@@ -658,6 +659,7 @@ __device__ __forceinline__ void prune_task3d(Smem3& sm, const ItemTable& tab, co
     t.voff = uint32_t(it.voff);
     t.toff = uint32_t(it.toff);
     t.pitch = uint32_t(it.pitch);
+    t.item = ii;
     t.code = o.code + it.coff;
     t.map = map;
     __syncthreads();  // everything in shared memory may still be read by the previous task
@@ -887,6 +889,8 @@ struct WarpStage2 {
     uint64_t rtage[kCapWR];
     uint32_t r0node[kCapWR];
     uint32_t rtnode[kCapWR];
+    uint8_t r0item[kCapWR];
+    uint8_t rtitem[kCapWR];
 };
 
 struct Smem2 {
@@ -923,10 +927,10 @@ __device__ __forceinline__ void warp_flush(WS& ws, WarpCounts& c, const Outs& o)
         if (bt + i < o.cap_s) o.st[bt + i] = ws.st[i];
     for (uint32_t i = lane; i < c.r0; i += 32)
         if (CP_IN(ws.r0node[i], o.n_uf0, o.ctr))
-            put_root(o.uf0 + ws.r0node[i], br0 + i, o.cap_r0, ws.r0age[i], o.node0, o.age0, o.res0, false);
+            put_root(o.uf0 + ws.r0node[i], br0 + i, o.cap_r0, ws.r0age[i], o.node0, o.age0, o.res0, false, ws.r0item[i]);
     for (uint32_t i = lane; i < c.rt; i += 32)
         if (CP_IN(ws.rtnode[i], o.n_uft, o.ctr))
-            put_root(o.uft + ws.rtnode[i], brt + i, o.cap_rt, ws.rtage[i], o.nodet, o.aget, o.rest, true);
+            put_root(o.uft + ws.rtnode[i], brt + i, o.cap_rt, ws.rtage[i], o.nodet, o.aget, o.rest, true, ws.rtitem[i]);
     c.s0 = c.st = c.r0 = c.rt = 0;
     __syncwarp();
 }
@@ -1110,6 +1114,7 @@ __global__ void __launch_bounds__(kW2 * 32) k_prune2d(ItemTable tab, Outs o) {
                     if (root0) {
                         const uint32_t p = cnt.r0 + __popc(m_r0 & lt);
                         ws.r0node[p] = vg;
+                        ws.r0item[p] = uint8_t(ii);
                         ws.r0age[p] = make_key(ord, vg, 0);
                         const unsigned long long kk = (unsigned long long)(uint64_t(ord) << 32 | vl);
                         my_min = kk < my_min ? kk : my_min;
@@ -1122,6 +1127,7 @@ __global__ void __launch_bounds__(kW2 * 32) k_prune2d(ItemTable tab, Outs o) {
                         const uint32_t mg = voff + my * W + mx;
                         const uint32_t p = cnt.rt + __popc(m_rt & lt);
                         ws.rtnode[p] = self;
+                        ws.rtitem[p] = uint8_t(ii);
                         ws.rtage[p] = make_key(ord_bits(best), mg, (6u * (t >> 1) + 2u * (t & 1u)) << 1);
                     }
                     cnt.rt += __popc(m_rt);

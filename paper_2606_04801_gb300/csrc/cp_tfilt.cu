@@ -25,8 +25,8 @@
 // T grid, vertex coordinate c of J becomes pixel n-c of I.
 //
 // Kernels: J itself (with a check that every pixel lies below the largest
-// finite float, so that the frame comes first), and the in-place mapping of
-// the V pairs before the canonical output sort.
+// finite float, so that the frame comes first), and the frame's links.  The V
+// pairs are mapped where they are put in order (cp_order.cu).
 #include "cp_common.cuh"
 #include "cp_kernels.h"
 
@@ -36,7 +36,7 @@ namespace {
 constexpr int kTT = 256;
 // The frame value: below every value of -I as long as every pixel is below
 // the largest finite float (a pixel at that float, or above it, is flagged).
-constexpr float kFrame = -3.40282347e38f;
+constexpr float kFrame = kTFrame;
 
 // J four rows at a time, item blockIdx.y (the rows' divisions once per group;
 // consecutive threads write consecutive x and read consecutive, reversed,
@@ -133,82 +133,6 @@ __global__ void __launch_bounds__(kTT) k_t_flatten(uint32_t* __restrict__ uf0, u
     }
 }
 
-// Doubled-grid index in J -> doubled-grid index in the T-complex of I.
-__device__ __forceinline__ int32_t t_cell(const TDims& t, int32_t vc) {
-    if (vc < 0) return -1;
-    const int64_t GWv = 2 * (t.W + 2) - 1, GHv = 2 * (t.H + 2) - 1;
-    const int64_t X = vc % GWv, Y = (vc / GWv) % GHv, Z = vc / (GWv * GHv);
-    const int64_t GWt = 2 * t.W + 1, GHt = 2 * t.H + 1, GDt = t.ndim == 3 ? 2 * t.D + 1 : 1;
-    const int64_t tx = GWt - X, ty = GHt - Y, tz = t.ndim == 3 ? GDt - Z : 0;
-    if (tx < 0 || tx >= GWt || ty < 0 || ty >= GHt || tz < 0 || tz >= GDt) return -1;  // a frame cell
-    return int32_t((tz * GHt + ty) * GWt + tx);
-}
-
-// Vertex of J -> pixel of I.
-__device__ __forceinline__ int32_t t_pixel(const TDims& t, int32_t vp) {
-    if (vp < 0) return -1;
-    const int64_t Wj = t.W + 2, Hj = t.H + 2;
-    const int64_t x = vp % Wj, y = (vp / Wj) % Hj, z = vp / (Wj * Hj);
-    const int64_t iz = t.ndim == 3 ? t.D - z : 0;
-    return int32_t((iz * t.H + (t.H - y)) * t.W + (t.W - x));
-}
-
-__device__ __forceinline__ float neg_canon(float v) {
-    const float r = -v;
-    return r == 0.0f ? 0.0f : r;  // -0.0 reads as +0.0
-}
-
-__global__ void __launch_bounds__(kTT) k_t_map(cp_pair* __restrict__ pairs, const uint32_t* d_n, uint32_t cap,
-                                               const __grid_constant__ TItems ti, const uint32_t* bad,
-                                               Counters* ctr) {
-    const uint32_t n = min(*d_n, cap);
-    for (uint32_t i = blockIdx.x * kTT + threadIdx.x; i < n; i += gridDim.x * kTT) {
-        const cp_pair p = pairs[i];
-        const TDims& t = ti.d[(p.item >= 0 && p.item < ti.n) ? p.item : 0];
-        const int top = t.ndim - 1;
-        cp_pair q;
-        q.item = p.item;
-        if (p.dim == 0 && p.death_cell < 0) {
-            // an item's frame class (the outside of its T-complex): dropped; its
-            // item index one past the last sorts it after every kept pair,
-            // outside the kept count
-            q = p;
-            q.item = ti.n;
-            q.dim = 0;
-            q.birth_cell = 0;
-        } else if (p.dim == top && p.birth == kFrame) {
-            // the last merge into the outside, through a frame facet: the T
-            // essential class, born at the T vertex dual to the dying top cell
-            q.dim = 0;
-            q.birth = neg_canon(p.death);
-            q.death = __int_as_float(0x7F800000);
-            q.birth_cell = t_cell(t, p.death_cell);
-            q.death_cell = -1;
-            q.birth_pixel = t_pixel(t, p.death_pixel);
-            q.death_pixel = -1;
-        } else {
-            q.dim = p.dim == 0 ? top : 0;
-            q.birth = neg_canon(p.death);
-            q.death = neg_canon(p.birth);
-            q.birth_cell = t_cell(t, p.death_cell);
-            q.death_cell = t_cell(t, p.birth_cell);
-            q.birth_pixel = t_pixel(t, p.death_pixel);
-            q.death_pixel = t_pixel(t, p.birth_pixel);
-        }
-        pairs[i] = q;
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        ctr->t_keep = n > uint32_t(ti.n) ? n - uint32_t(ti.n) : 0u;  // one frame class per item
-        if (*bad) set_status(ctr, kStNonfinite);
-    }
-}
-
-int grid_of(int64_t n) {
-    const int64_t b = (n + kTT - 1) / kTT;
-    const int64_t cap = int64_t(device_sm_count()) * 8;
-    return int(b < 1 ? 1 : (b < cap ? b : cap));
-}
-
 }  // namespace
 
 cudaError_t launch_t_build(const TItems& t, uint32_t* bad, cudaStream_t s) {
@@ -225,13 +149,6 @@ cudaError_t launch_t_flatten(uint32_t* uf0, uint8_t* code, const TItems& t, cuda
     if (t.n < 1 || t.n > kMaxItems) return cudaErrorInvalidValue;
     const int gx = (device_sm_count() * 8 + t.n - 1) / t.n;
     k_t_flatten<<<dim3(gx, t.n), kTT, 0, s>>>(uf0, code, t);
-    note_launches(1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_t_map(cp_pair* pairs, const uint32_t* d_n, uint32_t cap, const TItems& t, const uint32_t* bad,
-                         Counters* ctr, cudaStream_t s) {
-    k_t_map<<<grid_of(cap), kTT, 0, s>>>(pairs, d_n, cap, t, bad, ctr);
     note_launches(1);
     return cudaGetLastError();
 }

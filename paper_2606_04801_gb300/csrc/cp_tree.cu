@@ -150,7 +150,9 @@ __global__ void __launch_bounds__(kTT) k_tree(const __grid_constant__ TreeArgs a
     if (lane_id() == 0 && hops) atomicAdd(&ctr->trace_hops[0][1], (unsigned long long)hops);
 }
 
-// The pair of every root that the tree connects with an older one.
+// The pair of every root that the tree connects with an older one (calls with
+// H1, whose reduction needs the committed survivors marked; the others emit in
+// k_order).
 __global__ void __launch_bounds__(kTT) k_tree_emit(const __grid_constant__ TreeEmitArgs a) {
     Counters* ctr = a.ctr;
     if (ld_acquire_u32(&ctr->status) & (kStTimeout | kStNonfinite)) return;
@@ -161,16 +163,7 @@ __global__ void __launch_bounds__(kTT) k_tree_emit(const __grid_constant__ TreeE
         cp_pair pr;
         if (g < n) {
             const int q = g >= r0 ? 1 : 0;
-            const TreeNode& nd = a.node[q][q ? g - r0 : g];
-            if (nd.key != ~0ull) {
-                const uint64_t key = q ? ~nd.key : nd.key;
-                const int item = item_of_vertex(a.tab, key_vertex(key));
-                if (a.h1flags[q] && a.tab.it[item].ndim == 3) {
-                    const uint32_t id = cell_id3(a.tab.it[item], key, q != 0);
-                    atomicOr(a.h1flags[q] + (id >> 5), 1u << (id & 31u));
-                }
-                emit = commit_pair(a.tab, q ? ~nd.age : nd.age, q, key, item, pr);
-            }
+            emit = tree_pair(a.tab, a.node[q][q ? g - r0 : g], q, a.h1flags[q], pr);
         }
         const uint32_t pp = warp_append(&ctr->n_pairs, emit);
         if (emit) {
