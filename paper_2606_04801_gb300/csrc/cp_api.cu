@@ -293,10 +293,24 @@ int make_plan(int n_items, const int32_t* ndims, const int64_t* dims, const floa
         places += g * (P.h1 ? 3u : 2u);
     }
     plan_order(places, &P.order_shift, &P.chunk_shift, &P.buckets);
-    P.o_count = take(sizeof(uint32_t) * ((size_t(P.buckets) + 3) & ~size_t(3)));
+    uint32_t room = P.buckets;
+    if (t_mode) {  // never less room than the same dims take without t_mode
+        uint64_t all = 0;
+        for (int i = 0; i < n_items; ++i) {
+            uint64_t g = 1;
+            for (int k = ndims[i] == 3 ? 0 : 1; k < 3; ++k) g *= uint64_t(2 * dims[3 * i + k] - 1);
+            all += g * (P.h1 ? 3u : 2u);
+        }
+        int sh, ch;
+        uint32_t b;
+        plan_order(all, &sh, &ch, &b);
+        room = std::max(room, b);
+    }
+    const size_t count_bytes = sizeof(uint32_t) * ((size_t(room) + 3) & ~size_t(3));
+    P.o_count = take(count_bytes);
     P.zero_bytes = o;
     P.o_chunk = take(sizeof(uint32_t) * order_chunks());
-    P.o_start = take(sizeof(uint32_t) * ((size_t(P.buckets) + 3) & ~size_t(3)));
+    P.o_start = take(count_bytes);
     P.o_uf0 = take(sizeof(uint32_t) * size_t(P.ntot));
     P.o_uft = take(sizeof(uint32_t) * size_t(P.ttot));
     P.o_code = take(size_t(P.n_code) + 16);
