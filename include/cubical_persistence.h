@@ -398,6 +398,16 @@ int cubical_persistence_loss_backward(const cp_pair *d_pairs, int64_t n_pairs, c
                                       void *stream);
 
 /*
+ * Copies n_items (<= 128) arrays of floats on the device, counts[i] floats
+ * from d_src[i] to d_dst[i], in one launch on `stream` (the inputs of a
+ * batch to their places).  counts[i] = 0 skips an item, whose pointers are
+ * then not read.  Pointers are 4-byte aligned; no source may overlap another
+ * item's destination.  The three arrays are read before the call returns.
+ */
+int cubical_persistence_load_items(int n_items, const float *const *d_src, float *const *d_dst, const int64_t *counts,
+                                   void *stream);
+
+/*
  * Backward scatter that allocates nothing (the paper has no counterpart: it
  * is a convenience of this library).  For callers that cannot allocate
  * device memory, such as code inside another framework's hooks without

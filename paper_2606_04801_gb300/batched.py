@@ -85,8 +85,26 @@ class BatchedPersistence:
     def load(self, inputs: Sequence[torch.Tensor]):
         if len(inputs) != self.k:
             raise ValueError("wrong number of items")
-        for v, a in zip(self.views, inputs):
+        # plain float tensors on the device go in one launch, the rest (host or
+        # other types, strided, recorded by autograd, parts of this batch) by copy_
+        counts = [0] * self.k
+        ptrs = [0] * self.k
+        lo, hi = self.x.data_ptr(), self.x.data_ptr() + 4 * self.total
+        for i, (v, a, n) in enumerate(zip(self.views, inputs, self.sizes)):
+            if (type(a) is torch.Tensor and a.dtype is torch.float32 and a.device == self.dev and a.numel() == n
+                    and a.is_contiguous() and not a.requires_grad and not a.is_neg()):
+                p = a.data_ptr()
+                if p & 3 == 0 and (p >= hi or p + 4 * n <= lo):
+                    counts[i], ptrs[i] = n, p
+                    continue
             v.copy_(torch.as_tensor(a).reshape(v.shape), non_blocking=True)
+        if any(counts):
+            with torch.cuda.device(self.dev):
+                rc = self.lib.cubical_persistence_load_items(
+                    self.k, (ctypes.c_void_p * self.k)(*ptrs), self._ptrs, (ctypes.c_int64 * self.k)(*counts),
+                    ctypes.c_void_p(torch.cuda.current_stream(self.dev).cuda_stream))
+            if rc != CP_OK:
+                raise CpError(rc, "load_items")
 
     def _enqueue(self, stream_ptr: int):
         lib = self.lib

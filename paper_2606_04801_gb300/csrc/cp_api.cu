@@ -1415,6 +1415,23 @@ int cp_stage_times(float* ms, int cap) {
     return kStages;
 }
 
+int cubical_persistence_load_items(int n_items, const float* const* d_src, float* const* d_dst, const int64_t* counts,
+                                   void* stream) {
+    if (n_items < 1 || n_items > kMaxItems || !d_src || !d_dst || !counts) return CP_ERR_ARG;
+    LoadItems t;
+    t.n = 0;
+    for (int i = 0; i < n_items; ++i) {
+        if (counts[i] < 0 || counts[i] > (int64_t(1) << kVBits)) return CP_ERR_ARG;
+        if (counts[i] == 0) continue;
+        if (!d_src[i] || !d_dst[i] || ((reinterpret_cast<uintptr_t>(d_src[i]) | reinterpret_cast<uintptr_t>(d_dst[i])) & 3u))
+            return CP_ERR_ARG;
+        t.src[t.n] = d_src[i];
+        t.dst[t.n] = d_dst[i];
+        t.count[t.n++] = counts[i];
+    }
+    return launch_load_items(t, static_cast<cudaStream_t>(stream)) == cudaSuccess ? CP_OK : CP_ERR_CUDA;
+}
+
 size_t cubical_persistence_loss_backward_workspace_size(int64_t n_pixels) {
     if (n_pixels <= 0) return 0;
     return align_up(sizeof(double) * size_t(n_pixels)) + align_up(sizeof(double) * size_t(loss_partials()));

@@ -323,6 +323,16 @@ cudaError_t launch_t_build(const TItems& t, uint32_t* bad, cudaStream_t s);
 // vertex 0 (3D: has the code that says so).
 cudaError_t launch_t_flatten(uint32_t* uf0, uint8_t* code, const TItems& t, cudaStream_t s);
 cudaError_t launch_essential(const ItemTable& tab, Counters* ctr, cp_pair* pairs, uint32_t pair_cap, cudaStream_t s);
+// Items copied to their places in one launch (cp_load.cu): the items with a
+// count, packed to the front.
+struct LoadItems {
+    const float* src[kMaxItems];
+    float* dst[kMaxItems];
+    int64_t count[kMaxItems];  // floats, >= 1
+    int32_t chunk0[kMaxItems], n, chunks;
+};
+cudaError_t launch_load_items(LoadItems& t, cudaStream_t s);
+
 // Emission (tree calls), output order and gather (cp_order.cu).
 struct OrderArgs {
     ItemTable tab;

@@ -1,0 +1,47 @@
+"""BatchedPersistence.load: the packed inputs hold every item's values, from
+sources and to places on every 16-byte phase, and from the tensors that take
+the general copy (host, other types, strided, parts of the batch itself)."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+SHAPES = [(2, 2), (3, 5), (64, 64), (33, 31, 4), (4096, 2), (4095, 3), (2, 2, 3), (61, 67), (16, 16, 16), (129, 257)]
+
+
+def _at(phase, shape, dev="cuda"):
+    n = 1
+    for v in shape:
+        n *= v
+    return torch.rand(n + 4, device=dev)[phase : phase + n].view(shape)
+
+
+@pytest.mark.parametrize("phase", [0, 1, 2, 3])
+def test_every_phase(phase):
+    import paper_2606_04801_gb300 as cp
+
+    bp = cp.BatchedPersistence(SHAPES)
+    for turn in range(2):
+        xs = [_at((phase + turn * i) % 4, s) for i, s in enumerate(SHAPES)]
+        bp.load(xs)
+        assert torch.equal(bp.x, torch.cat([v.reshape(-1) for v in xs]))
+
+
+def test_general_copies_and_refusals():
+    import paper_2606_04801_gb300 as cp
+
+    shapes = [(5, 6)] * 10
+    bp = cp.BatchedPersistence(shapes)
+    xs = [torch.rand(5, 6), torch.rand(5, 6).numpy(), torch.rand(5, 6).double().cuda(), torch.rand(6, 5).cuda().t(),
+          torch.rand(30).cuda(), torch.rand(1, 5, 6).cuda(), torch.rand(5, 6).tolist(), torch._neg_view(torch.rand(5, 6).cuda()),
+          torch.randint(0, 9, (5, 6)).cuda(), torch.rand(5, 6).cuda()]
+    bp.load(xs)
+    assert torch.equal(bp.x, torch.cat([torch.as_tensor(v).to("cuda", torch.float32).reshape(-1) for v in xs]))
+    before = bp.views[1].clone()
+    bp.load([bp.views[1]] + [bp.views[0]] + xs[2:])  # in order, as copies one after the other
+    assert torch.equal(bp.views[0], before) and torch.equal(bp.views[1], before)
+    with pytest.raises(RuntimeError):
+        bp.load(xs[:-1] + [torch.rand(5, 7).cuda()])
+    with pytest.raises(ValueError):
+        bp.load(xs[:-1])
