@@ -12,6 +12,7 @@ step of the computation runs in the library's CUDA kernels.
 from __future__ import annotations
 
 import ctypes
+import math
 from dataclasses import dataclass
 from typing import Optional, Sequence
 
@@ -31,9 +32,10 @@ def _check_image(img: torch.Tensor, min_extent: int = 2):
         raise TypeError("image must be a CUDA tensor")
     if img.dtype != torch.float32:
         raise TypeError("image must be float32")
-    if img.dim() not in (2, 3):
+    shape = img.shape
+    if len(shape) not in (2, 3):
         raise ValueError("image must be 2D (H, W) or 3D (D, H, W)")
-    if any(s < min_extent for s in img.shape):
+    if min(shape) < min_extent:
         raise ValueError(f"every axis must be at least {min_extent} long")
 
 
@@ -117,12 +119,12 @@ def persistence(img: torch.Tensor, max_survivors: int = 0, with_stats: bool = Fa
     if tmode:
         fn = lib.cubical_persistence_t_2d if nd == 2 else lib.cubical_persistence_t_3d
         wsize = lib.cubical_persistence_t_workspace_size
-        n_all = n + int(np.prod([s + 1 for s in img.shape]))
-        n_j = int(np.prod([s + 2 for s in img.shape]))
+        n_all = n + math.prod([s + 1 for s in img.shape])
+        n_j = math.prod([s + 2 for s in img.shape])
     else:
         fn = lib.cubical_persistence_2d if nd == 2 else lib.cubical_persistence_3d
         wsize = lib.cubical_persistence_workspace_size
-        n_all = n + int(np.prod([s - 1 for s in img.shape])) + 1
+        n_all = n + math.prod([s - 1 for s in img.shape]) + 1
         n_j = n
     ms = int(max_survivors)
     for _ in range(4):
@@ -207,19 +209,27 @@ def persistence_batched(imgs: Sequence[torch.Tensor], max_survivors: int = 0, wi
     k = len(imgs)
     if k > _lib.CP_MAX_ITEMS:
         raise ValueError(f"at most {_lib.CP_MAX_ITEMS} items per call")
-    ptrs = (ctypes.c_void_p * k)(*[im.data_ptr() for im in imgs])
-    ndims = (ctypes.c_int32 * k)(*[im.dim() for im in imgs])
-    flat = []
+    # one pass over the items: a batch of small images waits for this loop
+    flat, nds = [], []
+    n = t = 0
     for im in imgs:
-        flat += ([1] + list(im.shape)) if im.dim() == 2 else list(im.shape)
+        shape = im.shape
+        d, h, w = shape if len(shape) == 3 else (1, *shape)
+        flat += (d, h, w)
+        nds.append(len(shape))
+        size, zp = d * h * w, len(shape) == 3
+        if tmode:
+            n += (d + 2 if zp else 1) * (h + 2) * (w + 2)  # the dual images' vertices
+            t += size + (d + 1 if zp else 1) * (h + 1) * (w + 1)
+        else:
+            n += size
+            t += size + (d - 1 if zp else 1) * (h - 1) * (w - 1) + 1
+    ptrs = (ctypes.c_void_p * k)(*[im.data_ptr() for im in imgs])
+    ndims = (ctypes.c_int32 * k)(*nds)
     dims = (ctypes.c_int64 * (3 * k))(*flat)
     if tmode:
-        n = sum(int(np.prod([s + 2 for s in im.shape])) for im in imgs)  # the dual images' vertices
-        t = sum(im.numel() + int(np.prod([s + 1 for s in im.shape])) for im in imgs)
         wsize, fn = lib.cubical_persistence_t_batched_workspace_size, lib.cubical_persistence_t_batched
     else:
-        n = sum(im.numel() for im in imgs)
-        t = n + sum(int(np.prod([s - 1 for s in im.shape])) + 1 for im in imgs)
         wsize, fn = lib.cubical_persistence_batched_workspace_size, lib.cubical_persistence_batched
     ms = int(max_survivors)
     for _ in range(4):
@@ -392,7 +402,7 @@ class _DiagramFn(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gb, gd, _graw):
         (raw,) = ctx.saved_tensors
-        n = int(np.prod(ctx.shape))
+        n = math.prod(ctx.shape)
         if gb is None:
             gb = torch.zeros(raw.shape[0], dtype=torch.float32, device=raw.device)
         if gd is None:
