@@ -38,8 +38,15 @@
 // design it replaces as the default (8 radix passes over both lists, then
 // reservation rounds with two grid barriers each, cp_uf.cu), kernel times:
 //   2048^2, 256 levels (14 K survivors)     204 -> 37 us
-//   512^3 blurred (587 K survivors)         553 -> 198 us
-//   128^3 uniform noise (1.15 M survivors) 1110 -> 475 us
+//   512^3 blurred (587 K survivors)         553 -> 117 us
+//   128^3 uniform noise (1.15 M survivors) 1110 -> 270 us
+// The oldest root of an item is where the climbs of every survivor above the
+// percolation level end, and its word never changes: read each time, that one
+// sector held up the whole chip (244 and 475 us in the last two).  k_roots2
+// flags its id (kTop) and nothing reads it.  Tried and left out: the smallest
+// survivor of each root put in first (Boruvka's first step; its atomics cost
+// the walks what it saved here), words through L1 until the first swap (more
+// swaps fail: 117 -> 151 us).
 #include "cp_common.cuh"
 #include "cp_grid.cuh"
 #include "cp_kernels.h"
@@ -108,21 +115,24 @@ __global__ void __launch_bounds__(kTT) k_tree(const __grid_constant__ TreeArgs a
             set_status(ctr, kStTimeout);
             return true;
         };
+        // an item's oldest root (flagged id) is connected with nothing older
+        auto word = [&](uint32_t w) { return (w & kTop) ? Word{~0ull, w} : ld_word(T + w); };
+        auto inside = [&](uint32_t w) { return (w & kTop) || CP_IN(w, L.n_rids, ctr); };
         for (bool live = true; live;) {
-            if (!CP_IN(u, L.n_rids, ctr) || !CP_IN(v, L.n_rids, ctr)) break;
-            Word wu = ld_word(T + u), wv = ld_word(T + v);
+            if (!inside(u) || !inside(v)) break;
+            Word wu = word(u), wv = word(v);
             for (;;) {
                 const bool cu = wu.key < s, cv = wv.key < s;
                 if (!cu && !cv) break;
                 if (cu) {
                     u = uint32_t(wu.parent);
-                    if (!CP_IN(u, L.n_rids, ctr)) u = 0;
-                    wu = ld_word(T + u);
+                    if (!inside(u)) u = 0;
+                    wu = word(u);
                 }
                 if (cv) {
                     v = uint32_t(wv.parent);
-                    if (!CP_IN(v, L.n_rids, ctr)) v = 0;
-                    wv = ld_word(T + v);
+                    if (!inside(v)) v = 0;
+                    wv = word(v);
                 }
                 if (overdue()) {
                     live = false;
@@ -130,11 +140,16 @@ __global__ void __launch_bounds__(kTT) k_tree(const __grid_constant__ TreeArgs a
                 }
             }
             if (!live || u == v || overdue()) break;
-            if (T[u].age < T[v].age) {  // u: the younger (ages: smaller is older)
+            // u: the younger (ages: smaller is older)
+            if ((u & kTop) || (!(v & kTop) && __ldg(&T[u].age) < __ldg(&T[v].age))) {
                 const uint32_t tu = u;
                 u = v;
                 v = tu;
                 wu = wv;
+            }
+            if (u & kTop) {  // two items' oldest roots: a corrupted list
+                set_status(ctr, kStInternal);
+                break;
             }
             const Word got = cas_word(T + u, wu, Word{s, uint64_t(v)});
             if (got.key != wu.key || got.parent != wu.parent) continue;
