@@ -492,7 +492,8 @@ int cubical_persistence_debug_wait_timeout(void *d_workspace, size_t ws_bytes, i
  *   CP_TUNE_ZCHUNK_3D    planes per 3D pruning task at most (4..4096, default 64;
  *                        small volumes get smaller tasks, to fill the chip)
  *   CP_TUNE_CTAS_PER_SM  3D pruning CTAs per SM (0 = as many as fit, default)
- *   CP_TUNE_ROWS_2D      most rows per 2D pruning task (4 .. 4096; default 64)
+ *   CP_TUNE_ROWS_2D      4 .. 4096, default 64; kept for saved settings: the 2D
+ *                        pass has one tile size
  *   CP_TUNE_CROSS_PRUNE_2D  1: the top dimension of 2D images waits for H0
  *                        and takes only the edges H0 leaves positive (the
  *                        cross-pruning of Sec. 3.2, Sec. 4.1 step 4: two sorts

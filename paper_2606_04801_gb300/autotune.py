@@ -1,7 +1,7 @@
 """Autotuner for the pruning pass (K1) and the union-find design.
 
-Picks the 3D task depth (planes per task), the number of 3D pruning CTAs per
-SM and the rows per 2D task by timing the lookup + pruning pass alone
+Picks the 3D task depth (planes per task) and the number of 3D pruning CTAs
+per SM by timing the lookup + pruning pass alone
 (cubical_persistence_debug_prune) on the given inputs; then the union-find
 design (reservation rounds over every survivor, or Borůvka's spanning forest
 first and the rounds over its edges) by timing whole forward calls with
@@ -30,7 +30,6 @@ from . import _lib
 ZCHUNK_3D, CTAS_PER_SM, ROWS_2D, UF_VARIANT = 1, 2, 3, 7
 CAND_ZCHUNK = (16, 32, 64, 128, 256)
 CAND_CTAS = (0, 2, 3)
-CAND_ROWS = (16, 32, 64, 128)
 
 
 def _cache_path() -> str:
@@ -159,7 +158,6 @@ def _time_forward(inputs: Sequence[torch.Tensor], repeats: int) -> float:
 
 def tune(inputs: Sequence[torch.Tensor], repeats: int = 5) -> dict:
     """Time every candidate on these inputs; returns the fastest setting."""
-    has2 = any(t.dim() == 2 for t in inputs)
     has3 = any(t.dim() == 3 for t in inputs)
     saved = current()
     best, best_ms = dict(saved), float("inf")
@@ -167,13 +165,12 @@ def tune(inputs: Sequence[torch.Tensor], repeats: int = 5) -> dict:
     try:
         for zc in CAND_ZCHUNK if has3 else (saved["zchunk3d"],):
             for ctas in CAND_CTAS if has3 else (saved["ctas3d"],):
-                for rows in CAND_ROWS if has2 else (saved["rows2d"],):
-                    cfg = {"zchunk3d": zc, "ctas3d": ctas, "rows2d": rows, "uf_variant": saved["uf_variant"]}
-                    apply(cfg)
-                    ms = _time_prune(inputs, repeats)
-                    trials.append((ms, cfg))
-                    if ms < best_ms:
-                        best, best_ms = cfg, ms
+                cfg = {"zchunk3d": zc, "ctas3d": ctas, "rows2d": saved["rows2d"], "uf_variant": saved["uf_variant"]}
+                apply(cfg)
+                ms = _time_prune(inputs, repeats)
+                trials.append((ms, cfg))
+                if ms < best_ms:
+                    best, best_ms = cfg, ms
         # the union-find design, on whole forward calls with the best pruning setting
         uf_ms = {}
         for var in (0, 1):

@@ -123,28 +123,6 @@ struct Plan {
 size_t align_up(size_t x) { return (x + 255) & ~size_t(255); }
 void plan_boruvka(Plan& P);
 
-// Owned rows per 2D pruning task: the fewest (at least 4) at which all of a
-// call's tasks run at once, at most the tuned bound.  A task is one warp that
-// takes its rows in series, at 0.6 us a row for a smooth image and 1.4 us for
-// noise, so an image that cannot fill the chip takes as long as its longest
-// task.  4864 warps run at once (152 SMs x 4 CTAs x 8 warps).  Measured at 64
-// rows and with this rule: 64^2 noise 96 -> 11 us, 160^2 42 -> 8, 769 x 1021
-// 45 -> 17, 1025 x 1539 46 -> 25, 2048^2 56 -> 50; at 4096^2 the bound holds.
-int plan_rows2d(const ItemTable& tab) {
-    constexpr int64_t kSlots = 4864;
-    int lo = 4, hi = std::max(4, prune_tile_y2d());
-    while (lo < hi) {
-        const int r = (lo + hi) / 2;
-        int64_t tasks = 0;
-        for (int j = 0; j < tab.n2d; ++j) tasks += int64_t(tab.it[j].tx) * ((tab.it[j].H + r - 1) / r);
-        if (tasks <= kSlots)
-            hi = r;
-        else
-            lo = r + 1;
-    }
-    return lo;
-}
-
 // Owned planes per 3D pruning task, at most the tuned bound: the value that
 // makes the fewest plane steps on the busiest CTA, counting kStart steps for
 // a task's start (its planes' first loads and the lead-in and lead-out steps).
@@ -227,12 +205,13 @@ int make_plan(int n_items, const int32_t* ndims, const int64_t* dims, const floa
         }
         if (voff > (int64_t(1) << kVBits) || toff > (int64_t(1) << kVBits) + kMaxItems) return CP_ERR_ARG;
     }
-    P.tab.rows2d = plan_rows2d(P.tab);
     for (int j = 0; j < P.tab.n2d; ++j) {
         Item& it = P.tab.it[j];
-        it.ty = (it.H + P.tab.rows2d - 1) / P.tab.rows2d;
+        it.ty = (it.H + prune_tile_y2d() - 1) / prune_tile_y2d();
         it.tile0 = t2;
         t2 += it.tx * it.ty;
+        it.coff = int64_t(P.n_code);  // 32 bytes per column of a tile (code_at2)
+        P.n_code += uint64_t(it.ty) * uint64_t(it.W) * 32u;
     }
     const int zc = plan_zchunk(P.tab);
     for (int j = P.tab.n2d; j < n_items; ++j) {
@@ -540,7 +519,7 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
     }
 
     CP_TRY(launch_prune(P.tab, po, P.tma, s));
-    if (tm) CP_TRY(launch_t_flatten(uf0, po.code, tm->items, s));
+    if (tm) CP_TRY(launch_t_flatten(po.code, tm->items, s));
     mark(1, s);
     nv.next("cp.roots+sort");
 
@@ -986,7 +965,7 @@ int t_run(int n_items, const float* const* h_images, const int32_t* ndims, const
     for (int j = 0; j < P.tab.n; ++j) {
         const Item& it = P.tab.it[j];
         tm.items.voff[it.user] = it.voff;
-        tm.items.coff[it.user] = it.ndim == 3 ? it.coff : 0;
+        tm.items.coff[it.user] = it.coff;
         tm.items.pitch[it.user] = it.ndim == 3 ? it.pitch : 0;
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);

@@ -37,14 +37,13 @@ struct Item {
     int32_t tma;              // 3D: index of the item's plane tensor map (TMA loads), or -1
     int32_t zc;               // 3D: owned planes per pruning task
     int32_t pitch;            // 3D: row pitch of the item's link codes (its width, rounded up to 4)
-    int64_t coff;             // 3D: the item's first link code
+    int64_t coff;             // the item's first link code
 };
 
 struct ItemTable {
     int32_t n;
     int32_t n2d, n3d;         // items 0..n2d-1 are 2D, n2d..n-1 are 3D
     int32_t tiles2d, tiles3d; // total pruning tiles of each kind
-    int32_t rows2d;           // vertex rows per 2D pruning task (4 .. 4096)
     int32_t zchunk3d;         // tuned bound on the planes of a 3D pruning task
     int32_t cross2d;          // 2D items: 1 = the dual list waits for H0 (cross-pruning), 0 = both at once
     Item it[kMaxItems];
@@ -145,19 +144,6 @@ __host__ __device__ __forceinline__ int64_t doubled_index(const Item& it, int z,
                                                           int dx) {
     int64_t GH = 2 * it.H - 1, GW = 2 * it.W - 1;
     return (int64_t(2 * z + dz) * GH + (2 * y + dy)) * GW + (2 * x + dx);
-}
-
-// Top cell (global id, or the item's outside vertex) in octant (sz, sy, sx)
-// (each +-1; sz ignored in 2D) of local vertex (z, y, x).
-__host__ __device__ __forceinline__ uint32_t top_of_octant(const Item& it, int z, int y, int x, int sz, int sy,
-                                                           int sx) {
-    int cz = it.ndim == 3 ? z + (sz < 0 ? -1 : 0) : 0;
-    int cy = y + (sy < 0 ? -1 : 0);
-    int cx = x + (sx < 0 ? -1 : 0);
-    bool out = cy < 0 || cy >= it.H - 1 || cx < 0 || cx >= it.W - 1 ||
-               (it.ndim == 3 && (cz < 0 || cz >= it.D - 1));
-    if (out) return uint32_t(it.toff + it.T);
-    return uint32_t(it.toff + (int64_t(cz) * (it.H - 1) + cy) * (it.W - 1) + cx);
 }
 
 // ---------------------------------------------------------------- device utils

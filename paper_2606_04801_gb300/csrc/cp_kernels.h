@@ -314,7 +314,7 @@ struct TItems {
     const float* img[kMaxItems];  // the image
     float* J[kMaxItems];          // its dual image: extents +2 along each image axis
     int64_t voff[kMaxItems];      // J's first vertex in the call's vertex space
-    int64_t coff[kMaxItems];      // 3D: J's first code and its codes' row pitch
+    int64_t coff[kMaxItems];      // J's first code; 3D: its codes' row pitch
     int32_t pitch[kMaxItems];
 };
 // J <- -image flipped along every axis, inside a one-voxel frame at -FLT_MAX;
@@ -322,7 +322,7 @@ struct TItems {
 cudaError_t launch_t_build(const TItems& t, uint32_t* bad, cudaStream_t s);
 // After the pruning pass: every frame vertex's H0 link points at the item's
 // vertex 0 (3D: has the code that says so).
-cudaError_t launch_t_flatten(uint32_t* uf0, uint8_t* code, const TItems& t, cudaStream_t s);
+cudaError_t launch_t_flatten(uint8_t* code, const TItems& t, cudaStream_t s);
 cudaError_t launch_essential(const ItemTable& tab, Counters* ctr, cp_pair* pairs, uint32_t pair_cap, cudaStream_t s);
 // Items copied to their places in one launch (cp_load.cu): the items with a
 // count, packed to the front.

@@ -838,9 +838,26 @@ __global__ void __launch_bounds__(kT3 + 64, 3) k_prune3d(const __grid_constant__
     }
 }
 
-// The words of a 3D item's forests from its codes, as the 2D pass writes them
-// (roots have theirs already).
-__global__ void __launch_bounds__(256) k_expand3d(const __grid_constant__ ItemTable tab, const __grid_constant__ Outs o) {
+// The words of every item's forests from its codes, links as ids (roots have
+// theirs already).
+__global__ void __launch_bounds__(256) k_expand(const __grid_constant__ ItemTable tab, const __grid_constant__ Outs o) {
+    for (int j = 0; j < tab.n2d; ++j) {
+        const Item& it = tab.it[j];
+        const int64_t n = int64_t(it.H) * it.W;
+        for (int64_t v = int64_t(blockIdx.x) * 256 + threadIdx.x; v < n; v += int64_t(gridDim.x) * 256) {
+            const int y = int(v / it.W), x = int(v - int64_t(y) * it.W);
+            const uint32_t c = o.code[it.coff + code_at2(it, y, x)];
+            int dy, dx;
+            if ((c & 15u) < 8u) {
+                link_offset2(0, c & 15u, dy, dx);
+                o.uf0[it.voff + v] = uint32_t(it.voff + v + int64_t(dy) * it.W + dx);
+            }
+            if (y >= it.H - 1 || x >= it.W - 1 || c >> 4 == 15u) continue;
+            const int64_t self = it.toff + int64_t(y) * (it.W - 1) + x;
+            link_offset2(1, c >> 4, dy, dx);
+            o.uft[self] = c >> 4 == 9u ? uint32_t(it.toff + it.T) : uint32_t(self + int64_t(dy) * (it.W - 1) + dx);
+        }
+    }
     for (int j = tab.n2d; j < tab.n; ++j) {
         const Item& it = tab.it[j];
         const int64_t n = int64_t(it.D) * it.H * it.W;
@@ -858,322 +875,261 @@ __global__ void __launch_bounds__(256) k_expand3d(const __grid_constant__ ItemTa
 }
 
 // ---------------------------------------------------------------- 2D
-// Each warp marches down a strip of one image on its own (no block
-// barriers): lane l handles column x0-1+l; lanes 1..31 own their columns (31
-// per strip), lane 0 is a halo whose lookup codes the top cells of column
-// x0-1 need.  The task owns rows [y0, y1) and computes lookups for rows
-// [y0, min(y1, H-1)].
+// A warp takes a tile of 32 x 32 vertices, of which it owns the inner 30 x
+// 30, and does all of it on words: lane = column, bit = row.
 //
-// Per row step y:
-//  1. cp.async prefetch of row y+kAhead2 (columns x0-2 .. x0+31) into the
-//     warp's 8-row shared-memory ring; out-of-image positions read +inf;
-//  2. the 8-neighbour mask of (y, x) from registers (rows y-1, y) and the
-//     ring (row y+1), direct table lookup, the H0 forest link (an up link
-//     continues the chain of (y-1, x), the same lane's previous step) and
-//     the survivors and H0 root of owned vertices;
-//  3. the top cell whose smallest corner is (y-1, x): its largest corner m
-//     among the 4 corner values holds, in its entry, where the top cell dies
-//     locally; the codes of rows y-1 and y of column x+1 come by shuffle, so
-//     each lane stores one coalesced dual forest link (or a dual root).
-constexpr int kW2 = 8;                   // warps per CTA (independent tasks)
-constexpr int kOX2 = 31;                 // owned columns per strip
-constexpr int kRW2 = 34;                 // ring row: columns x0-2 .. x0+31
-constexpr int kRing2 = 8, kAhead2 = 5;   // ring rows, rows in flight
-constexpr int kCap2 = 32 * 4;            // staged keys per warp and kind (one step's maximum)
-constexpr int kCapWR = 32;               // staged roots per warp and kind
-
-struct WarpStage2 {
-    uint64_t s0[kCap2];
-    uint64_t st[kCap2];
-    uint64_t r0age[kCapWR];
-    uint64_t rtage[kCapWR];
-    uint32_t r0node[kCapWR];
-    uint32_t rtnode[kCapWR];
-    uint8_t r0item[kCapWR];
-    uint8_t rtitem[kCapWR];
-};
+//   compare  of every vertex with its right, lower left, lower and lower
+//            right neighbour: the sign of a difference (exact: zero only for
+//            equal values), shifted into the lane's word.  The other four
+//            neighbours' bits are the complements of their own.
+//   logic    on those words, 32 x 32 vertices per instruction: the H0 link,
+//            the top cells in the lower stars and where each dies, the events
+//            (vertices whose lower star holds a survivor or a root: the lower
+//            link is not one arc).
+//   output   one code byte per vertex with both links (cp_walk.cuh), a
+//            column of a tile in one 32-byte sector.
+//   events   32 at a time: mask, table, and after one atomic per tile and
+//            array the keys, roots and ages.
+//
+// Closed forms used by the logic (equal to the table's entries on all 256
+// masks): the H0 link is the first of up, left, right, down in L(v); a top
+// cell in quadrant 0 or 1 of L(v) dies across +y, in 2 across +x, in 3 towards
+// the highest quadrant not in L(v), and is a dual root if all four are; there
+// is an event unless exactly one face of L(v) is not followed, around v, by a
+// quadrant of L(v).
+//
+// Small images are bound by a tile's events, which one warp takes 32 at a time:
+// up to eight warps then take a tile together, each with all of its words but
+// the events of its own rows.  Large ones are bound by issue.  Marching down a
+// strip with a mask, a table read and two 32-bit links per vertex took 273 warp
+// instructions per 32 vertices and wrote eight bytes per vertex instead of
+// one: 4096^2 smooth 188 -> 38 us, 2048^2 49 -> 11, 2048^2 noise 113 -> 60,
+// 769 x 1021 18 -> 7, 64^2 noise 10 -> 8.
+constexpr int kW2 = 4;                   // warps per CTA (independent tiles)
 
 struct Smem2 {
-    uint2 lut[256];
-    float ring[kW2][kRing2][kRW2];
-    WarpStage2 ws[kW2];
+    uint32_t n[kW2][8][32];              // neighbour words: bit set = the neighbour precedes
+    uint32_t queue[kW2][kTile2 * kTile2];  // events: row << 5 | lane; then | h0 << 10 | dual << 14 | roots << 18
 };
 
-struct WarpCounts {
-    uint32_t s0, st, r0, rt;
+struct Words2 {
+    uint32_t r, d, dr, a;  // right < v, below < v, lower right < v, below < right
 };
 
-template <class WS>
-__device__ __forceinline__ void warp_flush(WS& ws, WarpCounts& c, const Outs& o) {
-    __syncwarp();
-    const unsigned lane = lane_id();
-    uint32_t b0 = 0, bt = 0, br0 = 0, brt = 0;
-    if (lane == 0) {
-        if (c.s0) b0 = atomicAdd(&o.ctr->n_s0, c.s0);
-        if (c.st) bt = atomicAdd(&o.ctr->n_st, c.st);
-        if (c.r0) br0 = atomicAdd(&o.ctr->n_r0, c.r0);
-        if (c.rt) brt = atomicAdd(&o.ctr->n_rt, c.rt);
-        bool over = (c.s0 && b0 + c.s0 > o.cap_s) || (c.st && bt + c.st > o.cap_s) ||
-                    (c.r0 && br0 + c.r0 > o.cap_r0) || (c.rt && brt + c.rt > o.cap_rt);
-        if (over) set_status(o.ctr, kStCapacity);
+// The words of 32 rows from row y (the tile's first, y0 - 1) on; kIn: every
+// position read lies inside the image.  Outside it, values are +inf.
+template <bool kIn>
+__device__ __forceinline__ Words2 words2(const float* __restrict__ img, int W, int H, int x, int y, float& bad) {
+    constexpr int kB = 8;  // rows loaded at a time
+    const float inf = __int_as_float(0x7F800000);
+    const bool in0 = kIn || unsigned(x) < unsigned(W), in1 = kIn || unsigned(x + 1) < unsigned(W);
+    const float* p = img + (int64_t(y) * W + x);
+    auto get = [&](int i, float& a, float& b) {
+        const bool row = kIn || unsigned(y + i) < unsigned(H);
+        a = b = inf;
+        if (row && in0) a = __ldg(p + int64_t(i) * W);
+        if (row && in1) b = __ldg(p + int64_t(i) * W + 1);
+    };
+    auto check = [&](int i, float a) {  // NaN from the first NaN or infinity on
+        if (kIn || (in0 && unsigned(y + i) < unsigned(H))) bad = fmaf(a, 0.0f, bad);
+    };
+    Words2 w = {0, 0, 0, 0};
+    float a, b;
+    get(0, a, b);
+    check(0, a);
+    a = __fadd_rn(a, 0.0f);  // -0 and +0 are equal: +0, so that their difference is +0
+    b = __fadd_rn(b, 0.0f);
+#pragma unroll 1
+    for (int i0 = 1; i0 < 33; i0 += kB) {
+        float c[kB], d[kB];
+#pragma unroll
+        for (int k = 0; k < kB; ++k) get(i0 + k, c[k], d[k]);
+#pragma unroll
+        for (int k = 0; k < kB; ++k) {
+            check(i0 + k, c[k]);
+            const float e = __fadd_rn(c[k], 0.0f), f = __fadd_rn(d[k], 0.0f);
+            w.r = __funnelshift_l(__float_as_uint(__fsub_rn(b, a)), w.r, 1);
+            w.d = __funnelshift_l(__float_as_uint(__fsub_rn(e, a)), w.d, 1);
+            w.dr = __funnelshift_l(__float_as_uint(__fsub_rn(f, a)), w.dr, 1);
+            w.a = __funnelshift_l(__float_as_uint(__fsub_rn(e, b)), w.a, 1);
+            a = e;
+            b = f;
+        }
     }
-    b0 = __shfl_sync(0xFFFFFFFFu, b0, 0);
-    bt = __shfl_sync(0xFFFFFFFFu, bt, 0);
-    br0 = __shfl_sync(0xFFFFFFFFu, br0, 0);
-    brt = __shfl_sync(0xFFFFFFFFu, brt, 0);
-    for (uint32_t i = lane; i < c.s0; i += 32)
-        if (b0 + i < o.cap_s) o.s0[b0 + i] = ws.s0[i];
-    for (uint32_t i = lane; i < c.st; i += 32)
-        if (bt + i < o.cap_s) o.st[bt + i] = ws.st[i];
-    for (uint32_t i = lane; i < c.r0; i += 32)
-        if (CP_IN(ws.r0node[i], o.n_uf0, o.ctr))
-            put_root(o.uf0 + ws.r0node[i], br0 + i, o.cap_r0, ws.r0age[i], o.node0, o.age0, o.res0, false, ws.r0item[i]);
-    for (uint32_t i = lane; i < c.rt; i += 32)
-        if (CP_IN(ws.rtnode[i], o.n_uft, o.ctr))
-            put_root(o.uft + ws.rtnode[i], brt + i, o.cap_rt, ws.rtage[i], o.nodet, o.aget, o.rest, true, ws.rtitem[i]);
-    c.s0 = c.st = c.r0 = c.rt = 0;
-    __syncwarp();
+    w.r = __brev(w.r);
+    w.d = __brev(w.d);
+    w.dr = __brev(w.dr);
+    w.a = __brev(w.a);
+    return w;
 }
 
-struct Row {
-    float l, c, r;  // columns x-1, x, x+1
-};
-
-__device__ __forceinline__ void read_row(const float* slot, int lane, Row& R) {
-    R.l = slot[lane];
-    R.c = slot[lane + 1];
-    R.r = slot[lane + 2];
-}
-
-struct RowPos {
-    const float* img;
-    uint32_t W, H;
-    int gx0, gx1;     // image columns copied by this lane
-    int idx1;         // ring position of the second column
-    bool in0, in1;    // inside the image
-};
-
-// kCheck false: the caller knows that row y lies inside the image
-template <bool kCheck = true>
-__device__ __forceinline__ void issue_row(float (*ring)[kRW2], const RowPos& p, int lane, int y) {
-    float* slot = ring[(y + kRing2) & (kRing2 - 1)];
-    if (!kCheck || unsigned(y) < p.H) {
-        const float* base = p.img + uint32_t(y) * p.W;
-        if (p.in0) cp_async4(slot + lane + 1, base + p.gx0);
-        if (p.in1) cp_async4(slot + p.idx1, base + p.gx1);
-    } else {  // a row outside the image: every position +inf
-        const float inf = __int_as_float(0x7F800000);
-        if (p.in0) slot[lane + 1] = inf;
-        if (p.in1) slot[p.idx1] = inf;
-    }
-    cp_async_commit();
-}
-
-__global__ void __launch_bounds__(kW2 * 32) k_prune2d(ItemTable tab, Outs o) {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    Smem2& sm = *reinterpret_cast<Smem2*>(smem_raw);
+__global__ void __launch_bounds__(kW2 * 32) k_prune2d(const __grid_constant__ ItemTable tab, const __grid_constant__ Outs o,
+                                                      const int parts) {
+    __shared__ Smem2 sm;
     const int warp = threadIdx.x >> 5;
     const int lane = int(lane_id());
     const unsigned lt = (1u << lane) - 1u;
-    for (int i = threadIdx.x; i < 256; i += kW2 * 32) sm.lut[i] = g_lut2d[i];
-    __syncthreads();
-    WarpStage2& ws = sm.ws[warp];
-    float(*ring)[kRW2] = sm.ring[warp];
-    WarpCounts cnt = {0, 0, 0, 0};
-    const float inf = __int_as_float(0x7F800000);
-    for (int task = blockIdx.x * kW2 + warp; task < tab.tiles2d; task += gridDim.x * kW2) {
-        const int ii = tile_item(tab, 0, tab.n2d - 1, task);
+    constexpr unsigned kAll = 0xFFFFFFFFu;
+    for (int task = blockIdx.x * kW2 + warp; task < tab.tiles2d * parts; task += gridDim.x * kW2) {
+        const int tile = task / parts, part = task - tile * parts;
+        const int ii = tile_item(tab, 0, tab.n2d - 1, tile);
         const Item& it = tab.it[ii];
-        const int ltask = task - it.tile0;
-        const int x0 = (ltask % it.tx) * kOX2, y0 = (ltask / it.tx) * tab.rows2d;
-        const int y1 = min(it.H, y0 + tab.rows2d);  // owned rows [y0, y1)
-        const int ylast = min(y1, it.H - 1);        // lookups for rows [y0, ylast]
+        const int ltask = tile - it.tile0;
+        const int W = it.W, H = it.H, ty = ltask / it.tx;
+        const int x0 = (ltask - ty * it.tx) * kTile2, y0 = ty * kTile2;
         const int x = x0 - 1 + lane;
-        const uint32_t W = uint32_t(it.W), H = uint32_t(it.H), W1 = W - 1u;
-        const uint32_t voff = uint32_t(it.voff), toff = uint32_t(it.toff), OUT = uint32_t(it.toff + it.T);
-        const bool owned_x = lane >= 1 && x < it.W;
-        const bool cube_x = lane <= 30 && x >= 0 && x < it.W - 1;
-        RowPos rp;
-        rp.img = it.img;
-        rp.W = W;
-        rp.H = H;
-        rp.gx0 = x;
-        rp.in0 = unsigned(x) < W;
-        rp.gx1 = lane == 0 ? x0 - 2 : x0 + 31;
-        rp.idx1 = lane == 0 ? 0 : kRW2 - 1;
-        rp.in1 = (lane == 0 || lane == 31) && unsigned(rp.gx1) < W;
-        const bool has1 = lane == 0 || lane == 31;
-        __syncwarp();  // the ring may still be read by the previous task
-#pragma unroll
-        for (int s = 0; s < kRing2; ++s) {
-            if (!rp.in0) ring[s][lane + 1] = inf;
-            if (has1 && !rp.in1) ring[s][rp.idx1] = inf;
+        // ---- compare
+        float bad = 0.0f;
+        const bool inside = x0 > 0 && y0 > 0 && x0 + 31 < W && y0 + 31 < H;
+        const Words2 w = inside ? words2<true>(it.img, W, H, x, y0 - 1, bad) : words2<false>(it.img, W, H, x, y0 - 1, bad);
+        if (__any_sync(kAll, bad != bad) && lane == 0) set_status(o.ctr, kStNonfinite);
+        // ---- logic: neighbours before in linear order by complement, from the row above and the lane to the left
+        const uint32_t rl = __shfl_up_sync(kAll, w.r, 1), drl = __shfl_up_sync(kAll, w.dr, 1), al = __shfl_up_sync(kAll, w.a, 1);
+        const uint32_t nul = ~(drl << 1), nu = ~(w.d << 1), nur = ~(w.a << 1), nl = ~rl, nr = w.r, ndl = al, nd = w.d, ndr = w.dr;
+        const uint32_t q0 = nul & nu & nl, q1 = nur & nu & nr, q2 = ndl & nd & nl, q3 = ndr & nd & nr;
+        const bool own_x = lane >= 1 && lane <= kTile2 && x < W;
+        const uint32_t own = own_x ? (H - y0 >= kTile2 ? 0x7FFFFFFEu : (2u << (H - y0)) - 2u) : 0u;
+        uint32_t ev;
+        {
+            const uint32_t a = nu & ~q1, b = nr & ~q3, c = nd & ~q2, d = nl & ~q0;
+            const uint32_t two = (a & b) | (c & d) | ((a | b) & (c | d));
+            // this part's rows
+            const uint32_t rows = ((2u << ((part + 1) * kTile2 / parts)) - 1u) & ~((2u << (part * kTile2 / parts)) - 1u);
+            ev = ~((a | b | c | d) & ~two) & own & rows;
         }
+        // ---- code bytes: the byte of row i (bit i + 1) of the lane's column
+        if (part == 0) {
+            const uint32_t px = __shfl_down_sync(kAll, q2, 1), py = (q1 | __shfl_down_sync(kAll, q0, 1)) >> 1;
+            const uint32_t last_x = x == W - 2 ? kAll : 0u, first_x = x == 0 ? kAll : 0u, first_y = y0 == 0 ? 2u : 0u;
+            const int ly = H - 1 - y0;  // the bit of row H - 2
+            const uint32_t last_y = unsigned(ly) < 32u ? 1u << ly : 0u;
+            const uint32_t mx = q3 & ~q2, my = q3 & q2 & ~q1, dg = q3 & q2 & q1 & ~q0, root = q3 & q2 & q1 & q0;
+            const uint32_t out = (px & last_x) | (py & last_y) | ((mx | dg) & first_x) | ((my | dg) & first_y);
+            // runs of links up, and of links down (+y), at least 1, 2, 4, 8, 16 long
+            const uint32_t u1 = nu & ~1u, u2 = u1 & (u1 << 1), u4 = u2 & (u2 << 2), u8 = u4 & (u4 << 4), u16 = u8 & (u8 << 8);
+            const uint32_t d1 = py & ~out & 0x7FFFFFFEu, d2 = d1 & (d1 >> 1), d4 = d2 & (d2 >> 2), d8 = d4 & (d4 >> 4),
+                           d16 = d8 & (d8 >> 8);
+            uint32_t acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+            spread<0>(acc, ((nu & ((u2 & ~u4) | (u8 & ~u16))) | (~nu & (nl | (~nr & nd)))) >> 1);
+            spread<1>(acc, ((nu & u4 & ~u16) | (~nu & ~nl)) >> 1);
+            spread<2>(acc, (u16 | ~nu) >> 1);
+            spread<3>(acc, ~(nu | nl | nr | nd) >> 1);
+            spread<4>(acc, ((d2 & ~d4) | (d8 & ~d16) | ((px | my) & ~out) | out | root) >> 1);
+            spread<5>(acc, ((d4 & ~d16) | ((mx | my) & ~out) | root) >> 1);
+            spread<6>(acc, (d16 | ((px | mx | my) & ~out) | root) >> 1);
+            spread<7>(acc, (dg | out | root) >> 1);
+            const uint64_t at = uint64_t(it.coff) + uint64_t(code_at2(it, y0, x));
+            if (own_x && CP_IN(at + 31u, o.n_code, o.ctr)) {
+                uint4* dst = reinterpret_cast<uint4*>(o.code + at);
+                dst[0] = make_uint4(acc[0], acc[1], acc[2], acc[3]);
+                dst[1] = make_uint4(acc[4], acc[5], acc[6], acc[7]);
+            }
+        }
+        // ---- events
+        uint32_t incl = __popc(ev);
 #pragma unroll
-        for (int k = -1; k < kAhead2; ++k) issue_row(ring, rp, lane, y0 + k);
-        cp_async_wait<kAhead2 - 2>();  // rows y0-1 .. y0+1 have landed
+        for (int s = 1; s < 32; s <<= 1) {
+            const uint32_t u = __shfl_up_sync(kAll, incl, s);
+            if (lane >= s) incl += u;
+        }
+        const uint32_t total = __shfl_sync(kAll, incl, 31);
+        if (total == 0) continue;
+        uint32_t(*n)[32] = sm.n[warp];
+        uint32_t* queue = sm.queue[warp];
+        __syncwarp();  // the last tile's events have been read
+        n[0][lane] = nul, n[1][lane] = nu, n[2][lane] = nur, n[3][lane] = nl;
+        n[4][lane] = nr, n[5][lane] = ndl, n[6][lane] = nd, n[7][lane] = ndr;
+        for (uint32_t at = incl - __popc(ev); ev; ev &= ev - 1u) queue[at++] = uint32_t(__ffs(ev) - 1) << 5 | uint32_t(lane);
         __syncwarp();
-        Row A, B, C;
-        read_row(ring[(y0 - 1 + kRing2) & (kRing2 - 1)], lane, A);
-        read_row(ring[y0 & (kRing2 - 1)], lane, B);
-        unsigned long long my_min = ~0ull;
-        uint32_t far = 0, far_t = 0, cprev = 0;  // last H0 link / dual link written by this lane
-        bool nonfinite = false;                   // an owned value is NaN or infinite (checked once per task)
-        // interior: a std::integral_constant; true for a row with y >= y0 + 2 and
-        // y + kAhead2 <= ylast, where no boundary row or end-of-task case arises
-        auto step = [&](const int y, auto interior) {
-            constexpr bool kIn = decltype(interior)::value;
-            issue_row<!kIn>(ring, rp, lane, y + kAhead2);
-            read_row(ring[(y + 1) & (kRing2 - 1)], lane, C);
-            // ---- lookup of (y, x): bit i of the mask is stencil offset n = i (i < 4) or
-            // i + 1 (i >= 4); offsets before the centre in linear order precede on ties
-            const float cv = B.c;
+        uint32_t c_s = 0, c_r = 0;  // survivors (H0 | dual << 16), roots (the same)
+#pragma unroll 2
+        for (uint32_t e = lane; e < total; e += 32) {
+            const uint32_t q = queue[e], l = q & 31u, row = q >> 5;
             uint32_t raw = 0;
-            or_if_precedes<1u << 0, true>(raw, A.l, cv);
-            or_if_precedes<1u << 1, true>(raw, A.c, cv);
-            or_if_precedes<1u << 2, true>(raw, A.r, cv);
-            or_if_precedes<1u << 3, true>(raw, B.l, cv);
-            or_if_precedes<1u << 4, false>(raw, B.r, cv);
-            or_if_precedes<1u << 5, false>(raw, C.l, cv);
-            or_if_precedes<1u << 6, false>(raw, C.c, cv);
-            or_if_precedes<1u << 7, false>(raw, C.r, cv);
-            const uint2 e = sm.lut[raw];
-            const bool owned = owned_x && (kIn || y < y1);
-            const uint32_t ord = ord_bits(cv);
-            const uint32_t vl = uint32_t(y) * W + uint32_t(x);
-            const uint32_t vg = voff + vl;
-            const uint32_t direct = e.x & 7u;
-            // H0: a local minimum becomes a root (registered in the staging block
-            // below); otherwise the link along the first edge (face slots: up,
-            // left, right, down), where a link up continues the chain that this
-            // lane started one row before
-            const bool root0 = owned && direct == 7u;
-            nonfinite |= owned && !(fabsf(cv) <= 3.40282347e38f);
-            {
-                const uint32_t mag = (direct == 0u || direct == 3u) ? W : 1u;
-                const uint32_t u = direct < 2u ? vg - mag : vg + mag;
-                if (owned) far = root0 ? vg : ((direct == 0u && (kIn || y > y0)) ? far : u);
-                if (owned && !root0 && CP_IN(vg, o.n_uf0, o.ctr)) o.uf0[vg] = far;
-            }
-            const uint32_t h0s = owned ? (e.x >> 3) & 0xFu : 0u;
-            const uint32_t ds = owned ? (e.x >> 9) & 0xFu : 0u;
-            // cross-pruning: dual survivors that are also H0 survivors wait for the
-            // H0 union-find (flag bit of the H0 key); otherwise every dual survivor
-            // goes to the dual list now (one that kills an H0 class closes a dual
-            // cycle there: a no-op)
-            const uint32_t flg = tab.cross2d ? ds : 0u;
-            const uint32_t dn = tab.cross2d ? ds & ~h0s : ds;
-            // ---- the top cell with smallest corner (y-1, x): its largest corner m
-            // (value, then linear index) holds it; m's code field for it says where
-            // it dies locally (8: a dual root, registered in the staging block
-            // below; 15: not held, non-finite input only)
-            const uint32_t cprev_r = __shfl_down_sync(0xFFFFFFFFu, cprev, 1);
-            const uint32_t ccur_r = __shfl_down_sync(0xFFFFFFFFu, e.y, 1);
-            const bool cube = cube_x && (kIn || y > y0);
-            const float cvals[4] = {A.c, A.r, B.c, B.r};
-            int k = 0;
-            float best = cvals[0];
 #pragma unroll
-            for (int j = 1; j < 4; ++j) {
-                const bool ge = cvals[j] >= best;
-                best = ge ? cvals[j] : best;
-                k = ge ? j : k;
+            for (int k = 0; k < 8; ++k) raw |= ((n[k][l] >> row) & 1u) << k;
+            const uint32_t en = __ldg(&g_lut2d[raw].x);
+            const uint32_t h0 = (en >> 3) & 15u, dual = (en >> 9) & 15u;
+            const uint32_t r0 = (en & 7u) == 7u ? 1u : 0u, rt = raw == 255u ? 1u : 0u;
+            queue[e] = q | h0 << 10 | dual << 14 | r0 << 18 | rt << 19;
+            // cross-pruning: dual survivors that are also H0 survivors wait for the H0 union-find
+            c_s += __popc(h0) | __popc(tab.cross2d ? dual & ~h0 : dual) << 16;
+            c_r += r0 | rt << 16;
+        }
+        c_s = __reduce_add_sync(kAll, c_s);
+        c_r = __reduce_add_sync(kAll, c_r);
+        // lanes 0 .. 3 take room in the four arrays
+        uint32_t base = 0;
+        {
+            const uint32_t want = ((lane & 2) ? c_r : c_s) >> ((lane & 1) * 16) & 0xFFFFu;
+            uint32_t* c = lane == 0 ? &o.ctr->n_s0 : (lane == 1 ? &o.ctr->n_st : (lane == 2 ? &o.ctr->n_r0 : &o.ctr->n_rt));
+            const uint32_t cap = lane < 2 ? o.cap_s : (lane == 2 ? o.cap_r0 : o.cap_rt);
+            if (lane < 4 && want) {
+                base = atomicAdd(c, want);
+                if (base + want > cap) set_status(o.ctr, kStCapacity);
             }
-            const uint32_t word = k == 0 ? cprev : (k == 1 ? cprev_r : (k == 2 ? e.y : ccur_r));
-            const uint32_t t = uint32_t(3 - k);  // quadrant of the top cell as seen from m
-            const uint32_t code = (word >> (4u * t)) & 15u;
-            const uint32_t self = toff + uint32_t(y - 1) * W1 + uint32_t(x);
-            const bool rootT = cube && code == 8u;
-            {
-                // the top cell across: quadrant `code` of m, smallest corner m - (negative axes)
-                const int my = y - 1 + (k >> 1), mx = x + (k & 1);
-                const int ty = my - int(((code >> 1) & 1u) ^ 1u);
-                const int tx = mx - int((code & 1u) ^ 1u);
-                const bool out = unsigned(ty) >= H - 1u || unsigned(tx) >= W1;
-                // a link to (y-2, x) continues the chain that this lane wrote for that top
-                // cell in the previous step; a code of 15 writes a root tag to keep the
-                // forest well formed
-                const bool chain = ty == y - 2 && tx == x && (kIn || y - 1 > y0);
-                const uint32_t tgt = code < 4u ? (out ? OUT : toff + uint32_t(ty) * W1 + uint32_t(tx)) : kTag;
-                if (cube) far_t = rootT ? self : ((code < 4u && chain) ? far_t : tgt);
-                if (cube && !rootT && CP_IN(self, o.n_uft, o.ctr)) o.uft[self] = far_t;
-            }
-            cprev = e.y;
-            // ---- stage survivors and roots
-            if (__any_sync(0xFFFFFFFFu, root0 || rootT || (h0s | dn) != 0u)) {
-                const unsigned m_r0 = __ballot_sync(0xFFFFFFFFu, root0);
-                const unsigned m_rt = __ballot_sync(0xFFFFFFFFu, rootT);
-                const uint32_t or0 = __reduce_or_sync(0xFFFFFFFFu, h0s);
-                const uint32_t ort = __reduce_or_sync(0xFFFFFFFFu, dn);
-                const uint32_t n0 = __reduce_add_sync(0xFFFFFFFFu, uint32_t(__popc(h0s)));  // <= 32 * 4
-                const uint32_t nt = __reduce_add_sync(0xFFFFFFFFu, uint32_t(__popc(dn)));   // <= 32 * 4
-                if (cnt.s0 + n0 > uint32_t(kCap2) || cnt.st + nt > uint32_t(kCap2) ||
-                    cnt.r0 + __popc(m_r0) > uint32_t(kCapWR) || cnt.rt + __popc(m_rt) > uint32_t(kCapWR))
-                    warp_flush(ws, cnt, o);
-                if (m_r0) {
-                    if (root0) {
-                        const uint32_t p = cnt.r0 + __popc(m_r0 & lt);
-                        ws.r0node[p] = vg;
-                        ws.r0item[p] = uint8_t(ii);
-                        ws.r0age[p] = make_key(ord, vg, 0);
-                        const unsigned long long kk = (unsigned long long)(uint64_t(ord) << 32 | vl);
-                        my_min = kk < my_min ? kk : my_min;
-                    }
-                    cnt.r0 += __popc(m_r0);
-                }
-                if (m_rt) {
-                    if (rootT) {
-                        const uint32_t my = uint32_t(y - 1 + (k >> 1)), mx = uint32_t(x + (k & 1));
-                        const uint32_t mg = voff + my * W + mx;
-                        const uint32_t p = cnt.rt + __popc(m_rt & lt);
-                        ws.rtnode[p] = self;
-                        ws.rtitem[p] = uint8_t(ii);
-                        ws.rtage[p] = make_key(ord_bits(best), mg, (6u * (t >> 1) + 2u * (t & 1u)) << 1);
-                    }
-                    cnt.rt += __popc(m_rt);
-                }
-                uint32_t bits = or0;
-                while (bits) {
-                    const int s = __ffs(bits) - 1;
-                    bits &= bits - 1;
-                    const bool mine = (h0s >> s) & 1u;
-                    const unsigned m = __ballot_sync(0xFFFFFFFFu, mine);
-                    if (mine)  // face slot s is stencil offset 2s+1; low bit: the dual waits for it
-                        ws.s0[cnt.s0 + __popc(m & lt)] = make_key(ord, vg, (uint32_t(2 * s + 1) << 1) | ((flg >> s) & 1u));
-                    cnt.s0 += __popc(m);
-                }
-                bits = ort;
-                while (bits) {
-                    const int f = __ffs(bits) - 1;
-                    bits &= bits - 1;
-                    const bool mine = (dn >> f) & 1u;
-                    const unsigned m = __ballot_sync(0xFFFFFFFFu, mine);
-                    if (mine) ws.st[cnt.st + __popc(m & lt)] = ~make_key(ord, vg, uint32_t(2 * f + 1) << 1);
-                    cnt.st += __popc(m);
-                }
-                __syncwarp();
-            }
-            cp_async_wait<kAhead2 - 2>();  // row y+2 has landed (for the next step)
-            __syncwarp();
-            A = B;
-            B = C;
+        }
+        uint32_t b0 = __shfl_sync(kAll, base, 0), bt = __shfl_sync(kAll, base, 1), br0 = __shfl_sync(kAll, base, 2),
+                 brt = __shfl_sync(kAll, base, 3);
+        unsigned long long gmin = ~0ull;
+        __syncwarp();
+        // a batch's values are loaded during the one before
+        auto take = [&](uint32_t e, uint32_t& q, float& v) {
+            q = e < total ? queue[e] : 0u;
+            const int64_t at = int64_t(y0 - 1 + int((q >> 5) & 31u)) * W + (x0 - 1 + int(q & 31u));
+            v = e < total ? __ldg(it.img + at) : 0.0f;
         };
-        // the first two rows and the last few take every check; the interior rows
-        // are a second instantiation of the step without them
-        int y = y0;
-        for (; y <= ylast && y < y0 + 2; ++y) step(y, std::false_type());
-        for (; y + kAhead2 <= ylast; ++y) step(y, std::true_type());
-        for (; y <= ylast; ++y) step(y, std::false_type());
-        if (__any_sync(0xFFFFFFFFu, nonfinite) && lane == 0) set_status(o.ctr, kStNonfinite);
-        cp_async_wait<0>();
-        const unsigned long long w = warp_min_u64(my_min);
-        if (lane == 0 && w != ~0ull) atomicMin(&o.ctr->gmin[ii], w);
+        uint32_t q, q_next;
+        float val, val_next;
+        take(lane, q_next, val_next);
+        for (uint32_t e0 = 0; e0 < total; e0 += 32) {
+            q = q_next;
+            val = val_next;
+            take(e0 + 32 + lane, q_next, val_next);
+            uint32_t h0 = (q >> 10) & 15u, dual = (q >> 14) & 15u;
+            const uint32_t flg = tab.cross2d ? dual : 0u;
+            if (tab.cross2d) dual &= ~h0;
+            const bool root0 = (q >> 18) & 1u, rootT = (q >> 19) & 1u;
+            const int ex = x0 - 1 + int(q & 31u), ey = y0 - 1 + int((q >> 5) & 31u);
+            const uint32_t vl = uint32_t(ey) * uint32_t(W) + uint32_t(ex), vg = uint32_t(it.voff) + vl;
+            const uint32_t mine = __popc(h0) | __popc(dual) << 16;  // at most 128 each in a warp
+            uint32_t ex_s = mine;
+#pragma unroll
+            for (int s = 1; s < 32; s <<= 1) {
+                const uint32_t u = __shfl_up_sync(kAll, ex_s, s);
+                if (lane >= s) ex_s += u;
+            }
+            const uint32_t all = __shfl_sync(kAll, ex_s, 31);
+            ex_s -= mine;
+            const unsigned m0 = __ballot_sync(kAll, root0), mt = __ballot_sync(kAll, rootT);
+            const uint32_t ord = ord_bits(val);
+            for (uint32_t at = b0 + (ex_s & 0xFFFFu); h0; h0 &= h0 - 1u, ++at) {
+                const uint32_t s = uint32_t(__ffs(h0) - 1);  // face slot s is stencil offset 2 s + 1; low bit: the dual waits
+                if (at < o.cap_s) o.s0[at] = make_key(ord, vg, (2u * s + 1u) << 1 | ((flg >> s) & 1u));
+            }
+            for (uint32_t at = bt + (ex_s >> 16); dual; dual &= dual - 1u, ++at)
+                if (at < o.cap_s) o.st[at] = ~make_key(ord, vg, (2u * uint32_t(__ffs(dual) - 1) + 1u) << 1);
+            if (root0 && CP_IN(vg, o.n_uf0, o.ctr)) {
+                const unsigned long long k = (unsigned long long)(uint64_t(ord) << 32 | vl);
+                gmin = k < gmin ? k : gmin;
+                put_root(o.uf0 + vg, br0 + __popc(m0 & lt), o.cap_r0, make_key(ord, vg, 0), o.node0, o.age0, o.res0, false, ii);
+            }
+            if (rootT) {  // the top cell in quadrant 3 of its largest corner
+                const uint32_t self = uint32_t(it.toff) + uint32_t(ey) * uint32_t(W - 1) + uint32_t(ex);
+                if (CP_IN(self, o.n_uft, o.ctr))
+                    put_root(o.uft + self, brt + __popc(mt & lt), o.cap_rt, make_key(ord, vg, 16u), o.nodet, o.aget, o.rest, true, ii);
+            }
+            b0 += all & 0xFFFFu;
+            bt += all >> 16;
+            br0 += __popc(m0);
+            brt += __popc(mt);
+        }
+        gmin = warp_min_u64(gmin);
+        if (lane == 0 && gmin != ~0ull) atomicMin(&o.ctr->gmin[ii], gmin);
     }
-    if (__any_sync(0xFFFFFFFFu, (cnt.s0 | cnt.st | cnt.r0 | cnt.rt) != 0)) warp_flush(ws, cnt, o);
 }
 
 // ---------------------------------------------------------------- host side
-size_t prune_smem2d() { return sizeof(Smem2); }
 size_t prune_smem3d() { return sizeof(Smem3); }
 
 bool encode_plane_map(CUtensorMap* map, const float* img, int64_t D, int64_t H, int64_t W) {
@@ -1199,10 +1155,10 @@ bool encode_plane_map(CUtensorMap* map, const float* img, int64_t D, int64_t H, 
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NAN_REQUEST_ZERO_FMA) == CUDA_SUCCESS;
 }
-int prune_tile_x() { return kOX2; }
+int prune_tile_x() { return kTile2; }
 int prune_tile_x3d() { return kOX; }
 int g_rows2d = 64, g_zchunk3d = kZC, g_ctas3d = 0, g_cross2d = 0, g_uf_variant = 0;  // tuning (cp_set_tuning)
-int prune_tile_y2d() { return g_rows2d; }
+int prune_tile_y2d() { return kTile2; }
 int prune_tile_y3d() { return kOY; }
 int prune_zchunk3d() { return g_zchunk3d; }
 int prune_cross2d() { return g_cross2d; }
@@ -1295,8 +1251,7 @@ static Outs outs_of(const PruneOuts& po) {
 }
 
 cudaError_t launch_expand(const ItemTable& tab, const PruneOuts& po, cudaStream_t s) {
-    if (tab.n3d < 1) return cudaSuccess;
-    k_expand3d<<<device_sm_count() * 8, 256, 0, s>>>(tab, outs_of(po));
+    k_expand<<<device_sm_count() * 8, 256, 0, s>>>(tab, outs_of(po));
     note_launches(1);
     return cudaGetLastError();
 }
@@ -1310,14 +1265,19 @@ cudaError_t launch_prune(const ItemTable& tab, const PruneOuts& po, const TmaMap
         return device_sm_count() * (per_sm > 0 ? per_sm : 1);
     });
     const int blocks2d = device_cached(kCachePrune2d, [] {
-        cudaFuncSetAttribute(k_prune2d, cudaFuncAttributeMaxDynamicSharedMemorySize, int(prune_smem2d()));
         int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_prune2d, kW2 * 32, prune_smem2d());
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_prune2d, kW2 * 32, 0);
         return device_sm_count() * (per_sm > 0 ? per_sm : 1);
     });
     if (tab.tiles2d > 0) {
-        const int need2 = (tab.tiles2d + kW2 - 1) / kW2;
-        k_prune2d<<<need2 < blocks2d ? need2 : blocks2d, kW2 * 32, prune_smem2d(), s>>>(tab, o);
+        // warps per tile (its events' rows are split): as many as leave at most
+        // 16 warps per SM; uniform noise, 1 -> 8 parts: 64^2 20.0 -> 7.8 us,
+        // 480^2 20.5 -> 9.1; smooth, 2 parts: 769 x 1021 6.6 -> 7.0 us, 2048^2
+        // (one part) 11.6 -> 18.2
+        int parts = 8;
+        while (parts > 1 && int64_t(tab.tiles2d) * parts > 2432) parts >>= 1;
+        const int need2 = (tab.tiles2d * parts + kW2 - 1) / kW2;
+        k_prune2d<<<need2 < blocks2d ? need2 : blocks2d, kW2 * 32, 0, s>>>(tab, o, parts);
         note_launches(1);
     }
     if (tab.tiles3d > 0) {

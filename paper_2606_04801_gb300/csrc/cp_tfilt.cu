@@ -29,6 +29,7 @@
 // pairs are mapped where they are put in order (cp_order.cu).
 #include "cp_common.cuh"
 #include "cp_kernels.h"
+#include "cp_walk.cuh"
 
 namespace cp {
 namespace {
@@ -90,15 +91,15 @@ __global__ void __launch_bounds__(kTT) k_t_build(const __grid_constant__ TItems 
 // ancestor of every frame vertex (every frame vertex but 0 has an earlier
 // neighbour in the frame, and equal values order by index), so the shortcut
 // changes no root.  Item blockIdx.y.
-__global__ void __launch_bounds__(kTT) k_t_flatten(uint32_t* __restrict__ uf0, uint8_t* __restrict__ code,
-                                                   const __grid_constant__ TItems t) {
+__global__ void __launch_bounds__(kTT) k_t_flatten(uint8_t* __restrict__ code, const __grid_constant__ TItems t) {
     const int item = blockIdx.y;
     const TDims& d = t.d[item];
-    uint32_t* __restrict__ uf = uf0 + t.voff[item];
     uint8_t* __restrict__ cd = code + t.coff[item];
     const int64_t P = t.pitch[item];
-    const uint32_t root = uint32_t(t.voff[item]);
     const int64_t Dj = d.ndim == 3 ? d.D + 2 : 1, Hj = d.H + 2, Wj = d.W + 2;
+    Item j2;  // the shape that code_at2 wants
+    j2.W = int32_t(Wj);
+    auto at2 = [&](int64_t y, int64_t x) { return code_at2(j2, int(y), int(x)); };
     // whole frame rows, one block per row: both y faces of every plane, and
     // the two z faces (3D)
     const int64_t zf = d.ndim == 3 ? 2 * Hj : 0;  // rows of the two z faces
@@ -113,12 +114,11 @@ __global__ void __launch_bounds__(kTT) k_t_flatten(uint32_t* __restrict__ uf0, u
             z = d.ndim == 3 ? 1 + g / 2 : 0;
             y = (g & 1) ? Hj - 1 : 0;
         }
-        uint32_t* row = uf + (z * Hj + y) * Wj;
         uint8_t* crow = cd + (z * Hj + y) * P;
         for (int64_t x = threadIdx.x; x < Wj; x += kTT)
             if (z != 0 || y != 0 || x != 0) {
                 if (d.ndim == 3) crow[x] |= 7u;
-                else row[x] = root;
+                else cd[at2(y, x)] |= 15u;
             }
     }
     // the two x faces of the other rows
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kTT) k_t_flatten(uint32_t* __restrict__ uf0, u
         const int64_t z = d.ndim == 3 ? 1 + q / yi : 0, y = 1 + q % yi;
         const int64_t x = (k & 1) ? Wj - 1 : 0;
         if (d.ndim == 3) cd[(z * Hj + y) * P + x] |= 7u;
-        else uf[(z * Hj + y) * Wj + x] = root;
+        else cd[at2(y, x)] |= 15u;
     }
 }
 
@@ -145,10 +145,10 @@ cudaError_t launch_t_build(const TItems& t, uint32_t* bad, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_t_flatten(uint32_t* uf0, uint8_t* code, const TItems& t, cudaStream_t s) {
+cudaError_t launch_t_flatten(uint8_t* code, const TItems& t, cudaStream_t s) {
     if (t.n < 1 || t.n > kMaxItems) return cudaErrorInvalidValue;
     const int gx = (device_sm_count() * 8 + t.n - 1) / t.n;
-    k_t_flatten<<<dim3(gx, t.n), kTT, 0, s>>>(uf0, code, t);
+    k_t_flatten<<<dim3(gx, t.n), kTT, 0, s>>>(code, t);
     note_launches(1);
     return cudaGetLastError();
 }

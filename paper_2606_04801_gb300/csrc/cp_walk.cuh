@@ -1,15 +1,23 @@
 // Walks through the pruned forests, from a survivor's two endpoints to the
 // roots of their classes.
 //
-// 2D items: a 32-bit word per vertex / top cell, the parent's id or a tagged
-// root id.  3D items: a code byte per vertex, at (z H + y) pitch + x of the
-// item's codes: bits 0-2 the vertex's H0 link (face slot 0..5, 6: a root, 7: a
-// frame vertex of a T-filtration item, whose root is vertex 0), bits 3-6 the
-// dual link of the top cell with its smallest corner one plane below, at
-// (z - 1, y, x) (0..6: towards that slot as seen from that corner, 7: a root,
-// 8: the outside, 9, 10, 11: +z, +y, +x).  Only a root's word of the 32-bit arrays is written for 3D items (its
-// root id).  A 512^3 volume's codes (134 MB) mostly stay in L2 between the
-// pruning pass and the walks, where words (1,074 MB) did not.
+// Both are in a code byte per vertex; of the 32-bit arrays only a root's word
+// is written (its root id).
+//
+// 3D items: at (z H + y) pitch + x of the item's codes, bits 0-2 the vertex's
+// H0 link (face slot 0..5, 6: a root, 7: a frame vertex of a T-filtration
+// item, whose root is vertex 0), bits 3-6 the dual link of the top cell with
+// its smallest corner one plane below, at (z - 1, y, x) (0..6: towards that
+// slot as seen from that corner, 7: a root, 8: the outside, 9, 10, 11: +z, +y,
+// +x).  A 512^3 volume's codes (134 MB) mostly stay in L2 between the pruning
+// pass and the walks, where words (1,074 MB) did not.
+//
+// 2D items: 30 rows of a column at a time in one 32-byte sector (code_at2: a
+// column of a pruning tile), bits 0-3 the H0 link (0..4: up by 1 << d rows, all
+// of whose vertices but the last link up; 5, 6, 7: left, right, down; 14: a
+// root, 15: the frame as above), bits 4-7 the dual link of the top cell with
+// its smallest corner there (0..4: +y by 1 << d, likewise; 5..8: +x, -x, -y,
+// both; 9: the outside, 15: a root).  Runs end where the tile does.
 #pragma once
 #include "cp_common.cuh"
 
@@ -26,43 +34,140 @@ __host__ __device__ __forceinline__ int32_t link_offset3(int dual, uint32_t d, i
     return d == 9u ? hp : (d == 10u ? p : 1);
 }
 
+constexpr int kTile2 = 30;  // rows (and columns) of a 2D pruning tile
+
+// Where vertex (y, x) of a 2D item has its code byte (its first byte is the
+// item's).
+__host__ __device__ __forceinline__ uint32_t code_at2(const Item& it, int y, int x) {
+    const uint32_t t = uint32_t(y) / uint32_t(kTile2);
+    return (t * uint32_t(it.W) + uint32_t(x)) * 32u + (uint32_t(y) - t * uint32_t(kTile2));
+}
+
+// Offset of the 2D link with code field d (H0: 0..7; dual: 0..8).
+__host__ __device__ __forceinline__ void link_offset2(int dual, uint32_t d, int& dy, int& dx) {
+    const int run = d < 5u ? 1 << d : 0;
+    if (!dual) {
+        dy = d == 7u ? 1 : -run;
+        dx = d == 5u ? -1 : (d == 6u ? 1 : 0);
+    } else {
+        dy = d >= 7u ? -1 : run;
+        dx = d == 5u ? 1 : (d == 6u || d == 8u ? -1 : 0);
+    }
+}
+
 #ifdef __CUDACC__
 struct Forest {
-    const uint32_t* uf;    // 2D: links; 3D: root words
-    const uint8_t* code;   // 3D items' codes
+    const uint32_t* uf;    // root words
+    const uint8_t* code;   // codes
     uint32_t n_nodes;      // entries of uf / code (bounds-checked build)
     uint64_t n_code;
     int dual;
 };
 
-// One endpoint's path in a 3D item's codes.
-struct Path3 {
+// One endpoint's path in an item's codes: where it is, and whether it has
+// reached the outside (which has no code).
+struct Path {
     uint32_t at;
-    bool live, out;
+    bool out;
 };
 
-__device__ __forceinline__ void step3(const Forest& f, const Item& it, int32_t hp, Counters* ctr, Path3& p) {
+// What a link does, by its code field d, without branches, so that both paths
+// of every lane have a load in flight all the time.  A code that is no step
+// leaves the path where it is.  Bound by the latency of these loads (L2, or L1
+// for steps along a sector); with a branch per kind of link and path, k_roots2
+// took 185 us at 512^3 instead of 108, 84 instead of 59 for 128^3 noise.
+//
+// 3D: per unit of z, y and x, two bits at 2 d hold the offset + 1.
+template <class... P>
+constexpr uint32_t step_field(uint32_t w, uint32_t d, uint32_t v, P... rest) {
+    w = (w & ~(3u << (2 * d))) | v << (2 * d);
+    if constexpr (sizeof...(rest) > 0) return step_field(w, rest...);
+    return w;
+}
+constexpr uint32_t kStay = 0x55555555u;
+// H0: -z -y -x +x +y +z
+constexpr uint32_t kStepZ0 = step_field(kStay, 0u, 0u, 5u, 2u), kStepY0 = step_field(kStay, 1u, 0u, 4u, 2u),
+                   kStepX0 = step_field(kStay, 2u, 0u, 3u, 2u);
+// dual: the corners of slots 0 .. 6, then +z +y +x
+constexpr uint32_t kStepZ1 = step_field(kStay, 0u, 0u, 1u, 0u, 2u, 0u, 3u, 0u, 9u, 2u),
+                   kStepY1 = step_field(kStay, 0u, 0u, 1u, 0u, 4u, 0u, 5u, 0u, 10u, 2u),
+                   kStepX1 = step_field(kStay, 0u, 0u, 2u, 0u, 4u, 0u, 6u, 0u, 11u, 2u);
+struct Step3 {
+    uint32_t cz, cy, cx, shift, mask, hp, p;
+    __device__ __forceinline__ Step3(int dual, int32_t hp_, int32_t p_)
+        : cz(dual ? kStepZ1 : kStepZ0), cy(dual ? kStepY1 : kStepY0), cx(dual ? kStepX1 : kStepX0), shift(dual ? 3u : 0u),
+          mask(dual ? 15u : 7u), hp(uint32_t(hp_)), p(uint32_t(p_)) {}
+    __device__ __forceinline__ uint32_t field(uint32_t c) const { return (c >> shift) & mask; }
+    __device__ __forceinline__ uint32_t next(uint32_t at, uint32_t d) const {
+        const uint32_t s = 2u * d;
+        return at + ((cz >> s) & 3u) * hp + ((cy >> s) & 3u) * p + ((cx >> s) & 3u) - (hp + p + 1u);
+    }
+    __device__ __forceinline__ bool ends(uint32_t d) const { return mask == 7u ? d >= 6u : (0xF180u >> d) & 1u; }
+    __device__ __forceinline__ bool outside(uint32_t d) const { return mask == 15u && d == 8u; }
+    __device__ __forceinline__ bool frame(uint32_t d) const { return mask == 7u && d == 7u; }
+};
+struct Step2 {
+    uint32_t shift, last, band, far;  // far: what codes 5 .. 8 add, a signed byte each
+    int32_t sign;
+    __device__ __forceinline__ Step2(int dual, int32_t W)
+        : shift(dual ? 4u : 0u), last(dual ? 9u : 8u), band(32u * uint32_t(W)), far(dual ? 0xDFFFE020u : 0x000120E0u),
+          sign(dual ? 1 : -1) {}
+    __device__ __forceinline__ uint32_t field(uint32_t c) const { return (c >> shift) & 15u; }
+    __device__ __forceinline__ uint32_t next(uint32_t at, uint32_t d) const {
+        const int32_t step = d < 5u ? sign * (1 << d) : int32_t(far << (24u - 8u * ((d - 5u) & 3u))) >> 24;
+        at += d < last ? uint32_t(step) : 0u;
+        const uint32_t r = at & 31u;  // 30: one row below the tile, 31: one above it (and a column to the left)
+        if (r >= uint32_t(kTile2)) at += r == 31u ? uint32_t(kTile2) - band : band - uint32_t(kTile2);
+        return at;
+    }
+    __device__ __forceinline__ bool ends(uint32_t d) const { return d >= last; }
+    __device__ __forceinline__ bool outside(uint32_t d) const { return last == 9u && d == 9u; }
+    __device__ __forceinline__ bool frame(uint32_t d) const { return last == 8u && d == 15u; }
+};
+
+// Both paths in lockstep until neither has a link to follow.  False: the
+// bounded walk gave up (a corrupted forest).
+template <class Step>
+__device__ __forceinline__ bool follow(const Forest& f, uint64_t coff, const Step& st, Counters* ctr, Path& a, Path& b,
+                                       uint32_t& hops) {
+    uint64_t t0 = 0;
+    const uint8_t* code = f.code + coff;
+    uint32_t da, db;
     (void)ctr;
-    const uint64_t i = uint64_t(it.coff) + p.at;
-    if (!CP_IN(i, f.n_code, ctr)) {
-        p.live = false;
-        p.at = 0;
-        return;
+    for (uint32_t n = 1;; ++n) {
+        if (!CP_IN(coff + a.at, f.n_code, ctr)) a = Path{0, true};
+        if (!CP_IN(coff + b.at, f.n_code, ctr)) b = Path{0, true};
+        const uint32_t ca = __ldg(code + a.at), cb = __ldg(code + b.at);
+        da = st.field(ca);
+        db = st.field(cb);
+        a.at = a.out ? 0u : st.next(a.at, da);
+        b.at = b.out ? 0u : st.next(b.at, db);
+        ++hops;
+        if ((a.out || st.ends(da)) && (b.out || st.ends(db))) break;
+        if ((n & 1023u) == 0) {
+            const uint64_t now = global_timer_ns();
+            if (t0 == 0) t0 = now;
+            if (now - t0 > kWaitLimitNs) return false;
+        }
     }
-    const uint32_t c = __ldg(f.code + i);
-    const uint32_t d = f.dual ? c >> 3 : c & 7u;
-    if (f.dual ? d == 7u : d == 6u) {
-        p.live = false;
-    } else if (f.dual ? d == 8u : d == 7u) {
-        p.live = false;
-        p.out = f.dual;  // else: the frame of a T item, rooted at vertex 0
-        p.at = 0;
-    } else {
-        p.at += uint32_t(link_offset3(f.dual, d, hp, it.pitch));
-    }
+    // the frame of a T item is rooted at vertex 0
+    if (!a.out && st.frame(da)) a.at = 0;
+    if (!b.out && st.frame(db)) b.at = 0;
+    a.out |= st.outside(da);
+    b.out |= st.outside(db);
+    return true;
 }
 
-__device__ __forceinline__ uint32_t root_id3(const Forest& f, const Item& it, int item, Counters* ctr, const Path3& p) {
+__device__ __forceinline__ uint32_t root_id2(const Forest& f, const Item& it, int item, Counters* ctr, const Path& p) {
+    if (p.out) return uint32_t(item);
+    const uint32_t q = p.at >> 5, t = q / uint32_t(it.W), x = q - t * uint32_t(it.W);
+    const uint32_t y = t * uint32_t(kTile2) + (p.at & 31u);
+    const uint32_t node = f.dual ? uint32_t(it.toff) + y * uint32_t(it.W - 1) + x : uint32_t(it.voff) + y * uint32_t(it.W) + x;
+    (void)ctr;
+    return CP_IN(node, f.n_nodes, ctr) ? __ldg(f.uf + node) & ~kTag : 0u;
+}
+
+__device__ __forceinline__ uint32_t root_id3(const Forest& f, const Item& it, int item, Counters* ctr, const Path& p) {
     if (p.out) return uint32_t(item);
     const uint32_t row = p.at / uint32_t(it.pitch), x = p.at - row * uint32_t(it.pitch);
     uint32_t node;
@@ -89,17 +194,9 @@ __device__ __forceinline__ bool walk_roots(const ItemTable& tab, const Forest& f
     const uint32_t local = vg - uint32_t(it.voff), W = uint32_t(it.W), H = uint32_t(it.H);
     const uint32_t row = local / W;
     const int x = int(local - row * W);
-    uint64_t t0 = 0;
-    uint32_t steps = 0;
-    auto overdue = [&]() {
-        if ((++steps & 1023u) != 0) return false;
-        const uint64_t now = global_timer_ns();
-        if (t0 == 0) t0 = now;
-        return now - t0 > kWaitLimitNs;
-    };
     if (it.ndim == 3) {
         const int32_t p = it.pitch, hp = int32_t(H) * p;
-        Path3 a = {row * uint32_t(p) + uint32_t(x), true, false}, b = a;
+        Path a = {row * uint32_t(p) + uint32_t(x), false}, b = a;
         if (!f.dual) {
             b.at += uint32_t(dz * hp + dy * p + dx);
         } else {
@@ -109,51 +206,42 @@ __device__ __forceinline__ bool walk_roots(const ItemTable& tab, const Forest& f
             auto corner = [&](int s) {  // s: the zero coordinate's side (-1, +1)
                 const int qz = dz == 0 && s < 0 ? z - 1 : cz, qy = dy == 0 && s < 0 ? y - 1 : cy,
                           qx = dx == 0 && s < 0 ? x - 1 : cx;
-                Path3 q = {0, true, false};
-                if (qz < 0 || qz >= it.D - 1 || qy < 0 || qy >= it.H - 1 || qx < 0 || qx >= it.W - 1) {
-                    q.live = false;
-                    q.out = true;
-                } else {
-                    q.at = uint32_t((qz + 1) * hp + qy * p + qx);
-                }
-                return q;
+                const bool out = qz < 0 || qz >= it.D - 1 || qy < 0 || qy >= it.H - 1 || qx < 0 || qx >= it.W - 1;
+                return Path{out ? 0u : uint32_t((qz + 1) * hp + qy * p + qx), out};
             };
             a = corner(-1);
             b = corner(1);
         }
-        while (a.live || b.live) {
-            if (a.live) step3(f, it, hp, ctr, a);
-            if (b.live) step3(f, it, hp, ctr, b);
-            ++hops;
-            if (overdue()) {
-                ra = rb = 0;
-                return false;
-            }
+        if (!follow(f, uint64_t(it.coff), Step3(f.dual, hp, p), ctr, a, b, hops)) {
+            ra = rb = 0;
+            return false;
         }
         ra = root_id3(f, it, item, ctr, a);
         rb = root_id3(f, it, item, ctr, b);
         return true;
     }
-    uint32_t na = vg, nb = uint32_t(int64_t(vg) + int64_t(dy) * W + dx);
-    if (f.dual) {
-        // the facet's zero coordinate picks the side
-        const int y = int(row);
-        na = top_of_octant(it, 0, y, x, -1, dy == 0 ? -1 : dy, dy == 0 ? dx : -1);
-        nb = top_of_octant(it, 0, y, x, 1, dy == 0 ? 1 : dy, dy == 0 ? dx : 1);
+    const int y = int(row);
+    Path a = {0, false}, b = a;
+    if (!f.dual) {
+        a.at = code_at2(it, y, x);
+        b.at = code_at2(it, y + dy, x + dx);
+    } else {
+        // as in 3D
+        const int cy = y + (dy < 0 ? -1 : 0), cx = x + (dx < 0 ? -1 : 0);
+        auto corner = [&](int s) {
+            const int qy = dy == 0 && s < 0 ? y - 1 : cy, qx = dx == 0 && s < 0 ? x - 1 : cx;
+            const bool out = qy < 0 || qy >= it.H - 1 || qx < 0 || qx >= it.W - 1;
+            return Path{out ? 0u : code_at2(it, qy, qx), out};
+        };
+        a = corner(-1);
+        b = corner(1);
     }
-    uint32_t pa = CP_IN(na, f.n_nodes, ctr) ? __ldcg(f.uf + na) : kTag;
-    uint32_t pb = CP_IN(nb, f.n_nodes, ctr) ? __ldcg(f.uf + nb) : kTag;
-    while (!(pa & kTag) || !(pb & kTag)) {
-        ++hops;
-        if (!(pa & kTag)) pa = CP_IN(pa, f.n_nodes, ctr) ? __ldcg(f.uf + pa) : kTag;
-        if (!(pb & kTag)) pb = CP_IN(pb, f.n_nodes, ctr) ? __ldcg(f.uf + pb) : kTag;
-        if (overdue()) {
-            ra = rb = 0;
-            return false;
-        }
+    if (!follow(f, uint64_t(it.coff), Step2(f.dual, it.W), ctr, a, b, hops)) {
+        ra = rb = 0;
+        return false;
     }
-    ra = pa & ~kTag;
-    rb = pb & ~kTag;
+    ra = root_id2(f, it, item, ctr, a);
+    rb = root_id2(f, it, item, ctr, b);
     return true;
 }
 #endif

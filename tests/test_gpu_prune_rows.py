@@ -1,6 +1,6 @@
-"""The 2D pruning pass at the edges of its 31-column strips and of its row
-tasks (4 rows for small images, more where the strips would not all run at
-once), alone and batched, against the oracle: every field of every pair."""
+"""The 2D pruning pass at the edges of its 30 x 30 tiles, with one to eight
+warps per tile, alone and batched, against the oracle: every field of every
+pair."""
 import numpy as np
 import pytest
 
@@ -27,7 +27,7 @@ def _same(got, want, what):
 
 
 @pytest.mark.parametrize("shape", [(2, 2), (3, 32), (4, 31), (5, 62), (6, 30), (9, 63), (13, 1000), (3001, 7), (640, 962), (1301, 517),
-                                   (47, 12007)])
+                                   (47, 12007), (30, 30), (31, 60), (61, 91), (500, 600), (1500, 1501)])
 @pytest.mark.parametrize("kind", ["noise", "levels", "plateau"])
 def test_task_edges(shape, kind):
     import paper_2606_04801_gb300 as cp
@@ -39,7 +39,7 @@ def test_task_edges(shape, kind):
         _same(cp.persistence(x, filtration="T").numpy(), oracle.persistence_t(img), f"T {shape} {kind}")
 
 
-def test_one_row_count_for_a_batch():
+def test_batch_of_uneven_images():
     import paper_2606_04801_gb300 as cp
 
     imgs = [_image(s, "levels") for s in [(5, 31), (700, 901), (2, 63), (129, 33)]] + [workloads.uniform((3, 4, 5), 2)]
