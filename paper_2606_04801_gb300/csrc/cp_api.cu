@@ -16,6 +16,7 @@
 
 #include "cp_common.cuh"
 #include "cp_kernels.h"
+#include "cp_walk.cuh"
 #include "cp_lut.h"
 
 namespace cp {
@@ -126,13 +127,13 @@ void plan_boruvka(Plan& P);
 // Owned planes per 3D pruning task, at most the tuned bound: the value that
 // makes the fewest plane steps on the busiest CTA, counting kStart steps for
 // a task's start (its planes' first loads and the lead-in and lead-out steps).
-// One value for all items of a call; 456 CTAs run at once (152 SMs x 3).
+// One value for all items of a call; 1216 CTAs run at once (152 SMs x 8).
 int plan_zchunk(const ItemTable& tab) {
-    constexpr int kSlots = 456, kStart = 6;
+    constexpr int kSlots = 1216, kStart = 3;
     const int hi = prune_zchunk3d();
     int best = hi;
     int64_t best_cost = INT64_MAX;
-    for (int c = 4; c <= hi; ++c) {
+    for (int c = 1; c <= hi; ++c) {
         int64_t tasks = 0;
         int dmax = 0;
         for (int j = tab.n2d; j < tab.n; ++j) {
@@ -217,9 +218,9 @@ int make_plan(int n_items, const int32_t* ndims, const int64_t* dims, const floa
     for (int j = P.tab.n2d; j < n_items; ++j) {
         Item& it = P.tab.it[j];
         it.zc = zc;
-        it.pitch = (it.W + 3) & ~3;
+        it.bands = (it.H + kBand3 - 1) / kBand3;
         it.coff = int64_t(P.n_code);
-        P.n_code += uint64_t(it.D) * uint64_t(it.H) * uint64_t(it.pitch);
+        P.n_code += uint64_t(it.D) * uint64_t(it.bands) * uint64_t(it.W) * 32u;  // 32 bytes per column of a band (code_at3)
         it.tz = (it.D + zc - 1) / zc;
         it.tile0 = t3;
         t3 += it.tx * it.ty * it.tz;
@@ -966,7 +967,7 @@ int t_run(int n_items, const float* const* h_images, const int32_t* ndims, const
         const Item& it = P.tab.it[j];
         tm.items.voff[it.user] = it.voff;
         tm.items.coff[it.user] = it.coff;
-        tm.items.pitch[it.user] = it.ndim == 3 ? it.pitch : 0;
+        tm.items.bands[it.user] = it.ndim == 3 ? it.bands : 0;
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (launch_t_build(tm.items, bad, s) != cudaSuccess) return CP_ERR_CUDA;
@@ -1189,7 +1190,7 @@ int cubical_persistence_debug_layout(int n_items, const int32_t* ndims, const in
     Plan P;
     int rc = make_plan(n_items, ndims, dims, nullptr, max_survivors, P);
     if (rc != CP_OK) return rc;
-    const int64_t v[13] = {int64_t(P.o_ctr), int64_t(P.o_uf0),  int64_t(P.o_uft),  int64_t(P.o_s0),
+    const int64_t v[13] = {int64_t(P.o_ctr + offsetof(Counters, status)), int64_t(P.o_uf0),  int64_t(P.o_uft),  int64_t(P.o_s0),
                            int64_t(P.o_st),  int64_t(P.o_age0), int64_t(P.o_aget), int64_t(P.ntot),
                            int64_t(P.ttot),  int64_t(P.cap_s),  int64_t(P.cap_r0), int64_t(P.cap_rt),
                            int64_t(P.o_ctr + offsetof(Counters, tma_tasks))};

@@ -36,7 +36,7 @@ struct Item {
     int32_t user;             // the caller's index of the item
     int32_t tma;              // 3D: index of the item's plane tensor map (TMA loads), or -1
     int32_t zc;               // 3D: owned planes per pruning task
-    int32_t pitch;            // 3D: row pitch of the item's link codes (its width, rounded up to 4)
+    int32_t bands;            // 3D: bands of rows in a plane of the item's link codes (cp_walk.cuh)
     int64_t coff;             // the item's first link code
 };
 
@@ -51,7 +51,8 @@ struct ItemTable {
 
 // ---------------------------------------------------------------- counters
 // Lives at the start of the workspace.  Zeroed at the start of every call.
-struct Counters {
+struct alignas(8) Counters {
+    uint32_t spare;           // n_s0 and n_st, and n_r0 and n_rt, are added to in pairs
     uint32_t status;
     uint32_t n_s0;            // H0 survivors appended
     uint32_t n_st;            // dual survivors appended

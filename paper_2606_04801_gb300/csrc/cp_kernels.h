@@ -314,8 +314,8 @@ struct TItems {
     const float* img[kMaxItems];  // the image
     float* J[kMaxItems];          // its dual image: extents +2 along each image axis
     int64_t voff[kMaxItems];      // J's first vertex in the call's vertex space
-    int64_t coff[kMaxItems];      // J's first code; 3D: its codes' row pitch
-    int32_t pitch[kMaxItems];
+    int64_t coff[kMaxItems];      // J's first code; 3D: its planes' bands
+    int32_t bands[kMaxItems];
 };
 // J <- -image flipped along every axis, inside a one-voxel frame at -FLT_MAX;
 // *bad <- 1 if a pixel is not below FLT_MAX (the frame would not come first).

@@ -327,6 +327,7 @@ uint64_t check_words3(const Lut3D& lut) {
                 }
                 ok = ok && want == int(lut_dual(e, t));
             }
+            for (int b = 0; b < 27; ++b) ok = ok && (b == 13 || bit(relevant_plane(s, b)) == int((m >> b) & 1u));
             const bool needs = lut_h0_surv(e) || lut_dual_surv(e) || direct == 6 || lut_dual(e, 7) == 8;
             if (!ok || (needs && !bit(s.event))) ++bad;
         }

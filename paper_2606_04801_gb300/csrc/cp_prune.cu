@@ -92,6 +92,25 @@ __device__ __forceinline__ void put_root(uint32_t* word, uint32_t g, uint32_t ca
     *word = kTag | g;
 }
 
+// Room for a warp's survivors (H0, dual) and roots (the same) in their arrays:
+// lanes 0 and 1 add to the two pairs of counters.  (All of a noise volume's
+// events come through these: four atomics instead of two held them up.)
+__device__ __forceinline__ void reserve(const Outs& o, uint32_t s0, uint32_t st, uint32_t r0, uint32_t rt, uint32_t& b0,
+                                        uint32_t& bt, uint32_t& br0, uint32_t& brt) {
+    const unsigned lane = lane_id();
+    const uint32_t lo = lane == 0 ? s0 : r0, hi = lane == 0 ? st : rt;
+    unsigned long long base = 0;
+    if (lane < 2 && (lo | hi)) {
+        unsigned long long* c = reinterpret_cast<unsigned long long*>(lane == 0 ? &o.ctr->n_s0 : &o.ctr->n_r0);
+        base = atomicAdd(c, (unsigned long long)hi << 32 | lo);
+        if ((lo && uint32_t(base) + lo > (lane == 0 ? o.cap_s : o.cap_r0)) ||
+            (hi && uint32_t(base >> 32) + hi > (lane == 0 ? o.cap_s : o.cap_rt)))
+            set_status(o.ctr, kStCapacity);
+    }
+    const unsigned long long s = __shfl_sync(0xFFFFFFFFu, base, 0), r = __shfl_sync(0xFFFFFFFFu, base, 1);
+    b0 = uint32_t(s), bt = uint32_t(s >> 32), br0 = uint32_t(r), brt = uint32_t(r >> 32);
+}
+
 // Perfect hash of the 15,935 relevant masks (device layout, cp_mask3.cuh):
 // bucket -> displacement -> slot.
 __device__ __forceinline__ uint32_t hash_slot3(uint32_t rel, const uint16_t* disp) {
@@ -103,28 +122,24 @@ __device__ __forceinline__ uint32_t hash_slot3(uint32_t rel, const uint16_t* dis
 }  // namespace
 
 // ---------------------------------------------------------------- 3D
-// A CTA marches along z through a tile of 64 x 32 columns, of which it owns
-// 60 x 29.  The lookup of a vertex is done 32 vertices at a time, on words
-// that hold one bit per vertex:
+// A CTA of two warps marches along z through a tile of 60 x 29 columns.  A
+// warp compares 32 x 32 vertices of a plane, of which it owns 30 x 29, and
+// does all of it on words: lane = column, bit = row.
 //
-//   compare  (4 warps, 8 rows each) of every vertex p of a plane and each of
-//            the 13 neighbours q after it in linear order: does q precede p?
-//            A warp does a row of 64 columns, two per lane (even columns give
-//            one word, odd columns another): a compare and a ballot per
-//            neighbour.  The other 13 neighbours' bits are the complements of
-//            the neighbours' own.
-//   logic    (2 warps: even and odd columns; lane = row) the relevant mask
-//            (the collapse of Sec. 3.3 is one AND per edge and two per corner,
-//            for 32 vertices), the H0 link, the top cells in the lower stars
-//            and where each dies, and the vertices that need more than a link
-//            (events); a code byte per vertex with both links (cp_walk.cuh).
-//   output   (compare warps) the code bytes, two 4-byte stores per 8 columns.
-//   events   (compare warps, 32 at a time once a warp each has some) the
-//            vertices whose lower star holds a survivor or a root: their masks
-//            from the image, the lookup, the keys and roots.
-//
-// The two kinds of warps hand planes on through named barriers, either a plane
-// ahead of the other.
+//   compare  of every vertex with the 13 neighbours after it in linear order:
+//            the sign of a difference (exact: zero only for equal values),
+//            shifted into the lane's word.  The neighbours to the left belong
+//            to the next lane's vertex, whose value the lane has as well; the
+//            other 13 neighbours' bits are the complements of their own.
+//   logic    on those words, 32 x 32 vertices per instruction: the relevant
+//            mask (the collapse of Sec. 3.3 is one AND per edge and two per
+//            corner), the H0 link, the top cells in the lower stars and where
+//            each dies, and the vertices that need more than a link (events).
+//   output   one code byte per vertex with both links (cp_walk.cuh), a column
+//            of a band in one 32-byte sector.
+//   events   the vertices whose lower star holds a survivor or a root: each
+//            lane takes its relevant masks from the words; 32 at a time, once
+//            a warp has as many, the lookup, the keys and roots.
 //
 // Closed forms used by the logic (compared with the table's entry on all
 // 15,935 classes, check_words3):
@@ -136,124 +151,57 @@ __device__ __forceinline__ uint32_t hash_slot3(uint32_t rel, const uint16_t* dis
 //   - L(v) has survivors or a root only if the lower link is not a disc: its
 //     Euler characteristic is not 1 or it is not connected.
 //
-// Bound by the issue of compares, ballots and word logic (ALU pipe): 112 warp
-// instructions per 32 vertices at 256^3 (halo and chunk lead-in included; 280
-// with a 26-compare mask, a collapse and a table read per vertex, and links
-// stored as words), 40 of them the compares and ballots.  One byte per vertex
-// written instead of eight.  128^3 smooth 90 -> 28 us, 128^3 noise 282 -> 202
-// us, 512^3 1,430 -> 673 us.  Tried: eight compare warps per CTA (72
-// registers: spills, 1.2x the time), one logic warp (it bounds the step), a
-// CTA barrier per plane instead of the named ones, the row loop unrolled fully
-// (instruction cache misses), links as words with z chains (670 -> 840 us, and
-// the walks miss L2).
-constexpr int kW3 = 4;                     // compare warps per CTA (and two logic warps: even and odd columns)
-constexpr int kT3 = kW3 * 32;              // threads of the compare warps
-constexpr int kTX = 64, kTY = 32;          // compared columns / rows: x0-1 .. x0+62, y0-1 .. y0+30
-constexpr int kOX = 60, kOY = 29;          // owned: x0 .. x0+59, y0 .. y0+28
-constexpr int kRows = kTY / kW3;           // rows per warp
-constexpr int kUnrollC = 4;                // rows per turn of the compare loop (all eight: instruction cache misses)
-constexpr int kZC = 64;                    // default bound on the owned planes of a task
-constexpr int kRW = kTX + 2, kRH = kTY + 2;  // plane tile read: cols x0-2 .. x0+63, rows y0-2 .. y0+31
-constexpr int kRX = 2;                     // column x0-2 within a ring row (rows start at x0-4: 16-byte aligned)
-constexpr int kRS = 72;                    // ring row stride in floats (a TMA box row)
-constexpr int kSlot = 2464;                // ring slot in floats: kRH rows of kRS, padded to 128 bytes
-constexpr int kFix = (2 * kRH + 2 * kRW + 31) / 32;  // border positions set per lane of a logic warp
-constexpr int kRing = 3;                   // ring slots
-constexpr int kWR = 28;                    // words per row: 26, padded (16-byte rows; LDS.128 without conflicts)
-constexpr int kCR = 80;                    // code bytes per row: 64, padded
-constexpr int kQ = 4096;                   // event queue (two planes of 1,740 while fewer than kQMin wait)
-constexpr int kQMin = kT3;                 // events that a pass over the queue takes at least ...
-constexpr int kQAge = 16;                  // ... unless the oldest is this many planes back (entries hold z mod 32)
+// Positions outside the image read NaN, which precedes nothing; the complement
+// bits of such neighbours are masked.
+//
+// Bound by issue (63% of the slots, 12 warps per SM resident on average; a
+// fifth of the warps' time is one waiting for the other at a plane): 86 warp
+// instructions per 32 vertices at 384^3, 45 of them the differences and
+// shifts, which share the FMA and ALU pipes.  Two warps per CTA because they
+// wait for one another at every plane (eight: 44% of the time, 736 us at
+// 512^3).  Against compares and ballots in four warps that handed words to two
+// logic warps through shared memory: 512^3 smooth 673 -> 443 us, 256^3 smooth
+// (254 x 256 x 250) 121 -> 91, 128^3 smooth 27.6 -> 23.6, 128^3 noise 202 ->
+// 156.  Tried: slots freed by mbarriers instead of a CTA barrier (the same
+// waits, 468 us), four or two rows per turn of the compare loop (451, 455).
+constexpr int kWX3 = 2, kWY3 = 1;            // warps along x and y
+constexpr int kW3 = kWX3 * kWY3, kT3 = kW3 * 32;
+constexpr int kOWX = 30;                     // owned columns of a warp (owned rows: kBand3)
+constexpr int kOX = kWX3 * kOWX, kOY = kWY3 * kBand3;  // owned by the CTA: 60 x 29
+constexpr int kZC = 64;                      // default bound on the owned planes of a task
+constexpr int kRS = 68;                      // ring row: columns x0-4 .. x0+63 (16-byte aligned; a TMA box row)
+constexpr int kRX = 3;                       // column x0-1 within a ring row
+constexpr int kRW = kOX + 3;                 // columns read: x0-1 .. x0+61
+constexpr int kRH = kOY + 3;                 // rows y0-1 .. y0+30
+constexpr int kSlot = kRH * kRS;             // ring slot in floats
+constexpr int kRing = 3;                     // ring slots
+constexpr int kQ = 64;                       // events of a warp that wait (fewer than 32, and up to 32 more)
+static_assert(kSlot % 32 == 0, "slots start at 128-byte boundaries");
 
 // One task's place and constants (uniform over the CTA).
 struct Task3 {
     const float* img;
     int D, H, W, x0, y0, z0, z1, zlast;  // owned planes [z0, z1), zlast = z1 - 1
-    uint32_t HW, W1, HW1, voff, toff, pitch;
+    uint32_t HW, W1, HW1, voff, toff;
     int item;                // its index in the call's table
-    uint8_t* code;           // the item's link codes
     const CUtensorMap* map;  // nullptr: the planes come by cp.async
-    uint32_t own[2], cube[2];       // even / odd columns whose vertex / top cell the task owns
-    uint32_t first_x[2], last_x[2]; // the columns x = 0 and x = W - 2
 };
 
-// Ring slot of plane z >= -1.
-__device__ __forceinline__ int ring_slot(int z) { return int(unsigned(z + kRing) % unsigned(kRing)); }
+// Ring slot of plane z >= 0.
+__device__ __forceinline__ int ring_slot(int z) { return int(unsigned(z) % unsigned(kRing)); }
+
+struct Queue3 {
+    uint32_t rel[kQ], at[kQ];  // relevant mask (device layout); plane of the task << 10 | row << 5 | lane
+    float val[kQ];
+};
 
 struct Smem3 {
-    float ring[kRing][kSlot];  // first: slots 128-byte aligned (TMA destinations)
+    Queue3 queue[kW3];         // (a slot's first row is read one row up, into what lies before, and not used)
+    alignas(128) float ring[kRing][kSlot];  // TMA destinations
     uint64_t bar[kRing];       // mbarrier of each slot (TMA completion)
-    // compare words of a row: groups of {dx = -1, 0, +1} x {even, odd columns}
-    // for (dz, dy) = (1,-1) (1,0) (1,1) (0,1), then (0,0,+1)
-    alignas(16) uint32_t w[3][kTY][kWR];
-    alignas(16) uint8_t code[2][kTY][kCR];  // columns 2, 4 .. 62 (and a pad), then 1, 3 .. 63; dual << 3 | H0
-    // what the top cells below a plane need of the plane before, per row and parity
-    uint32_t low[2][6][kTY];
-    uint32_t xco[2][4][kTY], xev[2];  // between the two logic warps
-    uint16_t queue[kQ];        // event vertices: (z mod 32) << 11 | row << 6 | column
-    uint32_t tail[2];          // events queued up to the last even / odd plane
     Task3 t;
 };
-
-// raw |= kBit when the neighbour value u precedes the centre value c (kLe:
-// the neighbour comes earlier in linear order, so it also precedes on a tie;
-// NaN, the out-of-image fill, never precedes): a compare into a predicate and
-// a predicated OR, two instructions per bit
-template <uint32_t kBit, bool kLe>
-__device__ __forceinline__ void or_if_precedes(uint32_t& raw, float u, float c) {
-    if constexpr (kLe)
-        asm("{\n\t.reg .pred p;\n\tsetp.le.f32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
-            : "+r"(raw) : "f"(u), "f"(c), "n"(kBit));
-    else
-        asm("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
-            : "+r"(raw) : "f"(u), "f"(c), "n"(kBit));
-}
-
-struct Nbr {
-    float v[3][3];  // [row y-1, y, y+1][col x-1, x, x+1] of one plane
-};
-
-template <int n>
-__device__ __forceinline__ void mask_bit(uint32_t& raw, const Nbr& A, const Nbr& B, const Nbr& C, float cv) {
-    constexpr int a = n / 9, b = (n / 3) % 3, c = n % 3;
-    const Nbr& P = a == 0 ? A : (a == 1 ? B : C);
-    or_if_precedes<(1u << mask3_pos(n)), (n < 13)>(raw, P.v[b][c], cv);
-}
-
-// raw mask in the device layout (cp_mask3.cuh): the bit of canonical
-// neighbour n = 9a + 3b + c set when the neighbour at plane a, row b, column
-// c precedes the centre (ties: earlier linear index first)
-__device__ __forceinline__ uint32_t mask26(const Nbr& A, const Nbr& B, const Nbr& C) {
-    const float cv = B.v[1][1];
-    uint32_t raw = 0;
-    mask_bit<0>(raw, A, B, C, cv);
-    mask_bit<1>(raw, A, B, C, cv);
-    mask_bit<2>(raw, A, B, C, cv);
-    mask_bit<3>(raw, A, B, C, cv);
-    mask_bit<4>(raw, A, B, C, cv);
-    mask_bit<5>(raw, A, B, C, cv);
-    mask_bit<6>(raw, A, B, C, cv);
-    mask_bit<7>(raw, A, B, C, cv);
-    mask_bit<8>(raw, A, B, C, cv);
-    mask_bit<9>(raw, A, B, C, cv);
-    mask_bit<10>(raw, A, B, C, cv);
-    mask_bit<11>(raw, A, B, C, cv);
-    mask_bit<12>(raw, A, B, C, cv);
-    mask_bit<14>(raw, A, B, C, cv);
-    mask_bit<15>(raw, A, B, C, cv);
-    mask_bit<16>(raw, A, B, C, cv);
-    mask_bit<17>(raw, A, B, C, cv);
-    mask_bit<18>(raw, A, B, C, cv);
-    mask_bit<19>(raw, A, B, C, cv);
-    mask_bit<20>(raw, A, B, C, cv);
-    mask_bit<21>(raw, A, B, C, cv);
-    mask_bit<22>(raw, A, B, C, cv);
-    mask_bit<23>(raw, A, B, C, cv);
-    mask_bit<24>(raw, A, B, C, cv);
-    mask_bit<25>(raw, A, B, C, cv);
-    mask_bit<26>(raw, A, B, C, cv);
-    return raw;
-}
+static_assert(sizeof(Queue3) * kW3 >= sizeof(float) * kRS, "room for a row before the first slot");
 
 // ---- asynchronous copies into shared memory
 __device__ __forceinline__ void cp_async4(float* dst, const float* src) {
@@ -302,135 +250,96 @@ __device__ __forceinline__ void tma_load_plane(float* dst, const CUtensorMap* ma
         : "memory");
 }
 
-// Named barriers between the compare warps and the logic warp, two of each
-// kind (even and odd planes), so that either side can be a plane ahead.
-constexpr int kBarWords = 1;  // + plane parity: the compare words of a plane are complete
-constexpr int kBarCodes = 3;  // + plane parity: the codes of a plane are, and plane + 3 is in the ring
-constexpr int kBarRows = 5;   // among the compare warps (cp.async planes)
-constexpr int kBarLogic = 6;  // between the logic warps
-__device__ __forceinline__ void bar_arrive(int id) {
-    asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(kT3 + 64) : "memory");
-}
-__device__ __forceinline__ void bar_sync(int id) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kT3 + 64) : "memory");
-}
-
-// max(m, |v|), NaN if either is
-__device__ __forceinline__ float max_nan(float m, float v) {
-    float r;
-    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(m), "f"(fabsf(v)));
-    return r;
-}
-
 // Plane z of the tile.  TMA: one thread's tensor copy, completing on the
-// slot's mbarrier; positions outside the image read NaN (which precedes
-// nothing), and those next to an image vertex are set to +inf once the plane
-// has landed.  cp.async: a warp per row; +inf at positions outside the image,
-// set once per task.
-__device__ __forceinline__ void issue_tma(Smem3& sm, const Task3& t, int z) {  // one thread
-    if (z > t.zlast + 1 || unsigned(z) >= unsigned(t.D)) return;
-    uint64_t* bar = &sm.bar[ring_slot(z)];
-    // earlier generic-proxy accesses of the slot come before the copy
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_expect_tx(bar, uint32_t(kRH * kRS * sizeof(float)));
-    tma_load_plane(sm.ring[ring_slot(z)], t.map, bar, t.x0 - 2 - kRX, t.y0 - 2, z);
-}
-__device__ __forceinline__ void issue_rows(Smem3& sm, const Task3& t, int z) {  // the compare warps
-    if (z > t.zlast + 1 || unsigned(z) >= unsigned(t.D)) return;
+// slot's mbarrier; cp.async: a warp per row (positions outside the image hold
+// NaN for the whole task).
+__device__ __forceinline__ bool plane_read(const Task3& t, int z) { return z <= t.zlast + 1 && z < t.D; }
+__device__ __forceinline__ void issue_plane(Smem3& sm, const Task3& t, int z) {
+    if (!plane_read(t, z)) return;
     float* plane = sm.ring[ring_slot(z)];
+    if (t.map) {
+        if (threadIdx.x != 0) return;
+        uint64_t* bar = &sm.bar[ring_slot(z)];
+        // earlier generic-proxy accesses of the slot come before the copy
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_expect_tx(bar, uint32_t(kRH * kRS * sizeof(float)));
+        tma_load_plane(plane, t.map, bar, t.x0 - 1 - kRX, t.y0 - 1, z);
+        return;
+    }
     const int lane = int(lane_id());
     const float* src = t.img + uint32_t(z) * t.HW;
     for (int r = threadIdx.x >> 5; r < kRH; r += kW3) {
-        const int gy = t.y0 - 2 + r;
+        const int gy = t.y0 - 1 + r;
         if (unsigned(gy) >= unsigned(t.H)) continue;
         const float* row = src + uint32_t(gy) * uint32_t(t.W);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const int c = lane + 32 * k, gx = t.x0 - 2 + c;
+        for (int k = 0; k < 2; ++k) {
+            const int c = lane + 32 * k, gx = t.x0 - 1 + c;
             if (c < kRW && unsigned(gx) < unsigned(t.W)) cp_async4(plane + r * kRS + kRX + c, row + gx);
         }
     }
+    cp_async_commit();
 }
-// A plane outside the volume (z = D): every position +inf (the compare warps).
-__device__ __forceinline__ void fill_plane(Smem3& sm, int z) {
-    float* plane = sm.ring[ring_slot(z)];
-    for (int i = threadIdx.x; i < kRH * kRS; i += kT3) plane[i] = __int_as_float(0x7F800000);
-}
-
-// Four code bytes.
-__device__ __forceinline__ void put_code(const Outs& o, uint8_t* dst, uint32_t v) {
-    if (CP_IN(dst + 3 - o.code, o.n_code, o.ctr)) *reinterpret_cast<uint32_t*>(dst) = v;
-}
-
-// Before reading plane z: wait for its TMA copy (cp.async planes are covered
-// by the wait_group and the barrier of the step before).
+// Before reading plane z (every thread).
 __device__ __forceinline__ void wait_plane(Smem3& sm, const Task3& t, int z, uint32_t& par, Counters* ctr) {
-    if (!t.map || unsigned(z) >= unsigned(t.D)) return;
+    if (!plane_read(t, z)) return;
+    if (!t.map) {
+        cp_async_wait<0>();
+        return;
+    }
     const int slot = ring_slot(z);
     mbar_wait(&sm.bar[slot], (par >> slot) & 1u, ctr);
     par ^= 1u << slot;
 }
 
-// Compare words of this warp's rows in one plane (pl; up: the plane after it).
-// A position outside the image next to an image vertex holds +inf: everything
-// precedes it, so its neighbours' reversed bits are zero.
-// top_a, top_b: the largest magnitude of the two columns' values in image rows.
-__device__ __forceinline__ void compare_rows(const float* pl, const float* up, uint32_t (*w)[kWR], int warp, int lane,
-                                             float& top_a, float& top_b, int y_first, int H) {
-    struct Row {
-        float v[4];  // columns 2 lane - 1 .. 2 lane + 2 (tile columns)
-    };
-    auto read = [&](const float* p, int r) {
-        Row q;
-        const float2 a = *reinterpret_cast<const float2*>(p + r * kRS + kRX + 2 * lane);
-        const float2 b = *reinterpret_cast<const float2*>(p + r * kRS + kRX + 2 * lane + 2);
-        q.v[0] = a.x;
-        q.v[1] = a.y;
-        q.v[2] = b.x;
-        q.v[3] = b.y;
-        return q;
-    };
-    const int r0 = warp * kRows;
-    Row cur = read(pl, r0 + 1), u0 = read(up, r0), u1 = read(up, r0 + 1);
-#pragma unroll kUnrollC
-    for (int i = 0; i < kRows; ++i) {
-        const int r = r0 + i;
-        const Row nx = read(pl, r + 2), u2 = read(up, r + 2);
-        const float a = cur.v[1], b = cur.v[2];
-        if (unsigned(y_first + i) < unsigned(H)) {
-            top_a = max_nan(top_a, a);
-            top_b = max_nan(top_b, b);
-        }
-        uint32_t m[26];
-        auto put = [&](int k, const Row& q) {
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                m[k + 2 * d] = __ballot_sync(0xFFFFFFFFu, q.v[d] < a);
-                m[k + 2 * d + 1] = __ballot_sync(0xFFFFFFFFu, q.v[d + 1] < b);
-            }
-        };
-        put(0, u0);
-        put(6, u1);
-        put(12, u2);
-        put(18, nx);
-        m[24] = __ballot_sync(0xFFFFFFFFu, cur.v[2] < a);
-        m[25] = __ballot_sync(0xFFFFFFFFu, cur.v[3] < b);
-        if (lane == 0) {
-#pragma unroll
-            for (int k = 0; k < 24; k += 4)
-                *reinterpret_cast<uint4*>(&w[r][k]) = make_uint4(m[k], m[k + 1], m[k + 2], m[k + 3]);
-            *reinterpret_cast<uint2*>(&w[r][24]) = make_uint2(m[24], m[25]);
-        }
-        cur = nx;
-        u0 = u1;
-        u1 = u2;
-    }
-}
+// Compare words of a warp's rows in one plane: bit = row, set when the
+// neighbour precedes.
+struct Words3 {
+    uint32_t r, d, dr, a;      // in the plane: right < v, below < v, lower right < v, below < right
+    uint32_t c[3], p[3], m[3]; // the plane after, rows -1, 0, +1: same column < v, right < v, same column < right
+};
 
-// Bits of the columns lo .. hi (tile columns) in the even (par 0) or odd word.
-__device__ __forceinline__ uint32_t col_mask(int lo, int hi, int par) {
-    const int l0 = max(0, (lo - par + 1) >> 1), l1 = min(31, (hi - par) >> 1);
-    return l1 < l0 ? 0u : (0xFFFFFFFFu >> (31 - (l1 - l0))) << l0;
+// pl: this lane's column in the warp's first row; up: the same in the plane
+// after.  Rows from the last to the first, so that a row's bit is its number.
+__device__ __forceinline__ Words3 compare_rows(const float* pl, const float* up, int y_first, int H, float& bad) {
+    Words3 w = {};
+    // of row i + 1: v and right, up and right; of row i: up and right
+    float vna = 0.0f, vnb = 0.0f, una = 0.0f, unb = 0.0f;
+    float u0a = __fadd_rn(up[31 * kRS], 0.0f), u0b = __fadd_rn(up[31 * kRS + 1], 0.0f);  // -0 and +0 are equal
+#pragma unroll 1
+    for (int i0 = 24; i0 >= 0; i0 -= 8) {
+#pragma unroll
+        for (int k = 7; k >= 0; --k) {
+            const int i = i0 + k;
+            const float v = pl[i * kRS];
+            if (unsigned(y_first + i) < unsigned(H)) bad = fmaf(v, 0.0f, bad);  // NaN from the first NaN or infinity on
+            const float va = __fadd_rn(v, 0.0f), vb = __fadd_rn(pl[i * kRS + 1], 0.0f);
+            const float ua = __fadd_rn(up[(i - 1) * kRS], 0.0f), ub = __fadd_rn(up[(i - 1) * kRS + 1], 0.0f);
+            auto put = [](uint32_t& acc, float q, float c) {
+                acc = __funnelshift_l(__float_as_uint(__fsub_rn(q, c)), acc, 1);
+            };
+            put(w.r, vb, va);
+            put(w.d, vna, va);
+            put(w.dr, vnb, va);
+            put(w.a, vna, vb);
+            put(w.c[0], ua, va);
+            put(w.c[1], u0a, va);
+            put(w.c[2], una, va);
+            put(w.p[0], ub, va);
+            put(w.p[1], u0b, va);
+            put(w.p[2], unb, va);
+            put(w.m[0], ua, vb);
+            put(w.m[1], u0a, vb);
+            put(w.m[2], una, vb);
+            vna = va;
+            vnb = vb;
+            una = u0a;
+            unb = u0b;
+            u0a = ua;
+            u0b = ub;
+        }
+    }
+    return w;
 }
 
 // Eight words of 4 code bytes each |= plane b's bits of the word w.
@@ -444,163 +353,37 @@ __device__ __forceinline__ void spread(uint32_t (&acc)[8], uint32_t w) {
     }
 }
 
-// The logic of plane p for the even (par = 0) or odd columns; one warp, lane =
-// tile row.  wp, wl: the compare words of planes p and p - 1.  Returns the
-// event queue's new end (the even columns' events come first).
-template <int par>
-__device__ __forceinline__ uint32_t logic_plane(Smem3& sm, int p, const uint32_t (*wp)[kWR], const uint32_t (*wl)[kWR],
-                                                uint32_t tail) {
-    const Task3& t = sm.t;
-    const int r = int(lane_id()), rm = max(r - 1, 0), rp = min(r + 1, kTY - 1);
-    const int y = t.y0 - 1 + r;
-    const bool own_row = r >= 1 && r <= kOY && y < t.H, cube_row = own_row && y < t.H - 1;
-    const bool last_y = y == t.H - 2, first_y = y == 0;
-    Star3 st;
-    {
-        uint32_t n[27];
-        n[13] = 0;
-        // a row's word of one group for the column one to the left (dx = 1),
-        // the same (0) or one to the right (-1) of this parity's columns
-        auto at_col = [&](const uint32_t* g, int dx) -> uint32_t {
-            const uint32_t* q = g + 2 * (dx + 1);
-            if (dx == 0) return q[par];
-            if (par == 0) return dx > 0 ? q[1] << 1 : q[1];
-            return dx > 0 ? q[0] : q[0] >> 1;
-        };
-#pragma unroll
-        for (int dx = -1; dx <= 1; ++dx) {
-#pragma unroll
-            for (int dy = -1; dy <= 1; ++dy) {
-                n[13 + 9 + 3 * dy + dx] = wp[r][6 * (dy + 1) + 2 * (dx + 1) + par];
-                n[13 - 9 - 3 * dy - dx] = ~at_col(&wl[dy < 0 ? rp : (dy > 0 ? rm : r)][6 * (dy + 1)], dx);
-            }
-            n[13 + 3 + dx] = wp[r][18 + 2 * (dx + 1) + par];
-            n[13 - 3 - dx] = ~at_col(&wp[rm][18], dx);
-        }
-        n[14] = wp[r][24 + par];
-        n[12] = ~(par == 0 ? wp[r][25] << 1 : wp[r][24]);
-        star_words3(n, st);
-    }
-    const uint32_t own = own_row && p >= t.z0 ? t.own[par] : 0u;
-    const uint32_t cube = cube_row && p > 0 ? t.cube[par] : 0u;
-    uint32_t ev = st.event & own;
-    const uint32_t nev = __popc(ev);
-    uint32_t incl = nev;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (r >= o) incl += u;
-    }
-    // what the other parity's warp needs: its column one to the right is one of these
-#pragma unroll
-    for (int k = 0; k < 4; ++k) sm.xco[par][k][r] = st.co[2 * k];
-    if (r == 31) sm.xev[par] = incl;
-    asm volatile("bar.sync %0, 64;" ::"n"(kBarLogic) : "memory");
-    uint32_t xo[4];  // slots 0, 2, 4, 6 of the column one to the right
-#pragma unroll
-    for (int k = 0; k < 4; ++k) xo[k] = par == 0 ? sm.xco[1][k][r] : sm.xco[0][k][r] >> 1;
-    // ---- events, to the queue
-    {
-        uint32_t at = tail + (par == 0 ? 0u : sm.xev[0]) + incl - nev;
-        while (ev) {
-            const int l = __ffs(ev) - 1;
-            ev &= ev - 1;
-            sm.queue[at++ & (kQ - 1)] = uint16_t((p & 31) << 11 | r << 6 | (2 * l + par));
-        }
-        tail += sm.xev[0] + sm.xev[1];
-    }
-    // ---- the top cells between planes p - 1 and p: the slot that its largest
-    // corner sees it in.  Upper corners (slots 0..3 of plane p's vertices) send
-    // it to +z; plane p - 1's part comes from its own logic (sm.low).
-    const bool last_z = p == t.D - 1;  // the top cells across +z lie outside
-    const uint32_t up = st.co[3] | xo[1] | __shfl_down_sync(0xFFFFFFFFu, st.co[1] | xo[0], 1);
-    const uint32_t py_new = __shfl_down_sync(0xFFFFFFFFu, st.co[5] | xo[2], 1);
-    uint32_t* low = &sm.low[par][0][r];  // stride kTY
-    const uint32_t py = low[0], px = low[kTY], s0 = low[2 * kTY], s1 = low[3 * kTY], s2 = low[4 * kTY],
-                   s3 = low[5 * kTY];
-    const uint32_t upi = last_z ? 0u : up, pyi = last_y ? 0u : py, pxi = px & ~t.last_x[par];
-    uint32_t acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    // (the even columns' codes start at column 2, so that columns 1 + 8 k ..
-    // 8 + 8 k are one aligned word of each parity)
-    constexpr int sh = par == 0 ? 1 : 0;
-    spread<0>(acc, st.h[0] >> sh);
-    spread<1>(acc, st.h[1] >> sh);
-    spread<2>(acc, st.h[2] >> sh);
-    spread<3>(acc, (upi | pxi | s0 | ~cube) >> sh);
-    spread<4>(acc, (pyi | pxi | s1 | ~cube) >> sh);
-    spread<5>(acc, (s2 | ~cube) >> sh);
-    spread<6>(acc, (up | py | px | s3 | ~cube) >> sh);
-    uint4* dst = reinterpret_cast<uint4*>(&sm.code[p & 1][r][32 * par]);
-    dst[0] = make_uint4(acc[0], acc[1], acc[2], acc[3]);
-    dst[1] = make_uint4(acc[4], acc[5], acc[6], acc[7]);
-    // plane p's part for the top cells above it
-    uint32_t b0, b1, b2;
-    slot7_target(st.co, b0, b1, b2);
-    const uint32_t out = (~b0 & t.first_x[par]) | (first_y ? ~b1 : 0u) | (p == 0 ? ~b2 : 0u);
-    const uint32_t self = st.co[7] & ~out;
-    low[0] = py_new;
-    low[kTY] = xo[3];
-    low[2 * kTY] = self & b0;
-    low[3 * kTY] = self & b1;
-    low[4 * kTY] = self & b2;
-    low[5 * kTY] = st.co[7] & out;
-    return tail;
-}
+// What a warp keeps from one plane for the next.
+struct Carry3 {
+    uint32_t c[3], p[3], m[3];         // the compare words towards this plane (p: of the column to the left)
+    uint32_t py, px, s0, s1, s2, s3;   // the plane's part for the top cells above it
+};
 
-// 32 queued events (n: how many of them there are) from queue position `at`;
-// k: a plane within 31 planes after theirs.  Keys, roots and ages go straight
-// to the global arrays, with one atomic per array.
-__device__ __noinline__ unsigned long long event_batch(Smem3& sm, const Outs& o, int k, uint32_t at, uint32_t n) {
+// 32 queued events (n: how many of them there are) from queue position
+// `first` of the warp tile at (yw, xw).  Keys, roots and ages go straight to
+// the global arrays, with one atomic per array.
+__device__ __noinline__ unsigned long long event_batch(Smem3& sm, const Outs& o, const Queue3& queue, uint32_t first, uint32_t n) {
     const Task3& t = sm.t;
     const unsigned lane = lane_id(), lt = (1u << lane) - 1u;
+    const int warp = threadIdx.x >> 5;
     const bool live = lane < n;
-    const uint32_t e = live ? sm.queue[(at + lane) & (kQ - 1)] : 0u;
-    const int x = t.x0 - 1 + int(e & 63u), y = t.y0 - 1 + int((e >> 6) & 31u), z = k - ((k - int(e >> 11)) & 31);
-    bool root0 = false, rootT = false;
-    uint32_t sv = 0, ord = 0, vl = 0;
-    if (live) {
-        vl = uint32_t(z) * t.HW + uint32_t(y) * uint32_t(t.W) + uint32_t(x);
-        const float* c = t.img + vl;
-        // neighbours outside the image: read the nearest inside, drop the bit
-        const int dx[3] = {x > 0 ? -1 : 0, 0, x < t.W - 1 ? 1 : 0};
-        const int64_t dy[3] = {y > 0 ? -int64_t(t.W) : 0, 0, y < t.H - 1 ? int64_t(t.W) : 0};
-        const int64_t dz[3] = {z > 0 ? -int64_t(t.HW) : 0, 0, z < t.D - 1 ? int64_t(t.HW) : 0};
-        Nbr P[3];
-#pragma unroll
-        for (int k = 0; k < 27; ++k) P[k / 9].v[(k / 3) % 3][k % 3] = __ldg(c + dz[k / 9] + dy[(k / 3) % 3] + dx[k % 3]);
-        uint32_t raw = mask26(P[0], P[1], P[2]);
-        if (z == 0) raw &= ~mask3_side(0, -1);
-        if (z == t.D - 1) raw &= ~mask3_side(0, 1);
-        if (y == 0) raw &= ~mask3_side(1, -1);
-        if (y == t.H - 1) raw &= ~mask3_side(1, 1);
-        if (x == 0) raw &= ~mask3_side(2, -1);
-        if (x == t.W - 1) raw &= ~mask3_side(2, 1);
-        const uint32_t rel = collapse3_lattice(raw);
-        sv = __ldg(g_surv3d + hash_slot3(rel, g_disp3d));
-        root0 = (rel & kM3Faces) == 0u;
-        rootT = rel == kM3All;
-        ord = ord_bits(P[1].v[1][1]);
-    }
+    const uint32_t qi = (first + lane) & (kQ - 1), e = live ? queue.at[qi] : 0u, rel = live ? queue.rel[qi] : 0u;
+    const int x = t.x0 - 1 + (warp % kWX3) * kOWX + int(e & 31u), y = t.y0 - 1 + (warp / kWX3) * kBand3 + int((e >> 5) & 31u),
+              z = t.z0 + int(e >> 10);
+    const uint32_t sv = live ? __ldg(g_surv3d + hash_slot3(rel, g_disp3d)) : 0u;
+    const uint32_t ord = live ? ord_bits(queue.val[qi]) : 0u;
+    const uint32_t vl = uint32_t(z) * t.HW + uint32_t(y) * uint32_t(t.W) + uint32_t(x);
+    const bool root0 = live && (rel & kM3Faces) == 0u, rootT = rel == kM3All;
     const uint32_t vg = t.voff + vl;
     const uint32_t h0s = sv & 0x3Fu, ds = sv >> 6;
     const unsigned m_r0 = __ballot_sync(0xFFFFFFFFu, root0);
     const unsigned m_rt = __ballot_sync(0xFFFFFFFFu, rootT);
     const uint32_t n0 = __reduce_add_sync(0xFFFFFFFFu, uint32_t(__popc(h0s)));
     const uint32_t nt = __reduce_add_sync(0xFFFFFFFFu, uint32_t(__popc(ds)));
-    // lanes 0 .. 3 take room in the four arrays
-    uint32_t base = 0;
-    {
-        const uint32_t want = lane == 0 ? n0 : (lane == 1 ? nt : (lane == 2 ? __popc(m_r0) : __popc(m_rt)));
-        uint32_t* c = lane == 0 ? &o.ctr->n_s0 : (lane == 1 ? &o.ctr->n_st : (lane == 2 ? &o.ctr->n_r0 : &o.ctr->n_rt));
-        const uint32_t cap = lane < 2 ? o.cap_s : (lane == 2 ? o.cap_r0 : o.cap_rt);
-        if (lane < 4 && want) {
-            base = atomicAdd(c, want);
-            if (base + want > cap) set_status(o.ctr, kStCapacity);
-        }
-    }
-    uint32_t b0 = __shfl_sync(0xFFFFFFFFu, base, 0), bt = __shfl_sync(0xFFFFFFFFu, base, 1);
-    const uint32_t g0 = __shfl_sync(0xFFFFFFFFu, base, 2) + __popc(m_r0 & lt);
-    const uint32_t gt = __shfl_sync(0xFFFFFFFFu, base, 3) + __popc(m_rt & lt);
+    uint32_t b0, bt, g0, gt;
+    reserve(o, n0, nt, __popc(m_r0), __popc(m_rt), b0, bt, g0, gt);
+    g0 += __popc(m_r0 & lt);
+    gt += __popc(m_rt & lt);
     unsigned long long gmin = ~0ull;
     if (root0 && CP_IN(vg, o.n_uf0, o.ctr)) {
         gmin = (unsigned long long)(uint64_t(ord) << 32 | vl);
@@ -639,6 +422,7 @@ __device__ __noinline__ unsigned long long event_batch(Smem3& sm, const Outs& o,
 
 __device__ __forceinline__ void prune_task3d(Smem3& sm, const ItemTable& tab, const Outs& o, int ii, int ltask,
                                              const CUtensorMap* map, uint32_t& par) {
+    constexpr unsigned kAll = 0xFFFFFFFFu;
     const int warp = threadIdx.x >> 5, lane = int(lane_id());
     const Item& it = tab.it[ii];
     // task order: x segment fastest, then y segment, then z chunk
@@ -658,29 +442,15 @@ __device__ __forceinline__ void prune_task3d(Smem3& sm, const ItemTable& tab, co
     t.HW1 = (uint32_t(it.H) - 1u) * t.W1;
     t.voff = uint32_t(it.voff);
     t.toff = uint32_t(it.toff);
-    t.pitch = uint32_t(it.pitch);
     t.item = ii;
-    t.code = o.code + it.coff;
     t.map = map;
     __syncthreads();  // everything in shared memory may still be read by the previous task
-    if (threadIdx.x == 0) {
-        Task3 u = t;
-        const int xm = u.W - u.x0;  // tile column of the last image column
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            u.own[k] = col_mask(1, min(kOX, xm), k);
-            u.cube[k] = col_mask(1, min(kOX, xm - 1), k);
-            u.first_x[k] = col_mask(1 - u.x0, 1 - u.x0, k);
-            u.last_x[k] = col_mask(xm - 1, xm - 1, k);
-        }
-        sm.t = u;
-        sm.tail[0] = sm.tail[1] = 0;
-    }
-    if (!map) {  // positions outside the image stay +inf for the whole task
-        for (int i = threadIdx.x; i < kRH * kRW; i += kT3 + 64) {
+    if (threadIdx.x == 0) sm.t = t;
+    if (!map) {  // positions outside the image stay NaN for the whole task
+        for (int i = threadIdx.x; i < kRH * kRW; i += kT3) {
             const int ly = i / kRW, c = i - ly * kRW;
-            if (unsigned(t.y0 - 2 + ly) >= unsigned(it.H) || unsigned(t.x0 - 2 + c) >= unsigned(it.W))
-                for (int s = 0; s < kRing; ++s) sm.ring[s][ly * kRS + kRX + c] = __int_as_float(0x7F800000);
+            if (unsigned(t.y0 - 1 + ly) >= unsigned(it.H) || unsigned(t.x0 - 1 + c) >= unsigned(it.W))
+                for (int s = 0; s < kRing; ++s) sm.ring[s][ly * kRS + kRX + c] = __int_as_float(0x7FFFFFFF);
         }
     } else if (threadIdx.x == 0) {
         // counted in blocks of 31 x 8 columns by the tuned number of planes, whatever the tile
@@ -688,138 +458,158 @@ __device__ __forceinline__ void prune_task3d(Smem3& sm, const ItemTable& tab, co
         atomicAdd(&o.ctr->tma_tasks, blocks(t.x0, min(t.x0 + kOX, it.W), 31) * blocks(t.y0, min(t.y0 + kOY, it.H), 8) *
                                          blocks(t.z0, t.z1, tab.zchunk3d));
     }
-    __syncthreads();
-    // The code of a vertex holds the dual link of the top cell below it, which
-    // needs the logic of the plane before: planes first .. zlast are compared
-    // and first + 1 .. zlast go through the logic, the first of them only for
-    // the top cells above it.  Planes first .. zlast + 1 are read.
-    const int first = max(t.z0 - 2, -1);
-    //   compare warps, step k: wait for the codes of plane k - 2 (which come
-    //     with plane k + 1 in the ring); output plane k - 2, events; compare
-    //     plane k
-    //   logic warps, step k: wait for the words of plane k (the compare of
-    //     plane k was the last to read it); request plane k + 3 into its slot;
-    //     logic of plane k; wait for plane k + 3 to land
-    if (warp >= kW3) {
-        const bool even = warp == kW3;  // this warp also brings the planes in
-        // positions outside the image, next to it, are set to +inf in every
-        // plane (TMA path): columns x = -1 and x = W, rows y = -1 and y = H
-        const bool edge = t.x0 == 0 || t.y0 == 0 || t.x0 - 1 + kTX > t.W || t.y0 - 1 + kTY > t.H;
-        auto request = [&](int z) {
-            if (z <= t.zlast + 1 && unsigned(z) < unsigned(t.D) && map && even && lane == 0) issue_tma(sm, t, z);
-        };
-        auto landed = [&](int z) {
-            if (z > t.zlast + 1) return;
-            float* plane = sm.ring[ring_slot(z)];
-            if (unsigned(z) >= unsigned(t.D)) {  // a plane outside the volume: every position +inf
-                if (even)
-                    for (int i = lane; i < kRH * kRS; i += 32) plane[i] = __int_as_float(0x7F800000);
-            } else if (map) {
-                wait_plane(sm, t, z, par, o.ctr);
-                if (edge && even) {
-#pragma unroll
-                    for (int n = 0; n < kFix; ++n) {
-                        const int i = lane + 32 * n, j = i - 2 * kRH;
-                        const int c = j < 0 ? (i < kRH ? 1 - t.x0 : t.W + 2 - t.x0) : (j < kRW ? j : j - kRW);
-                        const int r = j < 0 ? (i < kRH ? i : i - kRH) : (j < kRW ? 1 - t.y0 : t.H + 2 - t.y0);
-                        if (j < 2 * kRW && unsigned(c) < unsigned(kRW) && unsigned(r) < unsigned(kRH))
-                            plane[r * kRS + kRX + c] = __int_as_float(0x7F800000);
-                    }
-                }
-            }
-        };
-#pragma unroll 1
-        for (int z = first; z < first + 3; ++z) request(z);
-#pragma unroll 1
-        for (int z = first; z < first + 2; ++z) landed(z);
-        bar_arrive(kBarCodes + (first & 1));
-        landed(first + 2);
-        bar_arrive(kBarCodes + ((first + 1) & 1));
-        uint32_t tail = 0;
-        int sc = 0;  // word slot of plane k
-#pragma unroll 1
-        for (int k = first; k <= t.zlast; ++k) {
-            bar_sync(kBarWords + (k & 1));
-            request(k + 3);
-            if (k > first) {
-                const uint32_t(*wl)[kWR] = sm.w[sc == 0 ? 2 : sc - 1];
-                tail = even ? logic_plane<0>(sm, k, sm.w[sc], wl, tail) : logic_plane<1>(sm, k, sm.w[sc], wl, tail);
-            }
-            if (even && lane == 0) sm.tail[k & 1] = tail;
-            landed(k + 3);
-            bar_arrive(kBarCodes + (k & 1));
-            sc = sc == 2 ? 0 : sc + 1;
-        }
-        return;
-    }
-    float top_a = 0.0f, top_b = 0.0f;  // largest magnitude of this lane's columns (NaN if one is)
+    // the warp's tile: columns xw .. xw + 31, rows yw .. yw + 31, the inner 30 x 29 owned
+    const int wx = warp % kWX3, wy = warp / kWX3;
+    const int x = t.x0 - 1 + wx * kOWX + lane, yw = t.y0 - 1 + wy * kBand3;
+    const int band = (yw + 1) / kBand3;
+    const bool idle = yw + 1 >= t.H || t.x0 + wx * kOWX >= t.W;  // owns nothing
+    const bool own_x = lane >= 1 && lane <= kOWX && x < t.W;
+    const int rows = t.H - (yw + 1);  // owned, if fewer than kBand3
+    const uint32_t own = own_x ? (rows >= kBand3 ? (2u << kBand3) - 2u : (2u << max(rows, 0)) - 2u) : 0u;
+    const uint32_t last_row = unsigned(rows) < 32u ? 1u << rows : 0u;  // the bit of row H - 1
+    const uint32_t cube_xy = x < t.W - 1 ? own & ~last_row : 0u;
+    const uint32_t mxm = x > 0 ? kAll : 0u, mxp = x < t.W - 1 ? kAll : 0u;  // columns with a neighbour on that side
+    const uint32_t mym = yw < 0 ? ~2u : kAll, myp = ~last_row;              // rows likewise
+    const uint32_t first_x = ~mxm, last_x = x == t.W - 2 ? kAll : 0u;
+    const uint32_t last_y = last_row >> 1;  // the bit of row H - 2
+    const int col = wy * kBand3 * kRS + kRX + wx * kOWX + lane;
+    Carry3 cr = {};
+    float bad = 0.0f;
     unsigned long long gmin = ~0ull;
-    uint32_t head = 0;  // events taken from the queue
-    int oldest = t.z0;  // no queued event lies before this plane
-    int sc = 0;         // word slot of plane k
-    if (!map) {
-        for (int z = first; z < first + 2; ++z) issue_rows(sm, t, z);
-        cp_async_commit();
-    }
+    Queue3& queue = sm.queue[warp];
+    uint32_t head = 0, tail = 0;  // events taken from the queue, put into it
+    const unsigned lt = (1u << lane) - 1u;
+    auto take = [&](uint32_t n) {
+        __syncwarp();
+        const unsigned long long g = event_batch(sm, o, queue, head, n);
+        gmin = g < gmin ? g : gmin;
+        head += n;
+        __syncwarp();
+    };
+    // The code of a vertex holds the dual link of the top cell below it, which
+    // needs the logic of the plane before, which needs the words of the plane
+    // before that: planes first .. zlast + 1 are read.
+    const int first = max(t.z0 - 2, 0);
+    __syncthreads();
+    issue_plane(sm, t, first);
+    issue_plane(sm, t, first + 1);
+    wait_plane(sm, t, first, par, o.ctr);
 #pragma unroll 1
-    for (int k = first; k <= t.zlast + 2; ++k) {
-        const int p = k - 2;
-        bar_sync(kBarCodes + (p & 1));
-        if (!map) {
-            asm volatile("bar.sync %0, %1;" ::"n"(kBarRows), "n"(kT3) : "memory");  // plane k - 1 has been compared
-            issue_rows(sm, t, k + 2);                                               // into its slot
-            cp_async_commit();
-            cp_async_wait<1>();
-            asm volatile("bar.sync %0, %1;" ::"n"(kBarRows), "n"(kT3) : "memory");  // plane k + 1 is there
+    for (int k = first; k <= t.zlast; ++k) {
+        wait_plane(sm, t, k + 1, par, o.ctr);
+        __syncthreads();  // plane k + 1 is there, plane k - 1 has been compared
+        issue_plane(sm, t, k + 2);
+        if (idle) continue;
+        Words3 w = compare_rows(sm.ring[ring_slot(k)] + col, sm.ring[ring_slot(k + 1)] + col, yw, t.H, bad);
+        if (k == t.D - 1) {  // no plane after
+#pragma unroll
+            for (int j = 0; j < 3; ++j) w.c[j] = w.p[j] = w.m[j] = 0u;
         }
-        const uint32_t tail = p >= t.z0 ? sm.tail[p & 1] : 0u;
-        if (p >= t.z0) {
-            // the codes of plane p: 8 columns (two words) of an owned row per thread and turn
-            uint8_t* plane = t.code + uint64_t(uint32_t(p) * uint32_t(t.H)) * t.pitch + uint32_t(t.x0);
-#pragma unroll 1
-                for (int i = threadIdx.x; i < 8 * kOY; i += kT3) {
-                    const int r = 1 + (i >> 3), c = i & 7, y = t.y0 - 1 + r;
-                    const uint32_t ev = *reinterpret_cast<const uint32_t*>(&sm.code[p & 1][r][4 * c]);
-                    const uint32_t od = *reinterpret_cast<const uint32_t*>(&sm.code[p & 1][r][32 + 4 * c]);
-                    const uint32_t x = 8u * c;
-                    uint8_t* dst = plane + uint64_t(uint32_t(y)) * t.pitch + x;
-                    if (y < t.H && uint32_t(t.x0) + x < t.pitch) {
-                        put_code(o, dst, __byte_perm(od, ev, 0x5140));
-                        if (c < 7 && uint32_t(t.x0) + x + 4 < t.pitch) put_code(o, dst + 4, __byte_perm(od, ev, 0x7362));
-                    }
+        if (k >= t.z0 - 1) {
+            Star3 st;
+            {
+                uint32_t n[27];
+                n[13] = 0;
+                const uint32_t mz = k > 0 ? kAll : 0u;
+                const uint32_t yz[3] = {mym & mz, mz, myp & mz};
+                n[14] = w.r;
+                n[12] = ~__shfl_up_sync(kAll, w.r, 1) & mxm;
+                n[16] = w.d;
+                n[10] = ~(w.d << 1) & mym;
+                n[17] = w.dr;
+                n[9] = ~(__shfl_up_sync(kAll, w.dr, 1) << 1) & mxm & mym;
+                n[15] = __shfl_up_sync(kAll, w.a, 1);
+                n[11] = ~(w.a << 1) & mxp & mym;
+#pragma unroll
+                for (int dy = -1; dy <= 1; ++dy) {
+                    n[22 + 3 * dy] = w.c[dy + 1];
+                    n[23 + 3 * dy] = w.p[dy + 1];
+                    n[21 + 3 * dy] = __shfl_up_sync(kAll, w.m[dy + 1], 1);
+                    // the words of the row one up or down, towards this row
+                    auto row = [&](uint32_t q) { return dy < 0 ? q << 1 : (dy > 0 ? q >> 1 : q); };
+                    n[4 + 3 * dy] = ~row(cr.c[1 - dy]) & yz[dy + 1];
+                    n[3 + 3 * dy] = ~row(cr.p[1 - dy]) & yz[dy + 1] & mxm;
+                    n[5 + 3 * dy] = ~row(cr.m[1 - dy]) & yz[dy + 1] & mxp;
                 }
-        }
-        if (tail - head >= uint32_t(kQMin) || (tail != head && (k - oldest >= kQAge || k == t.zlast + 2))) {
-            for (uint32_t at = head + 32u * warp; at < tail; at += kT3) {
-                const unsigned long long g = event_batch(sm, o, k, at, min(32u, tail - at));
-                gmin = g < gmin ? g : gmin;
+                star_words3(n, st);
             }
-            head = tail;
-        }
-        if (tail == head) oldest = p + 1;
-        if (k <= t.zlast) {
-            if (k < 0) {  // a plane outside the volume: all ones
-                wait_plane(sm, t, k + 1, par, o.ctr);
-                for (int i = threadIdx.x; i < kTY * kWR; i += kT3) (&sm.w[sc][0][0])[i] = 0xFFFFFFFFu;
-            } else {
-                if (k == first) wait_plane(sm, t, k, par, o.ctr);
-                wait_plane(sm, t, k + 1, par, o.ctr);
-                compare_rows(sm.ring[ring_slot(k)], sm.ring[ring_slot(k + 1)], sm.w[sc], warp, lane, top_a, top_b,
-                             t.y0 - 1 + warp * kRows, t.H);
+            // the column to the right's slots 0, 2, 4, 6
+            uint32_t xo[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) xo[j] = __shfl_down_sync(kAll, st.co[2 * j], 1);
+            if (k >= t.z0) {
+                // the top cells between planes k - 1 and k: the slot that its
+                // largest corner sees it in.  Upper corners (slots 0..3 of plane
+                // k's vertices) send it to +z; plane k - 1's part comes from its
+                // own logic.
+                const uint32_t cube = k > 0 ? cube_xy : 0u;
+                const uint32_t up = st.co[3] | xo[1] | ((st.co[1] | xo[0]) >> 1);
+                const uint32_t upi = k == t.D - 1 ? 0u : up, pyi = cr.py & ~last_y, pxi = cr.px & ~last_x;
+                uint32_t acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+                spread<0>(acc, st.h[0] >> 1);
+                spread<1>(acc, st.h[1] >> 1);
+                spread<2>(acc, st.h[2] >> 1);
+                spread<3>(acc, (upi | pxi | cr.s0 | ~cube) >> 1);
+                spread<4>(acc, (pyi | pxi | cr.s1 | ~cube) >> 1);
+                spread<5>(acc, (cr.s2 | ~cube) >> 1);
+                spread<6>(acc, (up | cr.py | cr.px | cr.s3 | ~cube) >> 1);
+                const uint64_t at = uint64_t(it.coff) + ((uint64_t(k) * uint32_t(it.bands) + uint32_t(band)) * uint32_t(t.W) + uint32_t(x)) * 32u;
+                if (own_x && CP_IN(at + 31u, o.n_code, o.ctr)) {
+                    uint4* dst = reinterpret_cast<uint4*>(o.code + at);
+                    dst[0] = make_uint4(acc[0], acc[1], acc[2], acc[3]);
+                    dst[1] = make_uint4(acc[4], acc[5], acc[6], acc[7]);
+                }
+                // events: each lane's next one, to the queue
+                uint32_t ev = st.event & own;
+                for (;;) {
+                    const unsigned have = __ballot_sync(kAll, ev != 0u);
+                    if (!have) break;
+                    const int row = ev ? __ffs(ev) - 1 : 0;
+                    uint32_t rel = 0;
+#pragma unroll
+                    for (int n = 0; n < 27; ++n)
+                        if (n != 13) rel |= ((relevant_plane(st, n) >> row) & 1u) << mask3_pos(n);
+                    if (ev) {
+                        const uint32_t q = (tail + __popc(have & lt)) & (kQ - 1);
+                        queue.rel[q] = rel;
+                        queue.at[q] = uint32_t(k - t.z0) << 10 | uint32_t(row) << 5 | uint32_t(lane);
+                        queue.val[q] = sm.ring[ring_slot(k)][col + row * kRS];
+                        ev &= ev - 1u;
+                    }
+                    tail += __popc(have);
+                    if (tail - head >= 32u) take(32u);
+                }
             }
-            bar_arrive(kBarWords + (k & 1));
-            sc = sc == 2 ? 0 : sc + 1;
+            // plane k's part for the top cells above it
+            uint32_t b0, b1, b2;
+            slot7_target(st.co, b0, b1, b2);
+            const uint32_t out = (~b0 & first_x) | (~b1 & ~mym) | (k == 0 ? ~b2 : 0u);
+            const uint32_t self = st.co[7] & ~out;
+            cr.py = (st.co[5] | xo[2]) >> 1;
+            cr.px = xo[3];
+            cr.s0 = self & b0;
+            cr.s1 = self & b1;
+            cr.s2 = self & b2;
+            cr.s3 = st.co[7] & out;
+        }
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            cr.c[j] = w.c[j];
+            cr.p[j] = __shfl_up_sync(kAll, w.p[j], 1);
+            cr.m[j] = w.m[j];
         }
     }
+    if (tail != head) take(tail - head);
     if (!map) cp_async_wait<0>();
-    const bool in_a = unsigned(t.x0 - 1 + 2 * lane) < unsigned(t.W), in_b = unsigned(t.x0 + 2 * lane) < unsigned(t.W);
-    const bool bad = (in_a && !(top_a <= 3.40282347e38f)) || (in_b && !(top_b <= 3.40282347e38f));
-    if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) set_status(o.ctr, kStNonfinite);
-    gmin = warp_min_u64(gmin);
-    if (lane == 0 && gmin != ~0ull) atomicMin(&o.ctr->gmin[ii], gmin);
+    if (!idle) {
+        const bool in = unsigned(x) < unsigned(t.W);
+        if (__any_sync(kAll, in && bad != bad) && lane == 0) set_status(o.ctr, kStNonfinite);
+        gmin = warp_min_u64(gmin);
+        if (lane == 0 && gmin != ~0ull) atomicMin(&o.ctr->gmin[ii], gmin);
+    }
 }
 
-__global__ void __launch_bounds__(kT3 + 64, 3) k_prune3d(const __grid_constant__ ItemTable tab, const __grid_constant__ Outs o,
+__global__ void __launch_bounds__(kT3, 8) k_prune3d(const __grid_constant__ ItemTable tab, const __grid_constant__ Outs o,
                                                     const __grid_constant__ TmaMaps maps) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     Smem3& sm = *reinterpret_cast<Smem3*>(smem_raw);
@@ -863,7 +653,7 @@ __global__ void __launch_bounds__(256) k_expand(const __grid_constant__ ItemTabl
         const int64_t n = int64_t(it.D) * it.H * it.W;
         for (int64_t v = int64_t(blockIdx.x) * 256 + threadIdx.x; v < n; v += int64_t(gridDim.x) * 256) {
             const int x = int(v % it.W), y = int((v / it.W) % it.H), z = int(v / (int64_t(it.W) * it.H));
-            const uint32_t c = o.code[it.coff + (int64_t(z) * it.H + y) * it.pitch + x];
+            const uint32_t c = o.code[it.coff + code_at3(it, z, y, x)];
             const uint32_t h = c & 7u, d = c >> 3;
             if (h < 6u) o.uf0[it.voff + v] = uint32_t(it.voff + v + link_offset3(0, h, it.H * it.W, it.W));
             if (z == 0 || y >= it.H - 1 || x >= it.W - 1 || d == 7u) continue;
@@ -1058,19 +848,8 @@ __global__ void __launch_bounds__(kW2 * 32) k_prune2d(const __grid_constant__ It
         }
         c_s = __reduce_add_sync(kAll, c_s);
         c_r = __reduce_add_sync(kAll, c_r);
-        // lanes 0 .. 3 take room in the four arrays
-        uint32_t base = 0;
-        {
-            const uint32_t want = ((lane & 2) ? c_r : c_s) >> ((lane & 1) * 16) & 0xFFFFu;
-            uint32_t* c = lane == 0 ? &o.ctr->n_s0 : (lane == 1 ? &o.ctr->n_st : (lane == 2 ? &o.ctr->n_r0 : &o.ctr->n_rt));
-            const uint32_t cap = lane < 2 ? o.cap_s : (lane == 2 ? o.cap_r0 : o.cap_rt);
-            if (lane < 4 && want) {
-                base = atomicAdd(c, want);
-                if (base + want > cap) set_status(o.ctr, kStCapacity);
-            }
-        }
-        uint32_t b0 = __shfl_sync(kAll, base, 0), bt = __shfl_sync(kAll, base, 1), br0 = __shfl_sync(kAll, base, 2),
-                 brt = __shfl_sync(kAll, base, 3);
+        uint32_t b0, bt, br0, brt;
+        reserve(o, c_s & 0xFFFFu, c_s >> 16, c_r & 0xFFFFu, c_r >> 16, b0, bt, br0, brt);
         unsigned long long gmin = ~0ull;
         __syncwarp();
         // a batch's values are loaded during the one before
@@ -1261,7 +1040,7 @@ cudaError_t launch_prune(const ItemTable& tab, const PruneOuts& po, const TmaMap
     const int blocks3d = device_cached(kCachePrune3d, [] {
         cudaFuncSetAttribute(k_prune3d, cudaFuncAttributeMaxDynamicSharedMemorySize, int(prune_smem3d()));
         int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_prune3d, kT3 + 64, prune_smem3d());
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_prune3d, kT3, prune_smem3d());
         return device_sm_count() * (per_sm > 0 ? per_sm : 1);
     });
     const int blocks2d = device_cached(kCachePrune2d, [] {
@@ -1284,7 +1063,7 @@ cudaError_t launch_prune(const ItemTable& tab, const PruneOuts& po, const TmaMap
         int cap = blocks3d;
         if (g_ctas3d > 0) cap = device_sm_count() * g_ctas3d < blocks3d ? device_sm_count() * g_ctas3d : blocks3d;
         int grid = tab.tiles3d < cap ? tab.tiles3d : cap;
-        k_prune3d<<<grid, kT3 + 64, prune_smem3d(), s>>>(tab, o, maps);
+        k_prune3d<<<grid, kT3, prune_smem3d(), s>>>(tab, o, maps);
         note_launches(1);
     }
     return cudaGetLastError();

@@ -95,11 +95,14 @@ __global__ void __launch_bounds__(kTT) k_t_flatten(uint8_t* __restrict__ code, c
     const int item = blockIdx.y;
     const TDims& d = t.d[item];
     uint8_t* __restrict__ cd = code + t.coff[item];
-    const int64_t P = t.pitch[item];
     const int64_t Dj = d.ndim == 3 ? d.D + 2 : 1, Hj = d.H + 2, Wj = d.W + 2;
-    Item j2;  // the shape that code_at2 wants
-    j2.W = int32_t(Wj);
-    auto at2 = [&](int64_t y, int64_t x) { return code_at2(j2, int(y), int(x)); };
+    Item j;  // the shape that code_at2 and code_at3 want
+    j.W = int32_t(Wj);
+    j.bands = t.bands[item];
+    auto code_at = [&](int64_t z, int64_t y, int64_t x) {
+        return d.ndim == 3 ? code_at3(j, int(z), int(y), int(x)) : code_at2(j, int(y), int(x));
+    };
+    const uint8_t frame = d.ndim == 3 ? 7u : 15u;
     // whole frame rows, one block per row: both y faces of every plane, and
     // the two z faces (3D)
     const int64_t zf = d.ndim == 3 ? 2 * Hj : 0;  // rows of the two z faces
@@ -114,12 +117,8 @@ __global__ void __launch_bounds__(kTT) k_t_flatten(uint8_t* __restrict__ code, c
             z = d.ndim == 3 ? 1 + g / 2 : 0;
             y = (g & 1) ? Hj - 1 : 0;
         }
-        uint8_t* crow = cd + (z * Hj + y) * P;
         for (int64_t x = threadIdx.x; x < Wj; x += kTT)
-            if (z != 0 || y != 0 || x != 0) {
-                if (d.ndim == 3) crow[x] |= 7u;
-                else cd[at2(y, x)] |= 15u;
-            }
+            if (z != 0 || y != 0 || x != 0) cd[code_at(z, y, x)] |= frame;
     }
     // the two x faces of the other rows
     const int64_t zi = d.ndim == 3 ? Dj - 2 : 1, yi = Hj - 2;
@@ -128,8 +127,7 @@ __global__ void __launch_bounds__(kTT) k_t_flatten(uint8_t* __restrict__ code, c
         const int64_t q = k >> 1;
         const int64_t z = d.ndim == 3 ? 1 + q / yi : 0, y = 1 + q % yi;
         const int64_t x = (k & 1) ? Wj - 1 : 0;
-        if (d.ndim == 3) cd[(z * Hj + y) * P + x] |= 7u;
-        else cd[at2(y, x)] |= 15u;
+        cd[code_at(z, y, x)] |= frame;
     }
 }
 

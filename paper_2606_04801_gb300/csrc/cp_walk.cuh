@@ -4,8 +4,8 @@
 // Both are in a code byte per vertex; of the 32-bit arrays only a root's word
 // is written (its root id).
 //
-// 3D items: at (z H + y) pitch + x of the item's codes, bits 0-2 the vertex's
-// H0 link (face slot 0..5, 6: a root, 7: a frame vertex of a T-filtration
+// 3D items: 29 rows of a column of a plane at a time in one 32-byte sector
+// (code_at3: a column of a pruning tile), bits 0-2 the vertex's H0 link (face slot 0..5, 6: a root, 7: a frame vertex of a T-filtration
 // item, whose root is vertex 0), bits 3-6 the dual link of the top cell with
 // its smallest corner one plane below, at (z - 1, y, x) (0..6: towards that
 // slot as seen from that corner, 7: a root, 8: the outside, 9, 10, 11: +z, +y,
@@ -23,8 +23,8 @@
 
 namespace cp {
 
-// Offset of the 3D link with code field d (H0: 0..5; dual: 0..6, 9..11) in the
-// codes' index space.
+// Offset of the 3D link with code field d (H0: 0..5; dual: 0..6, 9..11) between
+// ids, with hp and p the plane's and the row's.
 __host__ __device__ __forceinline__ int32_t link_offset3(int dual, uint32_t d, int32_t hp, int32_t p) {
     if (!dual) {
         const int32_t m = (d == 0u || d == 5u) ? hp : ((d == 1u || d == 4u) ? p : 1);
@@ -35,12 +35,19 @@ __host__ __device__ __forceinline__ int32_t link_offset3(int dual, uint32_t d, i
 }
 
 constexpr int kTile2 = 30;  // rows (and columns) of a 2D pruning tile
+constexpr int kBand3 = 29;  // rows of a warp's part of a 3D pruning tile
 
 // Where vertex (y, x) of a 2D item has its code byte (its first byte is the
 // item's).
 __host__ __device__ __forceinline__ uint32_t code_at2(const Item& it, int y, int x) {
     const uint32_t t = uint32_t(y) / uint32_t(kTile2);
     return (t * uint32_t(it.W) + uint32_t(x)) * 32u + (uint32_t(y) - t * uint32_t(kTile2));
+}
+
+// The same for vertex (z, y, x) of a 3D item.
+__host__ __device__ __forceinline__ uint32_t code_at3(const Item& it, int z, int y, int x) {
+    const uint32_t b = uint32_t(y) / uint32_t(kBand3);
+    return ((uint32_t(z) * uint32_t(it.bands) + b) * uint32_t(it.W) + uint32_t(x)) * 32u + (uint32_t(y) - b * uint32_t(kBand3));
 }
 
 // Offset of the 2D link with code field d (H0: 0..7; dual: 0..8).
@@ -93,14 +100,17 @@ constexpr uint32_t kStepZ1 = step_field(kStay, 0u, 0u, 1u, 0u, 2u, 0u, 3u, 0u, 9
                    kStepY1 = step_field(kStay, 0u, 0u, 1u, 0u, 4u, 0u, 5u, 0u, 10u, 2u),
                    kStepX1 = step_field(kStay, 0u, 0u, 2u, 0u, 4u, 0u, 6u, 0u, 11u, 2u);
 struct Step3 {
-    uint32_t cz, cy, cx, shift, mask, hp, p;
-    __device__ __forceinline__ Step3(int dual, int32_t hp_, int32_t p_)
+    uint32_t cz, cy, cx, shift, mask, hp, band;
+    __device__ __forceinline__ Step3(int dual, const Item& it)
         : cz(dual ? kStepZ1 : kStepZ0), cy(dual ? kStepY1 : kStepY0), cx(dual ? kStepX1 : kStepX0), shift(dual ? 3u : 0u),
-          mask(dual ? 15u : 7u), hp(uint32_t(hp_)), p(uint32_t(p_)) {}
+          mask(dual ? 15u : 7u), hp(32u * uint32_t(it.W) * uint32_t(it.bands)), band(32u * uint32_t(it.W)) {}
     __device__ __forceinline__ uint32_t field(uint32_t c) const { return (c >> shift) & mask; }
     __device__ __forceinline__ uint32_t next(uint32_t at, uint32_t d) const {
         const uint32_t s = 2u * d;
-        return at + ((cz >> s) & 3u) * hp + ((cy >> s) & 3u) * p + ((cx >> s) & 3u) - (hp + p + 1u);
+        at += ((cz >> s) & 3u) * hp + ((cx >> s) & 3u) * 32u + ((cy >> s) & 3u) - (hp + 33u);
+        const uint32_t r = at & 31u;  // 29: one row below the band, 31: one above it (and a column to the left)
+        if (r >= uint32_t(kBand3)) at += r == 31u ? uint32_t(kBand3) - band : band - uint32_t(kBand3);
+        return at;
     }
     __device__ __forceinline__ bool ends(uint32_t d) const { return mask == 7u ? d >= 6u : (0xF180u >> d) & 1u; }
     __device__ __forceinline__ bool outside(uint32_t d) const { return mask == 15u && d == 8u; }
@@ -169,14 +179,10 @@ __device__ __forceinline__ uint32_t root_id2(const Forest& f, const Item& it, in
 
 __device__ __forceinline__ uint32_t root_id3(const Forest& f, const Item& it, int item, Counters* ctr, const Path& p) {
     if (p.out) return uint32_t(item);
-    const uint32_t row = p.at / uint32_t(it.pitch), x = p.at - row * uint32_t(it.pitch);
-    uint32_t node;
-    if (!f.dual) {
-        node = uint32_t(it.voff) + row * uint32_t(it.W) + x;
-    } else {
-        const uint32_t z = row / uint32_t(it.H), y = row - z * uint32_t(it.H);
-        node = uint32_t(it.toff) + ((z - 1u) * uint32_t(it.H - 1) + y) * uint32_t(it.W - 1) + x;
-    }
+    const uint32_t q = p.at >> 5, t = q / uint32_t(it.W), x = q - t * uint32_t(it.W);
+    const uint32_t z = t / uint32_t(it.bands), y = (t - z * uint32_t(it.bands)) * uint32_t(kBand3) + (p.at & 31u);
+    const uint32_t node = f.dual ? uint32_t(it.toff) + ((z - 1u) * uint32_t(it.H - 1) + y) * uint32_t(it.W - 1) + x
+                                 : uint32_t(it.voff) + (z * uint32_t(it.H) + y) * uint32_t(it.W) + x;
     (void)ctr;
     return CP_IN(node, f.n_nodes, ctr) ? __ldg(f.uf + node) & ~kTag : 0u;
 }
@@ -195,24 +201,24 @@ __device__ __forceinline__ bool walk_roots(const ItemTable& tab, const Forest& f
     const uint32_t row = local / W;
     const int x = int(local - row * W);
     if (it.ndim == 3) {
-        const int32_t p = it.pitch, hp = int32_t(H) * p;
-        Path a = {row * uint32_t(p) + uint32_t(x), false}, b = a;
+        const int y = int(row % H), z = int(row / H);
+        Path a = {0, false}, b = a;
         if (!f.dual) {
-            b.at += uint32_t(dz * hp + dy * p + dx);
+            a.at = code_at3(it, z, y, x);
+            b.at = code_at3(it, z + dz, y + dy, x + dx);
         } else {
             // the facet's zero coordinate picks the side: smallest corners of its two top cells
-            const int y = int(row % H), z = int(row / H);
             const int cz = z + (dz < 0 ? -1 : 0), cy = y + (dy < 0 ? -1 : 0), cx = x + (dx < 0 ? -1 : 0);
             auto corner = [&](int s) {  // s: the zero coordinate's side (-1, +1)
                 const int qz = dz == 0 && s < 0 ? z - 1 : cz, qy = dy == 0 && s < 0 ? y - 1 : cy,
                           qx = dx == 0 && s < 0 ? x - 1 : cx;
                 const bool out = qz < 0 || qz >= it.D - 1 || qy < 0 || qy >= it.H - 1 || qx < 0 || qx >= it.W - 1;
-                return Path{out ? 0u : uint32_t((qz + 1) * hp + qy * p + qx), out};
+                return Path{out ? 0u : code_at3(it, qz + 1, qy, qx), out};
             };
             a = corner(-1);
             b = corner(1);
         }
-        if (!follow(f, uint64_t(it.coff), Step3(f.dual, hp, p), ctr, a, b, hops)) {
+        if (!follow(f, uint64_t(it.coff), Step3(f.dual, it), ctr, a, b, hops)) {
             ra = rb = 0;
             return false;
         }

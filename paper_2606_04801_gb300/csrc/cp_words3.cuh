@@ -13,7 +13,21 @@ struct Star3 {
     uint32_t h[3];   // planes of the H0 code: the first face slot of L(v) (0..5), 6: none (a local minimum)
     uint32_t co[8];  // octant t's top cell lies in L(v)
     uint32_t event;  // the lower link is not a disc (survivors or a root), or may not be
+    // the relevant mask's other planes: the faces in slot order, and the edges
+    // [dy][dx], [dz][dx], [dz][dy] (1: the positive side)
+    uint32_t f[6], xy[2][2], xz[2][2], yz[2][2];
 };
+
+// The relevant mask's plane of the canonical neighbour n (n != 13).
+CP_HD inline uint32_t relevant_plane(const Star3& s, int n) {
+    const int dz = n / 9 - 1, dy = (n / 3) % 3 - 1, dx = n % 3 - 1;
+    const int i = dz > 0, j = dy > 0, k = dx > 0;
+    if (dz && dy && dx) return s.co[4 * i + 2 * j + k];
+    if (!dz && dy && dx) return s.xy[j][k];
+    if (dz && !dy && dx) return s.xz[i][k];
+    if (dz && dy && !dx) return s.yz[i][j];
+    return s.f[dz ? 5 * i : (dy ? 1 + 3 * j : 2 + k)];
+}
 
 CP_HD inline void full_add(uint32_t a, uint32_t b, uint32_t c, uint32_t& sum, uint32_t& carry) {
     sum = a ^ b ^ c;
@@ -23,9 +37,10 @@ CP_HD inline void full_add(uint32_t a, uint32_t b, uint32_t c, uint32_t& sum, ui
 // r[n]: the canonical neighbour n = 9(dz+1) + 3(dy+1) + (dx+1) precedes v.
 CP_HD inline void star_words3(const uint32_t (&r)[27], Star3& o) {
     // faces in slot order z-, y-, x-, x+, y+, z+; the opposite of slot s is 5 - s
-    const uint32_t f[6] = {r[4], r[10], r[12], r[14], r[16], r[22]};
+    uint32_t(&f)[6] = o.f;
+    f[0] = r[4], f[1] = r[10], f[2] = r[12], f[3] = r[14], f[4] = r[16], f[5] = r[22];
     // the collapse: an edge with both its faces, a corner with its three edges
-    uint32_t xy[2][2], xz[2][2], yz[2][2];
+    uint32_t(&xy)[2][2] = o.xy, (&xz)[2][2] = o.xz, (&yz)[2][2] = o.yz;
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
