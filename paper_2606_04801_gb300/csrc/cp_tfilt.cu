@@ -39,40 +39,45 @@ constexpr int kTT = 256;
 // the largest finite float (a pixel at that float, or above it, is flagged).
 constexpr float kFrame = kTFrame;
 
-// J four rows at a time, item blockIdx.y (the rows' divisions once per group;
-// consecutive threads write consecutive x and read consecutive, reversed,
-// pixels of the mirrored rows of the image; four loads in flight per thread).
-constexpr int kTRows = 4;
+// J eight rows at a time, item blockIdx.y (consecutive threads write
+// consecutive x and read consecutive, reversed, pixels of the mirrored rows of
+// the image; eight loads in flight per thread).  Bound by memory: 254 x 256 x
+// 250 moves 131 MB in 37 us; with 64-bit divisions for each of four rows it was
+// bound by those, 60 us.
+constexpr int kTRows = 8;
 
 __global__ void __launch_bounds__(kTT) k_t_build(const __grid_constant__ TItems t, uint32_t* bad) {
     const int item = blockIdx.y;
     const TDims& d = t.d[item];
     const float* __restrict__ img = t.img[item];
     float* __restrict__ J = t.J[item];
-    const int64_t Dj = d.ndim == 3 ? d.D + 2 : 1, Hj = d.H + 2, Wj = d.W + 2;
-    const int64_t rows = Dj * Hj;
+    // (J has at most 2^27 vertices, so rows and positions fit 32 bits)
+    const uint32_t W = uint32_t(d.W), H = uint32_t(d.H), D = d.ndim == 3 ? uint32_t(d.D) : 0u;
+    const uint32_t Dj = d.ndim == 3 ? D + 2u : 1u, Hj = H + 2u, Wj = W + 2u, rows = Dj * Hj;
     bool flag = false;
-    for (int64_t r0 = int64_t(blockIdx.x) * kTRows; r0 < rows; r0 += int64_t(gridDim.x) * kTRows) {
-        const float* in[kTRows];
-        bool live[kTRows];  // an image row (else a frame row, or past the end)
+    for (uint32_t r0 = blockIdx.x * kTRows; r0 < rows; r0 += gridDim.x * kTRows) {
+        uint32_t in[kTRows];
+        uint32_t live = 0;  // image rows (else a frame row, or past the end)
+        uint32_t z = r0 / Hj, y = r0 - z * Hj;
 #pragma unroll
         for (int k = 0; k < kTRows; ++k) {
-            const int64_t r = r0 + k;
-            const int64_t z = r / Hj, y = r - z * Hj;
-            live[k] = r < rows && y != 0 && y != Hj - 1 && (d.ndim != 3 || (z != 0 && z != Dj - 1));
-            const int64_t iz = d.ndim == 3 ? d.D - z : 0;
-            in[k] = img + (iz * d.H + (d.H - y)) * d.W;  // dereferenced only when live
+            if (r0 + k < rows && y != 0 && y != Hj - 1u && (d.ndim != 3 || (z != 0 && z != Dj - 1u))) live |= 1u << k;
+            in[k] = ((d.ndim == 3 ? D - z : 0u) * H + (H - y)) * W + W;  // read only when live, at - x
+            if (++y == Hj) {
+                y = 0;
+                ++z;
+            }
         }
-        for (int64_t x = threadIdx.x; x < Wj; x += kTT) {
-            const bool inner = x > 0 && x < Wj - 1;
+        for (uint32_t x = threadIdx.x; x < Wj; x += kTT) {
+            const bool inner = x > 0 && x < Wj - 1u;
             float a[kTRows];
 #pragma unroll
-            for (int k = 0; k < kTRows; ++k) a[k] = (live[k] && inner) ? __ldg(in[k] + (d.W - x)) : 0.0f;
+            for (int k = 0; k < kTRows; ++k) a[k] = ((live >> k) & 1u) && inner ? __ldg(img + (in[k] - x)) : 0.0f;
 #pragma unroll
             for (int k = 0; k < kTRows; ++k) {
                 if (r0 + k >= rows) break;
                 float v = kFrame;
-                if (live[k] && inner) {
+                if (((live >> k) & 1u) && inner) {
                     flag |= !(a[k] < 3.40282347e38f);  // NaN, +inf, the largest float: the frame would not lie below
                     v = -a[k];
                 }
