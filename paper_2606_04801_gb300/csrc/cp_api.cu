@@ -548,7 +548,6 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
     ra.nb = nb0;
     ra.ctr = ctr;
     ra.n_nodes = uint32_t(P.ntot);
-    ra.node = nullptr;
     SortBufs sb;
     sb.keys_alt = salt;
     sb.vals = act1;
@@ -593,8 +592,6 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
         ra.pos = rt.pos = nullptr;
         rt.ra = na0;
         rt.rb = nb0;
-        ra.node = node0;
-        rt.node = nodet;
         CP_TRY(launch_roots2(ra, rt, s));
     } else if (joint) {
         // both lists walked, then sorted together (one launch per pass), then

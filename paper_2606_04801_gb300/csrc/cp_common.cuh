@@ -11,7 +11,6 @@ namespace cp {
 constexpr int kVBits = 27;                        // global vertex id bits in a key
 constexpr uint64_t kVMask = (1ull << kVBits) - 1;
 constexpr uint32_t kTag = 0x80000000u;            // union-find word: root tag | root id
-constexpr uint32_t kTop = 0x40000000u;            // merge tree: flag of the root id of an item's oldest root
 constexpr int kMaxItems = CP_MAX_ITEMS;
 constexpr float kTFrame = -3.40282347e38f;        // T-filtration: value of the dual image's frame
 

@@ -133,7 +133,6 @@ struct RootArgs {
     uint32_t* nb;
     Counters* ctr;
     uint32_t n_nodes;            // forest entries (bounds-checked build)
-    TreeNode* node;              // k_roots2: the merge tree's nodes, or nullptr
 };
 cudaError_t launch_roots(const RootArgs& r, cudaStream_t s);
 // Both lists' first-round walks in one launch (one work counter over both).
@@ -149,7 +148,7 @@ cudaError_t launch_uf(const ItemTable& tab, const UfParams* p, int nprob, cudaSt
 struct TreeList {
     const uint64_t* keys;   // survivor keys, unsorted (ascending order is the list's order)
     const uint32_t* d_n;
-    const uint32_t* ra;     // root ids of each survivor's endpoints (k_roots2), | kTop: the item's oldest root
+    const uint32_t* ra;     // root ids of each survivor's endpoints (k_roots2)
     const uint32_t* rb;
     TreeNode* node;
     uint32_t n_rids;        // nodes (bounds-checked build)

@@ -7,19 +7,18 @@
 // connected with the older root v by survivors of key at most s; (infinity,
 // u) while it is connected with nothing older.  A survivor (u, v, s) goes in
 // as follows:
-//   1. climb from u and from v while T's key is below s: the oldest known
-//      root of each class at level s;
-//   2. the same root: the survivor closes a cycle, done;
-//   3. else, with u' the younger of the two and v' the older: compare and
-//      swap T[u'] from the word (t, w) just read to (s, v').  If another
-//      survivor changed it meanwhile, back to 1;
-//   4. if t was infinity, done; else the displaced connection (u', w, t) is
-//      still owed, and u' ~ v' at level s < t: go on with (v', w, t).
+//   1. u: the younger of the two, v: the older.  The same root: the survivor
+//      closes a cycle, done;
+//   2. if T[u]'s key is below s, u becomes the older root in T[u]; back to 1;
+//   3. else compare and swap T[u] from the word (t, w) just read to (s, v).
+//      If another survivor changed it meanwhile, on with its new word at 2;
+//   4. if t was infinity, done; else the displaced connection (u, w, t) is
+//      still owed, and u ~ v at level s < t: go on with (v, w, t).
 // Why this is the sequential elder rule.  The connections in T and those
 // displaced ones still in some thread's hands connect, at every level a, what
 // all survivors taken so far with keys at most a connect: step 3 replaces
-// (u', w, t) by (u', v', s) and (v', w, t), and what step 2 drops is implied
-// by the rest.  Every T[u] points to an older root.  When all survivors are
+// (u, w, t) by (u, v, s) and (v, w, t), and what step 1 drops is implied by
+// the rest.  Every T[u] points to an older root.  When all survivors are
 // in, a class of k roots at level a is a tree of T's connections of key at
 // most a; each root gives at most one and the oldest none, so all but the
 // oldest have T's key at most a: T[u]'s key is the level at which u stops
@@ -33,20 +32,22 @@
 // its own: the full fence after a displacement rules that out (a connection
 // taken from T by a swap is owed by one thread alone until it is back in T).
 //
-// What bounds it: chains of dependent 16-byte L2 reads (a node's word), with
-// as many survivors in flight as threads fit.  Measured against the sorted
-// design it replaces as the default (8 radix passes over both lists, then
-// reservation rounds with two grid barriers each, cp_uf.cu), kernel times:
-//   2048^2, 256 levels (14 K survivors)     204 -> 37 us
-//   512^3 blurred (587 K survivors)         553 -> 117 us
-//   128^3 uniform noise (1.15 M survivors) 1110 -> 270 us
-// The oldest root of an item is where the climbs of every survivor above the
-// percolation level end, and its word never changes: read each time, that one
-// sector held up the whole chip (244 and 475 us in the last two).  k_roots2
-// flags its id (kTop) and nothing reads it.  Tried and left out: the smallest
-// survivor of each root put in first (Boruvka's first step; its atomics cost
-// the walks what it saved here), words through L1 until the first swap (more
-// swaps fail: 117 -> 151 us).
+// What bounds it: dependent L2 reads and swaps of a node's 16-byte word, 4 to 7
+// per survivor, with as many survivors in flight as threads fit.  Only the
+// younger end's word is read: the older an end, the more survivors end there,
+// and with both ends' words read the sectors of the oldest few roots held up
+// the chip.  Ages never change, so they come through L1, and a word keeps the
+// upper half of its parent's age with the parent, so that a climb reads one
+// word per step (ages with equal upper halves are looked up).  Times, first
+// with 8 radix passes over both lists and reservation rounds with two grid
+// barriers each (cp_uf.cu), then with both ends climbed, now:
+//   2048^2 blurred (97 K survivors)                46 -> 32 us
+//   512^3 blurred (587 K survivors)         553 -> 244 -> 67 us
+//   128^3 uniform noise (1.15 M survivors) 1110 -> 475 -> 127 us
+//   2048^2 uniform noise (2.61 M survivors)       495 -> 257 us
+// Tried and left out: the smallest survivor of each root put in first
+// (Boruvka's first step; its atomics cost the walks what it saved here), words
+// through L1 until the first swap (more swaps fail), fewer threads.
 #include "cp_common.cuh"
 #include "cp_grid.cuh"
 #include "cp_kernels.h"
@@ -60,7 +61,7 @@ constexpr int kTT = 256;
 // A node's word, read and swapped as 128 bits: {key, parent}.
 struct Word {
     uint64_t key;     // infinity (~0): connected with nothing older yet
-    uint64_t parent;  // root id
+    uint64_t parent;  // root id | upper half of its age << 32 (unused while key is infinity)
 };
 
 __device__ __forceinline__ Word ld_word(const TreeNode* n) {
@@ -115,49 +116,38 @@ __global__ void __launch_bounds__(kTT) k_tree(const __grid_constant__ TreeArgs a
             set_status(ctr, kStTimeout);
             return true;
         };
-        // an item's oldest root (flagged id) is connected with nothing older
-        auto word = [&](uint32_t w) { return (w & kTop) ? Word{~0ull, w} : ld_word(T + w); };
-        auto inside = [&](uint32_t w) { return (w & kTop) || CP_IN(w, L.n_rids, ctr); };
-        for (bool live = true; live;) {
-            if (!inside(u) || !inside(v)) break;
-            Word wu = word(u), wv = word(v);
-            for (;;) {
-                const bool cu = wu.key < s, cv = wv.key < s;
-                if (!cu && !cv) break;
-                if (cu) {
-                    u = uint32_t(wu.parent);
-                    if (!inside(u)) u = 0;
-                    wu = word(u);
-                }
-                if (cv) {
-                    v = uint32_t(wv.parent);
-                    if (!inside(v)) v = 0;
-                    wv = word(v);
-                }
-                if (overdue()) {
-                    live = false;
-                    break;
-                }
-            }
-            if (!live || u == v || overdue()) break;
+        auto age = [&](uint32_t w) { return __ldg(&T[w].age); };
+        if (u == v || !CP_IN(u, L.n_rids, ctr) || !CP_IN(v, L.n_rids, ctr)) continue;
+        uint32_t hu = uint32_t(age(u) >> 32), hv = uint32_t(age(v) >> 32);
+        while (u != v) {
             // u: the younger (ages: smaller is older)
-            if ((u & kTop) || (!(v & kTop) && __ldg(&T[u].age) < __ldg(&T[v].age))) {
-                const uint32_t tu = u;
-                u = v;
-                v = tu;
-                wu = wv;
+            if (hu < hv || (hu == hv && age(u) < age(v))) {
+                const uint32_t t = u, h = hu;
+                u = v, hu = hv;
+                v = t, hv = h;
             }
-            if (u & kTop) {  // two items' oldest roots: a corrupted list
-                set_status(ctr, kStInternal);
-                break;
+            Word w = ld_word(T + u);
+            bool in = false, late = overdue();
+            while (w.key > s && !in && !late) {
+                const Word got = cas_word(T + u, w, Word{s, uint64_t(hv) << 32 | v});
+                in = got.key == w.key && got.parent == w.parent;
+                if (!in) {
+                    w = got;
+                    late = overdue();
+                }
             }
-            const Word got = cas_word(T + u, wu, Word{s, uint64_t(v)});
-            if (got.key != wu.key || got.parent != wu.parent) continue;
-            if (wu.key == ~0ull) break;
-            asm volatile("fence.sc.gpu;" ::: "memory");
-            s = wu.key;
-            u = v;
-            v = uint32_t(wu.parent);
+            if (late) break;
+            if (in) {
+                if (w.key == ~0ull) break;
+                asm volatile("fence.sc.gpu;" ::: "memory");
+                s = w.key;
+                u = v, hu = hv;
+                v = uint32_t(w.parent), hv = uint32_t(w.parent >> 32);
+                if (!CP_IN(v, L.n_rids, ctr)) break;
+            } else {  // connected with an older root below s
+                u = uint32_t(w.parent), hu = uint32_t(w.parent >> 32);
+                if (!CP_IN(u, L.n_rids, ctr)) break;
+            }
         }
         hops += steps;
     }

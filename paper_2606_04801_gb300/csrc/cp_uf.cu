@@ -113,35 +113,12 @@ constexpr int kFT = 256;
 
 __device__ __forceinline__ Forest forest_of(const RootArgs& r) { return Forest{r.uf, r.code, r.n_nodes, r.n_code, r.dual}; }
 
-// A lane's last item and list, and the id of that item's oldest root (the
-// smallest vertex's, or the outside's); no id while there is no merge tree.
-struct TopRoot {
-    uint32_t of = ~0u, id = ~0u;
-};
-
-// Survivor i of the list r (one lane): its endpoints' root ids and its
-// position.  For the merge tree the item's oldest root is flagged: a third to
-// a half of all climbs end there, and unflagged they all read its one word
-// (k_tree).
-__device__ __forceinline__ void place_walk(const ItemTable& tab, const RootArgs& r, uint32_t i, uint32_t& hops,
-                                           TopRoot& tr) {
+// Survivor i of the list r (one lane): its endpoints' root ids and its position.
+__device__ __forceinline__ void place_walk(const ItemTable& tab, const RootArgs& r, uint32_t i, uint32_t& hops) {
     uint64_t key = r.keys[i];
     if (r.dual) key = ~key;
     uint32_t ra, rb;
-    if (r.node) {
-        const int item = item_of_vertex(tab, key_vertex(key));
-        const uint32_t k = uint32_t(item) << 1 | uint32_t(r.dual);
-        if (k != tr.of) {
-            tr.of = k;
-            tr.id = ~0u;
-            const uint64_t v = uint64_t(tab.it[item].voff) + uint32_t(r.ctr->gmin[item]);
-            if (r.dual) tr.id = uint32_t(item);
-            else if (v < r.n_nodes) tr.id = __ldg(r.uf + v) & ~kTag;
-        }
-    }
     if (!walk_roots(tab, forest_of(r), r.ctr, key, ra, rb, hops)) set_status(r.ctr, kStTimeout);
-    if (ra == tr.id) ra |= kTop;
-    if (rb == tr.id) rb |= kTop;
     __stcg(r.ra + i, ra);
     __stcg(r.rb + i, rb);
     if (r.pos) __stcg(r.pos + i, i);
@@ -153,13 +130,12 @@ __global__ void __launch_bounds__(kFT) k_roots(const __grid_constant__ RootArgs 
     const uint32_t n = min(*r.d_n, r.cap);
     const unsigned lane = lane_id();
     uint32_t hops = 0;
-    TopRoot tr;
     for (;;) {
         uint32_t base = 0;
         if (lane == 0) base = atomicAdd(&ctr->find_ctr, 32u);
         base = __shfl_sync(0xFFFFFFFFu, base, 0);
         if (base >= n) break;
-        if (base + lane < n) place_walk(r.tab, r, base + lane, hops, tr);
+        if (base + lane < n) place_walk(r.tab, r, base + lane, hops);
         __syncwarp();
     }
     for (int o = 16; o > 0; o >>= 1) hops += __shfl_xor_sync(0xFFFFFFFFu, hops, o);
@@ -178,7 +154,6 @@ __global__ void __launch_bounds__(kFT) k_roots2(const __grid_constant__ RootArgs
     const uint32_t n = n0 + n1;
     const unsigned lane = lane_id();
     uint32_t hops[2] = {0, 0};
-    TopRoot tr;
     for (;;) {
         uint32_t base = 0;
         if (lane == 0) base = atomicAdd(&ctr->find_ctr, 32u);
@@ -186,7 +161,7 @@ __global__ void __launch_bounds__(kFT) k_roots2(const __grid_constant__ RootArgs
         if (base >= n) break;
         const uint32_t g = base + lane;
         const int l = g >= n0 ? 1 : 0;  // this lane's list
-        if (g < n) place_walk(r0.tab, l ? r1 : r0, l ? g - n0 : g, hops[l], tr);
+        if (g < n) place_walk(r0.tab, l ? r1 : r0, l ? g - n0 : g, hops[l]);
         __syncwarp();
     }
     for (int l = 0; l < 2; ++l) {

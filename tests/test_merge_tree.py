@@ -40,6 +40,27 @@ def insert(T, age, s, u, v):
         s, u, v = wu[0], v, wu[1]
 
 
+def insert_younger(T, age, s, u, v):
+    """The same with only the younger end's word read (cp_tree.cu)."""
+    while u != v:
+        if age[u] < age[v]:
+            u, v = v, u
+        yield
+        w = T[u]
+        while w[0] > s:
+            yield
+            if T[u] == w:
+                T[u] = (s, v)
+                break
+            w = T[u]
+        else:
+            u = w[1]
+            continue
+        if w[0] == INF:
+            return
+        s, u, v = w[0], v, w[1]
+
+
 def sequential(n, age, edges):
     par, death = list(range(n)), [INF] * n
 
@@ -61,7 +82,8 @@ def sequential(n, age, edges):
 
 @pytest.mark.parametrize("width", [1, 2, 3, 8, 64])
 @pytest.mark.parametrize("kind", ["random", "path", "staircase", "star"])
-def test_any_schedule_gives_the_elder_rule(kind, width):
+@pytest.mark.parametrize("insert", [insert, insert_younger])
+def test_any_schedule_gives_the_elder_rule(insert, kind, width):
     rng = random.Random(f"{kind}{width}")
     for trial in range(60):
         n = rng.randint(1, 24)
