@@ -150,6 +150,14 @@ __host__ __device__ __forceinline__ int64_t doubled_index(const Item& it, int z,
 #ifdef __CUDACC__
 __device__ __forceinline__ void set_status(Counters* c, uint32_t bit) { atomicOr(&c->status, bit); }
 
+// A kernel launched by launch_after may start while the one before it on the
+// stream still runs: it waits for that one's end (and its writes) here, before
+// it touches memory, and then lets its own successor start waiting.
+__device__ __forceinline__ void wait_for_previous() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // CP_IN(i, n, ctr): in the bounds-checked build (-DCP_CHECKED), true when the
 // data-dependent index i lies in [0, n), else the call is flagged
 // (kStBounds) and the caller skips the access; in the normal build, true.

@@ -8,13 +8,26 @@ namespace cp {
 namespace {
 
 constexpr int kT = 256;
+constexpr int kIT = 256;  // k_init
 
-// One outside vertex per item: the oldest dual vertex (Sec. 3.1), never
-// paired (Appendix A.4); it takes dual root id = item index.
-__global__ void k_init(const __grid_constant__ ItemTable tab, Counters* ctr, uint32_t* uft, uint64_t* aget, uint64_t* rest,
-                       TreeNode* nodet) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < tab.n) {
+// The counters and the order's bucket counts (zero_bytes from ctr on, a
+// multiple of 16) to zero, by all blocks but the first, which takes the counters
+// and then sets what starts elsewhere: one outside vertex per item, the oldest
+// dual vertex (Sec. 3.1), never paired (Appendix A.4), with dual root id = item
+// index.  (A memset before this kernel took longer than both together.)
+__global__ void __launch_bounds__(kIT) k_init(const __grid_constant__ ItemTable tab, Counters* ctr, size_t zero_bytes, uint32_t* uft,
+                                              uint64_t* aget, uint64_t* rest, TreeNode* nodet) {
+    constexpr size_t kHead = (sizeof(Counters) + 15) / 16;
+    uint4* z = reinterpret_cast<uint4*>(ctr);
+    const uint4 zero = make_uint4(0, 0, 0, 0);
+    if (blockIdx.x > 0) {
+        for (size_t i = kHead + size_t(blockIdx.x - 1) * kIT + threadIdx.x; i < zero_bytes / 16; i += size_t(gridDim.x - 1) * kIT)
+            z[i] = zero;
+        return;
+    }
+    for (size_t i = threadIdx.x; i < kHead; i += kIT) z[i] = zero;
+    __syncthreads();
+    for (int i = threadIdx.x; i < tab.n; i += kIT) {
         const Item& it = tab.it[i];
         uft[it.toff + it.T] = kTag | uint32_t(i);
         aget[i] = ~0ull;
@@ -22,7 +35,7 @@ __global__ void k_init(const __grid_constant__ ItemTable tab, Counters* ctr, uin
         if (nodet) nodet[i] = TreeNode{~0ull, uint64_t(i), 0, uint64_t(i)};  // older than every top cell
         ctr->gmin[i] = ~0ull;
     }
-    if (i == 0) ctr->n_rt = uint32_t(tab.n);
+    if (threadIdx.x == 0) ctr->n_rt = uint32_t(tab.n);
 }
 
 // The essential H0 class of each item.
@@ -168,9 +181,10 @@ cudaError_t launch_loss_backward(const cp_pair* pairs, int64_t n, const int64_t*
     return cudaGetLastError();
 }
 
-cudaError_t launch_init(const ItemTable& tab, Counters* ctr, uint32_t* uft, uint64_t* aget, uint64_t* rest,
+cudaError_t launch_init(const ItemTable& tab, Counters* ctr, size_t zero_bytes, uint32_t* uft, uint64_t* aget, uint64_t* rest,
                         TreeNode* nodet, cudaStream_t s) {
-    k_init<<<1, kMaxItems, 0, s>>>(tab, ctr, uft, aget, rest, nodet);
+    const size_t blocks = 2 + zero_bytes / (16 * 2 * kIT);  // two stores per thread
+    k_init<<<unsigned(blocks < 512 ? blocks : 512), kIT, 0, s>>>(tab, ctr, zero_bytes, uft, aget, rest, nodet);
     note_launches(1);
     return cudaGetLastError();
 }

@@ -760,6 +760,7 @@ __global__ void __launch_bounds__(kW2 * 32) k_prune2d(const __grid_constant__ It
     const int lane = int(lane_id());
     const unsigned lt = (1u << lane) - 1u;
     constexpr unsigned kAll = 0xFFFFFFFFu;
+    wait_for_previous();
     for (int task = blockIdx.x * kW2 + warp; task < tab.tiles2d * parts; task += gridDim.x * kW2) {
         const int tile = task / parts, part = task - tile * parts;
         const int ii = tile_item(tab, 0, tab.n2d - 1, tile);
@@ -1056,8 +1057,8 @@ cudaError_t launch_prune(const ItemTable& tab, const PruneOuts& po, const TmaMap
         int parts = 8;
         while (parts > 1 && int64_t(tab.tiles2d) * parts > 2432) parts >>= 1;
         const int need2 = (tab.tiles2d * parts + kW2 - 1) / kW2;
-        k_prune2d<<<need2 < blocks2d ? need2 : blocks2d, kW2 * 32, 0, s>>>(tab, o, parts);
-        note_launches(1);
+        const cudaError_t e = launch_after(true, k_prune2d, need2 < blocks2d ? need2 : blocks2d, kW2 * 32, 0, s, tab, o, parts);
+        if (e != cudaSuccess) return e;
     }
     if (tab.tiles3d > 0) {
         int cap = blocks3d;

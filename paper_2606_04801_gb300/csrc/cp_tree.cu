@@ -87,6 +87,7 @@ __device__ __forceinline__ Word cas_word(TreeNode* n, Word expect, Word desired)
 // survivor per thread.
 __global__ void __launch_bounds__(kTT) k_tree(const __grid_constant__ TreeArgs a) {
     Counters* ctr = a.ctr;
+    wait_for_previous();
     // non-finite input, or walks that gave up: the call fails anyway
     if (ld_acquire_u32(&ctr->status) & (kStTimeout | kStNonfinite)) return;
     const uint32_t n0 = min(*a.l[0].d_n, a.cap), n1 = min(*a.l[1].d_n, a.cap), n = n0 + n1;
@@ -186,9 +187,7 @@ cudaError_t launch_tree(const TreeArgs& a, cudaStream_t s) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tree, kTT, 0);
         return device_sm_count() * (per_sm > 0 ? per_sm : 1);
     });
-    k_tree<<<blocks, kTT, 0, s>>>(a);
-    note_launches(1);
-    return cudaGetLastError();
+    return launch_after(true, k_tree, blocks, kTT, 0, s, a);
 }
 
 cudaError_t launch_tree_emit(const TreeEmitArgs& a, cudaStream_t s) {

@@ -149,6 +149,7 @@ __global__ void __launch_bounds__(kFT) k_roots(const __grid_constant__ RootArgs 
 __global__ void __launch_bounds__(kFT) k_roots2(const __grid_constant__ RootArgs r0,
                                                 const __grid_constant__ RootArgs r1) {
     Counters* ctr = r0.ctr;
+    wait_for_previous();
     if (ld_acquire_u32(&ctr->status) & (kStTimeout | kStNonfinite)) return;
     const uint32_t n0 = min(*r0.d_n, r0.cap), n1 = min(*r1.d_n, r1.cap);
     const uint32_t n = n0 + n1;
@@ -611,9 +612,7 @@ cudaError_t launch_roots(const RootArgs& r, cudaStream_t s) {
 
 cudaError_t launch_roots2(const RootArgs& r0, const RootArgs& r1, cudaStream_t s) {
     // (find_ctr is zero: the call's own memset, and no other walk before this)
-    k_roots2<<<find_blocks(), kFT, 0, s>>>(r0, r1);
-    note_launches(1);
-    return cudaGetLastError();
+    return launch_after(r0.tab.n3d == 0, k_roots2, find_blocks(), kFT, 0, s, r0, r1);
 }
 
 cudaError_t launch_place_roots(const RootArgs& r, cudaStream_t s) {
