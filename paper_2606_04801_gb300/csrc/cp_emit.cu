@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kT) k_loss_scatter(const cp_pair* __restrict__
 // gradient, so the accumulators of those pixels alone are cleared, filled and
 // rounded; the output is zeroed as a whole first.  kLoss: only those of the
 // pairs in the loss (few of a smooth field's: bound by the scattered sectors,
-// the two passes took 13 and 16 us over all pairs of 512^3 and take 5 and 5).
+// the two passes took 13 and 16 us over all pairs of 512^3 and take 5 and 8).
 template <bool kLoss>
 __device__ __forceinline__ bool in_loss(const cp_pair& p, float tau) {
     return !kLoss || (p.death_pixel >= 0 && double(p.death) - double(p.birth) > double(tau));
@@ -123,18 +123,24 @@ __global__ void k_touch_clear(const cp_pair* __restrict__ pairs, int64_t n, cons
     }
 }
 
-// The first block also sums the loss: one warp, in a fixed order (a launch of
-// its own that summed them one after the other took 15 us).
+// The first block also sums the loss: one warp, in a fixed order and with the
+// additions' rounding errors carried along, so that the order costs no accuracy
+// (a launch of its own that summed them one after the other took 15 us).
 template <bool kLoss>
 __global__ void k_touch_round(const cp_pair* __restrict__ pairs, int64_t n, const int64_t* d_n, float tau,
                               const int64_t* __restrict__ offs, const double* __restrict__ acc,
                               float* __restrict__ grad, int64_t n_pixels, const double* __restrict__ partials, double* loss) {
     if (kLoss && blockIdx.x == 0 && threadIdx.x < 32) {
-        double t = 0.0;
+        double hi = 0.0, lo = 0.0;  // the sum and what its additions round off (two-sum)
+        auto add = [&](double v, double rest) {
+            const double t = hi + v, b = t - hi;
+            lo += ((hi - (t - b)) + (v - b)) + rest;
+            hi = t;
+        };
 #pragma unroll
-        for (int i = 0; i < kLossBlocks; i += 32) t += partials[i + threadIdx.x];
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
-        if (threadIdx.x == 0) *loss = t;
+        for (int i = 0; i < kLossBlocks; i += 32) add(partials[i + threadIdx.x], 0.0);
+        for (int o = 16; o > 0; o >>= 1) add(__shfl_down_sync(0xFFFFFFFFu, hi, o), __shfl_down_sync(0xFFFFFFFFu, lo, o));
+        if (threadIdx.x == 0) *loss = hi + lo;
     }
     if (d_n) n = *d_n < n ? *d_n : n;
     for (int64_t i = int64_t(blockIdx.x) * kT + threadIdx.x; i < n; i += int64_t(gridDim.x) * kT) {
