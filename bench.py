@@ -35,7 +35,7 @@ SIGMA = 3.0
 METRIC = "Mvoxels/s for exact H0+top-dim diagrams (512^3 fp32), % HBM roofline; fwd+bwd batched vs plain"
 WORKLOAD = "3D 512^3 float32 blurred noise (sigma 3 vox), H0 + H2 pairs, fwd + total-persistence loss bwd"
 TAU = 0.05  # persistence threshold of the loss
-COUNTERS_BYTES = 4056  # status/count block the forward call copies back (sizeof the library's counters)
+COUNTERS_BYTES = 4064  # status/count block the forward call copies back (sizeof the library's counters)
 
 
 def _volume(seed: int) -> np.ndarray:
@@ -501,7 +501,6 @@ def run_2d(args):
     names = ["grf", "grf_256_levels"]
     H, W = imgs[0].shape
     N = H * W
-    T = (H - 1) * (W - 1)
     stream = torch.cuda.current_stream(dev)
     sp = ctypes.c_void_p(int(stream.cuda_stream))
     dims = (ctypes.c_int64 * 2)(H, W)
@@ -580,7 +579,7 @@ def run_2d(args):
             raise cp.CpError(bp.status()["rc"], "2D graph steps")
         elapsed = job_time(total, ws, dev)
         k1s = statistics.mean(k1) / 1e3 if k1 else None
-        alg = 4 * N + 4 * N + 4 * (T + 1) + 8 * (st["h0_survivors"] + st["top_survivors"]) + 16 * (st["h0_roots"] + st["top_roots"])
+        alg = 4 * N + N + 8 * (st["h0_survivors"] + st["top_survivors"]) + 36 * (st["h0_roots"] + st["top_roots"])
         lines[name] = {
             "value": job_value(N, ws, args.steps, elapsed), "ms_per_step": elapsed / args.steps * 1e3,
             "eager_ms_per_step": eager_elapsed / args.steps * 1e3,
@@ -1090,7 +1089,6 @@ def main():
     if args.uf_variant != "auto":  # profiling one union-find design regardless of the tuner's pick
         lib.cp_set_tuning(7, int(args.uf_variant))
         tuned["uf_variant"] = int(args.uf_variant)
-    T = (SIDE - 1) ** 3
     x = torch.from_numpy(vol).to(dev)
     stream = torch.cuda.current_stream(dev)
     sp = ctypes.c_void_p(int(stream.cuda_stream))
@@ -1258,7 +1256,8 @@ def main():
     peak, peak_kind = _peaks()
     k1 = statistics.mean(k1_ms) / 1e3 if k1_ms else None
     s0, stp, r0, rt = st["h0_survivors"], st["top_survivors"], st["h0_roots"], st["top_roots"]
-    alg = 4 * N + 4 * N + 4 * (T + 1) + 8 * (s0 + stp) + 16 * (r0 + rt)
+    # the image read, a code byte per vertex, a key per survivor, a node and a word per root
+    alg = 4 * N + N + 8 * (s0 + stp) + 36 * (r0 + rt)
     achieved = alg / k1 / 1e9 if k1 else None
     traffic = None
     limiter = None
@@ -1350,7 +1349,7 @@ def _k1_hash():
     import hashlib
 
     h = hashlib.sha256()
-    for f in ("cp_prune.cu", "cp_common.cuh", "cp_mask3.cuh"):
+    for f in ("cp_prune.cu", "cp_common.cuh", "cp_mask3.cuh", "cp_words3.cuh", "cp_walk.cuh"):
         with open(os.path.join(ROOT, "paper_2606_04801_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

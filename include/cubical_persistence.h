@@ -498,8 +498,8 @@ int cubical_persistence_debug_wait_timeout(void *d_workspace, size_t ws_bytes, i
  *                        and takes only the edges H0 leaves positive (the
  *                        cross-pruning of Sec. 3.2, Sec. 4.1 step 4: two sorts
  *                        and two union-find launches in sequence); 0 (default):
- *                        both dimensions run at once (one sort and one
- *                        union-find launch), the dual list keeping the edges
+ *                        both dimensions run at once (one union-find
+ *                        launch), the dual list keeping the edges
  *                        the table cannot settle, which the dual union-find
  *                        then finds closing dual cycles.  Same pairs.
  *   CP_TUNE_H1_BUDGET_MS wall-clock budget in milliseconds of the cross-star
@@ -543,12 +543,12 @@ long long cp_launch_count(void);
 /*
  * cp_profile(1) makes every following forward call record CUDA events on its
  * stream between its stages; cp_stage_times() then waits for the last call
- * and writes the six stage durations in milliseconds (prune, sort H0,
- * union-find H0, sort dual, union-find dual, emit) into ms[0..5] and returns
- * 6 (or a negative CP_ERR_* code; cap must be >= 6).  Each sort stage
- * includes the first-round root walks of its list.  In a call with volumes
- * only, both lists are walked and sorted together and both union-finds run in
- * one launch: ms[1] and ms[2] hold those joint times and ms[3], ms[4] are 0.
+ * and writes the six stage durations in milliseconds (prune, walks and sort
+ * H0, union-find H0, walks and sort dual, union-find dual, emission and order)
+ * into ms[0..5] and returns 6 (or a negative CP_ERR_* code; cap must be >= 6).
+ * Unless images are cross-pruned, both lists go together: ms[1] and ms[2] hold
+ * the walks (with CP_TUNE_UF_VARIANT = 1 and in slab calls the sort as well)
+ * and the union-find of both, and ms[3], ms[4] are 0.
  * In a cubical_persistence_slabs call, ms[2] holds stage 1 (the split and the
  * slabs' union-finds) and ms[4] stage 2 (marking, compaction and the merge
  * union-find).  cp_profile(0) stops recording.  Not thread-safe across concurrent calls.

@@ -1,10 +1,11 @@
 // C-ABI entry points: argument checks, workspace layout, lookup-table set-up
 // and the enqueueing of the pipeline
-//   init -> K1 prune -> root walks -> K3 merge trees of both lists -> essential pairs
-//        (slab split, Borůvka variant: K2 sort of both lists -> K3 rounds; 2D
-//        cross-pruning: sort and rounds of H0, then of the dual)
-//        [-> H1 of the volumes: columns, sort, reduction, pairs]
-//        -> K2 sort (pairs, canonical order) -> gather.
+//   init -> K1 prune -> root walks -> K3 merge trees of both lists
+//        -> K4: pairs emitted, put in canonical order and gathered.
+// Slab split and Borůvka variant: after the walks K2 sort of both lists -> K3
+// rounds -> essential pairs -> K4 in order; 2D cross-pruning: walks, sort and
+// rounds of H0, then of the dual.  Calls with H1: after the trees their pairs,
+// the essential pairs and the H1 columns, reduction and pairs, then K4 in order.
 #include <algorithm>
 #include <atomic>
 #include <cstddef>

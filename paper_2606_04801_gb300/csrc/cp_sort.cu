@@ -1,5 +1,8 @@
 // K2: LSD radix sort of 64-bit keys (optional 32-bit payload), 8-bit
 // digits, one kernel per digit pass with decoupled look-back ("onesweep").
+// For the calls whose union-finds take their survivors in order: the slab
+// split, the Borůvka variant and 2D cross-pruning (the merge tree of the
+// others takes them in any order).
 //
 // The filtration order of the survivors (Sec. 2.3) is a total order on
 // their 64-bit keys, so sorting the keys orders the union-find input

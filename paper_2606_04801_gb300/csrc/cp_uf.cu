@@ -1,6 +1,8 @@
 // K3: elder-rule union-find over the sorted survivors, H0 (Sec. 4.1 step 3,
 // Sec. 4.2 step 2) and the dual graph (Sec. 3.1, Appendix A; Sec. 4.1 step 5,
-// Sec. 4.2 step 3), plus the 2D cross-pruning of Sec. 3.2 / Sec. 4.1 step 4.
+// Sec. 4.2 step 3), plus the 2D cross-pruning of Sec. 3.2 / Sec. 4.1 step 4;
+// and the root walks of every call.  The rounds serve the slab split, the
+// Borůvka variant and cross-pruning; other calls use the merge tree (cp_tree.cu).
 //
 // Sequential union-find processes the sorted survivors one at a time; the
 // pairs depend on that order.  Here every unresolved survivor is processed
