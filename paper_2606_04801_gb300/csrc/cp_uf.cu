@@ -157,15 +157,17 @@ __global__ void __launch_bounds__(kFT) k_roots2(const __grid_constant__ RootArgs
     const uint32_t n = n0 + n1;
     const unsigned lane = lane_id();
     uint32_t hops[2] = {0, 0};
-    for (;;) {
-        uint32_t base = 0;
-        if (lane == 0) base = atomicAdd(&ctr->find_ctr, 32u);
-        base = __shfl_sync(0xFFFFFFFFu, base, 0);
-        if (base >= n) break;
+    // a warp's first 32 by its number, the others from the counter (with the
+    // first from the counter too, small calls waited for 7,296 warps' atomics on
+    // it: 2048^2 31 -> 22 us, 254 x 256 x 250 43 -> 33)
+    const uint32_t warps = gridDim.x * (kFT / 32);
+    for (uint32_t base = (blockIdx.x * (kFT / 32) + (threadIdx.x >> 5)) * 32u; base < n;) {
         const uint32_t g = base + lane;
         const int l = g >= n0 ? 1 : 0;  // this lane's list
         if (g < n) place_walk(r0.tab, l ? r1 : r0, l ? g - n0 : g, hops[l]);
         __syncwarp();
+        if (lane == 0) base = atomicAdd(&ctr->find_ctr, 32u) + warps * 32u;
+        base = __shfl_sync(0xFFFFFFFFu, base, 0);
     }
     for (int l = 0; l < 2; ++l) {
         uint32_t h = hops[l];
@@ -614,7 +616,9 @@ cudaError_t launch_roots(const RootArgs& r, cudaStream_t s) {
 
 cudaError_t launch_roots2(const RootArgs& r0, const RootArgs& r1, cudaStream_t s) {
     // (find_ctr is zero: the call's own memset, and no other walk before this)
-    return launch_after(r0.tab.n3d == 0, k_roots2, find_blocks(), kFT, 0, s, r0, r1);
+    // (overlapped for small images only: in place of the 2D pass's shared memory
+    // the walks want L1; 2048^2 noise 139 us overlapped, 89 not)
+    return launch_after(r0.tab.n3d == 0 && r0.tab.tiles2d <= 1216, k_roots2, find_blocks(), kFT, 0, s, r0, r1);
 }
 
 cudaError_t launch_place_roots(const RootArgs& r, cudaStream_t s) {
