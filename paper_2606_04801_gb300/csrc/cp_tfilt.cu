@@ -39,12 +39,12 @@ constexpr int kTT = 256;
 // the largest finite float (a pixel at that float, or above it, is flagged).
 constexpr float kFrame = kTFrame;
 
-// J eight rows at a time, item blockIdx.y (consecutive threads write
+// J four rows at a time, item blockIdx.y (consecutive threads write
 // consecutive x and read consecutive, reversed, pixels of the mirrored rows of
-// the image; eight loads in flight per thread).  Bound by memory: 254 x 256 x
-// 250 moves 131 MB in 37 us; with 64-bit divisions for each of four rows it was
-// bound by those, 60 us.
-constexpr int kTRows = 8;
+// the image; four loads in flight per thread).  Bound by memory: 510^3 moves
+// 1,068 MB in 188 us (5.7 TB/s; 227 us with eight rows), 254 x 256 x 250 131 MB
+// in 37 us; with 64-bit divisions for each row it was bound by those, 60 us.
+constexpr int kTRows = 4;
 
 __global__ void __launch_bounds__(kTT) k_t_build(const __grid_constant__ TItems t, uint32_t* bad) {
     const int item = blockIdx.y;
