@@ -4,18 +4,17 @@
 // Per vertex v:
 //   1. the mask of the neighbours that precede v (value, then index): 8 in 2D,
 //      26 in 3D;
-//   2. what it says about the lower star of v: 2D by a direct 256-entry table,
-//      3D by closed forms on words of 32 vertices, with a perfect-hash lookup
-//      for the vertices that leave survivors;
+//   2. what it says about the lower star of v, by closed forms on words of 32
+//      vertices, with a lookup (2D: 256 entries, 3D: a perfect hash) for the
+//      vertices that leave survivors or a root;
 //   3. the H0 forest link of v (first edge of L(v)), or v as an H0 root (local
 //      minimum);
 //   4. the dual forest link of each top cell, from its largest corner's lower
 //      star: the top cell across the facet where it dies locally, the outside
 //      vertex, or itself as a dual root;
 //   5. the surviving edges and facets as 64-bit order keys.
-// Rows (2D) and planes (3D) ahead are brought into shared memory
-// asynchronously; positions outside the image hold values that precede
-// nothing.
+// Planes (3D) ahead are brought into shared memory asynchronously; positions
+// outside the image hold values that precede nothing.
 #include "cp_common.cuh"
 #include "cp_kernels.h"
 #include "cp_mask3.cuh"
