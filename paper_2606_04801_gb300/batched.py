@@ -86,7 +86,9 @@ class BatchedPersistence:
         if len(inputs) != self.k:
             raise ValueError("wrong number of items")
         # plain float tensors on the device go in one launch, the rest (host or
-        # other types, strided, recorded by autograd, parts of this batch) by copy_
+        # other types, strided, recorded by autograd, parts of this batch) by
+        # copy_; those on the device may read items of this batch that come
+        # before them in the list, so what waits is copied first
         counts = [0] * self.k
         ptrs = [0] * self.k
         lo, hi = self.x.data_ptr(), self.x.data_ptr() + 4 * self.total
@@ -97,14 +99,21 @@ class BatchedPersistence:
                 if p & 3 == 0 and (p >= hi or p + 4 * n <= lo):
                     counts[i], ptrs[i] = n, p
                     continue
-            v.copy_(torch.as_tensor(a).reshape(v.shape), non_blocking=True)
+            a = torch.as_tensor(a)
+            if a.is_cuda and any(counts):
+                self._load_plain(ptrs, counts)
+                counts = [0] * self.k
+            v.copy_(a.reshape(v.shape), non_blocking=True)
         if any(counts):
-            with torch.cuda.device(self.dev):
-                rc = self.lib.cubical_persistence_load_items(
-                    self.k, (ctypes.c_void_p * self.k)(*ptrs), self._ptrs, (ctypes.c_int64 * self.k)(*counts),
-                    ctypes.c_void_p(torch.cuda.current_stream(self.dev).cuda_stream))
-            if rc != CP_OK:
-                raise CpError(rc, "load_items")
+            self._load_plain(ptrs, counts)
+
+    def _load_plain(self, ptrs, counts):
+        with torch.cuda.device(self.dev):
+            rc = self.lib.cubical_persistence_load_items(
+                self.k, (ctypes.c_void_p * self.k)(*ptrs), self._ptrs, (ctypes.c_int64 * self.k)(*counts),
+                ctypes.c_void_p(torch.cuda.current_stream(self.dev).cuda_stream))
+        if rc != CP_OK:
+            raise CpError(rc, "load_items")
 
     def _enqueue(self, stream_ptr: int):
         lib = self.lib

@@ -45,3 +45,21 @@ def test_general_copies_and_refusals():
         bp.load(xs[:-1] + [torch.rand(5, 7).cuda()])
     with pytest.raises(ValueError):
         bp.load(xs[:-1])
+
+
+def test_items_of_the_batch_as_sources_in_list_order():
+    """A source that is a part of the batch sees the items before it in the
+    list loaded and those after it not, whatever way each is copied."""
+    import paper_2606_04801_gb300 as cp
+
+    bp = cp.BatchedPersistence([(5, 6)] * 6)
+    old = [torch.rand(5, 6).cuda() for _ in range(6)]
+    bp.load(old)
+    new = [torch.rand(5, 6).cuda() for _ in range(6)]
+    src = [new[0], bp.views[0], bp.views[3], new[3], bp.views[3].double(), bp.views[2].t().contiguous().t()]
+    want = [new[0], new[0], old[3], new[3], old[3], old[2]]  # (the last two are copies made before the call)
+    bp.load(src)
+    for i, v in enumerate(want):
+        assert torch.equal(bp.views[i], v), i
+    bp.load([new[1], bp.views[0].view(6, 5).t(), new[2], new[3], new[4], new[5]])  # strided
+    assert torch.equal(bp.views[1], new[1].view(6, 5).t())
