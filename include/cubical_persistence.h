@@ -485,6 +485,16 @@ int cubical_persistence_debug_layout(int n_items, const int32_t *ndims, const in
  * `stream`.
  */
 int cubical_persistence_debug_wait_timeout(void *d_workspace, size_t ws_bytes, int64_t limit_us, void *stream);
+/*
+ * The same of the output launch's grid barriers: a forward call (arguments as
+ * for cubical_persistence_2d / _3d, max_survivors 0) whose barriers wait for
+ * one thread block more than there is and give up after limit_us microseconds
+ * (1 .. 2,000,000).  Returns CP_ERR_TIMEOUT with both counts 0, no pair
+ * written and the context usable.
+ */
+int cubical_persistence_debug_order_timeout(int ndim, const float *d_image, const int64_t *dims, cp_pair *d_out_pairs,
+                                            int64_t capacity, int64_t *h_out_count, int64_t *d_out_count,
+                                            void *d_workspace, size_t ws_bytes, int64_t limit_us, void *stream);
 
 /*
  * Tuning of the pruning pass (process-wide; read by the following calls;

@@ -432,8 +432,14 @@ struct TMode {
     const uint32_t* bad;
 };
 
+// How the output launch's grid barriers wait (OrderArgs).
+struct OrderWait {
+    uint32_t absent = 0;
+    uint64_t limit_ns = kWaitLimitNs;
+};
+
 int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, int64_t* d_out_count, void* ws,
-        size_t ws_bytes, cudaStream_t s, bool prune_only = false, const TMode* tm = nullptr) {
+        size_t ws_bytes, cudaStream_t s, bool prune_only = false, const TMode* tm = nullptr, OrderWait wait = {}) {
     if (!ws || (!d_out && capacity > 0) || capacity < 0) return CP_ERR_ARG;
     if (ws_bytes < P.bytes + kWsSlack) return CP_ERR_ARG;
     int rc = ensure_device_tables();
@@ -874,6 +880,8 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
     oa.out_cap = capacity;
     oa.out16 = (reinterpret_cast<uintptr_t>(d_out) & 15u) == 0 ? 1 : 0;
     oa.d_out_count = d_out_count;
+    oa.absent = wait.absent;
+    oa.limit_ns = wait.limit_ns;
     oa.ctr = ctr;
     CP_TRY(launch_order(oa, s));
     mark(6, s);
@@ -1322,6 +1330,19 @@ int cubical_persistence_debug_wait_timeout(void* d_workspace, size_t ws_bytes, i
     if (cudaMemcpyAsync(&h, ctr, sizeof(Counters), cudaMemcpyDeviceToHost, s) != cudaSuccess) return CP_ERR_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return CP_ERR_CUDA;
     return status_to_code(h.status);
+}
+
+int cubical_persistence_debug_order_timeout(int ndim, const float* d_image, const int64_t* dims, cp_pair* d_out_pairs,
+                                            int64_t capacity, int64_t* h_out_count, int64_t* d_out_count,
+                                            void* d_workspace, size_t ws_bytes, int64_t limit_us, void* stream) {
+    if ((ndim != 2 && ndim != 3) || !d_image || !dims || limit_us <= 0 || limit_us > 2000000) return CP_ERR_ARG;
+    int32_t nd = ndim;
+    int64_t d3[3] = {ndim == 3 ? dims[0] : 1, dims[ndim - 2], dims[ndim - 1]};
+    Plan P;
+    const int rc = make_plan(1, &nd, d3, &d_image, 0, P);
+    if (rc != CP_OK) return rc;
+    return run(P, d_out_pairs, capacity, h_out_count, d_out_count, d_workspace, ws_bytes, static_cast<cudaStream_t>(stream),
+               false, nullptr, OrderWait{1, uint64_t(limit_us) * 1000u});
 }
 
 int cp_set_tuning(int key, int value) {

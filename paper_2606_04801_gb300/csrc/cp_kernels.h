@@ -385,6 +385,8 @@ struct OrderArgs {
     int64_t out_cap;
     int out16;                  // out is 16-byte aligned
     int64_t* d_out_count;
+    uint32_t absent;            // CTAs that the grid barriers wait for and that never come (tests of their giving up; else 0)
+    uint64_t limit_ns;          // after which they give up
     Counters* ctr;
 };
 void plan_order(uint64_t places, int* shift, int* chunk_shift, uint32_t* buckets);

@@ -76,22 +76,37 @@ __device__ __forceinline__ uint64_t place_of(const OrderArgs& a, const cp_pair& 
     return a.base[p.item] + uint64_t(c) * a.cells[p.item] + uint32_t(p.birth_cell);
 }
 
+// The number of pairs to the caller (thread 0 of the grid), or none (any CTA
+// that gives up): a CTA that gives up flags the call before it writes 0, and
+// the number is taken back if the flag shows after it, so a failed call never
+// reports pairs.
+__device__ __forceinline__ void put_count(const OrderArgs& a, int64_t n) {
+    volatile int64_t* c = &a.ctr->out_count;
+    volatile int64_t* d = a.d_out_count;
+    *c = n;
+    if (d) *d = n;
+}
+
 // Grid barrier on the call's own counter (zero at the start of the call).
-__device__ __forceinline__ void order_barrier(Counters* ctr, uint32_t& epoch) {
+// False: the wait gave up and the CTA has to leave, since what other CTAs were
+// to write may not be there.  It then arrives at no later barrier, so no CTA
+// gets past one with another's part missing.
+__device__ __forceinline__ bool order_barrier(const OrderArgs& a, uint32_t& epoch) {
     __syncthreads();
     ++epoch;
+    bool late = false;
     if (threadIdx.x == 0) {
-        const uint32_t target = epoch * gridDim.x;
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&ctr->order_bar) : "memory");
+        const uint32_t target = epoch * gridDim.x + a.absent;
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&a.ctr->order_bar) : "memory");
         const uint64_t t0 = global_timer_ns();
-        while (ld_acquire_u32(&ctr->order_bar) < target) {
-            if (global_timer_ns() - t0 > kWaitLimitNs) {
-                set_status(ctr, kStTimeout);
-                break;
-            }
+        while (!late && ld_acquire_u32(&a.ctr->order_bar) < target) late = global_timer_ns() - t0 > a.limit_ns;
+        if (late) {
+            set_status(a.ctr, kStTimeout);
+            __threadfence();
+            put_count(a, 0);
         }
     }
-    __syncthreads();
+    return !__syncthreads_or(late);
 }
 
 // Pair i of the list: mapped (T calls), counted in its bucket.
@@ -135,10 +150,7 @@ __global__ void __launch_bounds__(kOT) k_order(const __grid_constant__ OrderArgs
     // a bounded wait that gave up, or non-finite input: the call fails anyway
     // (set by the launches before: every CTA reads the same)
     if (ld_acquire_u32(&ctr->status) & (kStTimeout | kStNonfinite)) {
-        if (gtid == 0) {
-            ctr->out_count = 0;
-            if (a.d_out_count) *a.d_out_count = 0;
-        }
+        if (gtid == 0) put_count(a, 0);
         return;
     }
     // ---- the pairs, each counted in its bucket
@@ -176,7 +188,7 @@ __global__ void __launch_bounds__(kOT) k_order(const __grid_constant__ OrderArgs
             count_pair(a, i, p);
         }
     }
-    order_barrier(ctr, epoch);
+    if (!order_barrier(a, epoch)) return;
     // ---- where each bucket starts within its chunk of 2^chunk_shift buckets
     // (a chunk per CTA), and the chunks' totals
     if (threadIdx.x == 0) sh_n = min(ld_acquire_u32(&ctr->n_pairs), a.pair_cap);
@@ -199,7 +211,7 @@ __global__ void __launch_bounds__(kOT) k_order(const __grid_constant__ OrderArgs
         }
         if (threadIdx.x == 0) __stcg(a.chunk + blockIdx.x, run);
     }
-    order_barrier(ctr, epoch);
+    if (!order_barrier(a, epoch)) return;
     {
         const uint32_t c = threadIdx.x < nchunks ? __ldcg(a.chunk + threadIdx.x) : 0u;
         const uint32_t at = block_scan(c, sh_warp);
@@ -220,7 +232,7 @@ __global__ void __launch_bounds__(kOT) k_order(const __grid_constant__ OrderArgs
         if (CP_IN(at, n, ctr))
             __stcg(a.sorted + at, make_uint2(uint32_t(place & ((uint64_t(1) << a.shift) - 1u)), i));
     }
-    order_barrier(ctr, epoch);
+    if (!order_barrier(a, epoch)) return;
     // ---- each to its place: the bucket's start and its rank among the members
     for (uint32_t d = gtid; d < n; d += gsize) {
         const uint2 e = __ldcg(a.sorted + d);
@@ -249,8 +261,9 @@ __global__ void __launch_bounds__(kOT) k_order(const __grid_constant__ OrderArgs
         }
     }
     if (gtid == 0) {
-        ctr->out_count = int64_t(n);
-        if (a.d_out_count) *a.d_out_count = int64_t(n);
+        put_count(a, int64_t(n));
+        __threadfence();
+        if (ld_acquire_u32(&ctr->status) & kStTimeout) put_count(a, 0);
         if (int64_t(n) > a.out_cap) set_status(ctr, kStCapacity);
         if (a.t_bad && *a.t_bad) set_status(ctr, kStNonfinite);
     }
