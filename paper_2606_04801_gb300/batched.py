@@ -91,9 +91,10 @@ class BatchedPersistence:
         # before them in the list, so what waits is copied first
         counts = [0] * self.k
         ptrs = [0] * self.k
+        dev = self.x.device  # with its index, which self.dev may leave out
         lo, hi = self.x.data_ptr(), self.x.data_ptr() + 4 * self.total
         for i, (v, a, n) in enumerate(zip(self.views, inputs, self.sizes)):
-            if (type(a) is torch.Tensor and a.dtype is torch.float32 and a.device == self.dev and a.numel() == n
+            if (type(a) is torch.Tensor and a.dtype is torch.float32 and a.device == dev and a.numel() == n
                     and a.is_contiguous() and not a.requires_grad and not a.is_neg()):
                 p = a.data_ptr()
                 if p & 3 == 0 and (p >= hi or p + 4 * n <= lo):

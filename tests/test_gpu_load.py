@@ -63,3 +63,16 @@ def test_items_of_the_batch_as_sources_in_list_order():
         assert torch.equal(bp.views[i], v), i
     bp.load([new[1], bp.views[0].view(6, 5).t(), new[2], new[3], new[4], new[5]])  # strided
     assert torch.equal(bp.views[1], new[1].view(6, 5).t())
+
+
+def test_device_without_index_takes_one_launch():
+    import paper_2606_04801_gb300 as cp
+
+    lib = cp.load()
+    for device in (None, "cuda", "cuda:0"):
+        bp = cp.BatchedPersistence([(5, 6)] * 4, device=device)
+        xs = [torch.rand(5, 6).cuda() for _ in range(4)]
+        before = lib.cp_launch_count()
+        bp.load(xs)
+        assert lib.cp_launch_count() - before == 1, device
+        assert torch.equal(bp.x, torch.cat([v.reshape(-1) for v in xs]))
