@@ -20,6 +20,7 @@ from typing import Optional, Sequence
 
 import numpy as np
 import torch
+from torch.autograd import forward_ad
 
 from . import _lib
 from ._lib import CP_ERR_CAPACITY, CP_OK, CpError
@@ -85,16 +86,19 @@ class BatchedPersistence:
     def load(self, inputs: Sequence[torch.Tensor]):
         if len(inputs) != self.k:
             raise ValueError("wrong number of items")
-        # plain float tensors on the device go in one launch, the rest (host or
-        # other types, strided, recorded by autograd, parts of this batch) by
-        # copy_; those on the device may read items of this batch that come
-        # before them in the list, so what waits is copied first
+        # plain float tensors on the device go in one launch, the rest by copy_:
+        # host or other types, strided, recorded by autograd (by forward mode: any
+        # in its scope), parts of this batch; all of a batch made in inference
+        # mode, which copy_ refuses outside it.  Those on the device may read
+        # items of this batch that come before them in the list, so what waits is
+        # copied first
         counts = [0] * self.k
         ptrs = [0] * self.k
+        plain = forward_ad._current_level < 0 and (torch.is_inference_mode_enabled() or not self.x.is_inference())
         dev = self.x.device  # with its index, which self.dev may leave out
         lo, hi = self.x.data_ptr(), self.x.data_ptr() + 4 * self.total
         for i, (v, a, n) in enumerate(zip(self.views, inputs, self.sizes)):
-            if (type(a) is torch.Tensor and a.dtype is torch.float32 and a.device == dev and a.numel() == n
+            if (plain and type(a) is torch.Tensor and a.dtype is torch.float32 and a.device == dev and a.numel() == n
                     and a.is_contiguous() and not a.requires_grad and not a.is_neg()):
                 p = a.data_ptr()
                 if p & 3 == 0 and (p >= hi or p + 4 * n <= lo):
@@ -109,6 +113,8 @@ class BatchedPersistence:
             self._load_plain(ptrs, counts)
 
     def _load_plain(self, ptrs, counts):
+        # as copy_ does: autograd learns that the batch changed
+        torch.autograd.graph.increment_version(self.x)
         with torch.cuda.device(self.dev):
             rc = self.lib.cubical_persistence_load_items(
                 self.k, (ctypes.c_void_p * self.k)(*ptrs), self._ptrs, (ctypes.c_int64 * self.k)(*counts),

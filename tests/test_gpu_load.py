@@ -76,3 +76,34 @@ def test_device_without_index_takes_one_launch():
         bp.load(xs)
         assert lib.cp_launch_count() - before == 1, device
         assert torch.equal(bp.x, torch.cat([v.reshape(-1) for v in xs]))
+
+
+def test_autograd_sees_a_load_as_it_sees_a_copy():
+    """A value saved for backward that a load overwrites is an error, not a
+    gradient of the new values; tangents of forward mode are copied; a batch
+    made in inference mode takes loads there alone."""
+    import torch.autograd.forward_ad as fw
+
+    import paper_2606_04801_gb300 as cp
+
+    def one():
+        return torch.rand(5, 6).cuda()
+
+    bp = cp.BatchedPersistence([(5, 6)] * 2)
+    bp.load([one(), one()])
+    w = torch.rand(5, 6, device="cuda", requires_grad=True)
+    y = (bp.views[1] * w).sum()
+    bp.load([one(), one()])
+    with pytest.raises(RuntimeError, match="modified by an inplace operation"):
+        y.backward()
+    with fw.dual_level():
+        t = torch.rand(5, 6).cuda()
+        bp.load([fw.make_dual(one(), t), one()])
+        assert torch.equal(fw.unpack_dual(bp.views[0]).tangent, t)
+    with torch.inference_mode():
+        bi = cp.BatchedPersistence([(5, 6)] * 2)
+        xs = [one(), one()]
+        bi.load(xs)
+        assert torch.equal(bi.x, torch.cat([v.reshape(-1) for v in xs]))
+    with pytest.raises(RuntimeError):
+        bi.load([one(), one()])
