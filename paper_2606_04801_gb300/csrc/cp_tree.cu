@@ -24,6 +24,14 @@
 // oldest have T's key at most a: T[u]'s key is the level at which u stops
 // being the oldest of its class, which is the survivor that kills it.  The
 // keys (so the pairs) do not depend on the schedule; the parents may.
+//
+// Long climbs shorten their way: with u connected with p at s1 (u's word) and p
+// with w at s2 < s1 (p's), u's word becomes (s1, w).  Its key stays, so the
+// pairs do; w is older than p; and what the word said follows from it and the
+// words of p, a root older than u: a connection displaced from or dropped at a
+// root rests on words, present or past, of older roots alone, so no two rest
+// on one another.
+//
 // This is the triplet merge tree of Smirnov and Morozov (TopoInVis 2017), in
 // root-id space.
 //
@@ -45,6 +53,12 @@
 //   512^3 blurred (587 K survivors)         553 -> 244 -> 67 us
 //   128^3 uniform noise (1.15 M survivors) 1110 -> 475 -> 127 us
 //   2048^2 uniform noise (2.61 M survivors)       495 -> 257 us
+// On a slope with noise (each basin drains into the one below it) the paths of
+// a survivor's ends meet far down, and a climb is as long as that: shortened
+// after 4, 8, 16, 32, 64 steps or never, 2048 x 8192 noise on a ramp takes
+// 1.22, 1.26, 1.41, 1.55, 1.75 or 9.17 ms (sort and rounds: 5.9), 2048^2 valleys
+// 88, 85, 88, 97, 121 or 908 us, but 128^3 noise, whose swaps it adds to, 192,
+// 173, 152, 141, 138 or 137 us and 512^3 blurred 123, 113, 102, 97, 97 or 96.
 // Tried and left out: the smallest survivor of each root put in first
 // (Boruvka's first step; its atomics cost the walks what it saved here), words
 // through L1 until the first swap (more swaps fail), fewer threads.
@@ -57,6 +71,7 @@ namespace cp {
 namespace {
 
 constexpr int kTT = 256;
+constexpr uint32_t kFar = 32;  // steps after which a climb shortens the paths it takes
 
 // A node's word, read and swapped as 128 bits: {key, parent}.
 struct Word {
@@ -146,7 +161,15 @@ __global__ void __launch_bounds__(kTT) k_tree(const __grid_constant__ TreeArgs a
                 v = uint32_t(w.parent), hv = uint32_t(w.parent >> 32);
                 if (!CP_IN(v, L.n_rids, ctr)) break;
             } else {  // connected with an older root below s
-                u = uint32_t(w.parent), hu = uint32_t(w.parent >> 32);
+                const uint32_t p = uint32_t(w.parent);
+                if (!CP_IN(p, L.n_rids, ctr)) break;
+                Word x = w;
+                if (steps > kFar) {  // two steps at once, and one from now on if the second is below the first
+                    x = ld_word(T + p);
+                    if (x.key >= s) x = w;
+                    else if (x.key < w.key) cas_word(T + u, w, Word{w.key, x.parent});
+                }
+                u = uint32_t(x.parent), hu = uint32_t(x.parent >> 32);
                 if (!CP_IN(u, L.n_rids, ctr)) break;
             }
         }
