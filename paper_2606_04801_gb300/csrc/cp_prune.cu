@@ -637,7 +637,7 @@ __global__ void __launch_bounds__(256) k_expand(const __grid_constant__ ItemTabl
             const int y = int(v / it.W), x = int(v - int64_t(y) * it.W);
             const uint32_t c = o.code[it.coff + code_at2(it, y, x)];
             int dy, dx;
-            if ((c & 15u) < 8u) {
+            if ((c & 15u) < 14u) {
                 link_offset2(0, c & 15u, dy, dx);
                 o.uf0[it.voff + v] = uint32_t(it.voff + v + int64_t(dy) * it.W + dx);
             }
@@ -692,7 +692,7 @@ __global__ void __launch_bounds__(256) k_expand(const __grid_constant__ ItemTabl
 // the events of its own rows.  Large ones are bound by issue.  Marching down a
 // strip with a mask, a table read and two 32-bit links per vertex took 273 warp
 // instructions per 32 vertices and wrote eight bytes per vertex instead of
-// one: 4096^2 smooth 188 -> 38 us, 2048^2 49 -> 11, 2048^2 noise 113 -> 60,
+// one: 4096^2 smooth 188 -> 40 us, 2048^2 49 -> 12, 2048^2 noise 113 -> 60,
 // 769 x 1021 18 -> 7, 64^2 noise 10 -> 8.
 constexpr int kW2 = 4;                   // warps per CTA (independent tiles)
 
@@ -799,15 +799,30 @@ __global__ void __launch_bounds__(kW2 * 32) k_prune2d(const __grid_constant__ It
             const uint32_t u1 = nu & ~1u, u2 = u1 & (u1 << 1), u4 = u2 & (u2 << 2), u8 = u4 & (u4 << 4), u16 = u8 & (u8 << 8);
             const uint32_t d1 = py & ~out & 0x7FFFFFFEu, d2 = d1 & (d1 >> 1), d4 = d2 & (d2 >> 2), d8 = d4 & (d4 >> 4),
                            d16 = d8 & (d8 >> 8);
+            // of the other links, at least 4 (and 16 along y) long; a lane whose own
+            // link depends on what lies beyond the tile is in none
+            auto four = [&](uint32_t q, bool left) {
+                if (lane == (left ? 0 : 31)) q = 0u;
+                q &= left ? __shfl_up_sync(kAll, q, 1) : __shfl_down_sync(kAll, q, 1);
+                return q & (left ? __shfl_up_sync(kAll, q, 2) : __shfl_down_sync(kAll, q, 2));
+            };
+            const uint32_t hl = ~nu & nl, hr = ~nu & ~nl & nr, hd = ~nu & ~nl & ~nr & nd, h0 = ~(nu | nl | nr | nd);
+            const uint32_t hl4 = four(hl, true), hr4 = four(hr, false);
+            const uint32_t e1 = hd & 0x7FFFFFFEu, e2 = e1 & (e1 >> 1), hd4 = e2 & (e2 >> 2), e8 = hd4 & (hd4 >> 4),
+                           hd16 = e8 & (e8 >> 8);
+            const uint32_t cx = px & ~out, cm = mx & ~out, cy = my & ~out;
+            const uint32_t cx4 = four(cx, false), cm4 = four(cm, true);
+            const uint32_t g1 = cy & 0x7FFFFFFEu, g2 = g1 & (g1 << 1), cy4 = g2 & (g2 << 2), g8 = cy4 & (cy4 << 4),
+                           cy16 = g8 & (g8 << 8);
             uint32_t acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-            spread<0>(acc, ((nu & ((u2 & ~u4) | (u8 & ~u16))) | (~nu & (nl | (~nr & nd)))) >> 1);
-            spread<1>(acc, ((nu & u4 & ~u16) | (~nu & ~nl)) >> 1);
-            spread<2>(acc, (u16 | ~nu) >> 1);
-            spread<3>(acc, ~(nu | nl | nr | nd) >> 1);
-            spread<4>(acc, ((d2 & ~d4) | (d8 & ~d16) | ((px | my) & ~out) | out | root) >> 1);
-            spread<5>(acc, ((d4 & ~d16) | ((mx | my) & ~out) | root) >> 1);
-            spread<6>(acc, (d16 | ((px | mx | my) & ~out) | root) >> 1);
-            spread<7>(acc, (dg | out | root) >> 1);
+            spread<0>(acc, ((u2 & ~u4) | (u8 & ~u16) | (hl & ~hl4) | hr4 | (hd & ~hd4) | hd16) >> 1);
+            spread<1>(acc, ((u4 & ~u16) | (hr & ~hr4) | hd | h0) >> 1);
+            spread<2>(acc, (u16 | (hl & ~hl4) | (hr & ~hr4) | (hd & ~hd4) | h0) >> 1);
+            spread<3>(acc, (hl4 | hr4 | hd4 | h0) >> 1);
+            spread<4>(acc, ((d2 & ~d4) | (d8 & ~d16) | (cx & ~cx4) | (cy & ~cy4) | cm4 | cy16 | out | root) >> 1);
+            spread<5>(acc, ((d4 & ~d16) | cm | (cy & ~cy4) | cx4 | root) >> 1);
+            spread<6>(acc, (d16 | (cx & ~cx4) | (cm & ~cm4) | cy | root) >> 1);
+            spread<7>(acc, (dg | out | cx4 | cm4 | cy4 | root) >> 1);
             const uint64_t at = uint64_t(it.coff) + uint64_t(code_at2(it, y0, x));
             if (own_x && CP_IN(at + 31u, o.n_code, o.ctr)) {
                 uint4* dst = reinterpret_cast<uint4*>(o.code + at);

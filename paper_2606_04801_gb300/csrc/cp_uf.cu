@@ -112,21 +112,23 @@ __device__ __forceinline__ void cross_prune(const ItemTable& tab, const UfParams
 // separate, non-cooperative launch: warps take 32 survivors at a time from a
 // counter, so a warp held up by a long path delays no other warp.
 constexpr int kFT = 256;
+constexpr int kFC = 6;  // CTAs per SM: 512^3 blurred 106 us, 119 with five (seven and eight: slower too)
 
 __device__ __forceinline__ Forest forest_of(const RootArgs& r) { return Forest{r.uf, r.code, r.n_nodes, r.n_code, r.dual}; }
 
 // Survivor i of the list r (one lane): its endpoints' root ids and its position.
+template <int kDim = 0>
 __device__ __forceinline__ void place_walk(const ItemTable& tab, const RootArgs& r, uint32_t i, uint32_t& hops) {
     uint64_t key = r.keys[i];
     if (r.dual) key = ~key;
     uint32_t ra, rb;
-    if (!walk_roots(tab, forest_of(r), r.ctr, key, ra, rb, hops)) set_status(r.ctr, kStTimeout);
+    if (!walk_roots<kDim>(tab, forest_of(r), r.ctr, key, ra, rb, hops)) set_status(r.ctr, kStTimeout);
     __stcg(r.ra + i, ra);
     __stcg(r.rb + i, rb);
     if (r.pos) __stcg(r.pos + i, i);
 }
 
-__global__ void __launch_bounds__(kFT) k_roots(const __grid_constant__ RootArgs r) {
+__global__ void __launch_bounds__(kFT, kFC) k_roots(const __grid_constant__ RootArgs r) {
     Counters* ctr = r.ctr;
     if (ld_acquire_u32(&ctr->status) & (kStTimeout | kStNonfinite)) return;
     const uint32_t n = min(*r.d_n, r.cap);
@@ -148,7 +150,8 @@ __global__ void __launch_bounds__(kFT) k_roots(const __grid_constant__ RootArgs 
 // survivors at a time from one counter running over the H0 list and then the
 // dual list, so the long walks of one list overlap those of the other instead
 // of following them.  Each lane walks its own list's forest.
-__global__ void __launch_bounds__(kFT) k_roots2(const __grid_constant__ RootArgs r0,
+template <int kDim>
+__global__ void __launch_bounds__(kFT, kFC) k_roots2(const __grid_constant__ RootArgs r0,
                                                 const __grid_constant__ RootArgs r1) {
     Counters* ctr = r0.ctr;
     wait_for_previous();
@@ -164,7 +167,7 @@ __global__ void __launch_bounds__(kFT) k_roots2(const __grid_constant__ RootArgs
     for (uint32_t base = (blockIdx.x * (kFT / 32) + (threadIdx.x >> 5)) * 32u; base < n;) {
         const uint32_t g = base + lane;
         const int l = g >= n0 ? 1 : 0;  // this lane's list
-        if (g < n) place_walk(r0.tab, l ? r1 : r0, l ? g - n0 : g, hops[l]);
+        if (g < n) place_walk<kDim>(r0.tab, l ? r1 : r0, l ? g - n0 : g, hops[l]);
         __syncwarp();
         if (lane == 0) base = atomicAdd(&ctr->find_ctr, 32u) + warps * 32u;
         base = __shfl_sync(0xFFFFFFFFu, base, 0);
@@ -618,7 +621,8 @@ cudaError_t launch_roots2(const RootArgs& r0, const RootArgs& r1, cudaStream_t s
     // (find_ctr is zero: the call's own memset, and no other walk before this)
     // (overlapped for small images only: in place of the 2D pass's shared memory
     // the walks want L1; 2048^2 noise 139 us overlapped, 89 not)
-    return launch_after(r0.tab.n3d == 0 && r0.tab.tiles2d <= 1216, k_roots2, find_blocks(), kFT, 0, s, r0, r1);
+    const auto kernel = r0.tab.n3d == 0 ? k_roots2<2> : (r0.tab.n2d == 0 ? k_roots2<3> : k_roots2<0>);
+    return launch_after(r0.tab.n3d == 0 && r0.tab.tiles2d <= 1216, kernel, find_blocks(), kFT, 0, s, r0, r1);
 }
 
 cudaError_t launch_place_roots(const RootArgs& r, cudaStream_t s) {

@@ -14,10 +14,16 @@
 //
 // 2D items: 30 rows of a column at a time in one 32-byte sector (code_at2: a
 // column of a pruning tile), bits 0-3 the H0 link (0..4: up by 1 << d rows, all
-// of whose vertices but the last link up; 5, 6, 7: left, right, down; 14: a
-// root, 15: the frame as above), bits 4-7 the dual link of the top cell with
-// its smallest corner there (0..4: +y by 1 << d, likewise; 5..8: +x, -x, -y,
-// both; 9: the outside, 15: a root).  Runs end where the tile does.
+// of whose vertices but the last link up; 5, 6, 7: left, right, down by one, 8,
+// 9, 10: by four, 11: down by 16, likewise; 14: a root, 15: the frame as above),
+// bits 4-7 the dual link of the top cell with its smallest corner there (0..4:
+// +y by 1 << d, likewise; 5..8: +x, -x, -y, both; 9: the outside; 10, 11, 12:
+// +x, -x, -y by four, 13: -y by 16, likewise; 15: a root).  Runs end where the
+// tile does.  The runs shorten long straight descents: with runs of links up
+// and +y alone, the walks of 2048^2 straight valleys took 337 us (falling along
+// +y) and 670 us (along x) and take 91 and 284; ordinary fields' differ little
+// (2048^2 noise 89 -> 84 us, 4096^2 blurred 46 -> 39), and the pruning pass pays
+// 2 us at 4096^2 for them.
 #pragma once
 #include "cp_common.cuh"
 
@@ -50,16 +56,19 @@ __host__ __device__ __forceinline__ uint32_t code_at3(const Item& it, int z, int
     return ((uint32_t(z) * uint32_t(it.bands) + b) * uint32_t(it.W) + uint32_t(x)) * 32u + (uint32_t(y) - b * uint32_t(kBand3));
 }
 
-// Offset of the 2D link with code field d (H0: 0..7; dual: 0..8).
+// Offset of the 2D link with code field d (H0: 0..11; dual: 0..8, 10..13), a
+// signed byte for each of the 16 fields (0: no step).
+struct Offsets2 {
+    uint32_t y[4], x[4];
+};
+__host__ __device__ __forceinline__ Offsets2 offsets2(int dual) {
+    return dual ? Offsets2{{0x08040201u, 0xFF000010u, 0x000000FFu, 0x0000F0FCu}, {0u, 0x00FF0100u, 0xFC0400FFu, 0u}}
+                : Offsets2{{0xF8FCFEFFu, 0x010000F0u, 0x10040000u, 0u}, {0u, 0x0001FF00u, 0x000004FCu, 0u}};
+}
 __host__ __device__ __forceinline__ void link_offset2(int dual, uint32_t d, int& dy, int& dx) {
-    const int run = d < 5u ? 1 << d : 0;
-    if (!dual) {
-        dy = d == 7u ? 1 : -run;
-        dx = d == 5u ? -1 : (d == 6u ? 1 : 0);
-    } else {
-        dy = d >= 7u ? -1 : run;
-        dx = d == 5u ? 1 : (d == 6u || d == 8u ? -1 : 0);
-    }
+    const Offsets2 o = offsets2(dual);
+    dy = int8_t(o.y[d >> 2] >> (8u * (d & 3u)));
+    dx = int8_t(o.x[d >> 2] >> (8u * (d & 3u)));
 }
 
 #ifdef __CUDACC__
@@ -117,22 +126,27 @@ struct Step3 {
     __device__ __forceinline__ bool frame(uint32_t d) const { return mask == 7u && d == 7u; }
 };
 struct Step2 {
-    uint32_t shift, last, band, far;  // far: what codes 5 .. 8 add, a signed byte each
-    int32_t sign;
+    uint32_t shift, band, end;  // end: the codes that are no step
+    Offsets2 o;
     __device__ __forceinline__ Step2(int dual, int32_t W)
-        : shift(dual ? 4u : 0u), last(dual ? 9u : 8u), band(32u * uint32_t(W)), far(dual ? 0xDFFFE020u : 0x000120E0u),
-          sign(dual ? 1 : -1) {}
+        : shift(dual ? 4u : 0u), band(32u * uint32_t(W)), end(dual ? 0x8200u : 0xC000u), o(offsets2(dual)) {}
     __device__ __forceinline__ uint32_t field(uint32_t c) const { return (c >> shift) & 15u; }
+    // Byte d of the 16 in t, with its sign.
+    static __device__ __forceinline__ uint32_t pick(const uint32_t (&t)[4], uint32_t d) {
+        const uint32_t sel = (d & 7u) * 0x1111u | 0x8880u;
+        uint32_t v;
+        asm("prmt.b32 %0, %1, %2, %3;" : "=r"(v) : "r"(d < 8u ? t[0] : t[2]), "r"(d < 8u ? t[1] : t[3]), "r"(sel));
+        return v;
+    }
     __device__ __forceinline__ uint32_t next(uint32_t at, uint32_t d) const {
-        const int32_t step = d < 5u ? sign * (1 << d) : int32_t(far << (24u - 8u * ((d - 5u) & 3u))) >> 24;
-        at += d < last ? uint32_t(step) : 0u;
+        at += pick(o.x, d) * 32u + pick(o.y, d);
         const uint32_t r = at & 31u;  // 30: one row below the tile, 31: one above it (and a column to the left)
         if (r >= uint32_t(kTile2)) at += r == 31u ? uint32_t(kTile2) - band : band - uint32_t(kTile2);
         return at;
     }
-    __device__ __forceinline__ bool ends(uint32_t d) const { return d >= last; }
-    __device__ __forceinline__ bool outside(uint32_t d) const { return last == 9u && d == 9u; }
-    __device__ __forceinline__ bool frame(uint32_t d) const { return last == 8u && d == 15u; }
+    __device__ __forceinline__ bool ends(uint32_t d) const { return (end >> d) & 1u; }
+    __device__ __forceinline__ bool outside(uint32_t d) const { return end == 0x8200u && d == 9u; }
+    __device__ __forceinline__ bool frame(uint32_t d) const { return end == 0xC000u && d == 15u; }
 };
 
 // Both paths in lockstep until neither has a link to follow.  False: the
@@ -190,6 +204,9 @@ __device__ __forceinline__ uint32_t root_id3(const Forest& f, const Item& it, in
 // Root ids of the two endpoints of the survivor with key k (the key itself,
 // not its complement), both paths in lockstep (two loads in flight); hops
 // counts the steps.  False: a bounded walk gave up (a corrupted forest).
+// kDim: the items are all 2D or all 3D (0: both kinds; in one kernel for all,
+// the 3D walks take 2 to 5% longer).
+template <int kDim = 0>
 __device__ __forceinline__ bool walk_roots(const ItemTable& tab, const Forest& f, Counters* ctr, uint64_t k,
                                            uint32_t& ra, uint32_t& rb, uint32_t& hops) {
     const uint32_t vg = key_vertex(k);
@@ -200,7 +217,7 @@ __device__ __forceinline__ bool walk_roots(const ItemTable& tab, const Forest& f
     const uint32_t local = vg - uint32_t(it.voff), W = uint32_t(it.W), H = uint32_t(it.H);
     const uint32_t row = local / W;
     const int x = int(local - row * W);
-    if (it.ndim == 3) {
+    if (kDim == 3 || (kDim == 0 && it.ndim == 3)) {
         const int y = int(row % H), z = int(row / H);
         Path a = {0, false}, b = a;
         if (!f.dual) {
