@@ -472,8 +472,9 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
     // variant and cross-pruning of images need the sorted lists and the rounds
     const bool joint = P.tab.n2d == 0 || !P.tab.cross2d;
     const bool tree = joint && P.slabs == 0 && !P.boruvka;
-    TreeNode* node0 = tree ? at<TreeNode>(ws, P.o_node0) : nullptr;
-    TreeNode* nodet = tree ? at<TreeNode>(ws, P.o_nodet) : nullptr;
+    // (the pruning pass alone leaves the roots' ages, whatever takes them in a call)
+    TreeNode* node0 = tree && !prune_only ? at<TreeNode>(ws, P.o_node0) : nullptr;
+    TreeNode* nodet = tree && !prune_only ? at<TreeNode>(ws, P.o_nodet) : nullptr;
     CP_TRY(launch_init(P.tab, ctr, P.zero_bytes, uft, aget, rest, nodet, s));
     mark(0, s);
     PruneOuts po;

@@ -142,3 +142,33 @@ def test_prune_stage_3d_tma_planes(cp, seed):
     img = rng.random((10, 12, 41), dtype=np.float32)
     _check(cp, lib, img)
     assert _check.tma_tasks == 0
+
+
+@pytest.mark.parametrize("shape", [(2, 2), (37, 29), (64, 33), (2, 3, 2), (9, 12, 40), (7, 30, 13)])
+def test_prune_stage_root_ages(cp, shape):
+    """The ages of the roots, by root id, at the two offsets of the layout: the
+    vertex's key (H0), that of the dying top cell's largest corner (dual), all
+    ones for the outside."""
+    lib = cp.load()
+    nd = len(shape)
+    img = np.random.default_rng(17).integers(0, 50, shape).astype(np.float32)
+    t = torch.from_numpy(img).cuda()
+    ptrs = (ctypes.c_void_p * 1)(t.data_ptr())
+    ndims = (ctypes.c_int32 * 1)(nd)
+    dims = (ctypes.c_int64 * 3)(*(((1,) + shape) if nd == 2 else shape))
+    off = (ctypes.c_int64 * 13)()
+    assert lib.cubical_persistence_debug_layout(1, ndims, dims, 0, off, 13) == 13
+    ws_bytes = lib.cubical_persistence_batched_workspace_size(1, ndims, dims, 0)
+    ws = torch.full((ws_bytes,), 0x5A, dtype=torch.uint8, device="cuda")
+    assert lib.cubical_persistence_debug_prune(1, ptrs, ndims, dims, ctypes.c_void_p(ws.data_ptr()), ws_bytes, 0, None) == 0
+    torch.cuda.synchronize()
+    w = ws.cpu().numpy()
+    n_r0, n_rt = (int(v) for v in w[off[0] : off[0] + 20].view(np.uint32)[3:5])
+    ref = Pruned(lib, img)
+    for forest, size, ages, n, want in (
+            (off[1], off[7], off[5], n_r0, {v: ref.key(ref.K(v), 0, v) for v, p in enumerate(ref.par0) if p == v}),
+            (off[2], off[8], off[6], n_rt, {**{c: ref.key(kv, b, kv[1]) for c, (kv, b) in ref.tage.items()}, ref.OUT: 2 ** 64 - 1})):
+        words = w[forest : forest + 4 * size].view(np.uint32)
+        age = w[ages : ages + 8 * n].view(np.uint64)
+        got = {int(r): int(age[int(words[r]) & ~TAG]) for r in np.flatnonzero(words & TAG)}
+        assert got == want
