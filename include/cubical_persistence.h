@@ -476,6 +476,15 @@ int cubical_persistence_debug_layout(int n_items, const int32_t *ndims, const in
                                      int64_t *h_offsets, int cap);
 
 /*
+ * The lookup + pruning pass of a batched call and nothing after it (arguments
+ * as for cubical_persistence_debug_prune, whose forests take a second pass
+ * over every code): what a tuner of that pass times.  Enqueued on `stream`;
+ * leaves nothing to read.
+ */
+int cubical_persistence_prune_pass(int n_items, const float *const *h_images, const int32_t *ndims, const int64_t *dims,
+                                   void *d_workspace, size_t ws_bytes, int64_t max_survivors, void *stream);
+
+/*
  * Failure-path test: a kernel waits, through the library's bounded-wait
  * routine (every device-side wait gives up the same way, after 2 s in
  * production), on a workspace word that nothing sets, and gives up after

@@ -2,7 +2,7 @@
 
 Picks the 3D task depth (planes per task) and the number of 3D pruning CTAs
 per SM by timing the lookup + pruning pass alone
-(cubical_persistence_debug_prune) on the given inputs; then the union-find
+(cubical_persistence_prune_pass) on the given inputs; then the union-find
 design (reservation rounds over every survivor, or Borůvka's spanning forest
 first and the rounds over its edges) by timing whole forward calls with
 each.  Which design is faster depends on the data (i.i.d. noise leaves many
@@ -83,7 +83,7 @@ def _time_prune(inputs: Sequence[torch.Tensor], repeats: int) -> float:
     wp = ctypes.c_void_p(ws.data_ptr())
 
     def once():
-        rc = lib.cubical_persistence_debug_prune(k, ptrs, ndims, dims, wp, wsb, 0, sp)
+        rc = lib.cubical_persistence_prune_pass(k, ptrs, ndims, dims, wp, wsb, 0, sp)
         if rc != 0:
             raise _lib.CpError(rc, "prune")
 

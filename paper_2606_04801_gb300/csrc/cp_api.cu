@@ -434,6 +434,11 @@ struct TMode {
     const uint32_t* bad;
 };
 
+// How far a call goes: to the pairs; to the forests, keys and ages of the
+// pruning pass (stage tests); to the end of the pruning pass as the calls run
+// it (timing).
+enum Until { kPairs, kStage, kPrune };
+
 // How the output launch's grid barriers wait (OrderArgs).
 struct OrderWait {
     uint32_t absent = 0;
@@ -441,7 +446,7 @@ struct OrderWait {
 };
 
 int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, int64_t* d_out_count, void* ws,
-        size_t ws_bytes, cudaStream_t s, bool prune_only = false, const TMode* tm = nullptr, OrderWait wait = {}) {
+        size_t ws_bytes, cudaStream_t s, Until until = kPairs, const TMode* tm = nullptr, OrderWait wait = {}) {
     if (!ws || (!d_out && capacity > 0) || capacity < 0) return CP_ERR_ARG;
     if (ws_bytes < P.bytes + kWsSlack) return CP_ERR_ARG;
     int rc = ensure_device_tables();
@@ -472,9 +477,9 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
     // variant and cross-pruning of images need the sorted lists and the rounds
     const bool joint = P.tab.n2d == 0 || !P.tab.cross2d;
     const bool tree = joint && P.slabs == 0 && !P.boruvka;
-    // (the pruning pass alone leaves the roots' ages, whatever takes them in a call)
-    TreeNode* node0 = tree && !prune_only ? at<TreeNode>(ws, P.o_node0) : nullptr;
-    TreeNode* nodet = tree && !prune_only ? at<TreeNode>(ws, P.o_nodet) : nullptr;
+    // (the stage test reads the roots' ages, whatever takes them in a call)
+    TreeNode* node0 = tree && until != kStage ? at<TreeNode>(ws, P.o_node0) : nullptr;
+    TreeNode* nodet = tree && until != kStage ? at<TreeNode>(ws, P.o_nodet) : nullptr;
     CP_TRY(launch_init(P.tab, ctr, P.zero_bytes, uft, aget, rest, nodet, s));
     mark(0, s);
     PruneOuts po;
@@ -496,10 +501,10 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
     po.ctr = ctr;
     po.n_uf0 = uint32_t(P.ntot);
     po.n_uft = uint32_t(P.ttot);
-    if (prune_only) {
+    if (until != kPairs) {
         CP_TRY(launch_prune(P.tab, po, P.tma, s));
         mark(1, s);
-        CP_TRY(launch_expand(P.tab, po, s));
+        if (until == kStage) CP_TRY(launch_expand(P.tab, po, s));
         return CP_OK;
     }
 
@@ -980,7 +985,7 @@ int t_run(int n_items, const float* const* h_images, const int32_t* ndims, const
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (launch_t_build(tm.items, bad, s) != cudaSuccess) return CP_ERR_CUDA;
     tm.bad = bad;
-    return run(P, d_out, capacity, h_out_count, d_out_count, base, v_bytes + kWsSlack, s, false, &tm);
+    return run(P, d_out, capacity, h_out_count, d_out_count, base, v_bytes + kWsSlack, s, kPairs, &tm);
 }
 
 int t_single(int ndim, const float* d_image, const int64_t* dims, cp_pair* d_out, int64_t capacity,
@@ -1189,7 +1194,16 @@ int cubical_persistence_debug_prune(int n_items, const float* const* h_images, c
     Plan P;
     int rc = make_plan(n_items, ndims, dims, h_images, max_survivors, P);
     if (rc != CP_OK) return rc;
-    return run(P, nullptr, 0, nullptr, nullptr, d_workspace, ws_bytes, static_cast<cudaStream_t>(stream), true);
+    return run(P, nullptr, 0, nullptr, nullptr, d_workspace, ws_bytes, static_cast<cudaStream_t>(stream), kStage);
+}
+
+int cubical_persistence_prune_pass(int n_items, const float* const* h_images, const int32_t* ndims, const int64_t* dims,
+                                   void* d_workspace, size_t ws_bytes, int64_t max_survivors, void* stream) {
+    if (!h_images) return CP_ERR_ARG;
+    Plan P;
+    int rc = make_plan(n_items, ndims, dims, h_images, max_survivors, P);
+    if (rc != CP_OK) return rc;
+    return run(P, nullptr, 0, nullptr, nullptr, d_workspace, ws_bytes, static_cast<cudaStream_t>(stream), kPrune);
 }
 
 int cubical_persistence_debug_layout(int n_items, const int32_t* ndims, const int64_t* dims, int64_t max_survivors,
@@ -1345,7 +1359,7 @@ int cubical_persistence_debug_order_timeout(int ndim, const float* d_image, cons
     const int rc = make_plan(1, &nd, d3, &d_image, 0, P);
     if (rc != CP_OK) return rc;
     return run(P, d_out_pairs, capacity, h_out_count, d_out_count, d_workspace, ws_bytes, static_cast<cudaStream_t>(stream),
-               false, nullptr, OrderWait{1, uint64_t(limit_us) * 1000u});
+               kPairs, nullptr, OrderWait{1, uint64_t(limit_us) * 1000u});
 }
 
 int cp_set_tuning(int key, int value) {
