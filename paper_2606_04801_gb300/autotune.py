@@ -8,7 +8,9 @@ first and the rounds over its edges) by timing whole forward calls with
 each.  Which design is faster depends on the data (i.i.d. noise leaves many
 survivors that close cycles, which Borůvka drops early; smooth fields leave
 few), so the cache key holds the survivor fraction's power of two besides
-the shape bucket.  The winners are cached per GPU and key in a JSON file
+the shape bucket.  It also holds a hash of the library's sources: what was
+fastest with other kernels says nothing about these, so a decision made for
+them is not applied but made again.  The winners are cached per GPU and key in a JSON file
 (default ~/.cache/cp_gb300/autotune.json, or $CP_AUTOTUNE_CACHE).  The pairs
 never depend on these settings; only the time does.
 
@@ -18,6 +20,8 @@ never depend on these settings; only the time does.
 from __future__ import annotations
 
 import ctypes
+import functools
+import hashlib
 import json
 import os
 from typing import Optional, Sequence
@@ -25,7 +29,7 @@ from typing import Optional, Sequence
 import numpy as np
 import torch
 
-from . import _lib
+from . import _lib, build
 
 ZCHUNK_3D, CTAS_PER_SM, ROWS_2D, UF_VARIANT = 1, 2, 3, 7
 CAND_ZCHUNK = (16, 32, 64, 128, 256)
@@ -34,6 +38,18 @@ CAND_CTAS = (0, 2, 3)
 
 def _cache_path() -> str:
     return os.environ.get("CP_AUTOTUNE_CACHE", os.path.join(os.path.expanduser("~"), ".cache", "cp_gb300", "autotune.json"))
+
+
+@functools.lru_cache(maxsize=None)
+def kernels() -> str:
+    """Hash of the sources that the library is built from."""
+    h = hashlib.sha256()
+    for name in sorted(build.CU + build.CPP + build.HEADERS):
+        path = os.path.join(build.CSRC, name)
+        if os.path.exists(path):
+            with open(path, "rb") as fh:
+                h.update(fh.read())
+    return h.hexdigest()[:12]
 
 
 def bucket(shapes: Sequence[Sequence[int]]) -> str:
@@ -193,7 +209,7 @@ def autotune(inputs: Sequence[torch.Tensor], cache: Optional[str] = None, retune
     dev = inputs[0].device
     frac = survivor_fraction(inputs)
     sbin = int(np.floor(np.log2(max(frac, 1e-9))))
-    key = f"{torch.cuda.get_device_name(dev)}|{bucket([tuple(t.shape) for t in inputs])}|surv:{sbin}"
+    key = f"{torch.cuda.get_device_name(dev)}|{bucket([tuple(t.shape) for t in inputs])}|surv:{sbin}|lib:{kernels()}"
     table = {}
     if os.path.exists(path):
         try:
