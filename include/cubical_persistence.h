@@ -504,6 +504,13 @@ int cubical_persistence_debug_wait_timeout(void *d_workspace, size_t ws_bytes, i
 int cubical_persistence_debug_order_timeout(int ndim, const float *d_image, const int64_t *dims, cp_pair *d_out_pairs,
                                             int64_t capacity, int64_t *h_out_count, int64_t *d_out_count,
                                             void *d_workspace, size_t ws_bytes, int64_t limit_us, void *stream);
+/*
+ * A forward call whose output launch has at most max_blocks (>= 1) thread
+ * blocks, as on a device or partition with that many SMs.  Same pairs.
+ */
+int cubical_persistence_debug_order_blocks(int ndim, const float *d_image, const int64_t *dims, cp_pair *d_out_pairs,
+                                           int64_t capacity, int64_t *h_out_count, int64_t *d_out_count,
+                                           void *d_workspace, size_t ws_bytes, int max_blocks, void *stream);
 
 /*
  * Tuning of the pruning pass (process-wide; read by the following calls;

@@ -111,6 +111,10 @@ _SIGS = {
         [_P, _I64, _P, ctypes.c_float, _P, _P, _P, _I64, _P, ctypes.c_size_t, _P],
     ),
     "cubical_persistence_load_items": (ctypes.c_int, [ctypes.c_int, _P, _P, _P, _P]),
+    "cubical_persistence_debug_order_blocks": (
+        ctypes.c_int,
+        [ctypes.c_int, _P, _P, _P, _I64, _P, _P, _P, ctypes.c_size_t, ctypes.c_int, _P],
+    ),
     "cubical_persistence_backward_noalloc_max_pixels": (ctypes.c_int64, []),
     "cubical_persistence_backward_noalloc": (ctypes.c_int, [_P, _I64, _P, _P, _P, _P, _I64, _P]),
     "cubical_persistence_uf_trace": (ctypes.c_int, [_P, ctypes.c_int, _P, _P, ctypes.c_int, _P]),

@@ -439,14 +439,16 @@ struct TMode {
 // it (timing).
 enum Until { kPairs, kStage, kPrune };
 
-// How the output launch's grid barriers wait (OrderArgs).
-struct OrderWait {
+// How the output launch runs: its grid barriers' waits (OrderArgs), its blocks
+// (launch_order).
+struct OrderLaunch {
     uint32_t absent = 0;
     uint64_t limit_ns = kWaitLimitNs;
+    int max_ctas = 0;
 };
 
 int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, int64_t* d_out_count, void* ws,
-        size_t ws_bytes, cudaStream_t s, Until until = kPairs, const TMode* tm = nullptr, OrderWait wait = {}) {
+        size_t ws_bytes, cudaStream_t s, Until until = kPairs, const TMode* tm = nullptr, OrderLaunch ol = {}) {
     if (!ws || (!d_out && capacity > 0) || capacity < 0) return CP_ERR_ARG;
     if (ws_bytes < P.bytes + kWsSlack) return CP_ERR_ARG;
     int rc = ensure_device_tables();
@@ -888,10 +890,10 @@ int run(const Plan& P, cp_pair* d_out, int64_t capacity, int64_t* h_out_count, i
     oa.out_cap = capacity;
     oa.out16 = (reinterpret_cast<uintptr_t>(d_out) & 15u) == 0 ? 1 : 0;
     oa.d_out_count = d_out_count;
-    oa.absent = wait.absent;
-    oa.limit_ns = wait.limit_ns;
+    oa.absent = ol.absent;
+    oa.limit_ns = ol.limit_ns;
     oa.ctr = ctr;
-    CP_TRY(launch_order(oa, s));
+    CP_TRY(launch_order(oa, ol.max_ctas, s));
     mark(6, s);
 #undef CP_TRY
     if (h_out_count) {
@@ -1359,7 +1361,22 @@ int cubical_persistence_debug_order_timeout(int ndim, const float* d_image, cons
     const int rc = make_plan(1, &nd, d3, &d_image, 0, P);
     if (rc != CP_OK) return rc;
     return run(P, d_out_pairs, capacity, h_out_count, d_out_count, d_workspace, ws_bytes, static_cast<cudaStream_t>(stream),
-               kPairs, nullptr, OrderWait{1, uint64_t(limit_us) * 1000u});
+               kPairs, nullptr, OrderLaunch{1, uint64_t(limit_us) * 1000u});
+}
+
+int cubical_persistence_debug_order_blocks(int ndim, const float* d_image, const int64_t* dims, cp_pair* d_out_pairs,
+                                           int64_t capacity, int64_t* h_out_count, int64_t* d_out_count,
+                                           void* d_workspace, size_t ws_bytes, int max_blocks, void* stream) {
+    if ((ndim != 2 && ndim != 3) || !d_image || !dims || max_blocks < 1) return CP_ERR_ARG;
+    int32_t nd = ndim;
+    int64_t d3[3] = {ndim == 3 ? dims[0] : 1, dims[ndim - 2], dims[ndim - 1]};
+    Plan P;
+    const int rc = make_plan(1, &nd, d3, &d_image, 0, P);
+    if (rc != CP_OK) return rc;
+    OrderLaunch ol;
+    ol.max_ctas = max_blocks;
+    return run(P, d_out_pairs, capacity, h_out_count, d_out_count, d_workspace, ws_bytes, static_cast<cudaStream_t>(stream),
+               kPairs, nullptr, ol);
 }
 
 int cp_set_tuning(int key, int value) {

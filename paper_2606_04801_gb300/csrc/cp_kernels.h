@@ -391,7 +391,8 @@ struct OrderArgs {
 };
 void plan_order(uint64_t places, int* shift, int* chunk_shift, uint32_t* buckets);
 size_t order_chunks();
-cudaError_t launch_order(const OrderArgs& a, cudaStream_t s);
+// max_ctas: thread blocks at most (0: one per SM).
+cudaError_t launch_order(const OrderArgs& a, int max_ctas, cudaStream_t s);
 cudaError_t launch_backward(const cp_pair* pairs, int64_t n, const float* gb, const float* gd, const int64_t* offs,
                             double* acc, float* grad, int64_t n_pixels, cudaStream_t s);
 

@@ -23,7 +23,7 @@ namespace cp {
 namespace {
 
 constexpr int kOT = 1024;        // one CTA per SM: the grid barriers cost least (512 x 2: the same, 256 x 4: slower)
-constexpr int kMaxChunks = 128;  // CTAs that scan the buckets (at most kOT, and the grid)
+constexpr int kMaxChunks = 128;  // chunks of buckets, each scanned by a CTA (at most kOT)
 
 // The T pair of a V pair of the dual image J (see cp_tfilt.cu): doubled
 // coordinate a of J becomes 2n+1-a of the T grid, vertex coordinate c of J
@@ -190,13 +190,13 @@ __global__ void __launch_bounds__(kOT) k_order(const __grid_constant__ OrderArgs
     }
     if (!order_barrier(a, epoch)) return;
     // ---- where each bucket starts within its chunk of 2^chunk_shift buckets
-    // (a chunk per CTA), and the chunks' totals
+    // (a chunk per CTA at a time), and the chunks' totals
     if (threadIdx.x == 0) sh_n = min(ld_acquire_u32(&ctr->n_pairs), a.pair_cap);
     __syncthreads();
     const uint32_t n = sh_n;
-    const uint32_t nchunks = (a.buckets + (1u << a.chunk_shift) - 1u) >> a.chunk_shift;  // <= kMaxChunks, the grid
-    if (blockIdx.x < nchunks) {
-        const uint32_t first = blockIdx.x << a.chunk_shift, last = min(a.buckets, first + (1u << a.chunk_shift));
+    const uint32_t nchunks = (a.buckets + (1u << a.chunk_shift) - 1u) >> a.chunk_shift;  // <= kMaxChunks
+    for (uint32_t k = blockIdx.x; k < nchunks; k += gridDim.x) {
+        const uint32_t first = k << a.chunk_shift, last = min(a.buckets, first + (1u << a.chunk_shift));
         uint32_t run = 0;
         // four buckets per thread and turn (the arrays are padded to a multiple of 4)
         for (uint32_t b0 = first; b0 < last; b0 += 4 * kOT) {
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(kOT) k_order(const __grid_constant__ OrderArgs
             run += sh_warp[kOT / 32];
             __syncthreads();
         }
-        if (threadIdx.x == 0) __stcg(a.chunk + blockIdx.x, run);
+        if (threadIdx.x == 0) __stcg(a.chunk + k, run);
     }
     if (!order_barrier(a, epoch)) return;
     {
@@ -284,15 +284,15 @@ void plan_order(uint64_t places, int* shift, int* chunk_shift, uint32_t* buckets
 
 size_t order_chunks() { return kMaxChunks; }
 
-cudaError_t launch_order(const OrderArgs& a, cudaStream_t s) {
+cudaError_t launch_order(const OrderArgs& a, int max_ctas, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     const int blocks = device_cached(kCacheOrder, [] {
         int per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_order, kOT, 0);
-        return per_sm > 0 && device_sm_count() >= kMaxChunks ? device_sm_count() : -1;
+        return per_sm > 0 ? device_sm_count() : -1;
     });
     if (blocks <= 0) return cudaErrorLaunchOutOfResources;
-    cfg.gridDim = dim3(unsigned(blocks));
+    cfg.gridDim = dim3(unsigned(max_ctas > 0 && max_ctas < blocks ? max_ctas : blocks));
     cfg.blockDim = dim3(kOT);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
