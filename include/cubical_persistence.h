@@ -529,13 +529,14 @@ int cubical_persistence_debug_order_blocks(int ndim, const float *d_image, const
  *                        the table cannot settle, which the dual union-find
  *                        then finds closing dual cycles.  Same pairs.
  *   CP_TUNE_H1_BUDGET_MS wall-clock budget in milliseconds of the cross-star
- *                        reduction rounds of the _full calls (0 .. 3,600,000;
- *                        default 30,000).  Those rounds (and, with the same
- *                        budget, the rewriting of the columns before them) run in one
- *                        non-preemptible cooperative launch; once the budget
- *                        is spent, every block leaves at the next round
- *                        boundary and the call returns CP_ERR_TIMEOUT (no
- *                        H1 pairs).  0 stops after the first round.
+ *                        reduction rounds of the _full calls and the rewriting
+ *                        of the columns before them, together (0 .. 3,600,000;
+ *                        default 30,000).  Those run in non-preemptible
+ *                        launches; once the budget is spent, the rewriting
+ *                        leaves the columns as they are, every block of the
+ *                        rounds leaves at the next round boundary and the call
+ *                        returns CP_ERR_TIMEOUT (no H1 pairs).  0 stops after
+ *                        the first round.
  *   CP_TUNE_H1_SOLO      the cross-star rounds: once at most this many
  *                        columns enter a round, the first CTA runs the rounds
  *                        alone while the others wait, until more than twice

@@ -433,7 +433,7 @@ struct ReduceArgs {
     ItemTable tab;
     H1Bufs b;
     Counters* ctr;
-    uint64_t budget_ns;  // wall-clock budget of the rounds
+    uint64_t budget_ns;  // wall-clock budget, from H1Ctl::t_begin on
     uint32_t solo_cols;  // see kSoloDefault (0: never alone)
 };
 
@@ -948,7 +948,7 @@ struct FlowArgs {
     ItemTable tab;
     H1Bufs b;
     Counters* ctr;
-    uint64_t budget_ns;
+    uint64_t budget_ns;  // wall-clock budget of the replacement and the rounds together
 };
 
 // The warp takes n entries of the replacement's part of the pool; ~0: none
@@ -961,7 +961,7 @@ __device__ uint64_t pool_take(const H1Bufs& b, uint64_t n) {
     return at + n <= flow_room(b) ? at : ~0ull;
 }
 
-// One column; false: left as it is (no room).
+// One column; false: left as it is (no room, or the budget is spent).
 template <class W>
 __device__ bool flow_column(const FlowArgs& a, W& s, uint32_t q, uint64_t& scratch, uint32_t& scratch_cap,
                             uint64_t t_start) {
@@ -975,10 +975,8 @@ __device__ bool flow_column(const FlowArgs& a, W& s, uint32_t q, uint64_t& scrat
     uint32_t which = 0, nout = 0, batches = 0;
     bool in_smem = true, changed = false;
     while (n > 0) {
-        if ((batches++ & 15u) == 0 && global_timer_ns() - t_start > a.budget_ns) {
-            if (lane == 0) set_status(a.ctr, kStTimeout);
-            return false;
-        }
+        // over the budget: left to the rounds, which stop after the next one
+        if ((batches++ & 15u) == 0 && global_timer_ns() - t_start > a.budget_ns) return false;
         // ---- the first entries and their owners
         const uint32_t take = min(32u, n);
         const uint64_t key = lane < take ? (in_smem ? cur[lane] : __ldcg(cur + lane)) : 0ull;
@@ -1131,7 +1129,9 @@ __global__ void __launch_bounds__(kFW * 32, W::kBig ? 1 : 3) k_h1_flow(const __g
     const uint32_t n = W::kBig ? b.ctl->flow_left : nl;
     const uint32_t* list = W::kBig ? b.list[0] : b.list0;
     uint32_t* next = W::kBig ? &b.ctl->flow_next2 : &b.ctl->flow_next;
-    const uint64_t t_start = global_timer_ns();
+    // the budget's clock: the first launch starts it, all later ones read it
+    const uint64_t t_start = W::kBig ? b.ctl->t_begin : global_timer_ns();
+    if (!W::kBig && blockIdx.x == 0 && threadIdx.x == 0) b.ctl->t_begin = t_start;
     uint64_t scratch = 0;
     uint32_t scratch_cap = 0;
     for (;;) {
@@ -1164,8 +1164,8 @@ __global__ void __launch_bounds__(kRT) k_h1_reduce(const __grid_constant__ Reduc
     __shared__ MergeJob sh_jobs[kJobs];           // the first CTA alone: the round's long merges
     __shared__ uint32_t sh_njobs, sh_scan[35];
     uint32_t epoch = 0;
-    const uint64_t t_start = global_timer_ns();  // read by thread 0 of CTA 0 only
-    uint64_t t_mode = t_start;   // start of the current mode (thread 0 of CTA 0)
+    const uint64_t t_start = ctl->t_begin;  // of the budget (k_h1_flow)
+    uint64_t t_mode = global_timer_ns();  // start of the current mode (thread 0 of CTA 0)
     uint32_t pgen = 0;           // wake-ups of the parked CTAs so far
     __shared__ uint32_t sh_wake[3];
     uint32_t nchg = min(ctl->nl, b.mcap);  // round 0: every column that left its star

@@ -252,6 +252,7 @@ struct H1Ctl {
     uint32_t rounds;              // reduction rounds run
     uint32_t stop[2];             // a round's merges hit an error (read one round later, by parity)
     uint32_t solo_round;          // the round from which the first CTA ran the rounds alone (0: never)
+    unsigned long long t_begin;   // device time at which the budget's clock started
     unsigned long long grown;     // pool entries taken by merged columns
     unsigned long long flow_grown;  // pool entries asked for by the star replacement (before them in the pool)
     unsigned long long t_grid_ns, t_solo_ns;  // wall time of the rounds on the whole grid / in one CTA
@@ -289,8 +290,9 @@ struct H1Bufs {
 // rounds, and appends the H1 pairs (zero persistence omitted) to pairs.
 cudaError_t launch_h1(const ItemTable& tab, const H1Bufs& b, Counters* ctr, cp_pair* pairs, uint32_t pair_cap,
                       cudaStream_t s);
-// Wall-clock budget of the cross-star rounds (one non-preemptible launch):
-// once it is spent, the rounds stop at the next round boundary and the call
+// Wall-clock budget of the star replacement and the cross-star rounds together
+// (non-preemptible launches): once it is spent, the replacement leaves the
+// columns as they are, the rounds stop at the next round boundary and the call
 // returns CP_ERR_TIMEOUT.
 void set_h1_budget_ms(int ms);
 int get_h1_budget_ms();
