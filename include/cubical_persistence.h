@@ -118,10 +118,10 @@ int cp_lut_num_classes(int ndim);
 int cp_lut_lookup(int ndim, uint32_t raw, uint32_t *relevant, uint64_t *entry);
 
 /*
- * Self-check of the 3D pruning kernel's mask form (host only, for tests):
- * the kernel builds the 26 neighbour comparisons into its own bit layout
- * and collapses them there with a few multiplications and masks (Sec. 3.3's
- * rule that an offset matters only when every nonzero sub-offset precedes).
+ * Self-check of the 3D lookup's mask form (host only, for tests): relevant
+ * masks are looked up in a bit layout of their own, in which a raw mask
+ * collapses with a few multiplications and masks (Sec. 3.3's rule that an
+ * offset matters only when every nonzero sub-offset precedes).
  * This runs that collapse on the host for all 2^26 raw masks and compares it
  * with the definition, and the pruning kernel's closed forms with the table
  * on all 15,935 classes; *n_mismatch receives the number of masks and
@@ -465,9 +465,11 @@ int cubical_persistence_uf_trace2(const void *d_workspace, int dual, uint32_t *h
  * capacity and dual root capacity.  Forest words with the top bit set are
  * roots (low bits: root id).  Survivor and root counts are the 2nd to 5th
  * uint32 of the counters.  With cap >= 13 a 13th value follows: the byte
- * offset of a uint32 counting the 3D pruning tasks whose image planes were
- * loaded by TMA (the others use cp.async).  Returns the number of values
- * written (12 or 13) or a CP_ERR_* code.
+ * offset of a uint32 that counts what of the volumes was loaded by TMA (the
+ * rest by cp.async), in blocks of 31 x 8 columns by the tuned planes
+ * (CP_TUNE_ZCHUNK_3D): a unit of its own, not the pruning pass's tiles.
+ * Offsets count from the first 256-byte boundary of the workspace.  Returns
+ * the number of values written (12 or 13) or a CP_ERR_* code.
  */
 int cubical_persistence_debug_prune(int n_items, const float *const *h_images, const int32_t *ndims,
                                     const int64_t *dims, void *d_workspace, size_t ws_bytes, int64_t max_survivors,

@@ -256,9 +256,9 @@ def persistence_batched(imgs: Sequence[torch.Tensor], max_survivors: int = 0, wi
 
 # Volumes beyond this many voxels (in all) need allow_large=True for H1: the
 # cross-star rounds grow with the area of the longest-lived loops, not with
-# the voxel count (smooth fields, one GB300: 0.11 s at 128^3, 0.84 s at
-# 256^3; at 512^3 the growing columns outran a 45 GB workspace).  The device
-# stops the rounds once cp_get_tuning(CP_TUNE_H1_BUDGET_MS) is spent, whatever
+# the voxel count (smooth fields, one GB300: 2.2 ms at 128^3, 7.7 ms at 256^3;
+# at 512^3, before the columns were rewritten ahead of the rounds, they outran a
+# 45 GB workspace).  The device stops the rounds once cp_get_tuning(CP_TUNE_H1_BUDGET_MS) is spent, whatever
 # the size.
 H1_PRACTICAL_VOXELS = 256 ** 3
 

@@ -3,11 +3,10 @@
 Picks the 3D task depth (planes per task) and the number of 3D pruning CTAs
 per SM by timing the lookup + pruning pass alone
 (cubical_persistence_prune_pass) on the given inputs; then the union-find
-design (reservation rounds over every survivor, or Borůvka's spanning forest
-first and the rounds over its edges) by timing whole forward calls with
-each.  Which design is faster depends on the data (i.i.d. noise leaves many
-survivors that close cycles, which Borůvka drops early; smooth fields leave
-few), so the cache key holds the survivor fraction's power of two besides
+design (the merge tree, or sorted survivors, Borůvka's spanning forest and
+reservation rounds over its edges) by timing whole forward calls with
+each.  What is fastest depends on the data (i.i.d. noise leaves many
+survivors, smooth fields few), so the cache key holds the survivor fraction's power of two besides
 the shape bucket.  It also holds a hash of the library's sources: what was
 fastest with other kernels says nothing about these, so a decision made for
 them is not applied but made again.  The winners are cached per GPU and key in a JSON file

@@ -101,7 +101,7 @@ struct Plan {
     int chunk_shift = 0;
     size_t o_count, o_chunk, o_start, zero_bytes;
     size_t o_node0, o_nodet;  // merge-tree nodes
-    size_t o_code;            // link codes of the 3D items
+    size_t o_code;            // link codes
     uint64_t n_code = 0;
     // H1 of the volumes (calls that ask for it): see H1Bufs
     bool h1 = false;

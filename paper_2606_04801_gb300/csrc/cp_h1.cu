@@ -795,8 +795,10 @@ __device__ void add_winner_warp(const ReduceArgs& a, uint32_t q, uint32_t r, uin
 // the largest first keeps an entry from being replaced twice.)  An entry
 // without owner is final once nothing larger is pending.
 //
-// What bounds it: latency.  A batch is three dependent L2 reads, a sort of up to
-// 128 keys and a merge, and a column takes some 100 batches.  Whole-diagram
+// What bounds it: issue (54% of the slots at 128^3, DRAM 3%): a batch sorts up
+// to 128 keys and merges entries one by one, after three dependent L2 reads, and
+// a column takes some 100 batches; few columns (small volumes, the second
+// launch) are bound by those reads' latency.  Whole-diagram
 // forward with the rounds alone (each addition of a star column a round of its
 // own) and with this first:
 //   128^3 sigma 2 (10,223 columns)   84 -> 2.4 ms (5,650 -> 97 rounds)

@@ -13,14 +13,14 @@ namespace cp {
 // older root `parent` by survivors of key at most `key`.  One 32-byte sector.
 struct alignas(32) TreeNode {
     uint64_t key;     // ~0: connected with nothing older yet
-    uint64_t parent;  // root id
+    uint64_t parent;  // its root id, and the upper half of its age << 32
     uint64_t age;     // smaller is older (the dual's age keys complemented)
     uint64_t item;    // index of its item in the call's table
 };
 struct PruneOuts {
-    uint32_t* uf0;   // H0 forest over global vertices (3D items: root words only)
-    uint32_t* uft;   // dual forest over global top cells (+ one outside vertex per item; 3D: root words only)
-    uint8_t* code;   // 3D items: both links of each vertex (cp_walk.cuh)
+    uint32_t* uf0;   // H0 roots' words, over global vertices
+    uint32_t* uft;   // dual roots' words, over global top cells (+ one outside vertex per item)
+    uint8_t* code;   // both links of each vertex (cp_walk.cuh)
     uint64_t n_code;
     uint64_t* s0;    // H0 survivor keys
     uint64_t* st;    // dual survivor keys (complemented: ascending sort = descending order)
@@ -34,7 +34,6 @@ struct PruneOuts {
     Counters* ctr;
     uint32_t n_uf0, n_uft;  // forest sizes (for the bounds-checked build)
 };
-size_t prune_smem2d();
 size_t prune_smem3d();
 int prune_tile_x();
 int prune_tile_x3d();
@@ -56,7 +55,7 @@ struct TmaMaps {
 // Encodes the plane map of a D x H x W float volume; false if it cannot be used.
 bool encode_plane_map(CUtensorMap* map, const float* img, int64_t D, int64_t H, int64_t W);
 cudaError_t launch_prune(const ItemTable& tab, const PruneOuts& po, const TmaMaps& maps, cudaStream_t s);
-// The 3D items' forests as words, from their codes (stage tests).
+// The forests as words, from their codes (stage tests).
 cudaError_t launch_expand(const ItemTable& tab, const PruneOuts& po, cudaStream_t s);
 
 // ---- K2 radix sort (LSD, 8-bit digits, decoupled look-back)
@@ -86,7 +85,7 @@ struct UfParams {
     const uint32_t* d_nkeys;
     uint32_t cap_keys;
     uint32_t* uf;
-    const uint8_t* code = nullptr;  // 3D items' links (cp_walk.cuh)
+    const uint8_t* code = nullptr;  // links (cp_walk.cuh)
     uint64_t n_code = 0;
     const uint64_t* age;
     uint64_t* res;
@@ -119,7 +118,7 @@ struct RootArgs {
     const uint32_t* d_n;
     uint32_t cap;
     const uint32_t* uf;
-    const uint8_t* code;         // 3D items' links (cp_walk.cuh)
+    const uint8_t* code;         // links (cp_walk.cuh)
     uint64_t n_code;
     int dual;
     uint32_t* ra;                // root id of each survivor's endpoints, by unsorted position
@@ -223,7 +222,7 @@ struct BoruvkaArgs {
     Counters* ctr;
 };
 cudaError_t launch_boruvka(const BoruvkaArgs& a, cudaStream_t s);
-int uf_variant();  // 0: reservation rounds over every survivor; 1: Borůvka, then rounds over its forest
+int uf_variant();  // 0: the merge tree; 1: Borůvka, then reservation rounds over its forest
 
 // Entries of SlabArgs::vcnt for a scratch capacity.
 uint32_t slab_vblocks_cap(uint32_t cap);

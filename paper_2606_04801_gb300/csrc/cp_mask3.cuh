@@ -1,7 +1,8 @@
-// Device form of the 3D lower-neighbour mask (Sec. 3.3): the bit layout the
-// pruning kernel builds its 26 comparisons into, and the collapse to the
-// relevant mask in that layout.  Host code uses the same functions to hash
-// the lookup table's keys and to check the layout against the definition.
+// Device form of the 3D lower-neighbour mask (Sec. 3.3): the bit layout of the
+// relevant masks that the pruning kernel looks up (it takes them from words of
+// 32 vertices, cp_words3.cuh) and that the table's hash is made for, and the
+// collapse of a raw mask in that layout, which host code compares with the
+// definition.
 //
 // The canonical numbering of a neighbour at offset (dz, dy, dx) is
 // n = 9(dz+1) + 3(dy+1) + (dx+1).  The device layout places the bits on a

@@ -27,7 +27,8 @@ namespace cp {
 
 // Lookup tables in global memory, read through the read-only cache (lanes of
 // a warp look up different entries, which constant memory would serialise).
-__device__ uint2 g_lut2d[256];  // same two-word entry layout as the 3D table
+// 2D: direct (3 bits) | h0_surv << 3 (6) | dual_surv << 9 (12) of each mask.
+__device__ uint32_t g_lut2d[256];
 // 3D: the perfect hash of the relevant masks (bucket -> displacement -> slot),
 // and per slot h0_surv | dual_surv << 6, read for event vertices only (the
 // links come from closed forms, cp_words3.cuh).
@@ -853,7 +854,7 @@ __global__ void __launch_bounds__(kW2 * 32) k_prune2d(const __grid_constant__ It
             uint32_t raw = 0;
 #pragma unroll
             for (int k = 0; k < 8; ++k) raw |= ((n[k][l] >> row) & 1u) << k;
-            const uint32_t en = __ldg(&g_lut2d[raw].x);
+            const uint32_t en = __ldg(g_lut2d + raw);
             const uint32_t h0 = (en >> 3) & 15u, dual = (en >> 9) & 15u;
             const uint32_t r0 = (en & 7u) == 7u ? 1u : 0u, rt = raw == 255u ? 1u : 0u;
             queue[e] = q | h0 << 10 | dual << 14 | r0 << 18 | rt << 19;
@@ -976,7 +977,7 @@ int set_tuning(int key, int value) {
             if (value != 0 && value != 1) return -1;
             g_cross2d = value;
             return 0;
-        case 7:  // union-find design: reservation rounds (0) or Borůvka's forest first (1)
+        case 7:  // union-find design: the merge tree (0) or Borůvka's forest and rounds over it (1)
             if (value != 0 && value != 1) return -1;
             g_uf_variant = value;
             return 0;
@@ -994,22 +995,11 @@ int get_tuning(int key) {
                       : -1;
 }
 
-// Table entry as two 32-bit words:
-//   x: direct (3 bits) | h0_surv << 3 (6) | dual_surv << 9 (12) | in_l << 21 (8)
-//   y: the eight 4-bit dual codes
-static uint2 pack_entry(uint64_t v) {
-    const uint32_t direct = uint32_t(v & 7u), h0s = uint32_t((v >> 3) & 0x3Fu);
-    const uint32_t ds = uint32_t((v >> 41) & 0xFFFu), in_l = uint32_t((v >> 53) & 0xFFu);
-    uint2 r;
-    r.x = direct | (h0s << 3) | (ds << 9) | (in_l << 21);
-    r.y = uint32_t((v >> 9) & 0xFFFFFFFFu);
-    return r;
-}
-
 cudaError_t upload_luts(const uint64_t* lut2d, const uint16_t* disp3d, const uint64_t* entries3d,
                         const uint32_t* keys3d) {
-    uint2 p2[256];
-    for (int i = 0; i < 256; ++i) p2[i] = pack_entry(lut2d[i]);
+    uint32_t p2[256];
+    for (int i = 0; i < 256; ++i)
+        p2[i] = uint32_t(lut2d[i] & 0x1FFu) | uint32_t((lut2d[i] >> 41) & 0xFFFu) << 9;
     cudaError_t e = cudaMemcpyToSymbol(g_lut2d, p2, sizeof(p2));
     if (e != cudaSuccess) return e;
     e = cudaMemcpyToSymbol(g_disp3d, disp3d, sizeof(uint16_t) * (1 << 12));

@@ -618,7 +618,7 @@ cudaError_t launch_roots(const RootArgs& r, cudaStream_t s) {
 }
 
 cudaError_t launch_roots2(const RootArgs& r0, const RootArgs& r1, cudaStream_t s) {
-    // (find_ctr is zero: the call's own memset, and no other walk before this)
+    // (find_ctr is zero: k_init, and no other walk before this)
     // (overlapped for small images only: in place of the 2D pass's shared memory
     // the walks want L1; 2048^2 noise 139 us overlapped, 89 not)
     const auto kernel = r0.tab.n3d == 0 ? k_roots2<2> : (r0.tab.n2d == 0 ? k_roots2<3> : k_roots2<0>);
