@@ -89,9 +89,9 @@ class BatchedPersistence:
         # plain float tensors on the device go in one launch, the rest by copy_:
         # host or other types, strided, recorded by autograd (by forward mode: any
         # in its scope), parts of this batch; all of a batch made in inference
-        # mode, which copy_ refuses outside it.  Those on the device may read
-        # items of this batch that come before them in the list, so what waits is
-        # copied first
+        # mode, which copy_ refuses outside it; tensors without memory (zero
+        # tensors).  Those on the device may read items of this batch that come
+        # before them in the list, so what waits is copied first
         counts = [0] * self.k
         ptrs = [0] * self.k
         plain = forward_ad._current_level < 0 and (torch.is_inference_mode_enabled() or not self.x.is_inference())
@@ -101,7 +101,7 @@ class BatchedPersistence:
             if (plain and type(a) is torch.Tensor and a.dtype is torch.float32 and a.device == dev and a.numel() == n
                     and a.is_contiguous() and not a.requires_grad and not a.is_neg()):
                 p = a.data_ptr()
-                if p & 3 == 0 and (p >= hi or p + 4 * n <= lo):
+                if p and p & 3 == 0 and (p >= hi or p + 4 * n <= lo):
                     counts[i], ptrs[i] = n, p
                     continue
             a = torch.as_tensor(a)

@@ -107,3 +107,13 @@ def test_autograd_sees_a_load_as_it_sees_a_copy():
         assert torch.equal(bi.x, torch.cat([v.reshape(-1) for v in xs]))
     with pytest.raises(RuntimeError):
         bi.load([one(), one()])
+
+
+def test_a_tensor_without_memory_is_zeros():
+    import paper_2606_04801_gb300 as cp
+
+    bp = cp.BatchedPersistence([(5, 6)] * 2)
+    xs = [torch.rand(5, 6).cuda() for _ in range(2)]
+    bp.load(xs)
+    bp.load([torch._efficientzerotensor((5, 6), device="cuda"), xs[1]])
+    assert not bp.views[0].any() and torch.equal(bp.views[1], xs[1])
