@@ -108,22 +108,25 @@ __global__ void __launch_bounds__(kTT) k_t_flatten(uint8_t* __restrict__ code, c
         return d.ndim == 3 ? code_at3(j, int(z), int(y), int(x)) : code_at2(j, int(y), int(x));
     };
     const uint8_t frame = d.ndim == 3 ? 7u : 15u;
-    // whole frame rows, one block per row: both y faces of every plane, and
-    // the two z faces (3D)
-    const int64_t zf = d.ndim == 3 ? 2 * Hj : 0;  // rows of the two z faces
-    const int64_t nrows = zf + 2 * (d.ndim == 3 ? Dj - 2 : 1);
-    for (int64_t f = blockIdx.x; f < nrows; f += gridDim.x) {
+    // whole frame rows, a thread per vertex (a long row takes the whole grid: with
+    // a block per row the two rows of a 1 x 2^21 image took 3 ms): both y faces of
+    // every plane, and the two z faces (3D)
+    const uint32_t zf = d.ndim == 3 ? uint32_t(2 * Hj) : 0u;  // rows of the two z faces
+    const uint32_t frame_rows = zf + 2u * (d.ndim == 3 ? uint32_t(Dj - 2) : 1u);
+    const uint32_t n_frame = frame_rows * uint32_t(Wj);  // (J has at most 2^27 vertices)
+    for (uint32_t k = blockIdx.x * kTT + threadIdx.x; k < n_frame; k += gridDim.x * kTT) {
+        const uint32_t f = k / uint32_t(Wj);
+        const int64_t x = k - f * uint32_t(Wj);
         int64_t z, y;
         if (f < zf) {
-            z = f < Hj ? 0 : Dj - 1;
-            y = f % Hj;
+            z = f < uint32_t(Hj) ? 0 : Dj - 1;
+            y = f % uint32_t(Hj);
         } else {
-            const int64_t g = f - zf;
+            const uint32_t g = f - zf;
             z = d.ndim == 3 ? 1 + g / 2 : 0;
             y = (g & 1) ? Hj - 1 : 0;
         }
-        for (int64_t x = threadIdx.x; x < Wj; x += kTT)
-            if (z != 0 || y != 0 || x != 0) cd[code_at(z, y, x)] |= frame;
+        if (z != 0 || y != 0 || x != 0) cd[code_at(z, y, x)] |= frame;
     }
     // the two x faces of the other rows
     const int64_t zi = d.ndim == 3 ? Dj - 2 : 1, yi = Hj - 2;
