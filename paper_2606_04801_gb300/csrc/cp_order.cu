@@ -76,7 +76,7 @@ __device__ __forceinline__ uint64_t place_of(const OrderArgs& a, const cp_pair& 
     return a.base[p.item] + uint64_t(c) * a.cells[p.item] + uint32_t(p.birth_cell);
 }
 
-// The number of pairs to the caller (thread 0 of the grid), or none (any CTA
+// The number of pairs to the caller (one thread of the grid), or none (any CTA
 // that gives up): a CTA that gives up flags the call before it writes 0, and
 // the number is taken back if the flag shows after it, so a failed call never
 // reports pairs.
@@ -233,6 +233,14 @@ __global__ void __launch_bounds__(kOT) k_order(const __grid_constant__ OrderArgs
             __stcg(a.sorted + at, make_uint2(uint32_t(place & ((uint64_t(1) << a.shift) - 1u)), i));
     }
     if (!order_barrier(a, epoch)) return;
+    // the count, by a thread that has a pair to place only if all have
+    if (gtid == gsize - 1u) {
+        put_count(a, int64_t(n));
+        __threadfence();
+        if (ld_acquire_u32(&ctr->status) & kStTimeout) put_count(a, 0);
+        if (int64_t(n) > a.out_cap) set_status(ctr, kStCapacity);
+        if (a.t_bad && *a.t_bad) set_status(ctr, kStNonfinite);
+    }
     // ---- each to its place: the bucket's start and its rank among the members
     for (uint32_t d = gtid; d < n; d += gsize) {
         const uint2 e = __ldcg(a.sorted + d);
@@ -259,13 +267,6 @@ __global__ void __launch_bounds__(kOT) k_order(const __grid_constant__ OrderArgs
                 o[4] = w.x, o[5] = w.y, o[6] = w.z, o[7] = w.w;
             }
         }
-    }
-    if (gtid == 0) {
-        put_count(a, int64_t(n));
-        __threadfence();
-        if (ld_acquire_u32(&ctr->status) & kStTimeout) put_count(a, 0);
-        if (int64_t(n) > a.out_cap) set_status(ctr, kStCapacity);
-        if (a.t_bad && *a.t_bad) set_status(ctr, kStNonfinite);
     }
 }
 
